@@ -106,9 +106,11 @@ const char* qb_last_error(void);
  * exact_momentum = 0, the exact (possibly negative) sum otherwise; sectors come
  * in the order N ascending, then P ascending.  Copies and validates the model (conservation,
  * Hermiticity), builds the combinatorial ranking tables and uploads them to the
- * current device, with two per-ket tables the space owns: the diagonal of H
- * (16 B per ket) and the occupation vector packed into 64 bits (8 B per ket),
- * plus a double-float copy of an observed state (16 B per ket).
+ * current device, with the tables the space owns: per ket the diagonal of H
+ * (16 B), the occupation vector packed into 64 bits (8 B), the ket weight and its
+ * inverse (8 B each) and the number of its last modes' filling (4 B), plus a
+ * double-float copy of an observed state (16 B per ket); and the ranking tables of
+ * the stages (a few bytes per ket).
  * Limits: 1 <= M <= QB_MAX_MODES; M * bits(n_max) <= 64; n_max <= 250;
  * the largest ket weight sqrt(n_max! / prod_m n_m!) over occupations of n_max
  * particles at most 2^160 (the RK4 stages hold psi / w(n) as fp32 pairs, with the
@@ -161,7 +163,9 @@ int qb_init_field_number(qb_space* space, const double* z, int n_tot, void* d_ps
 /* ---- time evolution (Eq. Schr; the per-sector parallel scheme of Sec. III B) */
 
 /* Bytes of device workspace qb_evolve / qb_evolve_batch need for `batch`
- * state vectors. */
+ * state vectors: 48 per ket and member, plus, for a coupling that is one real number
+ * per momentum class (a contact interaction), 16 for every entry of the annihilated
+ * vectors (at most M per ket, for one member). */
 int64_t qb_workspace_bytes(const qb_space* space, int batch);
 
 /* out = H psi for one state vector (d_out and d_psi distinct, device). */
@@ -192,13 +196,10 @@ int qb_space_set_resident_max(qb_space* space, int resident_max_kets);
 
 /* Execution tuning of the RK4 stages of qb_evolve, qb_evolve_plain and
  * qb_evolve_observe for one state vector (the per-sector parallel scheme of
- * Sec. III B, mapped onto thread blocks): the tile shape of the stage kernel, one of
- * QB_TILE_SHAPES compiled shapes given as (warps per thread block, kets per warp
- * tile, thread blocks per SM the register budget is planned for):
- *   0 (32, 64, 1) the default;  1 (16, 64, 2);  2 (24, 64, 1);  3 (12, 64, 3);
- *   4 (32, 128, 1).
- * A shape whose shared memory (the coupling tables plus the warps' tiles) does not
- * fit a thread block on the device runs as shape 3 (large tables, e.g. M = 16).
+ * Sec. III B, mapped onto thread blocks): the tile shape of the stage kernels, the
+ * warps per thread block, one of QB_TILE_SHAPES (a warp takes 32 kets at a time):
+ *   0: 32, the default;  1: 16;  2: 24;  3: 12;  4: 8.
+ * A small space runs with fewer, so that its kets spread over every SM.
  * Every ket sums its terms in the same order under every shape, so results are
  * bit-identical; only the time differs (the Python binding's Space.autotune times
  * them on the caller's workload).  QB_EINVAL outside [0, QB_TILE_SHAPES). */

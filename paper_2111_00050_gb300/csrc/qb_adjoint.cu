@@ -247,7 +247,8 @@ AdjointLayout adjoint_layout(const Space& s, int64_t steps, int ckpt_every, unsi
   L.tape = ckpt_every > 0 ? nullptr : reinterpret_cast<float4*>(take(4 * V * steps));
   L.psi = reinterpret_cast<double2*>(take(V));
   L.lam = reinterpret_cast<double2*>(take(V));
-  L.w1 = reinterpret_cast<float4*>(take(3 * L.n * 16));  // w1, w2, psif back to back
+  // w1, w2, psif back to back, then the vector of B_k f (factored couplings)
+  L.w1 = reinterpret_cast<float4*>(take(workspace_bytes(s, 1)));
   L.w2 = L.w1 ? L.w1 + L.n : nullptr;
   L.psif = L.w2 ? L.w2 + L.n : nullptr;
   L.v4 = reinterpret_cast<float4*>(take(V));
@@ -318,6 +319,8 @@ static int adjoint_impl(qb_space* space, const double* z, double scale, double d
     f.row0 = 0;
     f.row1 = n;
     f.status = status;
+    f.g = L.psif + n;
+    f.low1 = sp->t.fa_on ? sp->t.fa_low : 0;
     f.psi = L.psi;
     for (int64_t j = 0; j < steps; ++j) {
       f.psif = slot(j, 0);
@@ -398,6 +401,8 @@ static int adjoint_impl(qb_space* space, const double* z, double scale, double d
   a.row0 = 0;
   a.row1 = n;
   a.status = status;
+  a.g = L.psif + n;
+  a.low1 = sp->t.fa_on ? sp->t.fa_low : 0;
   auto set_z = [&](double zre) {
     a.zre = zre;
     const float h = (float)zre;

@@ -1,0 +1,501 @@
+// The hot kernel: one Horner RK4 stage of every sector (and every member of a
+// batched coupling sweep) in one launch, with the matrix-free sector H psi in
+// double-float arithmetic, in the weighted basis f = psi / w(n).
+//
+//   stage d (d = 4, 3, 2):  out = f + (-i dt/d) W^-1 H W v    (double-float out)
+//   stage 1:                psi = psi + (-i dt) H v, f = psi / w
+//                                                     (FP64 psi, plus its weighted copy)
+//
+// H is Eq. (Ham) restricted to sectors of fixed N and momentum (Sec. III B).  Per row
+// (ket n) the off-diagonal terms are the disjoint pairs {r, s} -> {p, q} of equal
+// momentum; in the weighted basis, w(n) = sqrt(N! / prod n_m!) up to a power of two
+// per N, the element of target n' = n - e_r - e_s + e_p + e_q is
+// G_{pq,rs} n_r (n_s - [r = s]): the ratio w(n') / w(n) cancels the creation square
+// roots and squares the annihilation ones.  G is the multiplicity-summed symmetrised
+// coupling; the diagonal is precomputed per ket.
+//
+// Ranking by blocks.  The kets of a sector that share the occupations of the first P
+// modes are consecutive; such a block is the list of fillings of the last M - P modes
+// with a given particle number and momentum (its class), the same list wherever that
+// class occurs.  A term sends every ket of a block into one target block, so that the
+// target's index in the state vector splits into
+//   base[block][term]   where the target block starts: one row of 32-bit indices per
+//                       block, written when the space is built, and
+//   map[term][filling]  where the changed filling stands in its class: 16-bit places,
+//                       written once, read in order by consecutive lanes.
+// A warp takes 32 consecutive kets, one per lane, and walks the annihilation pairs in
+// step: the pair, its couplings and (nearly always) the bases are the same for all
+// lanes, the map is read coalesced and the gathered targets are near-consecutive.
+#pragma once
+#include "qb_device.cuh"
+
+namespace qb {
+
+// What a stage launch computes besides (or instead of) its output vector:
+//   KIND_STAGE  the RK4 / adjoint stage alone (modes 0 to 3);
+//   KIND_BIL    with the adjoint's bilinears fused (modes 2, 3);
+//   KIND_DOT    <x|H|x> only (mode 4): Re(conj(psi_n) (H psi)_n) summed in FP64,
+//               with each off-diagonal term and its Hermitian reverse taken once
+//               (the partners of a pair that come after it, counted twice).
+enum { KIND_STAGE = 0, KIND_BIL = 1, KIND_DOT = 2 };
+
+extern __shared__ __align__(16) unsigned char blk_smem[];
+
+// words of occupation bytes, four modes a word
+template <int MT>
+__host__ __device__ constexpr int occ_words() {
+  return MT > 0 ? (MT + 3) / 4 : 4;
+}
+
+// 2^23 + n_m as a float, exactly: the byte becomes the last one of 2^23.  The mode is in
+// the low bits of m (three for two or three words, then m8 = mode >= 8; the bits above pick
+// bytes that are dropped).
+template <int NW>
+__device__ __forceinline__ float occ_float23(const uint32_t (&ob)[NW], uint32_t m, bool m8) {
+  uint32_t w;
+  if constexpr (NW == 2) w = __byte_perm(ob[0], ob[1], m);
+  if constexpr (NW == 3) w = __byte_perm(m8 ? ob[2] : ob[0], ob[1], m);
+  if constexpr (NW == 4) w = __byte_perm(m8 ? ob[2] : ob[0], m8 ? ob[3] : ob[1], m);
+  return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7650u));
+}
+template <int NW>
+__device__ __forceinline__ float occ_float(const uint32_t (&ob)[NW], int m) {
+  return occ_float23<NW>(ob, (uint32_t)(m & 7), m >= 8) - 8388608.0f;
+}
+
+// Occupation bytes of a packed occupation word
+template <int MT, int NW>
+__device__ __forceinline__ void unpack_occ(const Tables& t, uint64_t word, uint32_t (&ob)[NW]) {
+  constexpr int kMB = (MT > 0) ? MT : 16;
+#pragma unroll
+  for (int k = 0; k < NW; ++k) ob[k] = 0u;
+#pragma unroll
+  for (int m = 0; m < kMB; ++m) {
+    if (MT == 0 && m >= t.M) break;
+    ob[m >> 2] |= (uint32_t)occ_of(word, m, t.occ_bits) << (8 * (m & 3));
+  }
+}
+
+// Terms per record: KC partners of a pair (odd M, momentum mod M: every pair has
+// (M - 1) / 2), or groups of up to four partners (KC = 0).  Slots of a record: the
+// first four terms side by side (two for KC = 2), a fifth in an array of its own.
+template <int KC>
+struct Rec {
+  static constexpr int n = KC == 0 ? 4 : KC;
+  static constexpr int w = KC == 2 ? 2 : 4;
+  static_assert(KC >= 0 && KC <= 5 && KC != 1, "partners per pair");
+};
+
+template <int KC>
+struct MapRec {  // one filling's map entries of one record
+  uint2 a;
+  uint32_t b;
+};
+
+template <int KC>
+__device__ __forceinline__ MapRec<KC> load_map(const unsigned char* mp, const uint16_t* mp5) {
+  MapRec<KC> r;
+  r.b = 0u;
+  if constexpr (KC == 2) {
+    r.a = make_uint2(__ldg(reinterpret_cast<const uint32_t*>(mp)), 0u);
+  } else {
+    r.a = __ldg(reinterpret_cast<const uint2*>(mp));
+    if constexpr (KC == 5) r.b = __ldg(mp5);
+  }
+  return r;
+}
+
+template <int KC>
+struct BaseRec {  // a block's bases of one record
+  uint4 a;
+  uint32_t b;
+};
+template <int KC>
+__device__ __forceinline__ BaseRec<KC> load_base(const uint32_t* base, int rec, int nrec) {
+  BaseRec<KC> r;
+  r.b = 0u;
+  if constexpr (KC == 2) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(base) + rec);
+    r.a = make_uint4(v.x, v.y, 0u, 0u);
+  } else {
+    r.a = __ldg(reinterpret_cast<const uint4*>(base) + rec);
+    if constexpr (KC == 5) r.b = __ldg(base + 4 * nrec + rec);
+  }
+  return r;
+}
+
+// Everything of a ket's row that the epilogue needs, and the epilogue: forms the
+// stage's output (or the bilinears, or the <x|H|x> summand) from the off-diagonal sum.
+// WHOLE: acc is the whole two-body part (factored couplings), else its off-diagonal part.
+template <int MT, int B, int KIND, bool WHOLE, int NW>
+__device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a, int mode, int64_t gr, int64_t ri,
+                                               const dfc (&acc)[B], const uint32_t (&ob)[NW], dfl& bil_l, dfl* bil_w,
+                                               double& dot64) {
+  constexpr bool BIL = (KIND == KIND_BIL), DOT = (KIND == KIND_DOT);
+  constexpr int kMB = (MT > 0) ? MT : 16;
+  const int M = (MT > 0) ? MT : t.M;
+  const int64_t total = t.total;
+  const float4 dg4 = a.diag[gr];
+  const dfl zf{a.zf.x, a.zf.y};
+  // the ket weight where true values are formed
+  double2 wk = make_double2(1.0, 1.0);
+  if (BIL || DOT || mode == 1 || mode == 3) wk = make_double2(__ldg(t.wk + gr), __ldg(t.wi + gr));
+#pragma unroll
+  for (int b = 0; b < B; ++b) {
+    dfl acc_r, acc_i;
+    f2_unpack(acc[b].h, acc_r.h, acc_i.h);
+    f2_unpack(acc[b].l, acc_r.l, acc_i.l);
+    if (DOT) {  // each term stands for itself and its reverse (H Hermitian): twice the real part
+      acc_r = dfl{2.f * acc_r.h, 2.f * acc_r.l};
+      acc_i = dfl{2.f * acc_i.h, 2.f * acc_i.l};
+    }
+    const dfl sc{a.scale[b].x, a.scale[b].y};
+    const dfl dg = WHOLE ? dfl{dg4.x, dg4.y} : df_add(dfl{dg4.x, dg4.y}, df_mul(sc, dfl{dg4.z, dg4.w}));
+    const float4 xo = a.vin[(size_t)b * total + ri];
+    const dfl hr = df_add(df_mul(dg, df_re(xo)), df_mul(sc, acc_r));
+    const dfl hi = df_add(df_mul(dg, df_im(xo)), df_mul(sc, acc_i));
+    if (DOT) {
+      // <x|H|x>: Re(conj(psi_n) (H psi)_n) = w^2 Re(conj(f_n) (W^-1 H W f)_n), w^2 in
+      // FP64 (w^2 alone may leave the fp32 range); no output
+      const dfl val = df_add(df_mul(df_re(xo), hr), df_mul(df_im(xo), hi));
+      dot64 += df_to(val) * wk.x * wk.x;
+      continue;
+    }
+    if (BIL && b == 0) {
+      // H_L x (two-body part at scale 1) and the pair vector of this row, as true
+      // values: each factor times w (w^2 alone may leave the fp32 range)
+      const float4 pp = a.pair[ri];
+      const dfl wd = df_of(wk.x);
+      const dfl dl{dg4.z, dg4.w};
+      const dfl lr = df_mul(wd, WHOLE ? acc_r : df_add(df_mul(dl, df_re(xo)), acc_r));
+      const dfl li = df_mul(wd, WHOLE ? acc_i : df_add(df_mul(dl, df_im(xo)), acc_i));
+      const dfl pr = df_mul(wd, df_re(pp)), pi = df_mul(wd, df_im(pp));
+      const dfl xr = df_mul(wd, df_re(xo)), xi = df_mul(wd, df_im(xo));
+      // Im(conj(p) h) = p.re h.im - p.im h.re
+      bil_l = df_add(bil_l, df_add(df_mul(pr, li), df_neg(df_mul(pi, lr))));
+      // Im(conj(x) p) = x.re p.im - x.im p.re, weighted by each occupation
+      const dfl tx = df_add(df_mul(xr, pi), df_neg(df_mul(xi, pr)));
+#pragma unroll
+      for (int q = 0; q < kMB; ++q) {
+        if (q >= M) break;
+        bil_w[q] = df_add(bil_w[q], df_mul(dfl{occ_float<NW>(ob, q), 0.f}, tx));
+      }
+    }
+    if (mode == 0 || mode == 2) {
+      dfl orr = df_mul(zf, hi), oi = df_neg(df_mul(zf, hr));  // z H x with z = -i zre
+      if (mode == 0) {
+        const float4 p0 = a.psif[(size_t)b * total + ri];
+        orr = df_add(df_re(p0), orr);
+        oi = df_add(df_im(p0), oi);
+      }
+      a.out[(size_t)b * total + ri] = df_pack(orr, oi);
+    } else {  // modes 1 and 3: back to the FP64 vector, one weight per ket
+      double sr = a.zre * df_to(hi), si = -a.zre * df_to(hr);
+      if (mode == 3) {
+        for (int k = 0; k < a.nbasef; ++k) {
+          const float4 e = a.basef[k][(size_t)b * total + ri];
+          sr += df_to(df_re(e));
+          si += df_to(df_im(e));
+        }
+      }
+      const double2 p0 = a.psi[(size_t)b * total + ri];
+      const double nr = p0.x + wk.x * sr, ni = p0.y + wk.x * si;
+      a.psi[(size_t)b * total + ri] = make_double2(nr, ni);
+      a.out[(size_t)b * total + ri] = df_pack(df_of(nr * wk.y), df_of(ni * wk.y));
+    }
+  }
+}
+
+// The kets of one warp round: 32 consecutive ones, lane by lane.  Fillings of different
+// classes are numbered with a gap, so that a ket belongs to the block of the ket before it
+// exactly when its filling follows that one's; the block of a round's first ket is stored.
+struct RoundIn {
+  uint64_t word;   // packed occupations
+  uint32_t fill;   // number of the filling
+  uint32_t first;  // block of lane 0
+};
+__device__ __forceinline__ RoundIn load_round(const uint64_t* occ, const uint32_t* fill, const uint32_t* rblk, int64_t r,
+                                              int64_t n, int lane) {
+  RoundIn in;
+  const int64_t g = min(r * 32 + lane, n - 1);
+  in.word = __ldg(occ + g);
+  in.fill = __ldg(fill + g);
+  in.first = __ldg(rblk + r);
+  return in;
+}
+__device__ __forceinline__ uint32_t block_of_lane(const RoundIn& in, int lane, bool inside) {
+  const uint32_t prev = __shfl_up_sync(0xffffffffu, in.fill, 1);
+  const uint32_t heads = __ballot_sync(0xffffffffu, inside && lane > 0 && in.fill != prev + 1u);
+  return in.first + __popc(heads & (0xffffffffu >> (31 - lane)));
+}
+
+// Threads a CTA's registers are planned for (65,536 registers per SM): the one-state
+// stages at 64 a thread, the wider ones (bilinear accumulators, sweep members) at 128.
+template <int B, int KIND>
+__host__ __device__ constexpr int blk_max_threads() {
+  return (B == 1 && KIND != KIND_BIL) ? 1024 : 512;
+}
+
+// per-CTA sums of the bilinears in a fixed order: lanes by shuffles, warps in turn
+template <int kMB>
+__device__ __forceinline__ void bil_reduce(const DfArgs& a, int M, const dfl& bil_l, const dfl* bil_w) {
+  __shared__ double red[16][17];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int nq = M + 1;
+  for (int q = 0; q < nq; ++q) {
+    double val = (q == 0) ? df_to(bil_l) : 0.0;
+#pragma unroll
+    for (int u = 0; u < kMB; ++u)
+      if (q == u + 1) val = df_to(bil_w[u]);
+    for (int o = 16; o > 0; o >>= 1) val += __shfl_down_sync(0xffffffffu, val, o);
+    if (lane == 0) red[warp][q] = val;
+  }
+  __syncthreads();
+  if (threadIdx.x < nq) {
+    double sum = 0.0;
+    for (int w = 0; w < warps; ++w) sum += red[w][threadIdx.x];
+    a.partial[(size_t)blockIdx.x * nq + threadIdx.x] = sum;
+  }
+}
+
+// Shared memory: couplings (real, imaginary) of the slots and the record words
+inline size_t blk_smem_bytes(const Tables& t, bool cplx) {
+  return (size_t)t.bk_T * 8 * (cplx ? 2 : 1) + (((size_t)t.bk_nrec * 8 + 15) & ~(size_t)15);
+}
+
+template <int MT, bool FIX, int B, bool CPLX, int KIND>
+__global__ void __launch_bounds__((blk_max_threads<B, KIND>()), 1)
+    blk_stage_kernel(const Tables t, const DfArgs a, const int mode) {
+  constexpr int KC = FIX ? (MT - 1) / 2 : 0;
+  constexpr int NT = Rec<KC>::n, RW = Rec<KC>::w, NW = occ_words<MT>();
+  constexpr bool BIL = (KIND == KIND_BIL), DOT = (KIND == KIND_DOT);
+  constexpr int kMB = (MT > 0) ? MT : 16;
+  const int M = (MT > 0) ? MT : t.M;
+  const int T = t.bk_T, nrec = t.bk_nrec;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+
+  float2* sG = reinterpret_cast<float2*>(blk_smem);
+  float2* sGi = sG + T;
+  uint2* sinfo = reinterpret_cast<uint2*>(sG + (CPLX ? 2 : 1) * T);
+  for (int i = threadIdx.x; i < T; i += blockDim.x) {
+    sG[i] = __ldg(t.bk_G + i);
+    if (CPLX) sGi[i] = __ldg(t.bk_Gi + i);
+  }
+  for (int i = threadIdx.x; i < nrec; i += blockDim.x) sinfo[i] = __ldg(t.bk_info + i);
+  __syncthreads();  // the only CTA-wide barrier: warps run independently afterwards
+
+  const int64_t total = t.total;
+  dfl bil_l{0.f, 0.f};
+  dfl bil_w[BIL ? kMB : 1];
+#pragma unroll
+  for (int q = 0; q < (BIL ? kMB : 1); ++q) bil_w[q] = dfl{0.f, 0.f};
+  double dot64 = 0.0;
+
+  // the last rounds (the most particles, the most pairs per ket) first
+  const int64_t r0 = a.row0 / 32, step = (int64_t)gridDim.x * warps;
+  int64_t rd = (a.row1 - 1) / 32 - ((int64_t)blockIdx.x * warps + warp);
+  RoundIn next = load_round(t.occ, t.fill, t.rblk, max(rd, r0), total, lane);
+  for (; rd >= r0; rd -= step) {
+      const int64_t g = rd * 32 + lane;
+      const bool valid = g >= a.row0 && g < a.row1;
+      const RoundIn in = next;
+      next = load_round(t.occ, t.fill, t.rblk, max(rd - step, r0), total, lane);
+      const uint32_t* base = t.bk_base + (size_t)block_of_lane(in, lane, g < total) * T;
+      uint32_t ob[NW];
+      unpack_occ<MT, NW>(t, valid ? in.word : 0ull, ob);  // an invalid lane: no pair acts
+      const unsigned char* mp = t.bk_map + (size_t)in.fill * (2 * RW);
+      const uint16_t* mp5 = t.bk_map5 + in.fill;
+
+      dfc acc[B];  // (re, im) of the off-diagonal sum, double-float, packed
+#pragma unroll
+      for (int b = 0; b < B; ++b) acc[b] = dfc{0ull, 0ull};
+      bool bad = false;  // a target fell outside the state
+
+      // ---- the annihilation pairs (r <= s) in step; the next record's map in flight.  A
+      // lane that lacks the pair has the coefficient 0 and keeps its last gathered values.
+      float4 x[NT];
+#pragma unroll
+      for (int c = 0; c < NT; ++c) x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+      MapRec<KC> mcur = load_map<KC>(mp, mp5);
+      BaseRec<KC> bcur = load_base<KC>(base, 0, nrec);
+      for (int rec = 0; rec < nrec; ++rec) {
+        if (rec + 1 < nrec) {
+          mp += (size_t)t.bk_S * (2 * RW);
+          if (KC == 5) mp5 += t.bk_S;
+        }
+        const MapRec<KC> mnext = load_map<KC>(mp, mp5);
+        const BaseRec<KC> bnext = load_base<KC>(base, min(rec + 1, nrec - 1), nrec);
+        const uint2 info = sinfo[rec];
+        const float Af = (occ_float23<NW>(ob, info.x, (info.x & 0x8000u) != 0u) - 8388608.0f) *
+                         (occ_float23<NW>(ob, info.x >> 16, (info.x & 0x80000000u) != 0u) - __uint_as_float(info.y));
+        const bool act = Af != 0.f;
+        if (__any_sync(0xffffffffu, act)) {
+          const int n = KC == 0 ? (int)((info.x >> 4) & 7) : NT;
+          const int c_first = DOT ? (int)((info.x >> 8) & 7) : 0;
+          uint32_t rk[NT];
+          rk[0] = bcur.a.x + (mcur.a.x & 0xffffu);
+          rk[1] = bcur.a.y + (mcur.a.x >> 16);
+          if constexpr (NT > 2) rk[2] = bcur.a.z + (mcur.a.y & 0xffffu);
+          if constexpr (NT > 3) rk[3] = bcur.a.w + (mcur.a.y >> 16);
+          if constexpr (NT > 4) rk[4] = bcur.b + mcur.b;
+          if constexpr (KC == 0) {
+#pragma unroll
+            for (int c = 1; c < NT; ++c)
+              if (c >= n) rk[c] = rk[0];  // unused slots
+          }
+          uint32_t top = rk[0];
+#pragma unroll
+          for (int c = 1; c < NT; ++c) top = max(top, rk[c]);
+          const bool ok = act && top < (uint32_t)total;
+          bad |= act && !ok;
+#pragma unroll
+          for (int b = 0; b < B; ++b) {
+#pragma unroll
+            for (int c = 0; c < NT; ++c)
+              if (ok && (KC > 0 || c < n) && (!DOT || c >= c_first)) x[c] = __ldg(a.vin + (size_t)b * total + rk[c]);
+#pragma unroll
+            for (int c = 0; c < NT; ++c) {
+              if ((KC == 0 && c >= n) || (DOT && c < c_first)) continue;  // the same for all lanes
+              const int sl = c < 4 ? RW * rec + c : 4 * nrec + rec;
+              const float2 g2 = sG[sl];
+              const dfl cr = df_mul_f(dfl{g2.x, g2.y}, Af);
+              const f2 xh = f2_pack(x[c].x, x[c].y), xl = f2_pack(x[c].z, x[c].w);
+              dfc_fma(acc[b], f2_pack(cr.h, cr.h), f2_pack(-cr.h, -cr.h), f2_pack(cr.l, cr.l), xh, xl);
+              if (CPLX) {
+                // + (-c_i x_im, c_i x_re): lanes of x swapped, coefficient (-c_i, c_i)
+                const float2 gi = sGi[sl];
+                const dfl ci = df_mul_f(dfl{gi.x, gi.y}, Af);
+                dfc_fma(acc[b], f2_pack(-ci.h, ci.h), f2_pack(ci.h, -ci.h), f2_pack(-ci.l, ci.l),
+                        f2_pack(x[c].y, x[c].x), f2_pack(x[c].w, x[c].z));
+              }
+            }
+          }
+          // keep |lo| below an ulp of hi between pairs
+          if (KC > 0 || (info.x & 0x80u)) {
+#pragma unroll
+            for (int b = 0; b < B; ++b) acc[b] = dfc_renorm(acc[b]);
+          }
+        }
+        mcur = mnext;
+        bcur = bnext;
+      }
+      if (bad) atomicOr(a.status, 1);
+      if (valid) stage_epilogue<MT, B, KIND, false, NW>(t, a, mode, g, g, acc, ob, bil_l, bil_w, dot64);
+  }
+
+  if constexpr (DOT) {
+    // the CTA's sum in a fixed order: lanes by shuffles, warps in turn; partial[block]
+    __shared__ double red[32];
+    for (int o = 16; o > 0; o >>= 1) dot64 += __shfl_down_sync(0xffffffffu, dot64, o);
+    if (lane == 0) red[warp] = dot64;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double sum = 0.0;
+      for (int w = 0; w < warps; ++w) sum += red[w];
+      a.partial[blockIdx.x] = sum;
+    }
+  }
+  if constexpr (BIL) bil_reduce<kMB>(a, M, bil_l, bil_w);
+}
+
+// Tile shapes: warps per CTA (a warp takes 32 kets at a time)
+constexpr int kTileShapes = 5;
+__host__ __device__ constexpr int tile_warps(int ts) { return ts == 1 ? 16 : ts == 2 ? 24 : ts == 3 ? 12 : ts == 4 ? 8 : 32; }
+
+// Warps per CTA and grid of a launch over `rows` kets.  While a small space leaves SMs
+// without work the CTA shrinks, so that its rounds spread over every SM.
+template <typename K>
+inline int stage_geometry(K k, int64_t rows, int shape, int max_warps, size_t smem, int* warps_out, int* grid) {
+  int per = 0, sms = 0, dev = 0;
+  QB_CUDA(cudaGetDevice(&dev));
+  QB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  int warps = std::min(tile_warps(shape), max_warps);
+  const int64_t rounds = rows / 32 + 2;  // unaligned ends: at most one more
+  while (warps > 2 && rounds <= (int64_t)sms * (warps / 2)) warps >>= 1;
+  const int rc = occupancy_cached(k, smem, &per, &sms, 32 * warps);
+  if (rc) return rc;
+  *warps_out = warps;
+  *grid = (int)std::min<int64_t>((int64_t)sms * std::min(per, 16), (rounds + warps - 1) / warps);
+  return QB_OK;
+}
+
+// One stage over the rows [a.row0, a.row1).
+template <int MT, bool FIX, int B, bool CPLX, int KIND>
+int blk_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream_t st, int* grid_out) {
+  auto k = blk_stage_kernel<MT, FIX, B, CPLX, KIND>;
+  const size_t smem = blk_smem_bytes(t, CPLX);
+  int warps = 0, grid = 0;
+  const int rc = stage_geometry(k, a.row1 - a.row0, shape, blk_max_threads<B, KIND>() / 32, smem, &warps, &grid);
+  if (rc) return rc;
+  k<<<grid, 32 * warps, smem, st>>>(t, a, mode);
+  QB_CUDA(cudaGetLastError());
+  if (grid_out) *grid_out = grid;
+  return QB_OK;
+}
+
+// the kinds and batch sizes of one kernel family (real or complex couplings)
+template <int MT, bool FIX>
+int blk_launch_kind(const Tables& t, const DfArgs& a, int mode, int B, bool bil, int shape, cudaStream_t st, int* grid) {
+  if (mode < 0 || mode > 4) return fail(QB_EINTERNAL, "bad stage mode");
+  if (mode == 4) {
+    if (B != 1) return fail(QB_EUNSUPPORTED, "the <x|H|x> reduction runs one state at a time");
+    return blk_launch<MT, FIX, 1, false, KIND_DOT>(t, a, mode, shape, st, grid);
+  }
+  if (bil) {
+    if (B != 1) return fail(QB_EUNSUPPORTED, "bilinear stages run one state at a time");
+    return blk_launch<MT, FIX, 1, false, KIND_BIL>(t, a, mode, shape, st, grid);
+  }
+  if (B != 1 && t.exact) return fail(QB_EUNSUPPORTED, "exact momentum: batched sweeps are not built");
+  switch (B) {
+    case 1: return blk_launch<MT, FIX, 1, false, KIND_STAGE>(t, a, mode, shape, st, grid);
+    case 2: return blk_launch<MT, FIX, 2, false, KIND_STAGE>(t, a, mode, shape, st, grid);
+    case 4: return blk_launch<MT, FIX, 4, false, KIND_STAGE>(t, a, mode, shape, st, grid);
+    case 8: return blk_launch<MT, FIX, 8, false, KIND_STAGE>(t, a, mode, shape, st, grid);
+    default: return fail(QB_EINVAL, "batch must be 1, 2, 4 or 8");
+  }
+}
+
+// one translation unit each (qb_stage_m*.cu): the mode counts with a fixed partner count
+// (odd M, momentum mod M, real couplings), and everything else; and the factored stages
+int stage_launch_m5(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+int stage_launch_m7(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+int stage_launch_m9(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+int stage_launch_m11(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+int stage_launch_any(const Tables&, const DfArgs&, int, int, bool, bool, int, cudaStream_t, int*);
+int fac_launch_m5(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+int fac_launch_m7(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+int fac_launch_m9(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+int fac_launch_m11(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+int fac_launch_any(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
+
+// One stage over rows [a.row0, a.row1) in the weighted basis (factored spaces: the lower
+// kets [a.low0, a.low1) and a.g as well).  bil: the bilinear instantiations (adjoint modes
+// 2, 3); mode 4 is the <x|H|x> reduction (partial[block]; a factored space: its two-body
+// part); shape: tile shape (0: the default).
+inline int stage_launch(const Tables& t, const DfArgs& a, int mode, int B, bool cplx, cudaStream_t st,
+                        int* grid_out = nullptr, bool bil = false, int shape = 0) {
+  if (t.fa_on) {
+    if (t.fa_nt > 0) {
+      switch (t.M) {
+        case 5: return fac_launch_m5(t, a, mode, B, bil, shape, st, grid_out);
+        case 7: return fac_launch_m7(t, a, mode, B, bil, shape, st, grid_out);
+        case 9: return fac_launch_m9(t, a, mode, B, bil, shape, st, grid_out);
+        case 11: return fac_launch_m11(t, a, mode, B, bil, shape, st, grid_out);
+        default: break;
+      }
+    }
+    return fac_launch_any(t, a, mode, B, bil, shape, st, grid_out);
+  }
+  if (t.bk_kc > 0 && !cplx) {
+    switch (t.M) {
+      case 5: return stage_launch_m5(t, a, mode, B, bil, shape, st, grid_out);
+      case 7: return stage_launch_m7(t, a, mode, B, bil, shape, st, grid_out);
+      case 9: return stage_launch_m9(t, a, mode, B, bil, shape, st, grid_out);
+      case 11: return stage_launch_m11(t, a, mode, B, bil, shape, st, grid_out);
+      default: break;
+    }
+  }
+  return stage_launch_any(t, a, mode, B, cplx, bil, shape, st, grid_out);
+}
+
+}  // namespace qb

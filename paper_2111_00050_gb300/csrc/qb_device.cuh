@@ -397,19 +397,21 @@ struct DfArgs {
   const float4* diag;  // per ket (w.hi, w.lo, L.hi, L.lo)
   float2 scale[8];     // two-body scale per member, double-float
   int64_t row0, row1;  // kets [row0, row1) of the launch (every sector: 0, total)
+  float4* g;           // factored couplings: B_k of the gathered vector(s), [B][fa_nG]
+  int64_t low0, low1;  // and the lower kets [low0, low1) that the launch fills (every one: 0, fa_low)
   double zre;          // z = -i zre
   float2 zf;           // zre as double-float
   int* status;
 };
 
 // Resident CTAs per SM of `kernel` with `smem` dynamic shared memory, cached
-// per (kernel, smem) so that launch loops do not repeat the occupancy query.
+// per (kernel, smem, block) so that launch loops do not repeat the occupancy query.
 template <typename K>
 static int occupancy_cached(K kernel, size_t smem, int* per_sm, int* sms, int block = kBlock) {
   struct Entry {
     const void* fn;
     size_t smem;
-    int dev, per, sms;
+    int block, dev, per, sms;
   };
   static thread_local Entry cache[64];
   static thread_local int used = 0;
@@ -417,7 +419,7 @@ static int occupancy_cached(K kernel, size_t smem, int* per_sm, int* sms, int bl
   QB_CUDA(cudaGetDevice(&dev));
   const void* fn = reinterpret_cast<const void*>(kernel);
   for (int i = 0; i < used; ++i)
-    if (cache[i].fn == fn && cache[i].smem == smem && cache[i].dev == dev) {
+    if (cache[i].fn == fn && cache[i].smem == smem && cache[i].block == block && cache[i].dev == dev) {
       *per_sm = cache[i].per;
       *sms = cache[i].sms;
       return QB_OK;
@@ -435,7 +437,7 @@ static int occupancy_cached(K kernel, size_t smem, int* per_sm, int* sms, int bl
                                optin - (int)fa.sharedSizeBytes));
   QB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, block, smem));
   if (per < 1) return fail(QB_EUNSUPPORTED, "kernel does not fit on an SM with this table size");
-  Entry e{fn, smem, dev, per, s};
+  Entry e{fn, smem, block, dev, per, s};
   cache[used < 64 ? used++ : 63] = e;
   *per_sm = per;
   *sms = s;

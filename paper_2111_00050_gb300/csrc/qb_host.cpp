@@ -85,6 +85,262 @@ static int prepare_model(const qb_model* model, std::vector<double>& w, std::vec
   return QB_OK;
 }
 
+// The block tables of the stage kernel (Tables::bk_*), all but the maps, which the
+// device fills.  The suffix takes as many modes as keep the maps within kMapBytes and a
+// class within 16-bit places: longer blocks mean fewer rows of bases, while the maps are
+// read beside the gathers and should stay in L2.  One step of the M = 9, N = 27 long-range
+// space (23.5M kets) takes 22.8 ms with 6 MB, 21.5 with 24 and 21.8 with 80; of the M = 7,
+// n_tot = 16 contact space 24.3, 23.9 and 23.9.
+constexpr int64_t kMapBytes = 24ll << 20;
+
+static void build_block_tables(Space& sp, bool factored) {
+  Tables& t = sp.t;
+  const std::vector<int>&annR = sp.combos.annR, &annS = sp.combos.annS, &annStart = sp.combos.annStart;
+  const std::vector<uint32_t>& pq = sp.combos.pq;
+  const std::vector<double>& G = sp.combos.G;
+  const std::vector<std::vector<int>>& delta = sp.combos.delta;
+  const unsigned char(*pairidx)[16] = sp.combos.pairidx;
+  const int M = sp.M, nmax = sp.nmax, Q = sp.Q, twoQ = 2 * Q;
+  t.bk_kc = (M % 2 == 1 && M >= 5 && M <= 11 && !sp.exact && !t.is_complex) ? (M - 1) / 2 : 0;
+  const int w = t.bk_kc == 2 ? 2 : 4, per = t.bk_kc > 0 ? t.bk_kc : 4;
+  struct Record {
+    int pair, first, n;
+    bool last;
+  };
+  std::vector<Record> recs;
+  for (size_t a = 0; a < annR.size(); ++a)
+    for (int j = annStart[a]; j < annStart[a + 1]; j += per)
+      recs.push_back({(int)a, j, std::min(per, annStart[a + 1] - j), j + per >= annStart[a + 1]});
+  const int nrec = (int)recs.size();
+  t.bk_nrec = nrec;
+  t.bk_T = std::max(4, (nrec * (t.bk_kc == 5 ? 5 : w) + 3) & ~3);
+  const int TS = t.bk_T + 4;
+
+  auto CI = [&](int m, int n, int k) { return ((size_t)m * (nmax + 1) + n) * Q + k; };
+  // map bytes per filling (factored: the pairs added, four a group, and taken away)
+  const int64_t per_fill = factored ? 8 * ((M * (M + 1) / 2 + 3) / 4 + (sp.exact ? 2 * M : M) * ((M + 8) / 8))
+                                    : (int64_t)std::max(1, nrec) * (t.bk_kc == 5 ? 10 : 2 * w);
+  int P = M - 1;
+  for (int q = M - 1; q >= 0; --q) {
+    int64_t S = 0, big = 0;
+    for (int n = 0; n <= nmax; ++n)
+      for (int k = 0; k < Q; ++k) {
+        const int64_t c = (int64_t)sp.cnt[CI(q, n, k)];
+        S += c + 1;
+        big = std::max(big, c);
+      }
+    if (q < M - 1 && (big > 65535 || S * per_fill > kMapBytes)) break;
+    P = q;
+    t.bk_S = (int)S;
+  }
+  t.bk_P = P;
+
+  std::vector<uint32_t> info(2 * (size_t)std::max(1, nrec));
+  std::vector<float> Gr(2 * (size_t)t.bk_T, 0.f), Gi(2 * (size_t)t.bk_T, 0.f);
+  std::vector<int32_t> psh((size_t)M * TS, 0), EC((size_t)t.rem_w * twoQ, 0), cls(2 * (size_t)(nmax + 1) * Q);
+  for (int i = 0; i < nrec; ++i) {
+    const Record& R = recs[i];
+    int after = 0;  // first partner with a larger pair index (partners ascend)
+    for (int c = 0; c < R.n; ++c) {
+      const int j = R.first + c, sl = c < 4 ? w * i + c : 4 * nrec + i;
+      if ((int)pairidx[pq[j] & 0xff][(pq[j] >> 8) & 0xff] < R.pair) after = c + 1;
+      for (int k = 0; k < 2; ++k) {
+        float* g = (k ? Gi : Gr).data() + 2 * (size_t)sl;
+        g[0] = (float)G[2 * j + k];
+        g[1] = (float)(G[2 * j + k] - (double)g[0]);
+      }
+      for (int m = 1; m < M; ++m) psh[(size_t)m * TS + sl] = delta[j][m];
+    }
+    const uint32_t r = (uint32_t)annR[R.pair], q = (uint32_t)annS[R.pair];
+    info[2 * i] = (r & 7) | ((uint32_t)R.n << 4) | (R.last ? 0x80u : 0u) | ((uint32_t)after << 8) |
+                  (r >= 8 ? 0x8000u : 0u) | ((q & 7) << 16) | (q >= 8 ? 0x80000000u : 0u);
+    info[2 * i + 1] = r == q ? 0x4B000001u : 0x4B000000u;  // 2^23 + [r = s]
+  }
+  for (int rr = 0; rr < t.rem_w; ++rr)
+    for (int kk = 0; kk < twoQ; ++kk) {
+      const int rem = rr - 2;
+      int64_t v = 0;
+      if (P >= 1 && rem >= 1 && rem - 1 <= nmax) v = (int64_t)sp.cnt[CI(P - 1, rem - 1, modp(kk - (P - 1), Q))];
+      if (rem >= 0 && rem <= nmax) v += (int64_t)sp.cnt[CI(P, rem, kk % Q)];
+      EC[(size_t)rr * twoQ + kk] = (int32_t)v;
+    }
+  int32_t first = 0;
+  for (int n = 0; n <= nmax; ++n)
+    for (int k = 0; k < Q; ++k) {
+      const int32_t c = (int32_t)sp.cnt[CI(P, n, k)];
+      cls[2 * ((size_t)n * Q + k)] = first;
+      cls[2 * ((size_t)n * Q + k) + 1] = c;
+      first += c + 1;
+    }
+  auto put = [&](int k, const void* p, size_t bytes) {
+    sp.bk_off[k] = sp.bk.size();
+    sp.bk.insert(sp.bk.end(), (const unsigned char*)p, (const unsigned char*)p + bytes);
+    sp.bk.resize((sp.bk.size() + 255) & ~(size_t)255);
+  };
+  put(0, info.data(), 4 * info.size());
+  put(1, Gr.data(), 4 * Gr.size());
+  put(2, Gi.data(), 4 * Gi.size());
+  put(3, psh.data(), 4 * psh.size());
+  put(4, EC.data(), 4 * EC.size());
+  put(5, cls.data(), 4 * cls.size());
+  sp.bk_off[6] = sp.bk.size();
+  sp.bk_map_bytes = ((size_t)std::max(1, nrec) * t.bk_S * 2 * w + 255) & ~(size_t)255;
+}
+
+// Whether the two-body part factors into one operator per momentum class,
+// sum_k lam_k B_k^dag B_k (a contact interaction): every symmetrised coupling of a class
+// is the same real number.  Then builds the tables of the factored stages (Tables::fa_*)
+// and the list of lower sectors; called once the sectors are known.
+//
+// Where the line lies (one stage, direct against factored kernels): two launches cost 5 us
+// more than one, so small spaces stay direct (M = 7, 19,448 kets: 13.0 against 13.3 us;
+// 245,157: 39.8 against 29.6), and with three pairs a class (M = 5) or fewer the second pass
+// costs what the fewer terms save (2.3M kets: 144 against 159 us).
+constexpr int64_t kFactorMin = 32768;
+constexpr int kFactorMinM = 6;
+
+
+static bool build_factored(Space& sp) {
+  Tables& t = sp.t;
+  const int M = sp.M, nmax = sp.nmax, Q = sp.Q, twoQ = 2 * Q;
+  t.fa_on = 0;
+  if (M < kFactorMinM || sp.secOff.back() < kFactorMin || sp.secOff.back() >= (int64_t)kNoIndex) return false;
+  const int nc = sp.exact ? 2 * M - 1 : M;
+  std::vector<std::vector<std::pair<int, int>>> cls(nc);  // pairs p < q first, then p = q
+  for (int d = 0; d < 2; ++d)
+    for (int p = 0; p < M; ++p)
+      for (int q = d ? p : p + 1; q < (d ? p + 1 : M); ++q) cls[(p + q) % (sp.exact ? 2 * M : M)].push_back({p, q});
+  auto LS = [&](std::pair<int, int> a, std::pair<int, int> b) {
+    const size_t ix = (((size_t)a.first * M + a.second) * M + b.first) * M + b.second;
+    return cd(sp.Lsym[2 * ix], sp.Lsym[2 * ix + 1]);
+  };
+  std::vector<float> lam(2 * (size_t)nc);
+  for (int k = 0; k < nc; ++k) {
+    const cd l0 = LS(cls[k][0], cls[k][0]);
+    if (l0.imag() != 0.0) return false;
+    for (auto a : cls[k])
+      for (auto b : cls[k])
+        if (LS(a, b) != l0) return false;
+    lam[2 * k] = (float)l0.real();
+    lam[2 * k + 1] = (float)(l0.real() - (double)lam[2 * k]);
+  }
+  // lower sectors and the vector of B_k f
+  sp.lowN.clear();
+  sp.lowK.clear();
+  sp.lowOff.assign(1, 0);
+  std::vector<int32_t> lowof((size_t)(nmax + 1) * Q, -1);
+  std::vector<uint32_t> goff;
+  int64_t nG = 0;
+  for (int n = std::max(0, sp.nmin - 2); n + 2 <= nmax; ++n)
+    for (int k0 = 0; k0 < Q; ++k0) {
+      // within a layer in the order of the space's sectors (ascending label sum)
+      const int c = label_shift(M);
+      const int K = sp.exact ? k0 : modp((long long)k0 + (long long)c * n, Q);
+      const int64_t D = (int64_t)sp.cnt[((size_t)0 * (nmax + 1) + n) * Q + K];
+      if (D == 0) continue;
+      bool any = false;
+      std::vector<uint32_t> row(nc, kNoIndex);
+      for (int k = 0; k < nc; ++k) {
+        if (sp.secOf[(size_t)(n + 2) * Q + (K + k) % Q] < 0) continue;
+        if (sp.exact && K + k > (M - 1) * (n + 2)) continue;
+        if (nG + D >= (int64_t)kNoIndex) return false;
+        row[k] = (uint32_t)nG;
+        nG += D;
+        any = true;
+      }
+      if (!any) continue;
+      lowof[(size_t)n * Q + K] = (int32_t)sp.lowN.size();
+      sp.lowN.push_back(n);
+      sp.lowK.push_back(K);
+      sp.lowOff.push_back(sp.lowOff.back() + D);
+      goff.insert(goff.end(), row.begin(), row.end());
+    }
+  const int nlow = (int)sp.lowN.size();
+  if (nlow == 0) return false;
+  sp.low_held = nlow <= (int)sp.secN.size();
+  for (int i = 0; i < nlow && sp.low_held; ++i)
+    sp.low_held = sp.secN[i] == sp.lowN[i] && sp.secK[i] == sp.lowK[i] && sp.secOff[i] == sp.lowOff[i];
+
+  // annihilation records
+  const bool fix = M % 2 == 1 && !sp.exact;
+  t.fa_nt = fix && M >= 5 && M <= 11 ? (M + 1) / 2 : 0;
+  t.fa_pl = t.fa_nt > 4 ? 2 : 1;
+  const int per = t.fa_nt > 0 ? t.fa_nt : 4;
+  std::vector<uint32_t> rec;
+  std::vector<std::pair<int, int>> slot;  // pair of each annihilation slot (first < 0: unused)
+  std::vector<int32_t> ka;
+  for (int k = 0; k < nc; ++k) {
+    const int n = (int)cls[k].size();
+    int noff = 0;
+    while (noff < n && cls[k][noff].first != cls[k][noff].second) ++noff;
+    for (int j = 0; j < n; j += per) {
+      const int m = std::min(per, n - j);
+      const int dbl = noff > j && noff <= j + m ? noff - j : 7;
+      rec.push_back((uint32_t)k | ((uint32_t)m << 8) | ((uint32_t)(t.fa_nt ? 7 : dbl) << 12) |
+                    (j + per >= n ? 0x10000u : 0u));
+      rec.push_back(0u);
+      for (int c = 0; c < 4 * t.fa_pl; ++c) {
+        slot.push_back(c < m ? cls[k][j + c] : std::pair<int, int>(-1, -1));
+        ka.push_back(k);
+      }
+    }
+  }
+  t.fa_nrec = (int)rec.size() / 2;
+  t.fa_nc = nc;
+  // creation groups: the pairs r <= s in order
+  std::vector<std::pair<int, int>> cre;
+  for (int r = 0; r < M; ++r)
+    for (int s = r; s < M; ++s) cre.push_back({r, s});
+  while (cre.size() % 4) cre.push_back({-1, -1});
+  t.fa_ng = (int)cre.size() / 4;
+  const int Ta = fa_Ta(t), Tc = fa_Tc(t);
+  std::vector<int32_t> kc(Tc, 0), psa((size_t)M * Ta, 0), psc((size_t)M * Tc, 0);
+  std::vector<uint32_t> info(Tc, 0u);
+  std::vector<float> coef(2 * (size_t)Tc, 0.f);
+  auto shift = [&](std::pair<int, int> pr, int m, int sign) {
+    const int dc = (pr.first >= m) + (pr.second >= m);
+    const int dk = (pr.first >= m ? pr.first : 0) + (pr.second >= m ? pr.second : 0);
+    return sign * dc * twoQ + modp((long long)sign * dk, Q);
+  };
+  for (int i = 0; i < Ta; ++i)
+    for (int m = 0; m < M && slot[i].first >= 0; ++m) psa[(size_t)m * Ta + i] = shift(slot[i], m, 1);
+  for (int i = 0; i < Tc; ++i) {
+    if (cre[i].first < 0) continue;
+    const uint32_t r = (uint32_t)cre[i].first, q = (uint32_t)cre[i].second;
+    kc[i] = sp.exact ? (int)(r + q) : (int)((r + q) % M);
+    for (int m = 0; m < M; ++m) psc[(size_t)m * Tc + i] = shift(cre[i], m, -1);
+    info[i] = (r & 7) | (r >= 8 ? 0x8000u : 0u) | ((q & 7) << 16) | (q >= 8 ? 0x80000000u : 0u);
+    coef[2 * i] = r == q ? 8388609.f : 8388608.f;
+    coef[2 * i + 1] = r == q ? 1.f : 2.f;
+  }
+  sp.fa.clear();
+  int at = 0;
+  auto put = [&](const void* p, size_t bytes) {
+    sp.fa_off[at++] = sp.fa.size();
+    sp.fa.insert(sp.fa.end(), (const unsigned char*)p, (const unsigned char*)p + bytes);
+    sp.fa.resize((sp.fa.size() + 255) & ~(size_t)255);
+  };
+  put(rec.data(), 4 * rec.size());
+  put(lam.data(), 4 * lam.size());
+  put(ka.data(), 4 * ka.size());
+  put(kc.data(), 4 * kc.size());
+  put(psa.data(), 4 * psa.size());
+  put(psc.data(), 4 * psc.size());
+  put(info.data(), 4 * info.size());
+  put(coef.data(), 4 * coef.size());
+  put(lowof.data(), 4 * lowof.size());
+  put(sp.lowOff.data(), 8 * sp.lowOff.size());
+  put(goff.data(), 4 * goff.size());
+  put(sp.lowN.data(), 4 * sp.lowN.size());
+  put(sp.lowK.data(), 4 * sp.lowK.size());
+  sp.fa_off[13] = sp.fa.size();
+  t.fa_nlow = nlow;
+  t.fa_low = sp.lowOff.back();
+  t.fa_nG = nG;
+  t.fa_on = 1;
+  return true;
+}
+
 // Builds the fill counts, ranking table, coupling combinations and the
 // shared-memory image of the space.
 static int build_tables(Space& sp) {
@@ -124,17 +380,18 @@ static int build_tables(Space& sp) {
     size_t ix = (((size_t)p * M + q) * M + r) * M + s;
     return cd(sp.Lsym[2 * ix], sp.Lsym[2 * ix + 1]);
   };
-  std::vector<int> annR, annS, annStart;
-  std::vector<uint32_t> pq;
-  std::vector<double> G;
-  std::vector<std::vector<int>> delta;  // [combo][16]
+  sp.combos = Combos();
+  std::vector<int>&annR = sp.combos.annR, &annS = sp.combos.annS, &annStart = sp.combos.annStart;
+  std::vector<uint32_t>& pq = sp.combos.pq;
+  std::vector<double>& G = sp.combos.G;
+  std::vector<std::vector<int>>& delta = sp.combos.delta;
   std::vector<std::vector<int>> dex;    // [combo][16] shifts of the compact exact index
   // exact momentum: width of mode m's window of suffix momenta, (M-1-m) nmax + 1
   int exw[16] = {0};
   for (int m = 1; m < M; ++m) exw[m] = (M - 1 - m) * nmax + 1;
   std::vector<double> gd;
-  unsigned char pairidx[16][16];
-  memset(pairidx, 0xff, sizeof(pairidx));
+  unsigned char(*pairidx)[16] = sp.combos.pairidx;
+  memset(pairidx, 0xff, 256);
   bool cplx = false;
   for (int r = 0; r < M; ++r)
     for (int s = r; s < M; ++s) {
@@ -182,6 +439,7 @@ static int build_tables(Space& sp) {
   annStart.push_back((int)pq.size());
   t.n_combo = (int)pq.size();
   t.is_complex = cplx ? 1 : 0;
+
 
   // shared-memory image: the stage kernels' tables first after the ranking table
   // (ann .. dsw), so that they stage [E, delta) (mod M) or [ann, sqrt) (exact)
@@ -587,6 +845,8 @@ int qb_sector_build(const qb_model* model, int n_min, int n_max, const int* p_li
     delete sp;
     return fail(QB_EINVAL, "no non-empty sector in the requested range");
   }
+  build_block_tables(*sp, build_factored(*sp));
+  sp->fa_off[14] = sp->fa_off[13] + (((size_t)sp->t.fa_nrec * sp->t.fa_pl * sp->t.bk_S * 8 + 255) & ~(size_t)255);
   rc = device_setup(*sp);
   if (rc) {
     qb_space_free(reinterpret_cast<qb_space*>(sp));
@@ -610,6 +870,14 @@ void qb_space_free(qb_space* space) {
   cudaFree(sp->d_wtab);
   cudaFree(sp->d_occ);
   cudaFree(sp->d_wi);
+  cudaFree(sp->d_bk);
+  cudaFree(sp->d_fa);
+  cudaFree(sp->d_fill);
+  cudaFree(sp->d_low);
+  for (int k = 0; k < 2; ++k) {
+    cudaFree(sp->d_blocks[k]);
+    cudaFree(sp->d_base[k]);
+  }
   if (sp->capture_stream) cudaStreamDestroy(sp->capture_stream);
   if (sp->side_stream) cudaStreamDestroy(sp->side_stream);
   if (sp->ev_fork) cudaEventDestroy(sp->ev_fork);

@@ -15,6 +15,9 @@ namespace qb {
 // (a shift lies in [-4M, 5M) for M <= 16).
 constexpr int kDeltaBias = 64;
 
+// 32-bit indices of kets and of entries of B_k f stay below this
+constexpr uint32_t kNoIndex = 0xffff0000u;
+
 // Everything a kernel needs to walk one space, passed by value.
 //
 // Ranking of a ket n within its sector (N, K), K = sum_i i n_i mod M (mode
@@ -93,6 +96,75 @@ struct Tables {
   int occ_bits;
   const uint64_t* occ;  // [total]
   const double* wi;     // [total] 1 / w(n) of every ket (the centred ket weight; ket_weight)
+  const double* wk;     // [total] w(n)
+  // Block tables of the stage kernel (qb_block.cuh).  A block is the run of kets of a
+  // sector that share the occupations of modes 0 .. P-1; its class (rem, kr) is the
+  // particle number and index momentum of the other modes, whose fillings are numbered
+  // class by class (rem, then kr; lexicographic within a class), S in all.  The terms are
+  // grouped into records: one annihilation pair with its bk_kc partners, or (bk_kc = 0)
+  // with up to four of them.
+  int bk_kc;                // partners per pair where that is fixed (2 to 5), else 0
+  int bk_P;                 // modes of the block prefix
+  int bk_S;                 // fillings of the modes bk_P .. M-1 with up to nmax particles, and one number
+                            //   left out after each class
+  const uint32_t* fill;     // [total] number of the filling of every ket
+  int bk_nrec;              // records
+  int bk_T;                 // term slots (a multiple of 4): record i holds [w i, w i + w), w = 2 for
+                            //   bk_kc = 2, else 4; a fifth partner sits at 4 n_rec + i
+  const uint32_t* rblk;     // [ceil(total / 32)] block of every 32nd ket
+  const uint32_t* bk_base;  // [blocks][T] index in the state of the first ket of each slot's target block
+  const uint2* bk_info;     // [n_rec] x: r mod 8 | terms << 4 | last record of its pair << 7 | first partner after
+                            //   the pair << 8 | (r >= 8) << 15 | s mod 8 << 16 | (s >= 8) << 31; y: the float
+                            //   2^23 + [r = s]
+  const float2* bk_G;       // [T] real coupling (hi, lo); bk_Gi: imaginary
+  const float2* bk_Gi;
+  const int32_t* bk_psh;    // [M][T + 4] shift of the suffix index at mode m (a term conserves N and K: 0 for m = 0; 0 for unused slots)
+  const int32_t* bk_EC;     // [rem_w][2Q] ranking-table rows of mode P plus the size of the class
+  const int2* bk_cls;       // [nmax + 1][Q] (first filling, size) of each class
+  const unsigned char* bk_map;  // [n_rec][S] place of the changed filling in its class, w 16-bit entries
+  const uint16_t* bk_map5;      // [n_rec][S] of the fifth partner
+  // Factored couplings (qb_factor.cuh): H_2 = sum_k lam_k B_k^dag B_k, B_k the sum of a_p a_q
+  // over the ordered pairs of momentum class k (fa_on = 1).  B_k f lives on the lower kets, the
+  // kets of two particles fewer; its entries of every (lower sector, class) whose raised
+  // sector is held form one vector of fa_nG.  Annihilation records: a class with its pairs in
+  // fa_pl groups of four (odd M, momentum mod M: fa_nt pairs, the pair p = q last), or
+  // (fa_nt = 0) up to four pairs of a class.  Creation groups: four pairs (r, s) each.
+  int fa_on, fa_nt, fa_pl, fa_nrec, fa_nc, fa_ng;
+  int fa_nlow;                 // lower sectors
+  int64_t fa_low;              // lower kets
+  int64_t fa_nG;
+  const uint2* fa_rec;         // [fa_nrec] x: class | pairs << 8 | double the sum before pair (0-4; 7: never) << 12 |
+                               //   last record of the class << 16
+  const float2* fa_lam;        // [fa_nc] lam_k (hi, lo)
+  const int32_t* fa_ka;        // [fa_Ta] class of each annihilation slot
+  const int32_t* fa_kc;        // [fa_Tc] class of each creation slot
+  const int32_t* fa_psa;       // [M][fa_Ta] shift of the suffix index when the slot's pair is added
+  const int32_t* fa_psc;       // [M][fa_Tc] when it is taken away
+  const uint4* fa_info;        // [fa_ng] mode selectors of four pairs, as bk_info's x
+  const float4* fa_coef;       // [2 fa_ng] (2^23 + [r = s], 2 - [r = s]; 0 for an unused slot) of two pairs each
+  const uint2* fa_mapa;        // [fa_nrec][fa_pl][S] places after adding the pairs
+  const uint2* fa_mapc;        // [fa_ng][S] places after taking the pairs away
+  const int32_t* fa_lowof;     // [nmax + 1][Q] lower sector of (N, K) or -1
+  const int64_t* fa_lowoff;    // [fa_nlow + 1]
+  const uint32_t* fa_goff;     // [fa_nlow][fa_nc] first entry of (lower sector, class), or kNoIndex
+  const uint64_t* fa_occ;      // [fa_low] packed occupations of the lower kets
+  const uint32_t* fa_fill;     // [fa_low] and the numbers of their fillings
+  const uint32_t* fa_rblk;     // [ceil(fa_low / 32)] block of every 32nd lower ket
+  const uint32_t* fa_basea;    // [lower blocks][fa_rowa] raised target blocks, then the classes' entries (qb_factor.cuh)
+  const uint32_t* fa_basec;    // [blocks][fa_Tc] index in the vector of B_k f of the lowered target blocks
+  const double* fa_wk;         // [fa_low] their ket weights, or NULL
+};
+__host__ __device__ inline int fa_rowa(const Tables& t) { return t.fa_nrec * t.fa_pl * 4 + ((t.fa_nc + 3) & ~3); }
+__host__ __device__ inline int fa_Ta(const Tables& t) { return t.fa_nrec * t.fa_pl * 4; }
+__host__ __device__ inline int fa_Tc(const Tables& t) { return t.fa_ng * 4; }
+
+// The (annihilation pair, creation pair) combinations of a space, pair by pair
+struct Combos {
+  std::vector<int> annR, annS, annStart;       // pairs (r <= s) and their first combos
+  std::vector<uint32_t> pq;                    // p | q << 8 | lo << 16 | hi << 24
+  std::vector<double> G;                       // coupling (re, im)
+  std::vector<std::vector<int>> delta;         // [16] shift of the suffix index at each mode
+  unsigned char pairidx[16][16];
 };
 
 struct Space {
@@ -107,6 +179,15 @@ struct Space {
   std::vector<uint64_t> cnt;              // host copy of the fill counts
   std::vector<int> secOf;                 // [(nmax+1) * Q]
   std::vector<unsigned char> blob;        // host copy of the shared-memory image
+  Combos combos;
+  std::vector<unsigned char> bk;          // block tables but the maps (image of d_bk's first bytes)
+  size_t bk_off[7] = {0};                 // byte offsets of info, G, Gi, psh, EC, cls and the maps in d_bk
+  std::vector<unsigned char> fa;          // tables of the factored couplings but the maps (image of d_fa's first bytes)
+  size_t fa_off[15] = {0};
+  std::vector<int> lowN, lowK;            // lower sectors
+  std::vector<int64_t> lowOff;
+  bool low_held = false;                  // the lower kets are the space's first kets
+  size_t bk_map_bytes = 0;
   int64_t maxDim = 0;
   // device allocations owned by the space
   unsigned char* d_blob = nullptr;
@@ -119,7 +200,13 @@ struct Space {
   float4* d_obsf = nullptr;     // double-float copy of the state being observed (qb_observables)
   double2* d_wtab = nullptr;    // ket-weight factors (Tables::wtab)
   uint64_t* d_occ = nullptr;    // packed occupation vectors (Tables::occ)
-  double* d_wi = nullptr;       // inverse ket weights (Tables::wi)
+  double* d_wi = nullptr;       // inverse ket weights and the weights (Tables::wi, wk)
+  unsigned char* d_bk = nullptr;  // block tables (Tables::bk_*)
+  unsigned char* d_fa = nullptr;  // tables of the factored couplings (Tables::fa_*)
+  uint32_t* d_fill = nullptr;     // fillings (Tables::fill)
+  unsigned char* d_low = nullptr; // occupations and fillings of the lower kets
+  uint32_t* d_blocks[2] = {nullptr, nullptr};  // rblk and the block starts of the kets, and of the lower kets
+  uint32_t* d_base[2] = {nullptr, nullptr};    // bases of the blocks, and of the lower blocks
   int64_t scratch_doubles = 0;
   Tables t{};
   cudaStream_t capture_stream = nullptr;  // private stream on which RK4 chunks are captured into graphs

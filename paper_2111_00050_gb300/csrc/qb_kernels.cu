@@ -17,6 +17,8 @@
 #include "qb_internal.h"
 
 #include "qb_device.cuh"
+#include "qb_block.cuh"
+#include "qb_factor.cuh"
 #include "qb_stage.cuh"
 
 namespace qb {
@@ -195,7 +197,46 @@ __global__ void __launch_bounds__(256) to_dfw_kernel(const Tables t, const doubl
 
 // per-ket diagonal of H, one-body and two-body parts, as double-float pairs; the
 // packed occupations and the inverse ket weight of every ket
-__global__ void __launch_bounds__(kBlock) diag_kernel(const Tables t, float4* diag, uint64_t* occ, double* wi) {
+// Number of the filling of the modes P .. M-1 of the row's ket (after setup_row)
+__device__ __forceinline__ uint32_t row_filling(const Tables& t, const View& v, const RowScratch& rs, int N, int K) {
+  const int tid = threadIdx.x, P = t.bk_P, twoQ = 2 * t.Q;
+  int cls = N * t.Q + K;  // P = 0: the whole ket
+  if (P > 0) {
+    const int flat = rs.idx[P * kBlock + tid] - (P * t.rem_w + 2) * twoQ;
+    cls = flat / twoQ * t.Q + flat % twoQ;
+  }
+  const int2 c = __ldg(t.bk_cls + cls);
+  return (uint32_t)(c.x + c.y - 1 - (rs.pe[(t.M - 1) * kBlock + tid] - rs.pe[P * kBlock + tid]));
+}
+
+// packed occupations and fillings of the lower kets of a factored space
+__global__ void __launch_bounds__(kBlock) lower_kernel(const Tables t, const int32_t* lowN, const int32_t* lowK,
+                                                        uint64_t* occ, uint32_t* fill) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  load_blob(t, smem);
+  const View v = make_view(t, smem);
+  const RowScratch rs = row_scratch(smem + blob_smem(t));
+  for (int64_t g = (int64_t)blockIdx.x * kBlock + threadIdx.x; g < t.fa_low; g += (int64_t)gridDim.x * kBlock) {
+    int lo = 0, hi = t.fa_nlow - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (__ldg(t.fa_lowoff + mid) <= g)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    const int64_t off = __ldg(t.fa_lowoff + lo);
+    const int N = __ldg(lowN + lo), K = __ldg(lowK + lo);
+    setup_row(t, v, rs, N, K, __ldg(t.fa_lowoff + lo + 1) - off, g - off);
+    uint64_t word = 0;
+    for (int m = 0; m < t.M; ++m) word |= (uint64_t)rs.occ[m * kBlock + threadIdx.x] << (m * t.occ_bits);
+    occ[g] = word;
+    fill[g] = row_filling(t, v, rs, N, K);
+  }
+}
+
+__global__ void __launch_bounds__(kBlock) diag_kernel(const Tables t, float4* diag, uint64_t* occ, double* wi,
+                                                        double* wk, uint32_t* fill) {
   extern __shared__ __align__(16) unsigned char smem[];
   load_blob(t, smem);
   const View v = make_view(t, smem);
@@ -207,7 +248,9 @@ __global__ void __launch_bounds__(kBlock) diag_kernel(const Tables t, float4* di
     const int sid = find_sector(t, g);
     const int64_t off = __ldg(t.sec_off + sid);
     const int64_t D = __ldg(t.sec_off + sid + 1) - off;
-    setup_row(t, v, rs, __ldg(t.sec_N + sid), __ldg(t.sec_K + sid), D, g - off);
+    const int N = __ldg(t.sec_N + sid), K = __ldg(t.sec_K + sid);
+    setup_row(t, v, rs, N, K, D, g - off);
+    fill[g] = row_filling(t, v, rs, N, K);
     double dw = 0.0, dl = 0.0;
     uint64_t word = 0;
     for (int r = 0; r < M; ++r) {
@@ -222,8 +265,309 @@ __global__ void __launch_bounds__(kBlock) diag_kernel(const Tables t, float4* di
     const dfl a = df_of(dw), b = df_of(dl);
     diag[g] = make_float4(a.h, a.l, b.h, b.l);
     occ[g] = word;
-    wi[g] = ket_weight<0>(t, rs.occ + tid, kBlock).y;
+    const double2 wt = ket_weight<0>(t, rs.occ + tid, kBlock);
+    wi[g] = wt.y;
+    wk[g] = wt.x;
   }
+}
+
+// A filling from its number: its class (particles crem, momentum ckr of the modes P ..
+// M-1), occupations and ranking-table indices.  False for the numbers left out.
+struct Filling {
+  int crem, ckr;
+  int occ[kMaxM], idx[kMaxM];
+};
+__device__ __forceinline__ bool filling_of(const Tables& t, int64_t f, Filling& F) {
+  const int M = t.M, Q = t.Q, P = t.bk_P, V = t.nmax + 1, twoQ = 2 * Q;
+  const uint32_t* cnt = reinterpret_cast<const uint32_t*>(t.blob + t.o_cnt);
+  int lo = 0, hi = V * Q - 1;  // the last class that starts at or before it
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (t.bk_cls[mid].x <= f)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  int64_t left = f - t.bk_cls[lo].x;
+  if (left >= t.bk_cls[lo].y) return false;
+  F.crem = lo / Q;
+  F.ckr = lo % Q;
+  int rem = F.crem, kr = F.ckr;
+  for (int m = 0; m < kMaxM; ++m) F.occ[m] = 0;
+  for (int m = P; m < M - 1; ++m) {  // lexicographic in (n_P, n_P+1, ...)
+    int val = 0;
+    while (val < rem) {
+      const int64_t c = cnt[((size_t)(m + 1) * V + rem - val) * Q + kr];
+      if (left < c) break;
+      left -= c;
+      ++val;
+      kr -= m;
+      while (kr < 0) kr += Q;
+    }
+    F.occ[m] = val;
+    rem -= val;
+  }
+  F.occ[M - 1] = rem;
+  int sr = 0, sk = 0;
+  for (int m = M - 1; m >= P; --m) {
+    sr += F.occ[m];
+    sk = (sk + m * F.occ[m]) % Q;
+    F.idx[m] = (m * t.rem_w + sr + 2) * twoQ + sk;
+  }
+  return true;
+}
+
+// Place in its class of the filling changed by the shifts sh[m * stride] of the suffix
+// indices; 0 outside the space
+__device__ __forceinline__ uint16_t place_of(const Tables& t, const Filling& F, const int32_t* sh, int stride) {
+  const int M = t.M, Q = t.Q, P = t.bk_P, twoQ = 2 * Q;
+  const int32_t* E = reinterpret_cast<const int32_t*>(t.blob + t.o_E);
+  const int flat = (F.crem + 2) * twoQ + F.ckr + sh[P * stride];
+  const int rr = flat / twoQ - 2, kk = (flat % twoQ) % Q;
+  if (rr < 0 || rr > t.nmax) return 0;
+  int place = t.bk_cls[rr * Q + kk].y - 1;
+  for (int m = P + 1; m < M; ++m) place -= E[F.idx[m] + sh[m * stride]];
+  return (uint16_t)(place < 0 || place > 65535 ? 0 : place);
+}
+
+// whether the filling supplies what the pair (r, s) takes from the modes P .. M-1
+__device__ __forceinline__ bool supplies(const Tables& t, const Filling& F, int r, int s) {
+  bool ok = r < t.bk_P || F.occ[r] >= (r == s ? 2 : 1);
+  return ok && (s < t.bk_P || r == s || F.occ[s] >= 1);
+}
+__device__ __forceinline__ int2 pair_of(uint32_t info) {  // the modes of a selector word
+  return make_int2((info & 7) | ((info >> 12) & 8), ((info >> 16) & 7) | ((info >> 28) & 8));
+}
+
+// Blocks.  A ket starts a block unless its filling follows the one before it.
+constexpr int kScanRounds = 2048;  // rounds of 32 kets per CTA of the block scan
+
+__device__ __forceinline__ uint32_t round_heads(const uint32_t* fill, int64_t r, int64_t n, int lane) {
+  const int64_t g = r * 32 + lane;
+  bool head = false;
+  if (g < n) head = g == 0 || __ldg(fill + g) != __ldg(fill + g - 1) + 1u;
+  return __ballot_sync(0xffffffffu, head);
+}
+
+// blocks that start in each run of kScanRounds rounds
+__global__ void __launch_bounds__(256) block_count_kernel(const uint32_t* fill, int64_t n, uint32_t* part) {
+  __shared__ uint32_t sum;
+  if (threadIdx.x == 0) sum = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int64_t r0 = (int64_t)blockIdx.x * kScanRounds, r1 = min(r0 + kScanRounds, (n + 31) / 32);
+  uint32_t c = 0;
+  for (int64_t r = r0 + (threadIdx.x >> 5); r < r1; r += 8) c += __popc(round_heads(fill, r, n, lane));
+  if (lane == 0) atomicAdd(&sum, c);
+  __syncthreads();
+  if (threadIdx.x == 0) part[blockIdx.x] = sum;
+}
+
+// part[i] = the blocks before run i; part[n] = all of them
+__global__ void __launch_bounds__(1024) block_scan_kernel(uint32_t* part, int n) {
+  __shared__ uint32_t s[1024];
+  __shared__ uint32_t carry;
+  if (threadIdx.x == 0) carry = 0;
+  for (int i0 = 0; i0 < n; i0 += 1024) {
+    const int i = i0 + threadIdx.x;
+    const uint32_t v = i < n ? part[i] : 0u;
+    s[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = 1; o < 1024; o <<= 1) {
+      const uint32_t x = threadIdx.x >= o ? s[threadIdx.x - o] : 0u;
+      __syncthreads();
+      s[threadIdx.x] += x;
+      __syncthreads();
+    }
+    const uint32_t before = carry + s[threadIdx.x] - v;
+    if (i < n) part[i] = before;
+    __syncthreads();
+    if (threadIdx.x == 1023) carry = before + v;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[n] = carry;
+}
+
+// rblk[r] = block of the first ket of round r; start[b] = first ket of block b
+__global__ void __launch_bounds__(256) block_start_kernel(const uint32_t* fill, int64_t n, const uint32_t* part,
+                                                           uint32_t* rblk, uint32_t* start) {
+  __shared__ uint32_t cnt[kScanRounds];
+  __shared__ uint32_t wsum[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t r0 = (int64_t)blockIdx.x * kScanRounds;
+  const int nr = (int)min((int64_t)kScanRounds, (n + 31) / 32 - r0);
+  for (int r = warp; r < nr; r += 8) {
+    const uint32_t h = round_heads(fill, r0 + r, n, lane);
+    if (lane == 0) cnt[r] = __popc(h);
+  }
+  __syncthreads();
+  // exclusive scan of cnt: 8 rounds a thread
+  uint32_t v[8], t = 0;
+  for (int k = 0; k < 8; ++k) {
+    const int r = threadIdx.x * 8 + k;
+    v[k] = r < nr ? cnt[r] : 0u;
+    t += v[k];
+  }
+  uint32_t x = t;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[warp] = x;
+  __syncthreads();
+  uint32_t run = part[blockIdx.x] + x - t;
+  for (int w = 0; w < warp; ++w) run += wsum[w];
+  for (int k = 0; k < 8; ++k) {
+    const int r = threadIdx.x * 8 + k;
+    if (r < nr) cnt[r] = run;
+    run += v[k];
+  }
+  __syncthreads();
+  for (int r = warp; r < nr; r += 8) {
+    const uint32_t h = round_heads(fill, r0 + r, n, lane);
+    if (lane == 0) rblk[r0 + r] = cnt[r] + (h & 1u) - 1u;
+    if ((h >> lane) & 1u) start[cnt[r] + __popc(h & ((1u << lane) - 1u))] = (uint32_t)((r0 + r) * 32 + lane);
+  }
+}
+
+// Suffix states of a block, lane m <= P holding mode m's: particles, momentum mod Q and the
+// ranking-table index (mode P: the row of bk_EC)
+struct BlockState {
+  int N, K, cls, my;
+};
+__device__ __forceinline__ BlockState block_state(const Tables& t, uint64_t word, int lane) {
+  int rem = 0, kr = 0;
+  for (int i = t.M - 1; i >= lane; --i) {
+    const int n = occ_of(word, i, t.occ_bits);
+    rem += n;
+    kr += i * n;
+  }
+  kr %= t.Q;
+  BlockState b;
+  b.N = __shfl_sync(0xffffffffu, rem, 0);
+  b.K = __shfl_sync(0xffffffffu, kr, 0);
+  b.cls = __shfl_sync(0xffffffffu, rem * t.Q + kr, t.bk_P);
+  b.my = ((lane < t.bk_P ? lane * t.rem_w : 0) + rem + 2) * 2 * t.Q + kr;
+  return b;
+}
+// sum of the ranking terms of modes 1 .. P of the block shifted by sh[m * stride], plus the
+// size of its class (all lanes take part; sh per lane)
+__device__ __forceinline__ uint32_t block_sum(const Tables& t, const BlockState& b, const int32_t* sh, int stride) {
+  const int32_t* E = reinterpret_cast<const int32_t*>(t.blob + t.o_E);
+  uint32_t sum = 0;
+  for (int m = 1; m < t.bk_P; ++m) sum += (uint32_t)__ldg(E + __shfl_sync(0xffffffffu, b.my, m) + (sh ? __ldg(sh + m * stride) : 0));
+  return sum + (uint32_t)__ldg(t.bk_EC + __shfl_sync(0xffffffffu, b.my, t.bk_P) + (sh ? __ldg(sh + t.bk_P * stride) : 0));
+}
+
+// Bases of the direct stage kernel, one warp a block; checks that the block starts where the
+// ranking says and with the first filling of its class.
+__global__ void __launch_bounds__(256) base_kernel(const Tables t, const uint32_t* start, int64_t nblocks, uint32_t* base,
+                                                    int* status) {
+  const int lane = threadIdx.x & 31, T = t.bk_T, TS = T + 4;
+  for (int64_t b = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5; b < nblocks; b += ((int64_t)gridDim.x * 256) >> 5) {
+    const int64_t g = start[b];
+    const BlockState s = block_state(t, __ldg(t.occ + g), lane);
+    const uint32_t end = (uint32_t)__ldg(t.sec_off + __ldg(t.sec_of + s.N * t.Q + s.K) + 1);
+    const uint32_t own = end - block_sum(t, s, nullptr, 0);
+    if (lane == 0 && (own != (uint32_t)g || __ldg(t.fill + g) != (uint32_t)__ldg(t.bk_cls + s.cls).x)) atomicOr(status, 2);
+    if (t.fa_on) continue;
+    for (int t0 = 0; t0 < T; t0 += 32) {
+      const int tt = min(t0 + lane, T - 1);
+      const uint32_t v = end - block_sum(t, s, t.bk_psh + tt, TS);
+      if (t0 + lane < T) base[(size_t)b * T + tt] = v;
+    }
+  }
+}
+
+// Bases of the factored stages: lowered targets of the blocks (basec), raised targets of
+// the lower blocks (basea) and where each class's entries start less the lower ket's number.
+__global__ void __launch_bounds__(256) lowered_base_kernel(const Tables t, const uint32_t* start, int64_t nblocks,
+                                                            uint32_t* basec) {
+  const int lane = threadIdx.x & 31, Tc = fa_Tc(t);
+  for (int64_t b = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5; b < nblocks; b += ((int64_t)gridDim.x * 256) >> 5) {
+    const BlockState s = block_state(t, __ldg(t.occ + start[b]), lane);
+    for (int t0 = 0; t0 < Tc; t0 += 32) {
+      const int tt = min(t0 + lane, Tc - 1);
+      const int k = __ldg(t.fa_kc + tt);
+      int kk = s.K - k;
+      while (kk < 0) kk += t.Q;
+      const uint32_t sum = block_sum(t, s, t.fa_psc + tt, Tc);
+      uint32_t v = kNoIndex;
+      if (s.N >= 2) {
+        const int lid = __ldg(t.fa_lowof + (s.N - 2) * t.Q + kk);
+        const uint32_t go = lid >= 0 ? __ldg(t.fa_goff + lid * t.fa_nc + k) : kNoIndex;
+        if (go != kNoIndex) v = go + (uint32_t)(__ldg(t.fa_lowoff + lid + 1) - __ldg(t.fa_lowoff + lid)) - sum;
+      }
+      if (t0 + lane < Tc) basec[(size_t)b * Tc + tt] = v;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) raised_base_kernel(const Tables t, const uint32_t* start, int64_t nblocks,
+                                                           uint32_t* basea) {
+  const int lane = threadIdx.x & 31, Ta = fa_Ta(t), row = fa_rowa(t);
+  for (int64_t b = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5; b < nblocks; b += ((int64_t)gridDim.x * 256) >> 5) {
+    const BlockState s = block_state(t, __ldg(t.fa_occ + start[b]), lane);
+    const int lid = __ldg(t.fa_lowof + s.N * t.Q + s.K);
+    for (int t0 = 0; t0 < Ta; t0 += 32) {
+      const int tt = min(t0 + lane, Ta - 1);
+      const int k = __ldg(t.fa_ka + tt);
+      const uint32_t sum = block_sum(t, s, t.fa_psa + tt, Ta);
+      uint32_t v = kNoIndex;
+      if (__ldg(t.fa_goff + lid * t.fa_nc + k) != kNoIndex)
+        v = (uint32_t)__ldg(t.sec_off + __ldg(t.sec_of + (s.N + 2) * t.Q + (s.K + k) % t.Q) + 1) - sum;
+      if (t0 + lane < Ta) basea[(size_t)b * row + tt] = v;
+    }
+    for (int k = lane; k < row - Ta; k += 32) {
+      uint32_t v = 0;
+      if (k < t.fa_nc) v = __ldg(t.fa_goff + lid * t.fa_nc + k) - (uint32_t)__ldg(t.fa_lowoff + lid);
+      basea[(size_t)b * row + Ta + k] = v;
+    }
+  }
+}
+
+// The maps of the direct stage kernel (Tables::bk_map): for every filling and every term,
+// the place of the changed filling in its class.  A thread takes one filling and the
+// records of its block row.
+__global__ void __launch_bounds__(kBlock) block_map_kernel(const Tables t, uint16_t* map, uint16_t* map5) {
+  const int64_t f = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+  Filling F;
+  if (f >= t.bk_S || !filling_of(t, f, F)) return;
+  const int w = t.bk_kc == 2 ? 2 : 4, TS = t.bk_T + 4;
+  for (int rec = blockIdx.y; rec < t.bk_nrec; rec += gridDim.y) {
+    const uint32_t info = t.bk_info[rec].x;
+    const int2 rs = pair_of(info);
+    const int n = (info >> 4) & 7;
+    const bool ok = supplies(t, F, rs.x, rs.y);
+    for (int c = 0; c < max(w, n); ++c) {
+      const int slot = c < 4 ? w * rec + c : 4 * t.bk_nrec + rec;
+      const uint16_t place = ok && c < n ? place_of(t, F, t.bk_psh + slot, TS) : 0;
+      if (c < w)
+        map[((size_t)rec * t.bk_S + f) * w + c] = place;
+      else
+        map5[(size_t)rec * t.bk_S + f] = place;
+    }
+  }
+}
+
+// The maps of the factored stages: places after a pair is added (fa_mapa) or taken away
+// (fa_mapc)
+__global__ void __launch_bounds__(kBlock) factor_map_kernel(const Tables t, uint16_t* mapa, uint16_t* mapc) {
+  const int64_t f = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+  Filling F;
+  if (f >= t.bk_S || !filling_of(t, f, F)) return;
+  const int Ta = fa_Ta(t), Tc = fa_Tc(t);
+  const uint32_t* info = reinterpret_cast<const uint32_t*>(t.fa_info);
+  for (int q = blockIdx.y; q < Ta / 4 + t.fa_ng; q += gridDim.y)
+    for (int c = 0; c < 4; ++c) {
+      if (q < Ta / 4) {
+        mapa[((size_t)q * t.bk_S + f) * 4 + c] = place_of(t, F, t.fa_psa + 4 * q + c, Ta);
+      } else {
+        const int i = 4 * (q - Ta / 4) + c;
+        const int2 rs = pair_of(info[i]);
+        mapc[((size_t)(q - Ta / 4) * t.bk_S + f) * 4 + c] = supplies(t, F, rs.x, rs.y) ? place_of(t, F, t.fa_psc + i, Tc) : 0;
+      }
+    }
 }
 
 // ------------------------------------------------------------- small kernels
@@ -557,6 +901,29 @@ int check_status(const Space& s, cudaStream_t st) {
   return QB_OK;
 }
 
+// Finds the blocks of n kets from their fillings: *d_out receives rblk [ceil(n / 32)] and,
+// from *start on, the first ket of each block.
+static int find_blocks(const uint32_t* fill, int64_t n, uint32_t** d_out, uint32_t** start, int64_t* nblocks) {
+  const int64_t nr = (n + 31) / 32;
+  const int np = (int)((nr + kScanRounds - 1) / kScanRounds);
+  uint32_t* part = nullptr;
+  QB_CUDA(cudaMalloc(&part, sizeof(uint32_t) * ((size_t)np + 1)));
+  block_count_kernel<<<np, 256>>>(fill, n, part);
+  block_scan_kernel<<<1, 1024>>>(part, np);
+  uint32_t total = 0;
+  cudaError_t e = cudaMemcpy(&total, part + np, sizeof(total), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMalloc(d_out, sizeof(uint32_t) * ((size_t)nr + total));
+  if (e == cudaSuccess) {
+    *start = *d_out + nr;
+    *nblocks = total;
+    block_start_kernel<<<np, 256>>>(fill, n, part, *d_out, *start);
+    e = cudaGetLastError();
+  }
+  cudaFree(part);  // waits for the kernels
+  QB_CUDA(e);
+  return QB_OK;
+}
+
 int device_setup(Space& s) {
   QB_CUDA(cudaGetDevice(&s.device));
   const size_t nsec = s.secN.size();
@@ -591,8 +958,9 @@ int device_setup(Space& s) {
   QB_CUDA(cudaMalloc(&s.d_diag, sizeof(float4) * (size_t)t.total));
   QB_CUDA(cudaMalloc(&s.d_obsf, sizeof(float4) * (size_t)t.total));
   QB_CUDA(cudaMalloc(&s.d_occ, sizeof(uint64_t) * (size_t)t.total));
-  QB_CUDA(cudaMalloc(&s.d_wi, sizeof(double) * (size_t)t.total));
+  QB_CUDA(cudaMalloc(&s.d_wi, 2 * sizeof(double) * (size_t)t.total));
   t.wi = s.d_wi;
+  t.wk = s.d_wi + t.total;
   t.occ_bits = 1;
   while ((1 << t.occ_bits) <= s.nmax) ++t.occ_bits;  // M * occ_bits <= 64 (checked by qb_sector_build)
   t.occ = s.d_occ;
@@ -629,20 +997,119 @@ int device_setup(Space& s) {
     t.wscale = s.d_wtab + (size_t)V * V;
   }
   {
+    const size_t five = t.bk_kc == 5 ? (size_t)t.bk_nrec * t.bk_S * 2 : 0;
+    QB_CUDA(cudaMalloc(&s.d_bk, s.bk_off[6] + (t.fa_on ? 0 : s.bk_map_bytes + five)));
+    QB_CUDA(cudaMemcpy(s.d_bk, s.bk.data(), s.bk.size(), cudaMemcpyHostToDevice));
+    t.bk_info = reinterpret_cast<const uint2*>(s.d_bk + s.bk_off[0]);
+    t.bk_G = reinterpret_cast<const float2*>(s.d_bk + s.bk_off[1]);
+    t.bk_Gi = reinterpret_cast<const float2*>(s.d_bk + s.bk_off[2]);
+    t.bk_psh = reinterpret_cast<const int32_t*>(s.d_bk + s.bk_off[3]);
+    t.bk_EC = reinterpret_cast<const int32_t*>(s.d_bk + s.bk_off[4]);
+    t.bk_cls = reinterpret_cast<const int2*>(s.d_bk + s.bk_off[5]);
+    t.bk_map = s.d_bk + s.bk_off[6];
+    t.bk_map5 = reinterpret_cast<const uint16_t*>(s.d_bk + s.bk_off[6] + s.bk_map_bytes);
+    QB_CUDA(cudaMalloc(&s.d_fill, sizeof(uint32_t) * (size_t)t.total));
+    t.fill = s.d_fill;
+  }
+  {
     const size_t smem = row_smem(t);
     int grid = 0;
     int rc = persistent_grid(diag_kernel, smem, t.total, &grid);
     if (rc) return rc;
-    diag_kernel<<<grid, kBlock, smem>>>(t, s.d_diag, s.d_occ, s.d_wi);
+    diag_kernel<<<grid, kBlock, smem>>>(t, s.d_diag, s.d_occ, s.d_wi, s.d_wi + t.total, s.d_fill);
     QB_CUDA(cudaGetLastError());
-    QB_CUDA(cudaDeviceSynchronize());
   }
+  uint32_t* start = nullptr;
+  int64_t nblocks = 0;
+  {
+    int rc = find_blocks(s.d_fill, t.total, &s.d_blocks[0], &start, &nblocks);
+    if (rc) return rc;
+    t.rblk = s.d_blocks[0];
+    const size_t T = t.fa_on ? (size_t)fa_Tc(t) : (size_t)t.bk_T;
+    QB_CUDA(cudaMalloc(&s.d_base[0], sizeof(uint32_t) * (size_t)nblocks * T));
+  }
+  const int base_grid = sms * 8;
+  base_kernel<<<base_grid, 256>>>(t, start, nblocks, s.d_base[0], reinterpret_cast<int*>(s.d_scratch));
+  QB_CUDA(cudaGetLastError());
+  if (!t.fa_on) {
+    t.bk_base = s.d_base[0];
+    if (t.bk_nrec > 0) {
+      const dim3 grid((unsigned)((t.bk_S + kBlock - 1) / kBlock), (unsigned)std::min(t.bk_nrec, 8));
+      block_map_kernel<<<grid, kBlock>>>(t, reinterpret_cast<uint16_t*>(s.d_bk + s.bk_off[6]),
+                                         const_cast<uint16_t*>(t.bk_map5));
+      QB_CUDA(cudaGetLastError());
+    }
+  } else {
+    const size_t total_bytes = s.fa_off[14] + (size_t)t.fa_ng * t.bk_S * 8;
+    QB_CUDA(cudaMalloc(&s.d_fa, total_bytes));
+    QB_CUDA(cudaMemcpy(s.d_fa, s.fa.data(), s.fa.size(), cudaMemcpyHostToDevice));
+    auto at = [&](int k) { return s.d_fa + s.fa_off[k]; };
+    t.fa_rec = reinterpret_cast<const uint2*>(at(0));
+    t.fa_lam = reinterpret_cast<const float2*>(at(1));
+    t.fa_ka = reinterpret_cast<const int32_t*>(at(2));
+    t.fa_kc = reinterpret_cast<const int32_t*>(at(3));
+    t.fa_psa = reinterpret_cast<const int32_t*>(at(4));
+    t.fa_psc = reinterpret_cast<const int32_t*>(at(5));
+    t.fa_info = reinterpret_cast<const uint4*>(at(6));
+    t.fa_coef = reinterpret_cast<const float4*>(at(7));
+    t.fa_lowof = reinterpret_cast<const int32_t*>(at(8));
+    t.fa_lowoff = reinterpret_cast<const int64_t*>(at(9));
+    t.fa_goff = reinterpret_cast<const uint32_t*>(at(10));
+    t.fa_basec = s.d_base[0];
+    t.fa_mapa = reinterpret_cast<const uint2*>(at(13));
+    t.fa_mapc = reinterpret_cast<const uint2*>(at(14));
+    uint32_t* lstart = start;
+    int64_t lblocks = nblocks;
+    if (s.low_held) {
+      t.fa_occ = s.d_occ;
+      t.fa_fill = s.d_fill;
+      t.fa_wk = t.wk;
+      t.fa_rblk = t.rblk;
+      // the lower kets' blocks are the first ones: up to the block of the ket after them
+      if (t.fa_low < t.total) {
+        const int64_t r = t.fa_low / 32;
+        uint32_t first = 0, f[32];
+        const int n = (int)(t.fa_low - 32 * r) + 1;
+        QB_CUDA(cudaMemcpy(&first, t.rblk + r, sizeof(first), cudaMemcpyDeviceToHost));
+        QB_CUDA(cudaMemcpy(f, s.d_fill + 32 * r, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
+        lblocks = first;
+        for (int k = 1; k < n; ++k) lblocks += f[k] != f[k - 1] + 1u;
+      }
+    } else {
+      QB_CUDA(cudaMalloc(&s.d_low, (size_t)t.fa_low * 12));
+      uint64_t* occ = reinterpret_cast<uint64_t*>(s.d_low);
+      uint32_t* fill = reinterpret_cast<uint32_t*>(occ + t.fa_low);
+      t.fa_occ = occ;
+      t.fa_fill = fill;
+      t.fa_wk = nullptr;
+      int grid = 0;
+      int rc = persistent_grid(lower_kernel, row_smem(t), t.fa_low, &grid);
+      if (rc) return rc;
+      lower_kernel<<<grid, kBlock, row_smem(t)>>>(t, reinterpret_cast<const int32_t*>(at(11)),
+                                                  reinterpret_cast<const int32_t*>(at(12)), occ, fill);
+      QB_CUDA(cudaGetLastError());
+      rc = find_blocks(fill, t.fa_low, &s.d_blocks[1], &lstart, &lblocks);
+      if (rc) return rc;
+      t.fa_rblk = s.d_blocks[1];
+    }
+    QB_CUDA(cudaMalloc(&s.d_base[1], sizeof(uint32_t) * (size_t)lblocks * fa_rowa(t)));
+    t.fa_basea = s.d_base[1];
+    lowered_base_kernel<<<base_grid, 256>>>(t, start, nblocks, s.d_base[0]);
+    raised_base_kernel<<<base_grid, 256>>>(t, lstart, lblocks, s.d_base[1]);
+    QB_CUDA(cudaGetLastError());
+    const dim3 grid((unsigned)((t.bk_S + kBlock - 1) / kBlock), (unsigned)std::min(fa_Ta(t) / 4 + t.fa_ng, 8));
+    factor_map_kernel<<<grid, kBlock>>>(t, reinterpret_cast<uint16_t*>(at(13)), reinterpret_cast<uint16_t*>(at(14)));
+    QB_CUDA(cudaGetLastError());
+  }
+  QB_CUDA(cudaDeviceSynchronize());
   return QB_OK;
 }
 
 // workspace: two double-float stage vectors and the double-float copy of psi,
-// each [batch][total] x 16 bytes
-int64_t workspace_bytes(const Space& s, int batch) { return 3 * (int64_t)batch * s.secOff.back() * 16; }
+// each [batch][total] x 16 bytes, and for factored couplings the vector of B_k f
+int64_t workspace_bytes(const Space& s, int batch) {
+  return 16 * (3 * (int64_t)batch * s.secOff.back() + (s.t.fa_on ? s.t.fa_nG : 0));
+}
 
 template <int MODE, int B, bool CPLX>
 static int launch_stage(const Space& s, const StageArgs& a, cudaStream_t st, int* grid_out = nullptr) {
@@ -685,6 +1152,16 @@ int launch_hpsi(const Space& s, const void* d_v, void* d_out, void* stream) {
 // the launches directly.
 constexpr int64_t kGraphSteps = 32;
 
+// lower kets whose entries a per-sector launch fills (factored couplings): the layer of two
+// particles fewer, before the first sector of its particle number
+static void lower_range(const Space& s, int sec, int64_t* low0, int64_t* low1) {
+  *low0 = *low1 = 0;
+  if (!s.t.fa_on || (sec > 0 && s.secN[sec] == s.secN[sec - 1])) return;
+  const auto r = std::equal_range(s.lowN.begin(), s.lowN.end(), s.secN[sec] - 2);
+  *low0 = s.lowOff[r.first - s.lowN.begin()];
+  *low1 = s.lowOff[r.second - s.lowN.begin()];
+}
+
 template <int B>
 static int rk4_issue(Space& s, DfArgs& a, double dt, int64_t steps, float4* w1, float4* w2, float4* psif,
                      cudaStream_t st, bool plain, int64_t row0 = 0) {
@@ -702,6 +1179,8 @@ static int rk4_issue(Space& s, DfArgs& a, double dt, int64_t steps, float4* w1, 
       const float zh = (float)a.zre;
       a.zf = make_float2(zh, (float)(a.zre - (double)zh));
       if (!plain) {
+        a.low0 = 0;
+        a.low1 = s.t.fa_on ? s.t.fa_low : 0;
         a.row0 = row0;
         a.row1 = s.t.total;
         int rc = stage_launch(s.t, a, d == 1 ? 1 : 0, B, cplx, st, nullptr, false, s.tile_shape);
@@ -710,6 +1189,7 @@ static int rk4_issue(Space& s, DfArgs& a, double dt, int64_t steps, float4* w1, 
         for (size_t sec = 0; sec + 1 < s.secOff.size(); ++sec) {
           a.row0 = s.secOff[sec];
           a.row1 = s.secOff[sec + 1];
+          lower_range(s, (int)sec, &a.low0, &a.low1);
           int rc = stage_launch(s.t, a, d == 1 ? 1 : 0, B, cplx, st, nullptr, false, s.tile_shape);
           if (rc) return rc;
         }
@@ -735,6 +1215,7 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
   a.diag = s.d_diag;
   a.psi = psi;
   a.psif = psif;
+  a.g = psif + (size_t)B * s.t.total;
   a.status = reinterpret_cast<int*>(s.d_scratch);
   a.nbasef = 0;
   if (plain) return rk4_issue<B>(s, a, dt, steps, w1, w2, psif, st, true);
@@ -742,7 +1223,7 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
   // stream, all steps in one launch, while the rest advances stage by stage.
   int64_t row0 = 0;
   bool forked = false;
-  if (B == 1) {
+  if (B == 1 && !s.t.fa_on) {
     int n_small = 0;
     const int nsec = (int)s.secDim.size();
     int optin = 0;

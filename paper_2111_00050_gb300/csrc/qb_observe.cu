@@ -857,6 +857,8 @@ int launch_moments(Space& s, const void* d_psi, double* out_host, void* stream) 
   a.scale[0] = make_float2(1.0f, 0.0f);
   a.row0 = 0;
   a.row1 = s.t.total;
+  a.low0 = 0;
+  a.low1 = s.t.fa_on ? s.t.fa_low : 0;
   a.status = reinterpret_cast<int*>(s.d_scratch);
   a.partial = dot_area(s);
   int g2 = 0;
@@ -889,6 +891,8 @@ int launch_moments(Space& s, const void* d_psi, double* out_host, void* stream) 
   for (int k = 0; k < nmom; ++k) out_host[k] = mom[k];
   out_host[0] = pre[0];
   out_host[1] = pre[1];
+  if (s.t.fa_on)  // the reduction holds the two-body part alone
+    for (int i = 0; i < M; ++i) h += s.w[i] * pre[2 + i];
   out_host[2] = h;
   out_host[3] = 0.0;
   const int oM = 4 + 2 * M;

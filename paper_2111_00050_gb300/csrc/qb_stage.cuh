@@ -1,18 +1,6 @@
-// The hot kernel: one Horner RK4 stage of every sector (and every member of a
-// batched coupling sweep) in one launch, with the matrix-free sector H psi in
-// double-float arithmetic, in the weighted basis f = psi / w(n).
-//
-//   stage d (d = 4, 3, 2):  out = f + (-i dt/d) W^-1 H W v    (double-float out)
-//   stage 1:                psi = psi + (-i dt) H v, f = psi / w
-//                                                     (FP64 psi, plus its weighted copy)
-//
-// H is Eq. (Ham) restricted to sectors of fixed N and momentum mod M (Sec. III B).
-// Per row (ket n) the off-diagonal terms are the disjoint pairs {r, s} -> {p, q}
-// with p + q = r + s (mod M); in the weighted basis, w(n) = sqrt(N! / prod n_m!) up
-// to a power of two per N, the element of target n' = n - e_r - e_s + e_p + e_q is
-// G_{pq,rs} n_r (n_s - [r = s]): the ratio w(n') / w(n) cancels the creation
-// square roots and squares the annihilation ones.  G is the multiplicity-summed
-// symmetrised coupling; the diagonal is precomputed per ket.
+// The shared-memory resident path of small sectors: one CTA runs every RK4 stage of a
+// sector, with the arithmetic and the order of sums of the direct stage kernel
+// (qb_block.cuh).
 //
 // Work layout: every warp owns tiles of kRows consecutive kets and runs without
 // CTA-wide barriers.  Phase 1 unpacks the tile's occupations (kRows/32 kets per
@@ -31,6 +19,7 @@
 //             signed value lo + 65536 hi, so the low half's borrow is part of it);
 //   RK_EXACT  exact momentum: 16-bit shifts, the ranking table in global memory.
 #pragma once
+#include "qb_block.cuh"
 #include "qb_device.cuh"
 
 #ifndef QB_UNROLL_PARTNERS
@@ -60,34 +49,6 @@ __device__ __forceinline__ int reg_occ(uint32_t ob0, uint32_t ob1, uint32_t ob2,
   if constexpr (MT <= 8) return (int)(__byte_perm(ob0, ob1, (uint32_t)m) & 0xffu);
   return m < 8 ? (int)(__byte_perm(ob0, ob1, (uint32_t)m) & 0xffu) : (int)((ob2 >> (8 * (m - 8))) & 0xffu);
 }
-
-// What a stage launch computes besides (or instead of) its output vector:
-//   KIND_STAGE  the RK4 / adjoint stage alone (modes 0 to 3);
-//   KIND_BIL    with the adjoint's bilinears fused (modes 2, 3);
-//   KIND_DOT    <x|H|x> only (mode 4): Re(conj(psi_n) (H psi)_n) summed in FP64,
-//               with each off-diagonal term and its Hermitian reverse taken once
-//               (the partners of a pair that come after it, counted twice).
-enum { KIND_STAGE = 0, KIND_BIL = 1, KIND_DOT = 2 };
-
-// Tile shapes of the stage kernel: warps per CTA, kets per warp tile and the
-// resident CTAs per SM its register budget is planned for (65,536 registers per SM
-// shared by warps x 32 x CTAs threads).  The CTA's warps share one copy of the
-// ranking table in shared memory.  Shape 0 is the default; the others are
-// compiled for the single-state stage (qb_space_set_tile_shape selects one).
-struct TileShape {
-  int warps, rows, min_blocks;
-};
-constexpr int kTileShapes = 5;
-__host__ __device__ constexpr TileShape tile_shape(int ts) {
-  return ts == 1   ? TileShape{16, 64, 2}
-         : ts == 2 ? TileShape{24, 64, 1}
-         : ts == 3 ? TileShape{12, 64, 3}
-         : ts == 4 ? TileShape{32, 128, 1}
-                   : TileShape{32, 64, 1};
-}
-// the shape of the batched sweeps and the bilinear stages (12 warps: room for the
-// registers of their extra accumulators)
-constexpr int kWideShape = 3;
 
 // Shared scratch of the stage kernel, after the table image, per warp (a tile of
 // `rows` kets):
@@ -555,69 +516,6 @@ __device__ __forceinline__ StageSmem stage_smem(const Tables& t, int M, int warp
   return S;
 }
 
-// Resident CTAs per SM the launch bounds plan for: the single-state stages at their
-// shape's count; the bilinear ones of the specialised mode counts at 2 CTAs per SM
-// (80 registers, more accumulators per lane); the batched ones and the generic
-// bilinear ones (16 accumulators) keep the compiler's choice (one CTA).
-template <int MT, int B, int KIND, int TS>
-__host__ __device__ constexpr int stage_min_blocks() {
-  return (B == 1 && KIND != KIND_BIL) ? tile_shape(TS).min_blocks : ((KIND == KIND_BIL && MT > 0) ? 2 : 1);
-}
-
-template <int MT, int B, bool CPLX, int KIND, int RK, int TS>
-__global__ void __launch_bounds__(32 * tile_shape(TS).warps, (stage_min_blocks<MT, B, KIND, TS>()))
-    stage_df_kernel(const Tables t, const DfArgs a, const int mode) {
-  constexpr bool BIL = (KIND == KIND_BIL), DOT = (KIND == KIND_DOT);
-  constexpr int kWarps = tile_shape(TS).warps, kRows = tile_shape(TS).rows;
-  const int M = (MT > 0) ? MT : t.M;
-  // the only CTA-wide barrier: warps run independently afterwards
-  const StageSmem S = stage_smem<RK>(t, M, kWarps, kRows);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t row1 = a.row1;
-  constexpr int kMB = (MT > 0) ? MT : 16;  // bilinear accumulators: one per mode + H_L
-  dfl bil_l{0.f, 0.f};
-  dfl bil_w[BIL ? kMB : 1];
-#pragma unroll
-  for (int q = 0; q < (BIL ? kMB : 1); ++q) bil_w[q] = dfl{0.f, 0.f};
-  double dot64 = 0.0;
-
-  for (int64_t base = a.row0 + ((int64_t)blockIdx.x * kWarps + warp) * kRows; base < row1;
-       base += (int64_t)gridDim.x * kWarps * kRows)
-    stage_tile<MT, B, CPLX, KIND, false, RK, kRows>(t, S.v, S.Gf, S.dtab, a, mode, base, row1, 0, S.sidx, S.socc, S.sD,
-                                                    S.sOff, S.sperm, S.hist, S.cursor, bil_l, bil_w, dot64);
-  if constexpr (DOT) {
-    // the CTA's sum in a fixed order: lanes by shuffles, warps in turn; partial[block]
-    __shared__ double red[kWarps];
-    for (int o = 16; o > 0; o >>= 1) dot64 += __shfl_down_sync(0xffffffffu, dot64, o);
-    if (lane == 0) red[warp] = dot64;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double sum = 0.0;
-      for (int w = 0; w < kWarps; ++w) sum += red[w];
-      a.partial[blockIdx.x] = sum;
-    }
-  }
-  if constexpr (BIL) {
-    // per-CTA sums of the bilinears in a fixed order: lanes by shuffles, warps in turn
-    __shared__ double red[kWarps][17];
-    const int nq = M + 1;
-    for (int q = 0; q < nq; ++q) {
-      double val = (q == 0) ? df_to(bil_l) : 0.0;
-#pragma unroll
-      for (int u = 0; u < kMB; ++u)
-        if (q == u + 1) val = df_to(bil_w[u]);
-      for (int o = 16; o > 0; o >>= 1) val += __shfl_down_sync(0xffffffffu, val, o);
-      if (lane == 0) red[warp][q] = val;
-    }
-    __syncthreads();
-    if (threadIdx.x < nq) {
-      double sum = 0.0;
-      for (int w = 0; w < kWarps; ++w) sum += red[w][threadIdx.x];
-      a.partial[(size_t)blockIdx.x * nq + threadIdx.x] = sum;
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Resident small sectors: each CTA takes sectors [0, n_small) from a static work
 // list (sector c, c + gridDim.x, ...), copies the sector's psi into shared
@@ -705,24 +603,6 @@ inline size_t stage_image_smem(const Tables& t, bool exact) {
   return (size_t)(kSmemEnd(t, exact) - kSmemFrom(t, exact) + 15) & ~(size_t)15;
 }
 
-// dynamic shared memory of a stage launch at tile shape ts
-inline size_t stage_shape_smem(const Tables& t, bool exact, int ts) {
-  const TileShape sh = tile_shape(ts);
-  return stage_image_smem(t, exact) +
-         (size_t)sh.warps * df_warp_scratch_bytes(sidx_words(t.M, exact), t.M, t.n_ann, sh.rows);
-}
-
-// The tile shape a stage launch runs at: the requested one where its shared memory
-// fits a CTA on the current device (with room for the kernels' static arrays),
-// otherwise the 12-warp shape (large tables, e.g. M = 16).
-inline int fitting_shape(const Tables& t, bool exact, int ts) {
-  int dev = 0, optin = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-    return kWideShape;
-  return stage_shape_smem(t, exact, ts) + 4096 <= (size_t)optin ? ts : kWideShape;
-}
-
 // Shared memory of the resident kernel holding `cap` kets per sector.
 inline size_t resident_smem(const Tables& t, int cap) {
   return stage_image_smem(t, t.exact != 0) +
@@ -755,100 +635,6 @@ int resident_launch_t(const Tables& t, const ResArgs& r, bool cplx, cudaStream_t
   return resident_launch_r<MT, RK_PAIR>(t, r, cplx, st);
 }
 
-// Launches one stage for mode count MT (0: any M), ranking variant RK and the
-// runtime batch size / coupling type / bilinear flag; `shape` selects the tile
-// shape of the single-state stage (others run shape 0).  *grid (if non-NULL)
-// receives the grid size.  Exact momentum: one state at a time.
-template <int MT, int RK>
-int stage_launch_r(const Tables& t, const DfArgs& a, int mode, int B, bool cplx, bool bil, int shape, cudaStream_t st,
-                   int* grid_out) {
-  int grid = 0, rc = QB_OK;
-#define QB_STAGE_CASE(BB, CC, LL, TT)                                                                   \
-  {                                                                                                     \
-    auto k = stage_df_kernel<MT, BB, CC, LL, RK, TT>;                                                   \
-    constexpr TileShape sh = tile_shape(TT);                                                            \
-    const size_t smem = stage_shape_smem(t, RK == RK_EXACT, TT);                                        \
-    rc = persistent_grid(k, smem, a.row1 - a.row0, &grid, 32 * sh.warps);                               \
-    if (rc) return rc;                                                                                  \
-    k<<<grid, 32 * sh.warps, smem, st>>>(t, a, mode);                                                   \
-  }
-  if (mode < 0 || mode > 4) return fail(QB_EINTERNAL, "bad stage mode");
-  // the launches of a fixed shape 0 drop to the 12-warp shape when shape 0 does not fit
-  const bool wide0 = fitting_shape(t, RK == RK_EXACT, 0) != 0;
-  shape = fitting_shape(t, RK == RK_EXACT, shape);
-  if (mode == 4) {  // <x|H|x>
-    if (B != 1) return fail(QB_EUNSUPPORTED, "the <x|H|x> reduction runs one state at a time");
-    if (cplx) {
-      if (wide0)
-        QB_STAGE_CASE(1, true, KIND_DOT, kWideShape)
-      else
-        QB_STAGE_CASE(1, true, KIND_DOT, 0)
-    } else {
-      if (wide0)
-        QB_STAGE_CASE(1, false, KIND_DOT, kWideShape)
-      else
-        QB_STAGE_CASE(1, false, KIND_DOT, 0)
-    }
-  } else if (bil) {
-    if (B != 1) return fail(QB_EUNSUPPORTED, "bilinear stages run one state at a time");
-    if (cplx)
-      QB_STAGE_CASE(1, true, KIND_BIL, kWideShape)
-    else
-      QB_STAGE_CASE(1, false, KIND_BIL, kWideShape)
-  } else if (cplx) {
-    if (B != 1) return fail(QB_EUNSUPPORTED, "batched sweeps need a real coupling");
-    if (wide0)
-      QB_STAGE_CASE(1, true, KIND_STAGE, kWideShape)
-    else
-      QB_STAGE_CASE(1, true, KIND_STAGE, 0)
-  } else {
-    if constexpr (RK == RK_EXACT) {
-      if (B != 1) return fail(QB_EUNSUPPORTED, "exact momentum: batched sweeps are not built");
-      // the widest of 32, 24 and 12 warps that fits beside the compact ranking table
-      if (!wide0)
-        QB_STAGE_CASE(1, false, KIND_STAGE, 0)
-      else if (fitting_shape(t, true, 2) == 2)
-        QB_STAGE_CASE(1, false, KIND_STAGE, 2)
-      else
-        QB_STAGE_CASE(1, false, KIND_STAGE, kWideShape)
-    } else {
-      switch (B) {
-        case 1:
-          switch (shape) {
-            case 1: QB_STAGE_CASE(1, false, KIND_STAGE, 1) break;
-            case 2: QB_STAGE_CASE(1, false, KIND_STAGE, 2) break;
-            case 3: QB_STAGE_CASE(1, false, KIND_STAGE, 3) break;
-            case 4: QB_STAGE_CASE(1, false, KIND_STAGE, 4) break;
-            default: QB_STAGE_CASE(1, false, KIND_STAGE, 0) break;
-          }
-          break;
-        case 2: QB_STAGE_CASE(2, false, KIND_STAGE, kWideShape) break;
-        case 4: QB_STAGE_CASE(4, false, KIND_STAGE, kWideShape) break;
-        case 8: QB_STAGE_CASE(8, false, KIND_STAGE, kWideShape) break;
-        default: return fail(QB_EINVAL, "batch must be 1, 2, 4 or 8");
-      }
-    }
-  }
-#undef QB_STAGE_CASE
-  QB_CUDA(cudaGetLastError());
-  if (grid_out) *grid_out = grid;
-  return QB_OK;
-}
-
-template <int MT>
-int stage_launch_t(const Tables& t, const DfArgs& a, int mode, int B, bool cplx, bool bil, int shape, cudaStream_t st,
-                   int* grid_out) {
-  if (rank_variant(t) == RK_EXACT) return stage_launch_r<MT, RK_EXACT>(t, a, mode, B, cplx, bil, shape, st, grid_out);
-  return stage_launch_r<MT, RK_PAIR>(t, a, mode, B, cplx, bil, shape, st, grid_out);
-}
-
-// one explicit specialisation per translation unit (qb_stage_m*.cu)
-int stage_launch_m5(const Tables&, const DfArgs&, int, int, bool, bool, int, cudaStream_t, int*);
-int stage_launch_m7(const Tables&, const DfArgs&, int, int, bool, bool, int, cudaStream_t, int*);
-int stage_launch_m9(const Tables&, const DfArgs&, int, int, bool, bool, int, cudaStream_t, int*);
-int stage_launch_m11(const Tables&, const DfArgs&, int, int, bool, bool, int, cudaStream_t, int*);
-int stage_launch_any(const Tables&, const DfArgs&, int, int, bool, bool, int, cudaStream_t, int*);
-
 int resident_launch_m5(const Tables&, const ResArgs&, bool, cudaStream_t);
 int resident_launch_m7(const Tables&, const ResArgs&, bool, cudaStream_t);
 int resident_launch_m9(const Tables&, const ResArgs&, bool, cudaStream_t);
@@ -862,20 +648,6 @@ inline int resident_launch(const Tables& t, const ResArgs& r, bool cplx, cudaStr
     case 9: return resident_launch_m9(t, r, cplx, st);
     case 11: return resident_launch_m11(t, r, cplx, st);
     default: return resident_launch_any(t, r, cplx, st);
-  }
-}
-
-// One stage over rows [a.row0, a.row1) in the weighted basis.  bil: the bilinear
-// instantiations (adjoint modes 2, 3); mode 4 is the <x|H|x> reduction (partial[block]);
-// shape: tile shape of the single-state stage (0: the default).
-inline int stage_launch(const Tables& t, const DfArgs& a, int mode, int B, bool cplx, cudaStream_t st,
-                        int* grid_out = nullptr, bool bil = false, int shape = 0) {
-  switch (t.M) {
-    case 5: return stage_launch_m5(t, a, mode, B, cplx, bil, shape, st, grid_out);
-    case 7: return stage_launch_m7(t, a, mode, B, cplx, bil, shape, st, grid_out);
-    case 9: return stage_launch_m9(t, a, mode, B, cplx, bil, shape, st, grid_out);
-    case 11: return stage_launch_m11(t, a, mode, B, cplx, bil, shape, st, grid_out);
-    default: return stage_launch_any(t, a, mode, B, cplx, bil, shape, st, grid_out);
   }
 }
 

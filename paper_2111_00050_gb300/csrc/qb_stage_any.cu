@@ -1,10 +1,15 @@
-// Stage-kernel specialisation for any M (see qb_stage.cuh).
+// Stage kernels for any M, exact momentum and complex couplings (see qb_block.cuh).
 #include "qb_stage.cuh"
 
 namespace qb {
 int stage_launch_any(const Tables& t, const DfArgs& a, int mode, int B, bool cplx, bool bil, int shape, cudaStream_t st,
-                   int* grid) {
-  return stage_launch_t<0>(t, a, mode, B, cplx, bil, shape, st, grid);
+                     int* grid) {
+  if (!cplx) return blk_launch_kind<0, false>(t, a, mode, B, bil, shape, st, grid);
+  if (B != 1) return fail(QB_EUNSUPPORTED, "batched sweeps need a real coupling");
+  if (mode < 0 || mode > 4) return fail(QB_EINTERNAL, "bad stage mode");
+  if (mode == 4) return blk_launch<0, false, 1, true, KIND_DOT>(t, a, mode, shape, st, grid);
+  if (bil) return blk_launch<0, false, 1, true, KIND_BIL>(t, a, mode, shape, st, grid);
+  return blk_launch<0, false, 1, true, KIND_STAGE>(t, a, mode, shape, st, grid);
 }
 int resident_launch_any(const Tables& t, const ResArgs& r, bool cplx, cudaStream_t st) {
   return resident_launch_t<0>(t, r, cplx, st);

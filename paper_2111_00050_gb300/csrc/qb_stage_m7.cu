@@ -1,10 +1,9 @@
-// Stage-kernel specialisation for M = 7 modes (see qb_stage.cuh).
+// Stage-kernel specialisation for M = 7 modes with 3 partners a pair (see qb_block.cuh).
 #include "qb_stage.cuh"
 
 namespace qb {
-int stage_launch_m7(const Tables& t, const DfArgs& a, int mode, int B, bool cplx, bool bil, int shape, cudaStream_t st,
-                   int* grid) {
-  return stage_launch_t<7>(t, a, mode, B, cplx, bil, shape, st, grid);
+int stage_launch_m7(const Tables& t, const DfArgs& a, int mode, int B, bool bil, int shape, cudaStream_t st, int* grid) {
+  return blk_launch_kind<7, true>(t, a, mode, B, bil, shape, st, grid);
 }
 int resident_launch_m7(const Tables& t, const ResArgs& r, bool cplx, cudaStream_t st) {
   return resident_launch_t<7>(t, r, cplx, st);
