@@ -184,14 +184,13 @@ int qb_evolve(qb_space* space, void* d_psi, double dt, int64_t steps, void* d_wo
 int qb_evolve_batch(qb_space* space, void* d_psi, int batch, const double* scale, double dt, int64_t steps,
                     void* d_work, void* stream);
 
-/* Execution tuning of qb_evolve for one state vector.  Leading sectors (in the
- * order of qb_space_sectors) of at most resident_max_kets kets run
- * shared-memory resident: each CTA takes such sectors from a work list and
- * advances them through every step of the call in one launch, on a side stream
- * beside the stage-by-stage launches of the larger sectors (which are captured
- * into CUDA graphs in chunks of 32 steps).  0 disables the resident path; the
- * default is 1024; values above what shared memory holds are clipped.  Results
- * do not depend on the setting: every ket goes through the same arithmetic. */
+/* Execution tuning of qb_evolve for one state vector.  A small space (at most 64 kets
+ * per SM of the device) whose sectors all have at most resident_max_kets kets and at
+ * most 256 (M = 5: 512) runs resident: one thread block per sector advances it through
+ * every step of the call in one launch, in registers and shared memory.  Other spaces
+ * run stage by stage, the launches captured into CUDA graphs in chunks of 32 steps.
+ * 0 disables the resident path; the default is 1024.  Results do not depend on the
+ * setting: every ket goes through the same arithmetic. */
 int qb_space_set_resident_max(qb_space* space, int resident_max_kets);
 
 /* Execution tuning of the RK4 stages of qb_evolve, qb_evolve_plain and

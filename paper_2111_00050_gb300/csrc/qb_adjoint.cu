@@ -24,7 +24,7 @@
 #include <vector>
 
 #include "qb_device.cuh"
-#include "qb_stage.cuh"
+#include "qb_block.cuh"
 
 namespace qb {
 

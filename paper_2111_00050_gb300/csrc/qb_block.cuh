@@ -124,6 +124,29 @@ __device__ __forceinline__ BaseRec<KC> load_base(const uint32_t* base, int rec, 
   return r;
 }
 
+// acc += the terms of one record: coefficient G n_r (n_s - [r = s]) = G Af, gathered values x
+template <int KC, bool CPLX, bool DOT>
+__device__ __forceinline__ void add_record(dfc& acc, const float4 (&x)[Rec<KC>::n], const float2* sG, const float2* sGi,
+                                           int rec, int nrec, int n, int c_first, float Af) {
+  constexpr int NT = Rec<KC>::n, RW = Rec<KC>::w;
+#pragma unroll
+  for (int c = 0; c < NT; ++c) {
+    if ((KC == 0 && c >= n) || (DOT && c < c_first)) continue;  // the same for all lanes
+    const int sl = c < 4 ? RW * rec + c : 4 * nrec + rec;
+    const float2 g2 = sG[sl];
+    const dfl cr = df_mul_f(dfl{g2.x, g2.y}, Af);
+    const f2 xh = f2_pack(x[c].x, x[c].y), xl = f2_pack(x[c].z, x[c].w);
+    dfc_fma(acc, f2_pack(cr.h, cr.h), f2_pack(-cr.h, -cr.h), f2_pack(cr.l, cr.l), xh, xl);
+    if (CPLX) {
+      // + (-c_i x_im, c_i x_re): lanes of x swapped, coefficient (-c_i, c_i)
+      const float2 gi = sGi[sl];
+      const dfl ci = df_mul_f(dfl{gi.x, gi.y}, Af);
+      dfc_fma(acc, f2_pack(-ci.h, ci.h), f2_pack(ci.h, -ci.h), f2_pack(-ci.l, ci.l), f2_pack(x[c].y, x[c].x),
+              f2_pack(x[c].w, x[c].z));
+    }
+  }
+}
+
 // Everything of a ket's row that the epilogue needs, and the epilogue: forms the
 // stage's output (or the bilinears, or the <x|H|x> summand) from the off-diagonal sum.
 // WHOLE: acc is the whole two-body part (factored couplings), else its off-diagonal part.
@@ -259,12 +282,15 @@ __device__ __forceinline__ void bil_reduce(const DfArgs& a, int M, const dfl& bi
 }
 
 // Shared memory: couplings (real, imaginary) of the slots and the record words
-inline size_t blk_smem_bytes(const Tables& t, bool cplx) {
+__host__ __device__ inline size_t blk_smem_bytes(const Tables& t, bool cplx) {
   return (size_t)t.bk_T * 8 * (cplx ? 2 : 1) + (((size_t)t.bk_nrec * 8 + 15) & ~(size_t)15);
 }
 
-template <int MT, bool FIX, int B, bool CPLX, int KIND>
-__global__ void __launch_bounds__((blk_max_threads<B, KIND>()), 1)
+// U: records whose gathers are in flight together.  One where every SM has its 32 warps;
+// four in CTAs of up to 256 threads (255 registers) for the spaces that leave a warp or two
+// per scheduler, where every gather's latency shows.
+template <int MT, bool FIX, int B, bool CPLX, int KIND, int U>
+__global__ void __launch_bounds__((U > 1 ? 256 : blk_max_threads<B, KIND>()), 1)
     blk_stage_kernel(const Tables t, const DfArgs a, const int mode) {
   constexpr int KC = FIX ? (MT - 1) / 2 : 0;
   constexpr int NT = Rec<KC>::n, RW = Rec<KC>::w, NW = occ_words<MT>();
@@ -311,73 +337,82 @@ __global__ void __launch_bounds__((blk_max_threads<B, KIND>()), 1)
       for (int b = 0; b < B; ++b) acc[b] = dfc{0ull, 0ull};
       bool bad = false;  // a target fell outside the state
 
-      // ---- the annihilation pairs (r <= s) in step; the next record's map in flight.  A
-      // lane that lacks the pair has the coefficient 0 and keeps its last gathered values.
-      float4 x[NT];
+      // ---- the annihilation pairs (r <= s) in step, U records' gathers and the next U records'
+      // maps and bases in flight.  A lane that lacks a pair has the coefficient 0 and keeps its
+      // last gathered values.
+      float4 x[U][NT];
 #pragma unroll
-      for (int c = 0; c < NT; ++c) x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-      MapRec<KC> mcur = load_map<KC>(mp, mp5);
-      BaseRec<KC> bcur = load_base<KC>(base, 0, nrec);
-      for (int rec = 0; rec < nrec; ++rec) {
-        if (rec + 1 < nrec) {
-          mp += (size_t)t.bk_S * (2 * RW);
-          if (KC == 5) mp5 += t.bk_S;
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int c = 0; c < NT; ++c) x[u][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+      MapRec<KC> mcur[U], mnext[U];
+      BaseRec<KC> bcur[U], bnext[U];
+      auto load = [&](int rec0, MapRec<KC> (&mr)[U], BaseRec<KC> (&br)[U]) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int rec = min(rec0 + u, nrec - 1);
+          mr[u] = load_map<KC>(mp + (size_t)rec * t.bk_S * (2 * RW), mp5 + (size_t)rec * t.bk_S);
+          br[u] = load_base<KC>(base, rec, nrec);
         }
-        const MapRec<KC> mnext = load_map<KC>(mp, mp5);
-        const BaseRec<KC> bnext = load_base<KC>(base, min(rec + 1, nrec - 1), nrec);
-        const uint2 info = sinfo[rec];
-        const float Af = (occ_float23<NW>(ob, info.x, (info.x & 0x8000u) != 0u) - 8388608.0f) *
-                         (occ_float23<NW>(ob, info.x >> 16, (info.x & 0x80000000u) != 0u) - __uint_as_float(info.y));
-        const bool act = Af != 0.f;
-        if (__any_sync(0xffffffffu, act)) {
+      };
+      if (nrec > 0) load(0, mcur, bcur);
+      for (int rec0 = 0; rec0 < nrec; rec0 += U) {
+        load(rec0 + U, mnext, bnext);
+        float Af[U];
+        uint32_t rk[U][NT], infox[U];
+        bool ok[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const bool in_list = U == 1 || rec0 + u < nrec;
+          const uint2 info = sinfo[in_list ? rec0 + u : rec0];
+          infox[u] = info.x;
+          Af[u] = (occ_float23<NW>(ob, info.x, (info.x & 0x8000u) != 0u) - 8388608.0f) *
+                  (occ_float23<NW>(ob, info.x >> 16, (info.x & 0x80000000u) != 0u) - __uint_as_float(info.y));
+          if (!in_list) Af[u] = 0.f;
           const int n = KC == 0 ? (int)((info.x >> 4) & 7) : NT;
+          rk[u][0] = bcur[u].a.x + (mcur[u].a.x & 0xffffu);
+          rk[u][1] = bcur[u].a.y + (mcur[u].a.x >> 16);
+          if constexpr (NT > 2) rk[u][2] = bcur[u].a.z + (mcur[u].a.y & 0xffffu);
+          if constexpr (NT > 3) rk[u][3] = bcur[u].a.w + (mcur[u].a.y >> 16);
+          if constexpr (NT > 4) rk[u][4] = bcur[u].b + mcur[u].b;
+          uint32_t top = rk[u][0];
+#pragma unroll
+          for (int c = 1; c < NT; ++c)
+            if (KC > 0 || c < n) top = max(top, rk[u][c]);
+          const bool act = Af[u] != 0.f;
+          ok[u] = act && top < (uint32_t)total;
+          bad |= act && !ok[u];
           const int c_first = DOT ? (int)((info.x >> 8) & 7) : 0;
-          uint32_t rk[NT];
-          rk[0] = bcur.a.x + (mcur.a.x & 0xffffu);
-          rk[1] = bcur.a.y + (mcur.a.x >> 16);
-          if constexpr (NT > 2) rk[2] = bcur.a.z + (mcur.a.y & 0xffffu);
-          if constexpr (NT > 3) rk[3] = bcur.a.w + (mcur.a.y >> 16);
-          if constexpr (NT > 4) rk[4] = bcur.b + mcur.b;
-          if constexpr (KC == 0) {
 #pragma unroll
-            for (int c = 1; c < NT; ++c)
-              if (c >= n) rk[c] = rk[0];  // unused slots
-          }
-          uint32_t top = rk[0];
+          for (int c = 0; c < NT; ++c)
+            if (ok[u] && (KC > 0 || c < n) && (!DOT || c >= c_first)) x[u][c] = __ldg(a.vin + rk[u][c]);
+        }
 #pragma unroll
-          for (int c = 1; c < NT; ++c) top = max(top, rk[c]);
-          const bool ok = act && top < (uint32_t)total;
-          bad |= act && !ok;
+        for (int u = 0; u < U; ++u) {
+          if (!__any_sync(0xffffffffu, Af[u] != 0.f)) continue;
+          const int rec = rec0 + u;
+          const int n = KC == 0 ? (int)((infox[u] >> 4) & 7) : NT;
+          const int c_first = DOT ? (int)((infox[u] >> 8) & 7) : 0;
 #pragma unroll
           for (int b = 0; b < B; ++b) {
+            if (b > 0) {
 #pragma unroll
-            for (int c = 0; c < NT; ++c)
-              if (ok && (KC > 0 || c < n) && (!DOT || c >= c_first)) x[c] = __ldg(a.vin + (size_t)b * total + rk[c]);
-#pragma unroll
-            for (int c = 0; c < NT; ++c) {
-              if ((KC == 0 && c >= n) || (DOT && c < c_first)) continue;  // the same for all lanes
-              const int sl = c < 4 ? RW * rec + c : 4 * nrec + rec;
-              const float2 g2 = sG[sl];
-              const dfl cr = df_mul_f(dfl{g2.x, g2.y}, Af);
-              const f2 xh = f2_pack(x[c].x, x[c].y), xl = f2_pack(x[c].z, x[c].w);
-              dfc_fma(acc[b], f2_pack(cr.h, cr.h), f2_pack(-cr.h, -cr.h), f2_pack(cr.l, cr.l), xh, xl);
-              if (CPLX) {
-                // + (-c_i x_im, c_i x_re): lanes of x swapped, coefficient (-c_i, c_i)
-                const float2 gi = sGi[sl];
-                const dfl ci = df_mul_f(dfl{gi.x, gi.y}, Af);
-                dfc_fma(acc[b], f2_pack(-ci.h, ci.h), f2_pack(ci.h, -ci.h), f2_pack(-ci.l, ci.l),
-                        f2_pack(x[c].y, x[c].x), f2_pack(x[c].w, x[c].z));
-              }
+              for (int c = 0; c < NT; ++c)
+                if (ok[u] && (KC > 0 || c < n)) x[u][c] = __ldg(a.vin + (size_t)b * total + rk[u][c]);
             }
+            add_record<KC, CPLX, DOT>(acc[b], x[u], sG, sGi, rec, nrec, n, c_first, Af[u]);
           }
           // keep |lo| below an ulp of hi between pairs
-          if (KC > 0 || (info.x & 0x80u)) {
+          if (KC > 0 || (infox[u] & 0x80u)) {
 #pragma unroll
             for (int b = 0; b < B; ++b) acc[b] = dfc_renorm(acc[b]);
           }
         }
-        mcur = mnext;
-        bcur = bnext;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          mcur[u] = mnext[u];
+          bcur[u] = bnext[u];
+        }
       }
       if (bad) atomicOr(a.status, 1);
       if (valid) stage_epilogue<MT, B, KIND, false, NW>(t, a, mode, g, g, acc, ob, bil_l, bil_w, dot64);
@@ -402,6 +437,13 @@ __global__ void __launch_bounds__((blk_max_threads<B, KIND>()), 1)
 constexpr int kTileShapes = 5;
 __host__ __device__ constexpr int tile_warps(int ts) { return ts == 1 ? 16 : ts == 2 ? 24 : ts == 3 ? 12 : ts == 4 ? 8 : 32; }
 
+// Rounds of 32 kets per SM up to which the four-record kernel runs: the CTA of 8 warps that
+// its registers allow is then one wave.  One stage, one record against four (us): M = 5,
+// 3,003 kets 7.6 / 6.0, 33,649 kets 8.1 / 7.2; M = 7, 19,448 kets 12.5 / 10.6; M = 11, 16,796
+// kets 28.4 / 19.2.  The generic kernel (partner counts that vary) gains nothing by it (M = 6,
+// 27,132 kets: 11.7 / 13.0).
+constexpr int kFewWarps = 8;
+
 // Warps per CTA and grid of a launch over `rows` kets.  While a small space leaves SMs
 // without work the CTA shrinks, so that its rounds spread over every SM.
 template <typename K>
@@ -420,17 +462,30 @@ inline int stage_geometry(K k, int64_t rows, int shape, int max_warps, size_t sm
 }
 
 // One stage over the rows [a.row0, a.row1).
-template <int MT, bool FIX, int B, bool CPLX, int KIND>
-int blk_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream_t st, int* grid_out) {
-  auto k = blk_stage_kernel<MT, FIX, B, CPLX, KIND>;
+template <int MT, bool FIX, int B, bool CPLX, int KIND, int U>
+int blk_launch_u(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream_t st, int* grid_out) {
+  auto k = blk_stage_kernel<MT, FIX, B, CPLX, KIND, U>;
   const size_t smem = blk_smem_bytes(t, CPLX);
   int warps = 0, grid = 0;
-  const int rc = stage_geometry(k, a.row1 - a.row0, shape, blk_max_threads<B, KIND>() / 32, smem, &warps, &grid);
+  const int rc = stage_geometry(k, a.row1 - a.row0, shape, (U > 1 ? 256 : blk_max_threads<B, KIND>()) / 32, smem, &warps,
+                                &grid);
   if (rc) return rc;
   k<<<grid, 32 * warps, smem, st>>>(t, a, mode);
   QB_CUDA(cudaGetLastError());
   if (grid_out) *grid_out = grid;
   return QB_OK;
+}
+
+template <int MT, bool FIX, int B, bool CPLX, int KIND>
+int blk_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream_t st, int* grid_out) {
+  if constexpr (FIX && B == 1 && KIND == KIND_STAGE) {
+    int dev = 0, sms = 0;
+    QB_CUDA(cudaGetDevice(&dev));
+    QB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if ((a.row1 - a.row0) / 32 <= (int64_t)sms * kFewWarps)
+      return blk_launch_u<MT, FIX, B, CPLX, KIND, 4>(t, a, mode, shape, st, grid_out);
+  }
+  return blk_launch_u<MT, FIX, B, CPLX, KIND, 1>(t, a, mode, shape, st, grid_out);
 }
 
 // the kinds and batch sizes of one kernel family (real or complex couplings)

@@ -879,9 +879,6 @@ void qb_space_free(qb_space* space) {
     cudaFree(sp->d_base[k]);
   }
   if (sp->capture_stream) cudaStreamDestroy(sp->capture_stream);
-  if (sp->side_stream) cudaStreamDestroy(sp->side_stream);
-  if (sp->ev_fork) cudaEventDestroy(sp->ev_fork);
-  if (sp->ev_join) cudaEventDestroy(sp->ev_join);
   delete sp;
 }
 

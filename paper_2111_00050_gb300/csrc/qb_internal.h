@@ -210,9 +210,7 @@ struct Space {
   int64_t scratch_doubles = 0;
   Tables t{};
   cudaStream_t capture_stream = nullptr;  // private stream on which RK4 chunks are captured into graphs
-  cudaStream_t side_stream = nullptr;     // resident small sectors run here, beside the large ones
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  int resident_max_kets = 1024;           // sectors up to this size run shared-memory resident
+  int resident_max_kets = 1024;           // spaces whose sectors are all up to this size run shared-memory resident
   int order = 4;                          // Taylor order of a time step (4: RK4)
   int tile_shape = 0;                     // tile shape of the single-state stage kernel (qb_stage.cuh)
   int device = 0;

@@ -1164,7 +1164,7 @@ static void lower_range(const Space& s, int sec, int64_t* low0, int64_t* low1) {
 
 template <int B>
 static int rk4_issue(Space& s, DfArgs& a, double dt, int64_t steps, float4* w1, float4* w2, float4* psif,
-                     cudaStream_t st, bool plain, int64_t row0 = 0) {
+                     cudaStream_t st, bool plain) {
   const bool cplx = s.t.is_complex != 0;
   const int K = s.order;
   for (int64_t it = 0; it < steps; ++it) {
@@ -1181,7 +1181,7 @@ static int rk4_issue(Space& s, DfArgs& a, double dt, int64_t steps, float4* w1, 
       if (!plain) {
         a.low0 = 0;
         a.low1 = s.t.fa_on ? s.t.fa_low : 0;
-        a.row0 = row0;
+        a.row0 = 0;
         a.row1 = s.t.total;
         int rc = stage_launch(s.t, a, d == 1 ? 1 : 0, B, cplx, st, nullptr, false, s.tile_shape);
         if (rc) return rc;
@@ -1219,26 +1219,13 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
   a.status = reinterpret_cast<int*>(s.d_scratch);
   a.nbasef = 0;
   if (plain) return rk4_issue<B>(s, a, dt, steps, w1, w2, psif, st, true);
-  // Leading sectors small enough to sit in shared memory run resident on a side
-  // stream, all steps in one launch, while the rest advances stage by stage.
-  int64_t row0 = 0;
-  bool forked = false;
+  // A space of small sectors runs resident, all steps in one launch.
   if (B == 1 && !s.t.fa_on) {
-    int n_small = 0;
-    const int nsec = (int)s.secDim.size();
-    int optin = 0;
+    int optin = 0, sms = 0;
     QB_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, s.device));
-    const size_t base_smem = resident_smem(s.t, 0);
-    const int64_t room = optin > (int)base_smem ? (optin - (int64_t)base_smem - 1024) / 64 : 0;
-    const int64_t limit = std::min<int64_t>(room, s.resident_max_kets);
-    int cap = 0;
-    while (n_small < nsec && s.secDim[n_small] <= limit) cap = std::max<int>(cap, (int)s.secDim[n_small++]);
-    if (n_small > 0) {
-      if (!s.side_stream) QB_CUDA(cudaStreamCreateWithFlags(&s.side_stream, cudaStreamNonBlocking));
-      if (!s.ev_fork) QB_CUDA(cudaEventCreateWithFlags(&s.ev_fork, cudaEventDisableTiming));
-      if (!s.ev_join) QB_CUDA(cudaEventCreateWithFlags(&s.ev_join, cudaEventDisableTiming));
-      QB_CUDA(cudaEventRecord(s.ev_fork, st));
-      QB_CUDA(cudaStreamWaitEvent(s.side_stream, s.ev_fork, 0));
+    QB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s.device));
+    const int cap = (int)std::min<int64_t>((s.maxDim + 3) & ~int64_t(3), 65536);
+    if (s.maxDim <= std::min(s.resident_max_kets, resident_most(s.t)) && s.t.total <= 64LL * sms && resident_smem(s.t, cap) + 1024 <= (size_t)optin) {
       ResArgs r{};
       r.psi = psi;
       r.psif = psif;
@@ -1247,28 +1234,14 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
       r.dt = dt;
       r.steps = steps;
       r.order = s.order;
-      r.n_small = n_small;
       r.cap = cap;
       r.status = a.status;
-      int rc = resident_launch(s.t, r, s.t.is_complex != 0, s.side_stream);
-      if (rc) return rc;
-      QB_CUDA(cudaEventRecord(s.ev_join, s.side_stream));
-      forked = true;
-      row0 = s.secOff[n_small];
+      return resident_launch(s.t, r, (int)std::min<int64_t>(1024, (s.maxDim + 31) & ~int64_t(31)), st);
     }
   }
-  auto join = [&]() -> int {
-    if (forked) QB_CUDA(cudaStreamWaitEvent(st, s.ev_join, 0));
-    return QB_OK;
-  };
-  if (row0 >= s.t.total) return join();
-  if (steps < 2 * kGraphSteps) {
-    int rc = rk4_issue<B>(s, a, dt, steps, w1, w2, psif, st, false, row0);
-    if (rc) return rc;
-    return join();
-  }
+  if (steps < 2 * kGraphSteps) return rk4_issue<B>(s, a, dt, steps, w1, w2, psif, st, false);
   // first step directly: fills the launch-geometry cache outside any capture
-  int rc = rk4_issue<B>(s, a, dt, 1, w1, w2, psif, st, false, row0);
+  int rc = rk4_issue<B>(s, a, dt, 1, w1, w2, psif, st, false);
   if (rc) return rc;
   int64_t left = steps - 1;
   cudaGraph_t graph = nullptr;
@@ -1278,7 +1251,7 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
   // stream, which cannot capture); the graph is launched on the caller's stream
   if (!s.capture_stream) QB_CUDA(cudaStreamCreateWithFlags(&s.capture_stream, cudaStreamNonBlocking));
   if (cudaStreamBeginCapture(s.capture_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-    rc = rk4_issue<B>(s, a, dt, kGraphSteps, w1, w2, psif, s.capture_stream, false, row0);
+    rc = rk4_issue<B>(s, a, dt, kGraphSteps, w1, w2, psif, s.capture_stream, false);
     const cudaError_t ec = cudaStreamEndCapture(s.capture_stream, &graph);
     if (rc) {
       if (graph) cudaGraphDestroy(graph);
@@ -1301,9 +1274,7 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
   } else if (graph) {
     cudaGraphDestroy(graph);
   }
-  rc = rk4_issue<B>(s, a, dt, left, w1, w2, psif, st, false, row0);
-  if (rc) return rc;
-  return join();
+  return rk4_issue<B>(s, a, dt, left, w1, w2, psif, st, false);
 }
 
 int launch_rk4(Space& s, void* d_psi, int batch, const double* scale, double dt, int64_t steps, void* d_work,

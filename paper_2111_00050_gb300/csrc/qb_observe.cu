@@ -28,9 +28,14 @@
 
 #include "qb_device.cuh"
 #include "qb_internal.h"
-#include "qb_stage.cuh"
+#include "qb_block.cuh"
 
 namespace qb {
+
+// The moments kernels' dynamic shared memory starts with the ranking table (momentum mod
+// M), so a byte offset into the table is one shared load with an immediate base.
+extern __shared__ __align__(16) unsigned char smem_raw[];
+__device__ __forceinline__ int32_t e_byte(uint32_t off) { return *reinterpret_cast<const int32_t*>(smem_raw + off); }
 
 constexpr int kObsBlock = 256;  // threads per CTA of the first pass
 // warps per CTA of the moments kernel (its CTAs share nothing but the staged table);
@@ -284,7 +289,6 @@ __global__ void __launch_bounds__(32 * mw_warps(kMwSpl), QB_MW_MIN_BLOCKS) momen
                                                                  double* partial, int nmom, int e_begin, int nent,
                                                                  int sec_smem, int* status, const float4* ketf,
                                                                  const int* tb) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int kMwWarps = mw_warps(kMwSpl), kMwBlock = 32 * kMwWarps;
   constexpr int kMB = (MT > 0) ? MT : kMaxM;
   constexpr int kIW = MwWords<MT, EXACT>::n;

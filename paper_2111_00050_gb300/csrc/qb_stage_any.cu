@@ -11,7 +11,8 @@ int stage_launch_any(const Tables& t, const DfArgs& a, int mode, int B, bool cpl
   if (bil) return blk_launch<0, false, 1, true, KIND_BIL>(t, a, mode, shape, st, grid);
   return blk_launch<0, false, 1, true, KIND_STAGE>(t, a, mode, shape, st, grid);
 }
-int resident_launch_any(const Tables& t, const ResArgs& r, bool cplx, cudaStream_t st) {
-  return resident_launch_t<0>(t, r, cplx, st);
+int resident_launch_any(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {
+  return t.is_complex ? resident_launch_k<0, false, true>(t, r, threads, st)
+                      : resident_launch_k<0, false, false>(t, r, threads, st);
 }
 }  // namespace qb

@@ -5,7 +5,7 @@ namespace qb {
 int stage_launch_m11(const Tables& t, const DfArgs& a, int mode, int B, bool bil, int shape, cudaStream_t st, int* grid) {
   return blk_launch_kind<11, true>(t, a, mode, B, bil, shape, st, grid);
 }
-int resident_launch_m11(const Tables& t, const ResArgs& r, bool cplx, cudaStream_t st) {
-  return resident_launch_t<11>(t, r, cplx, st);
+int resident_launch_m11(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {
+  return resident_launch_k<11, true, false>(t, r, threads, st);
 }
 }  // namespace qb

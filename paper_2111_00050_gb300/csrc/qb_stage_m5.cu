@@ -5,7 +5,8 @@ namespace qb {
 int stage_launch_m5(const Tables& t, const DfArgs& a, int mode, int B, bool bil, int shape, cudaStream_t st, int* grid) {
   return blk_launch_kind<5, true>(t, a, mode, B, bil, shape, st, grid);
 }
-int resident_launch_m5(const Tables& t, const ResArgs& r, bool cplx, cudaStream_t st) {
-  return resident_launch_t<5>(t, r, cplx, st);
+int resident_launch_m5(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {
+  if (threads <= reg_kets(5)) return resident_reg_launch<5>(t, r, threads, st);
+  return resident_launch_k<5, true, false>(t, r, threads, st);
 }
 }  // namespace qb
