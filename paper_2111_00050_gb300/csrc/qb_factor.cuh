@@ -47,7 +47,8 @@ inline size_t ann_smem_bytes(const Tables& t) { return ((size_t)t.fa_nrec * 8 + 
 // start less the number of the lower ket.  kNoIndex: the raised sector is not held.
 
 // DOT: no vector; sum_k lam_k |B_k psi|^2 in FP64 over CTAs, partial[block]
-template <int NT, bool DOT>
+// EVERY: every record of every lower ket is taken (all momenta held).
+template <int NT, bool DOT, bool EVERY>
 __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfArgs a) {
   constexpr int PL = NT > 4 ? 2 : 1;       // groups of four pairs a record
   constexpr int NS = NT > 0 ? NT : 4;      // pairs of a record
@@ -61,14 +62,22 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
   const int64_t total = t.total;
   double dot64 = 0.0;
 
+  // Rounds of a layer are taken in an order that walks its sectors side by side (fa_perm):
+  // a ket f(n) is read from every lower sector, at about the same place, and is still in
+  // L1 / L2 then.  (A launch over part of the lower kets takes them as they come.)
+  const uint32_t* perm = a.low0 == 0 && a.low1 == t.fa_low ? t.fa_perm : nullptr;
   const int64_t r0 = a.low0 / 32, step = (int64_t)gridDim.x * warps;
   int64_t rd = (a.low1 - 1) / 32 - ((int64_t)blockIdx.x * warps + warp);
-  RoundIn next = load_round(t.fa_occ, t.fa_fill, t.fa_rblk, max(rd, r0), t.fa_low, lane);
+  auto round_of = [&](int64_t r) { return perm ? (int64_t)__ldg(perm + max(r, r0)) : max(r, r0); };
+  int64_t rn = round_of(rd), rn2 = round_of(rd - step);
+  RoundIn next = load_round(t.fa_occ, t.fa_fill, t.fa_rblk, rn, t.fa_low, lane);
   for (; rd >= r0; rd -= step) {
-      const int64_t g = rd * 32 + lane;
+      const int64_t g = rn * 32 + lane;
       const bool valid = g >= a.low0 && g < a.low1;
       const RoundIn in = next;
-      next = load_round(t.fa_occ, t.fa_fill, t.fa_rblk, max(rd - step, r0), t.fa_low, lane);
+      rn = rn2;
+      next = load_round(t.fa_occ, t.fa_fill, t.fa_rblk, rn, t.fa_low, lane);
+      rn2 = round_of(rd - 2 * step);
       const uint32_t* base = t.fa_basea + (size_t)block_of_lane(in, lane, g < t.fa_low) * fa_rowa(t);
       const uint32_t* gb = base + fa_Ta(t);
       const uint2* mp = t.fa_mapa + in.fill;
@@ -86,22 +95,28 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
       float4 x[NS];
 #pragma unroll
       for (int c = 0; c < NS; ++c) x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+      // the records whose raised sector some lane's block has (one class of M where the
+      // space holds one momentum)
+      uint32_t mask = ~0u;
+      if (!EVERY && nrec <= 32) mask = __reduce_or_sync(0xffffffffu, valid ? __ldg(gb + nc) : 0u);
       uint2 mcur[PL];
       uint4 bcur[PL];
-#pragma unroll
-      for (int p = 0; p < PL; ++p) {
-        mcur[p] = __ldg(mp + (size_t)p * t.bk_S);
-        bcur[p] = __ldg(reinterpret_cast<const uint4*>(base) + p);
-      }
-      for (int rec = 0; rec < nrec; ++rec) {
-        if (rec + 1 < nrec) mp += (size_t)PL * t.bk_S;
-        uint2 mnext[PL];
-        uint4 bnext[PL];
+      auto load = [&](int rec) {
 #pragma unroll
         for (int p = 0; p < PL; ++p) {
-          mnext[p] = __ldg(mp + (size_t)p * t.bk_S);
-          bnext[p] = __ldg(reinterpret_cast<const uint4*>(base) + min(rec + 1, nrec - 1) * PL + p);
+          mcur[p] = __ldg(mp + (size_t)(rec * PL + p) * t.bk_S);
+          bcur[p] = __ldg(reinterpret_cast<const uint4*>(base) + rec * PL + p);
         }
+      };
+      auto following = [&](int rec) {  // the next record to take, or nrec
+        if (EVERY || nrec > 32) return rec + 1;
+        const uint32_t rest = rec < 31 ? mask & (~0u << (rec + 1)) : 0u;
+        return rest ? __ffs(rest) - 1 : nrec;
+      };
+      int rec = EVERY || (mask & 1u) ? 0 : following(0);
+      if (rec < nrec) load(rec);
+      for (int rnext; rec < nrec; rec = rnext) {
+        rnext = following(rec);
         uint32_t ix[NS];
         ix[0] = bcur[0].x + (mcur[0].x & 0xffffu);
         ix[1] = bcur[0].y + (mcur[0].x >> 16);
@@ -110,11 +125,7 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
         if constexpr (NS > 4) ix[4] = bcur[PL - 1].x + (mcur[PL - 1].x & 0xffffu);
         if constexpr (NS > 5) ix[5] = bcur[PL - 1].y + (mcur[PL - 1].x >> 16);
         const bool act = valid && bcur[0].x != kNoIndex;
-#pragma unroll
-        for (int p = 0; p < PL; ++p) {
-          mcur[p] = mnext[p];
-          bcur[p] = bnext[p];
-        }
+        if (rnext < nrec) load(rnext);
         if (!__any_sync(0xffffffffu, act)) continue;
         const uint32_t info = srec[rec].x;
         const int n = NT > 0 ? NT : (int)((info >> 8) & 15), dbl = NT > 0 ? NT - 1 : (int)((info >> 12) & 7);
@@ -175,6 +186,21 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
   }
 }
 
+// the creation pairs in order: r < s, then r = s
+template <int MT>
+struct PairList {
+  int r[MT * (MT + 1) / 2], s[MT * (MT + 1) / 2];
+  constexpr PairList() : r(), s() {
+    int i = 0;
+    for (int p = 0; p < MT; ++p)
+      for (int q = p + 1; q < MT; ++q, ++i) {
+        r[i] = p;
+        s[i] = q;
+      }
+    for (int p = 0; p < MT; ++p, ++i) r[i] = s[i] = p;
+  }
+};
+
 inline size_t cre_smem_bytes(const Tables& t) { return (size_t)fa_Tc(t) * 12; }
 
 template <int MT, int KIND>
@@ -212,41 +238,85 @@ __global__ void __launch_bounds__(KIND == KIND_BIL ? 512 : 1024, 1)
       const uint2* mp = t.fa_mapc + in.fill;
       dfc acc[1] = {dfc{0ull, 0ull}};
       bool bad = false;
-      float4 x[4];
+      if constexpr (MT > 0) {
+        // unrolled: the pairs are constants, a factor is one product of two registers; the
+        // pairs r < s first, their sum doubled, then the pairs r = s
+        constexpr PairList<MT> pr{};
+        constexpr int NP = MT * (MT + 1) / 2, NO = MT * (MT - 1) / 2, NG = (NP + 3) / 4;
+        float nf[MT];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-      uint2 mcur = __ldg(mp);
-      uint4 bcur = __ldg(base);
-      for (int gi = 0; gi < ng; ++gi) {
-        if (gi + 1 < ng) {
-          mp += t.bk_S;
-          ++base;
+        for (int m = 0; m < MT; ++m) nf[m] = occ_float<NW>(ob, m);
+        float4 x[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        uint2 mcur = __ldg(mp);
+        uint4 bcur = __ldg(base);
+#pragma unroll
+        for (int gi = 0; gi < NG; ++gi) {
+          const uint32_t ix[4] = {bcur.x + (mcur.x & 0xffffu), bcur.y + (mcur.x >> 16), bcur.z + (mcur.y & 0xffffu),
+                                  bcur.w + (mcur.y >> 16)};
+          if (gi + 1 < NG) {
+            mcur = __ldg(mp + (size_t)(gi + 1) * t.bk_S);
+            bcur = __ldg(base + gi + 1);
+          }
+          float A[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const int i = 4 * gi + c;
+            if (i >= NP) break;
+            A[c] = i < NO ? nf[pr.r[i]] * nf[pr.s[i]] : nf[pr.r[i]] * (nf[pr.r[i]] - 1.f);  // exact
+            const bool act = A[c] != 0.f, ok = act && ix[c] < nG;
+            bad |= act && !ok;
+            if (ok) x[c] = __ldg(a.g + ix[c]);
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const int i = 4 * gi + c;
+            if (i >= NP) break;
+            if (i == NO) acc[0] = dfc{f2_add(acc[0].h, acc[0].h), f2_add(acc[0].l, acc[0].l)};
+            if (__any_sync(0xffffffffu, A[c] != 0.f))
+              dfc_fma_int(acc[0], f2_pack(A[c], A[c]), f2_pack(-A[c], -A[c]), f2_pack(x[c].x, x[c].y),
+                          f2_pack(x[c].z, x[c].w));
+          }
+          acc[0] = dfc_renorm(acc[0]);  // keep |lo| below an ulp of hi
         }
-        const uint2 mnext = __ldg(mp);
-        const uint4 bnext = __ldg(base);
-        const uint4 sl = sinfo[gi];
-        const float4 ca = scoef[2 * gi], cb = scoef[2 * gi + 1];
-        const uint32_t sel[4] = {sl.x, sl.y, sl.z, sl.w};
-        const float del[4] = {ca.x, ca.z, cb.x, cb.z}, mul[4] = {ca.y, ca.w, cb.y, cb.w};
-        const uint32_t ix[4] = {bcur.x + (mcur.x & 0xffffu), bcur.y + (mcur.x >> 16), bcur.z + (mcur.y & 0xffffu),
-                                bcur.w + (mcur.y >> 16)};
-        float A[4];
+      } else {
+        float4 x[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          A[c] = (occ_float23<NW>(ob, sel[c], (sel[c] & 0x8000u) != 0u) - 8388608.0f) * mul[c] *
-                 (occ_float23<NW>(ob, sel[c] >> 16, (sel[c] & 0x80000000u) != 0u) - del[c]);  // exact
-          const bool act = A[c] != 0.f, ok = act && ix[c] < nG;
-          bad |= act && !ok;
-          if (ok) x[c] = __ldg(a.g + ix[c]);
+        for (int c = 0; c < 4; ++c) x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        uint2 mcur = __ldg(mp);
+        uint4 bcur = __ldg(base);
+        for (int gi = 0; gi < ng; ++gi) {
+          if (gi + 1 < ng) {
+            mp += t.bk_S;
+            ++base;
+          }
+          const uint2 mnext = __ldg(mp);
+          const uint4 bnext = __ldg(base);
+          const uint4 sl = sinfo[gi];
+          const float4 ca = scoef[2 * gi], cb = scoef[2 * gi + 1];
+          const uint32_t sel[4] = {sl.x, sl.y, sl.z, sl.w};
+          const float del[4] = {ca.x, ca.z, cb.x, cb.z}, mul[4] = {ca.y, ca.w, cb.y, cb.w};
+          const uint32_t ix[4] = {bcur.x + (mcur.x & 0xffffu), bcur.y + (mcur.x >> 16), bcur.z + (mcur.y & 0xffffu),
+                                  bcur.w + (mcur.y >> 16)};
+          float A[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            A[c] = (occ_float23<NW>(ob, sel[c], (sel[c] & 0x8000u) != 0u) - 8388608.0f) * mul[c] *
+                   (occ_float23<NW>(ob, sel[c] >> 16, (sel[c] & 0x80000000u) != 0u) - del[c]);  // exact
+            const bool act = A[c] != 0.f, ok = act && ix[c] < nG;
+            bad |= act && !ok;
+            if (ok) x[c] = __ldg(a.g + ix[c]);
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (__any_sync(0xffffffffu, A[c] != 0.f))
+              dfc_fma_int(acc[0], f2_pack(A[c], A[c]), f2_pack(-A[c], -A[c]), f2_pack(x[c].x, x[c].y),
+                          f2_pack(x[c].z, x[c].w));
+          acc[0] = dfc_renorm(acc[0]);  // keep |lo| below an ulp of hi
+          mcur = mnext;
+          bcur = bnext;
         }
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (__any_sync(0xffffffffu, A[c] != 0.f))
-            dfc_fma_int(acc[0], f2_pack(A[c], A[c]), f2_pack(-A[c], -A[c]), f2_pack(x[c].x, x[c].y),
-                        f2_pack(x[c].z, x[c].w));
-        acc[0] = dfc_renorm(acc[0]);  // keep |lo| below an ulp of hi
-        mcur = mnext;
-        bcur = bnext;
       }
       if (bad) atomicOr(a.status, 1);
       if (valid) stage_epilogue<MT, 1, KIND, true, NW>(t, a, mode, g, g, acc, ob, bil_l, bil_w, dot64);
@@ -256,7 +326,7 @@ __global__ void __launch_bounds__(KIND == KIND_BIL ? 512 : 1024, 1)
 
 template <int NT, bool DOT>
 int ann_launch(const Tables& t, const DfArgs& a, int shape, cudaStream_t st, int* grid_out) {
-  auto k = ann_kernel<NT, DOT>;
+  auto k = t.fa_every ? ann_kernel<NT, DOT, true> : ann_kernel<NT, DOT, false>;
   const size_t smem = ann_smem_bytes(t);
   int grid = 0, warps = 0;
   const int rc = stage_geometry(k, a.low1 - a.low0, shape, 32, smem, &warps, &grid);

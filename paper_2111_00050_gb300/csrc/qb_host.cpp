@@ -138,6 +138,7 @@ static void build_block_tables(Space& sp, bool factored) {
   std::vector<uint32_t> info(2 * (size_t)std::max(1, nrec));
   std::vector<float> Gr(2 * (size_t)t.bk_T, 0.f), Gi(2 * (size_t)t.bk_T, 0.f);
   std::vector<int32_t> psh((size_t)M * TS, 0), EC((size_t)t.rem_w * twoQ, 0), cls(2 * (size_t)(nmax + 1) * Q);
+  std::vector<uint32_t> combo(t.bk_T, 0xffffffffu);
   for (int i = 0; i < nrec; ++i) {
     const Record& R = recs[i];
     int after = 0;  // first partner with a larger pair index (partners ascend)
@@ -149,6 +150,7 @@ static void build_block_tables(Space& sp, bool factored) {
         g[0] = (float)G[2 * j + k];
         g[1] = (float)(G[2 * j + k] - (double)g[0]);
       }
+      combo[sl] = (uint32_t)j;
       for (int m = 1; m < M; ++m) psh[(size_t)m * TS + sl] = delta[j][m];
     }
     const uint32_t r = (uint32_t)annR[R.pair], q = (uint32_t)annS[R.pair];
@@ -183,6 +185,7 @@ static void build_block_tables(Space& sp, bool factored) {
   put(3, psh.data(), 4 * psh.size());
   put(4, EC.data(), 4 * EC.size());
   put(5, cls.data(), 4 * cls.size());
+  put(7, combo.data(), 4 * combo.size());
   sp.bk_off[6] = sp.bk.size();
   sp.bk_map_bytes = ((size_t)std::max(1, nrec) * t.bk_S * 2 * w + 255) & ~(size_t)255;
 }
@@ -215,12 +218,14 @@ static bool build_factored(Space& sp) {
     return cd(sp.Lsym[2 * ix], sp.Lsym[2 * ix + 1]);
   };
   std::vector<float> lam(2 * (size_t)nc);
+  std::vector<double> lam64(nc);
   for (int k = 0; k < nc; ++k) {
     const cd l0 = LS(cls[k][0], cls[k][0]);
     if (l0.imag() != 0.0) return false;
     for (auto a : cls[k])
       for (auto b : cls[k])
         if (LS(a, b) != l0) return false;
+    lam64[k] = l0.real();
     lam[2 * k] = (float)l0.real();
     lam[2 * k + 1] = (float)(l0.real() - (double)lam[2 * k]);
   }
@@ -287,15 +292,18 @@ static bool build_factored(Space& sp) {
   }
   t.fa_nrec = (int)rec.size() / 2;
   t.fa_nc = nc;
-  // creation groups: the pairs r <= s in order
+  // creation groups: the pairs r < s, then r = s
   std::vector<std::pair<int, int>> cre;
   for (int r = 0; r < M; ++r)
-    for (int s = r; s < M; ++s) cre.push_back({r, s});
+    for (int s = r + 1; s < M; ++s) cre.push_back({r, s});
+  for (int r = 0; r < M; ++r) cre.push_back({r, r});
   while (cre.size() % 4) cre.push_back({-1, -1});
   t.fa_ng = (int)cre.size() / 4;
   const int Ta = fa_Ta(t), Tc = fa_Tc(t);
   std::vector<int32_t> kc(Tc, 0), psa((size_t)M * Ta, 0), psc((size_t)M * Tc, 0);
-  std::vector<uint32_t> info(Tc, 0u);
+  std::vector<uint32_t> info(Tc, 0u), pqa(Ta, 0u);
+  for (int i = 0; i < Ta; ++i)
+    if (slot[i].first >= 0) pqa[i] = (uint32_t)slot[i].first | ((uint32_t)slot[i].second << 8);
   std::vector<float> coef(2 * (size_t)Tc, 0.f);
   auto shift = [&](std::pair<int, int> pr, int m, int sign) {
     const int dc = (pr.first >= m) + (pr.second >= m);
@@ -333,8 +341,12 @@ static bool build_factored(Space& sp) {
   put(goff.data(), 4 * goff.size());
   put(sp.lowN.data(), 4 * sp.lowN.size());
   put(sp.lowK.data(), 4 * sp.lowK.size());
+  at = 15;
+  put(lam64.data(), 8 * lam64.size());
+  put(pqa.data(), 4 * pqa.size());
   sp.fa_off[13] = sp.fa.size();
   t.fa_nlow = nlow;
+  t.fa_every = std::find(goff.begin(), goff.end(), kNoIndex) == goff.end() ? 1 : 0;
   t.fa_low = sp.lowOff.back();
   t.fa_nG = nG;
   t.fa_on = 1;
@@ -874,6 +886,8 @@ void qb_space_free(qb_space* space) {
   cudaFree(sp->d_fa);
   cudaFree(sp->d_fill);
   cudaFree(sp->d_low);
+  cudaFree(sp->d_perm);
+  cudaFree(sp->d_hpsi);
   for (int k = 0; k < 2; ++k) {
     cudaFree(sp->d_blocks[k]);
     cudaFree(sp->d_base[k]);

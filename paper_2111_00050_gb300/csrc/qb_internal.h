@@ -2,6 +2,7 @@
 // kernels (qb_kernels.cu).  Not part of the public ABI (include/qb.h).
 #pragma once
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -118,6 +119,7 @@ struct Tables {
                             //   2^23 + [r = s]
   const float2* bk_G;       // [T] real coupling (hi, lo); bk_Gi: imaginary
   const float2* bk_Gi;
+  const uint32_t* bk_combo; // [T] combination of the slot, or 0xffffffff
   const int32_t* bk_psh;    // [M][T + 4] shift of the suffix index at mode m (a term conserves N and K: 0 for m = 0; 0 for unused slots)
   const int32_t* bk_EC;     // [rem_w][2Q] ranking-table rows of mode P plus the size of the class
   const int2* bk_cls;       // [nmax + 1][Q] (first filling, size) of each class
@@ -130,12 +132,15 @@ struct Tables {
   // fa_pl groups of four (odd M, momentum mod M: fa_nt pairs, the pair p = q last), or
   // (fa_nt = 0) up to four pairs of a class.  Creation groups: four pairs (r, s) each.
   int fa_on, fa_nt, fa_pl, fa_nrec, fa_nc, fa_ng;
+  int fa_every;                // 1: every class of every lower sector has its raised sector
   int fa_nlow;                 // lower sectors
   int64_t fa_low;              // lower kets
   int64_t fa_nG;
   const uint2* fa_rec;         // [fa_nrec] x: class | pairs << 8 | double the sum before pair (0-4; 7: never) << 12 |
                                //   last record of the class << 16
   const float2* fa_lam;        // [fa_nc] lam_k (hi, lo)
+  const double* fa_lam64;      // [fa_nc] lam_k
+  const uint32_t* fa_pqa;      // [fa_Ta] p | q << 8 of each annihilation slot
   const int32_t* fa_ka;        // [fa_Ta] class of each annihilation slot
   const int32_t* fa_kc;        // [fa_Tc] class of each creation slot
   const int32_t* fa_psa;       // [M][fa_Ta] shift of the suffix index when the slot's pair is added
@@ -152,9 +157,11 @@ struct Tables {
   const uint32_t* fa_rblk;     // [ceil(fa_low / 32)] block of every 32nd lower ket
   const uint32_t* fa_basea;    // [lower blocks][fa_rowa] raised target blocks, then the classes' entries (qb_factor.cuh)
   const uint32_t* fa_basec;    // [blocks][fa_Tc] index in the vector of B_k f of the lowered target blocks
+  const uint32_t* fa_perm;     // [ceil(fa_low / 32)] order of the rounds (qb_factor.cuh), or NULL
   const double* fa_wk;         // [fa_low] their ket weights, or NULL
 };
-__host__ __device__ inline int fa_rowa(const Tables& t) { return t.fa_nrec * t.fa_pl * 4 + ((t.fa_nc + 3) & ~3); }
+// a row of fa_basea: the slots, the classes' entries, the mask of records with a held class
+__host__ __device__ inline int fa_rowa(const Tables& t) { return t.fa_nrec * t.fa_pl * 4 + ((t.fa_nc + 4) & ~3); }
 __host__ __device__ inline int fa_Ta(const Tables& t) { return t.fa_nrec * t.fa_pl * 4; }
 __host__ __device__ inline int fa_Tc(const Tables& t) { return t.fa_ng * 4; }
 
@@ -181,9 +188,9 @@ struct Space {
   std::vector<unsigned char> blob;        // host copy of the shared-memory image
   Combos combos;
   std::vector<unsigned char> bk;          // block tables but the maps (image of d_bk's first bytes)
-  size_t bk_off[7] = {0};                 // byte offsets of info, G, Gi, psh, EC, cls and the maps in d_bk
+  size_t bk_off[8] = {0};                 // byte offsets of info, G, Gi, psh, EC, cls, the maps and combo in d_bk
   std::vector<unsigned char> fa;          // tables of the factored couplings but the maps (image of d_fa's first bytes)
-  size_t fa_off[15] = {0};
+  size_t fa_off[17] = {0};
   std::vector<int> lowN, lowK;            // lower sectors
   std::vector<int64_t> lowOff;
   bool low_held = false;                  // the lower kets are the space's first kets
@@ -206,6 +213,9 @@ struct Space {
   uint32_t* d_fill = nullptr;     // fillings (Tables::fill)
   unsigned char* d_low = nullptr; // occupations and fillings of the lower kets
   uint32_t* d_blocks[2] = {nullptr, nullptr};  // rblk and the block starts of the kets, and of the lower kets
+  void* d_hpsi = nullptr;      // FP64 vector of B_k psi (qb_hpsi of a factored space), made by the first call
+  std::mutex hpsi_mu;          // held by the call that uses it
+  uint32_t* d_perm = nullptr;                  // Tables::fa_perm
   uint32_t* d_base[2] = {nullptr, nullptr};    // bases of the blocks, and of the lower blocks
   int64_t scratch_doubles = 0;
   Tables t{};
@@ -249,7 +259,8 @@ inline double* prep_area(const Space& s) { return init_final(s) + 2; }
 inline double* prep_final(const Space& s) { return prep_area(s) + max_grid_of(s) * nprep(s.M); }
 
 // launchers (qb_kernels.cu); all return a QB_* status
-int launch_hpsi(const Space& s, const void* d_v, void* d_out, void* stream);
+int launch_hpsi(Space& s, const void* d_v, void* d_out, void* stream);
+int launch_hpsi_rows(const Space& s, const void* d_v, void* d_out, cudaStream_t st);  // thread per row, no tables of blocks
 int launch_rk4(Space& s, void* d_psi, int batch, const double* scale, double dt, int64_t steps, void* d_work,
                void* stream, bool plain = false);
 int launch_unrank(const Space& s, int64_t first, int64_t count, int* d_occ, void* stream);

@@ -518,11 +518,53 @@ __global__ void __launch_bounds__(256) raised_base_kernel(const Tables t, const 
         v = (uint32_t)__ldg(t.sec_off + __ldg(t.sec_of + (s.N + 2) * t.Q + (s.K + k) % t.Q) + 1) - sum;
       if (t0 + lane < Ta) basea[(size_t)b * row + tt] = v;
     }
+    // bit i: the class of record i (of the first 32) has a raised sector
+    uint32_t held = 0;
+    if (lane < t.fa_nrec && __ldg(t.fa_goff + lid * t.fa_nc + (__ldg(&t.fa_rec[lane].x) & 0xffu)) != kNoIndex) held = 1u;
+    held = __ballot_sync(0xffffffffu, held != 0u);
     for (int k = lane; k < row - Ta; k += 32) {
       uint32_t v = 0;
       if (k < t.fa_nc) v = __ldg(t.fa_goff + lid * t.fa_nc + k) - (uint32_t)__ldg(t.fa_lowoff + lid);
+      if (k == t.fa_nc) v = held;
       basea[(size_t)b * row + Ta + k] = v;
     }
+  }
+}
+
+// Order of the lower rounds: within a layer (equal N) of S sectors, which are nearly equal
+// in size, position j of the layer's n rounds is round (j mod S) ceil(n / S) + j / S, the
+// positions beyond the last segment's end moved up.
+__global__ void __launch_bounds__(256) round_order_kernel(const Tables t, const int32_t* lowN, uint32_t* perm) {
+  const int64_t nr = (t.fa_low + 31) / 32;
+  for (int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x; r < nr; r += (int64_t)gridDim.x * 256) {
+    // the layer of round r: the rounds [floor(first / 32), floor(end / 32)) of its kets
+    int lo = 0, hi = t.fa_nlow - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (__ldg(t.fa_lowoff + mid) / 32 <= r)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    int a = lo, b = lo;
+    while (a > 0 && lowN[a - 1] == lowN[lo]) --a;
+    while (b + 1 < t.fa_nlow && lowN[b + 1] == lowN[lo]) ++b;
+    const int64_t ra = __ldg(t.fa_lowoff + a) / 32, rb = b + 1 < t.fa_nlow ? __ldg(t.fa_lowoff + b + 1) / 32 : nr;
+    const int64_t S = b - a + 1, n = rb - ra, len = (n + S - 1) / S, j = r - ra;
+    // full columns: len - 1 of them where the last segment is short
+    const int64_t lastlen = n - (S - 1) * len;  // of segment S - 1 (may be <= 0)
+    int64_t seg, pos;
+    if (lastlen < 0) {  // fewer rounds than segments need: as they come
+      seg = 0;
+      pos = j;
+    } else if (j < lastlen * S) {
+      seg = j % S;
+      pos = j / S;
+    } else {
+      seg = (j - lastlen * S) % (S - 1);
+      pos = lastlen + (j - lastlen * S) / (S - 1);
+    }
+    perm[r] = (uint32_t)(ra + seg * len + pos);
   }
 }
 
@@ -1006,6 +1048,7 @@ int device_setup(Space& s) {
     t.bk_psh = reinterpret_cast<const int32_t*>(s.d_bk + s.bk_off[3]);
     t.bk_EC = reinterpret_cast<const int32_t*>(s.d_bk + s.bk_off[4]);
     t.bk_cls = reinterpret_cast<const int2*>(s.d_bk + s.bk_off[5]);
+    t.bk_combo = reinterpret_cast<const uint32_t*>(s.d_bk + s.bk_off[7]);
     t.bk_map = s.d_bk + s.bk_off[6];
     t.bk_map5 = reinterpret_cast<const uint16_t*>(s.d_bk + s.bk_off[6] + s.bk_map_bytes);
     QB_CUDA(cudaMalloc(&s.d_fill, sizeof(uint32_t) * (size_t)t.total));
@@ -1056,6 +1099,8 @@ int device_setup(Space& s) {
     t.fa_lowoff = reinterpret_cast<const int64_t*>(at(9));
     t.fa_goff = reinterpret_cast<const uint32_t*>(at(10));
     t.fa_basec = s.d_base[0];
+    t.fa_lam64 = reinterpret_cast<const double*>(at(15));
+    t.fa_pqa = reinterpret_cast<const uint32_t*>(at(16));
     t.fa_mapa = reinterpret_cast<const uint2*>(at(13));
     t.fa_mapc = reinterpret_cast<const uint2*>(at(14));
     uint32_t* lstart = start;
@@ -1091,6 +1136,13 @@ int device_setup(Space& s) {
       rc = find_blocks(fill, t.fa_low, &s.d_blocks[1], &lstart, &lblocks);
       if (rc) return rc;
       t.fa_rblk = s.d_blocks[1];
+    }
+    {
+      const int64_t nr = (t.fa_low + 31) / 32;
+      QB_CUDA(cudaMalloc(&s.d_perm, sizeof(uint32_t) * (size_t)nr));
+      round_order_kernel<<<base_grid, 256>>>(t, reinterpret_cast<const int32_t*>(at(11)), s.d_perm);
+      QB_CUDA(cudaGetLastError());
+      t.fa_perm = s.d_perm;
     }
     QB_CUDA(cudaMalloc(&s.d_base[1], sizeof(uint32_t) * (size_t)lblocks * fa_rowa(t)));
     t.fa_basea = s.d_base[1];
@@ -1130,16 +1182,13 @@ static int launch_stage_c(const Space& s, const StageArgs& a, cudaStream_t st, i
                         : launch_stage<MODE, B, false>(s, a, st, grid_out);
 }
 
-int launch_hpsi(const Space& s, const void* d_v, void* d_out, void* stream) {
-  cudaStream_t st = (cudaStream_t)stream;
+int launch_hpsi_rows(const Space& s, const void* d_v, void* d_out, cudaStream_t st) {
   StageArgs a{};
   a.vin = (const double2*)d_v;
   a.out = (double2*)d_out;
   a.scale[0] = 1.0;
   a.status = reinterpret_cast<int*>(s.d_scratch);
-  int rc = launch_stage_c<MODE_HPSI, 1>(s, a, st);
-  if (rc) return rc;
-  return check_status(s, st);
+  return launch_stage_c<MODE_HPSI, 1>(s, a, st);
 }
 
 // plain = true: one launch per sector per stage (the comparison baseline of
