@@ -190,15 +190,6 @@ __global__ void __launch_bounds__(kBlock) mixed_kernel(const Tables t, const dou
   }
 }
 
-// acc[c] += weight * sum_k partial[k][c], summed in a fixed order
-__global__ void accumulate_kernel(const double* partial, int n, int width, double weight, double* acc) {
-  for (int c = threadIdx.x; c < width; c += blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < n; ++k) s += partial[(size_t)k * width + c];
-    acc[c] += weight * s;
-  }
-}
-
 struct AdjointLayout {
   int64_t n;  // kets
   int64_t nck;
@@ -413,7 +404,7 @@ static int adjoint_impl(qb_space* space, const double* z, double scale, double d
     int r = stage_launch(sp->t, a, mode, 1, cplx, st, &grid, bil, 0);
     if (r) return r;
     if (bil) {
-      accumulate_kernel<<<1, 32, 0, st>>>(L.partial, grid, M + 1, weight, L.acc);
+      sum_rows_kernel<<<M + 1, kSumThreads, 0, st>>>(L.partial, grid, M + 1, weight, true, L.acc);
       QB_CUDA(cudaGetLastError());
       // coupling gradient: <forward stage vector, O costate> for every two-body O
       if (grad_L) {
@@ -501,14 +492,14 @@ static int adjoint_impl(qb_space* space, const double* z, double scale, double d
     const int width = 2 * (M + 1);
     mixed_kernel<<<grid, kBlock, smem, st>>>(sp->t, L.lam, L.psi, L.partial, status);
     QB_CUDA(cudaGetLastError());
-    QB_CUDA(cudaMemsetAsync(L.fin, 0, 8 * width, st));
-    accumulate_kernel<<<1, 64, 0, st>>>(L.partial, grid, width, 1.0, L.fin);
+    sum_rows_kernel<<<width, kSumThreads, 0, st>>>(L.partial, grid, width, 1.0, false, L.fin);
+    QB_CUDA(cudaGetLastError());
     QB_CUDA(cudaMemcpyAsync(lamps.data(), L.fin, 8 * width, cudaMemcpyDeviceToHost, st));
     QB_CUDA(cudaStreamSynchronize(st));
     mixed_kernel<<<grid, kBlock, smem, st>>>(sp->t, L.psi, L.psi, L.partial, status);
     QB_CUDA(cudaGetLastError());
-    QB_CUDA(cudaMemsetAsync(L.fin, 0, 8 * width, st));
-    accumulate_kernel<<<1, 64, 0, st>>>(L.partial, grid, width, 1.0, L.fin);
+    sum_rows_kernel<<<width, kSumThreads, 0, st>>>(L.partial, grid, width, 1.0, false, L.fin);
+    QB_CUDA(cudaGetLastError());
     QB_CUDA(cudaMemcpyAsync(psips.data(), L.fin, 8 * width, cudaMemcpyDeviceToHost, st));
   }
   int hstat = 0;

@@ -152,7 +152,7 @@ __device__ __forceinline__ void add_record(dfc& acc, const float4 (&x)[Rec<KC>::
 // WHOLE: acc is the whole two-body part (factored couplings), else its off-diagonal part.
 template <int MT, int B, int KIND, bool WHOLE, int NW>
 __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a, int mode, int64_t gr, int64_t ri,
-                                               const dfc (&acc)[B], const uint32_t (&ob)[NW], dfl& bil_l, dfl* bil_w,
+                                               const dfc (&acc)[B], const uint32_t (&ob)[NW], dfl& bil_l, dfc* bil_w,
                                                double& dot64) {
   constexpr bool BIL = (KIND == KIND_BIL), DOT = (KIND == KIND_DOT);
   constexpr int kMB = (MT > 0) ? MT : 16;
@@ -198,10 +198,14 @@ __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a,
       bil_l = df_add(bil_l, df_add(df_mul(pr, li), df_neg(df_mul(pi, lr))));
       // Im(conj(x) p) = x.re p.im - x.im p.re, weighted by each occupation
       const dfl tx = df_add(df_mul(xr, pi), df_neg(df_mul(xi, pr)));
+      // two modes a packed sum, the occupations exact
+      const f2 th = f2_pack(tx.h, tx.h), tl = f2_pack(tx.l, tx.l);
 #pragma unroll
-      for (int q = 0; q < kMB; ++q) {
+      for (int q = 0; q < kMB; q += 2) {
         if (q >= M) break;
-        bil_w[q] = df_add(bil_w[q], df_mul(dfl{occ_float<NW>(ob, q), 0.f}, tx));
+        const float n0 = occ_float<NW>(ob, q), n1 = q + 1 < kMB ? occ_float<NW>(ob, q + 1) : 0.f;
+        dfc_fma_int(bil_w[q / 2], f2_pack(n0, n1), f2_pack(-n0, -n1), th, tl);
+        bil_w[q / 2] = dfc_renorm(bil_w[q / 2]);
       }
     }
     if (mode == 0 || mode == 2) {
@@ -252,24 +256,30 @@ __device__ __forceinline__ uint32_t block_of_lane(const RoundIn& in, int lane, b
   return in.first + __popc(heads & (0xffffffffu >> (31 - lane)));
 }
 
-// Threads a CTA's registers are planned for (65,536 registers per SM): the one-state
-// stages at 64 a thread, the wider ones (bilinear accumulators, sweep members) at 128.
+// Threads a CTA's registers are planned for (65,536 registers per SM): the one-state stages
+// at 64 a thread, the bilinear ones at 80 (one stage of 2.3M kets at M = 5: 265 us at 128,
+// 200 at 80, 192 at 64 where that does not spill), the sweep members at 128.
 template <int B, int KIND>
 __host__ __device__ constexpr int blk_max_threads() {
-  return (B == 1 && KIND != KIND_BIL) ? 1024 : 512;
+  return KIND == KIND_BIL ? 768 : (B == 1 ? 1024 : 512);
 }
 
 // per-CTA sums of the bilinears in a fixed order: lanes by shuffles, warps in turn
 template <int kMB>
-__device__ __forceinline__ void bil_reduce(const DfArgs& a, int M, const dfl& bil_l, const dfl* bil_w) {
-  __shared__ double red[16][17];
+__device__ __forceinline__ void bil_reduce(const DfArgs& a, int M, const dfl& bil_l, const dfc* bil_w) {
+  __shared__ double red[32][17];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const int nq = M + 1;
   for (int q = 0; q < nq; ++q) {
     double val = (q == 0) ? df_to(bil_l) : 0.0;
 #pragma unroll
     for (int u = 0; u < kMB; ++u)
-      if (q == u + 1) val = df_to(bil_w[u]);
+      if (q == u + 1) {
+        float h0, h1, l0, l1;
+        f2_unpack(bil_w[u / 2].h, h0, h1);
+        f2_unpack(bil_w[u / 2].l, l0, l1);
+        val = u % 2 ? (double)h1 + (double)l1 : (double)h0 + (double)l0;
+      }
     for (int o = 16; o > 0; o >>= 1) val += __shfl_down_sync(0xffffffffu, val, o);
     if (lane == 0) red[warp][q] = val;
   }
@@ -330,9 +340,9 @@ __global__ void __launch_bounds__((U > 1 ? 256 : blk_max_threads<B, KIND>()), 1)
 
   const int64_t total = t.total;
   dfl bil_l{0.f, 0.f};
-  dfl bil_w[BIL ? kMB : 1];
+  dfc bil_w[BIL ? (kMB + 1) / 2 : 1];
 #pragma unroll
-  for (int q = 0; q < (BIL ? kMB : 1); ++q) bil_w[q] = dfl{0.f, 0.f};
+  for (int q = 0; q < (BIL ? (kMB + 1) / 2 : 1); ++q) bil_w[q] = dfc{0ull, 0ull};
   double dot64 = 0.0;
 
   // the last rounds (the most particles, the most pairs per ket) first
@@ -582,14 +592,12 @@ int fac_launch_any(const Tables&, const DfArgs&, int, int, bool, int, cudaStream
 inline int stage_launch(const Tables& t, const DfArgs& a, int mode, int B, bool cplx, cudaStream_t st,
                         int* grid_out = nullptr, bool bil = false, int shape = 0) {
   if (t.fa_on) {
-    if (t.fa_nt > 0) {
-      switch (t.M) {
-        case 5: return fac_launch_m5(t, a, mode, B, bil, shape, st, grid_out);
-        case 7: return fac_launch_m7(t, a, mode, B, bil, shape, st, grid_out);
-        case 9: return fac_launch_m9(t, a, mode, B, bil, shape, st, grid_out);
-        case 11: return fac_launch_m11(t, a, mode, B, bil, shape, st, grid_out);
-        default: break;
-      }
+    switch (t.M) {
+      case 5: return fac_launch_m5(t, a, mode, B, bil, shape, st, grid_out);
+      case 7: return fac_launch_m7(t, a, mode, B, bil, shape, st, grid_out);
+      case 9: return fac_launch_m9(t, a, mode, B, bil, shape, st, grid_out);
+      case 11: return fac_launch_m11(t, a, mode, B, bil, shape, st, grid_out);
+      default: break;
     }
     return fac_launch_any(t, a, mode, B, bil, shape, st, grid_out);
   }

@@ -31,7 +31,6 @@ struct View {
   const double* G;
   const int8_t* delta;
   const int32_t* ann;
-  const int32_t* hs;
   const uint8_t* pairidx;
   const double* w;
   const double* gd;
@@ -47,7 +46,6 @@ __device__ __forceinline__ View view_at(const Tables& t, const unsigned char* s)
   v.G = (const double*)(s + t.o_G);
   v.delta = (const int8_t*)(s + t.o_delta);
   v.ann = (const int32_t*)(s + t.o_ann);
-  v.hs = (const int32_t*)(s + t.o_hs);
   v.pairidx = (const uint8_t*)(s + t.o_pairidx);
   v.w = (const double*)(s + t.o_w);
   v.gd = (const double*)(s + t.o_gd);
@@ -84,15 +82,6 @@ __device__ __forceinline__ View make_view(const Tables& t, const unsigned char* 
 __device__ __forceinline__ int delta_shift(const Tables& t, const View& v, int j, int m) {
   if (t.exact) return (int)reinterpret_cast<const int16_t*>(v.delta)[j * 16 + m];
   return (int)reinterpret_cast<const uint8_t*>(v.delta)[j * 16 + m] - kDeltaBias;
-}
-
-// Copies the table image from byte offset `from` on (16-byte aligned) into
-// shared memory; the stage kernels leave the fill counts in global memory.
-__device__ __forceinline__ void load_blob_from(const Tables& t, unsigned char* smem, int from) {
-  const int4* src = reinterpret_cast<const int4*>(t.blob + from);
-  int4* dst = reinterpret_cast<int4*>(smem);
-  for (int i = threadIdx.x; i < (t.blob_bytes - from) / 16; i += blockDim.x) dst[i] = __ldg(src + i);
-  __syncthreads();
 }
 
 // Per-thread scratch rows in shared memory, laid out [m][thread] so that the
@@ -370,6 +359,28 @@ __device__ __forceinline__ void dfc_fma(dfc& acc, f2 ch, f2 nch, f2 cl, f2 xh, f
   acc.l = f2_add(acc.l, f2_add(err, e));
 }
 
+// acc += x, both double-float: TwoSum of the high parts, the rest in acc.l
+__device__ __forceinline__ void dfc_add(dfc& acc, f2 xh, f2 xl) {
+  const f2 s = f2_add(acc.h, xh);
+  const f2 bb = f2_sub(s, acc.h);
+  const f2 err = f2_add(f2_sub(acc.h, f2_sub(s, bb)), f2_sub(xh, bb));
+  acc.h = s;
+  acc.l = f2_add(acc.l, f2_add(err, xl));
+}
+
+// acc += a * x for an exact small a (a2 = (a, a), na2 = -a2)
+__device__ __forceinline__ void dfc_fma_int(dfc& acc, f2 a2, f2 na2, f2 xh, f2 xl) {
+  const f2 pn = f2_mul(na2, xh);  // -fl(a x.h)
+  f2 e = f2_fma(a2, xh, pn);      // exact error of that product
+  e = f2_fma(a2, xl, e);
+  const f2 s = f2_sub(acc.h, pn);
+  const f2 bb = f2_sub(s, acc.h);
+  const f2 err = f2_sub(f2_sub(acc.h, f2_sub(s, bb)), f2_add(pn, bb));
+  acc.h = s;
+  acc.l = f2_add(acc.l, f2_add(err, e));
+}
+
+
 __device__ __forceinline__ dfc dfc_renorm(dfc a) {
   const f2 h = f2_add(a.h, a.l);
   return {h, f2_sub(a.l, f2_sub(h, a.h))};
@@ -403,6 +414,27 @@ struct DfArgs {
   float2 zf;           // zre as double-float
   int* status;
 };
+
+// Sums of the columns c0, c0 + 1, ... of partial[n][width], one CTA of kSumThreads a column:
+// rows dealt to the threads in order, then a tree (a fixed order, the same for every launch of the same
+// n).  out[c] = sum, or out[c] += weight * sum.  One thread adding 2,432 rows in turn took
+// 16 to 33 us a launch.
+constexpr int kSumThreads = 128;
+static __global__ void __launch_bounds__(kSumThreads) sum_rows_kernel(const double* partial, int n, int width,
+                                                                       double weight, bool add, double* out,
+                                                                       int c0 = 0) {
+  __shared__ double red[kSumThreads / 32];
+  const int c = c0 + blockIdx.x;
+  double s = 0.0;
+  for (int k = threadIdx.x; k < n; k += kSumThreads) s += partial[(size_t)k * width + c];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kSumThreads / 32; ++w) s += red[w];
+    out[c] = add ? out[c] + weight * s : s;
+  }
+}
 
 // Resident CTAs per SM of `kernel` with `smem` dynamic shared memory, cached
 // per (kernel, smem, block) so that launch loops do not repeat the occupancy query.

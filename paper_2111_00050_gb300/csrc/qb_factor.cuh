@@ -19,28 +19,6 @@
 
 namespace qb {
 
-// acc += x, both double-float: TwoSum of the high parts, the rest in acc.l
-__device__ __forceinline__ void dfc_add(dfc& acc, f2 xh, f2 xl) {
-  const f2 s = f2_add(acc.h, xh);
-  const f2 bb = f2_sub(s, acc.h);
-  const f2 err = f2_add(f2_sub(acc.h, f2_sub(s, bb)), f2_sub(xh, bb));
-  acc.h = s;
-  acc.l = f2_add(acc.l, f2_add(err, xl));
-}
-
-// acc += a * x for an exact small a (a2 = (a, a), na2 = -a2)
-__device__ __forceinline__ void dfc_fma_int(dfc& acc, f2 a2, f2 na2, f2 xh, f2 xl) {
-  const f2 pn = f2_mul(na2, xh);  // -fl(a x.h)
-  f2 e = f2_fma(a2, xh, pn);      // exact error of that product
-  e = f2_fma(a2, xl, e);
-  const f2 s = f2_sub(acc.h, pn);
-  const f2 bb = f2_sub(s, acc.h);
-  const f2 err = f2_sub(f2_sub(acc.h, f2_sub(s, bb)), f2_add(pn, bb));
-  acc.h = s;
-  acc.l = f2_add(acc.l, f2_add(err, e));
-}
-
-
 inline size_t ann_smem_bytes(const Tables& t) { return ((size_t)t.fa_nrec * 8 + t.fa_nc * 8 + 15) & ~(size_t)15; }
 
 // Rows of bases per lower block: the annihilation slots, then where each class's entries
@@ -204,7 +182,7 @@ struct PairList {
 inline size_t cre_smem_bytes(const Tables& t) { return (size_t)fa_Tc(t) * 12; }
 
 template <int MT, int KIND>
-__global__ void __launch_bounds__(KIND == KIND_BIL ? 512 : 1024, 1)
+__global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
     cre_kernel(const Tables t, const DfArgs a, const int mode) {
   constexpr int NW = occ_words<MT>();
   constexpr bool BIL = (KIND == KIND_BIL);
@@ -219,9 +197,9 @@ __global__ void __launch_bounds__(KIND == KIND_BIL ? 512 : 1024, 1)
   __syncthreads();
   const uint32_t nG = (uint32_t)t.fa_nG;
   dfl bil_l{0.f, 0.f};
-  dfl bil_w[BIL ? kMB : 1];
+  dfc bil_w[BIL ? (kMB + 1) / 2 : 1];
 #pragma unroll
-  for (int q = 0; q < (BIL ? kMB : 1); ++q) bil_w[q] = dfl{0.f, 0.f};
+  for (int q = 0; q < (BIL ? (kMB + 1) / 2 : 1); ++q) bil_w[q] = dfc{0ull, 0ull};
   double dot64 = 0.0;
 
   const int64_t r0 = a.row0 / 32, step = (int64_t)gridDim.x * warps;
@@ -342,7 +320,7 @@ int cre_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream
   auto k = cre_kernel<MT, KIND>;
   const size_t smem = cre_smem_bytes(t);
   int grid = 0, warps = 0;
-  const int rc = stage_geometry(k, a.row1 - a.row0, shape, KIND == KIND_BIL ? 16 : 32, smem, &warps, &grid);
+  const int rc = stage_geometry(k, a.row1 - a.row0, shape, blk_max_threads<1, KIND>() / 32, smem, &warps, &grid);
   if (rc) return rc;
   k<<<grid, 32 * warps, smem, st>>>(t, a, mode);
   QB_CUDA(cudaGetLastError());

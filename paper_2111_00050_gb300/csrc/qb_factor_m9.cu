@@ -3,6 +3,7 @@
 
 namespace qb {
 int fac_launch_m9(const Tables& t, const DfArgs& a, int mode, int B, bool bil, int shape, cudaStream_t st, int* grid) {
+  if (t.fa_nt == 0) return fac_launch<9, 0>(t, a, mode, B, bil, shape, st, grid);  // exact momentum
   return fac_launch<9, 5>(t, a, mode, B, bil, shape, st, grid);
 }
 }  // namespace qb

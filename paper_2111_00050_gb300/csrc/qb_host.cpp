@@ -195,19 +195,18 @@ static void build_block_tables(Space& sp, bool factored) {
 // is the same real number.  Then builds the tables of the factored stages (Tables::fa_*)
 // and the list of lower sectors; called once the sectors are known.
 //
-// Where the line lies (one stage, direct against factored kernels): two launches cost 5 us
-// more than one, so small spaces stay direct (M = 7, 19,448 kets: 13.0 against 13.3 us;
-// 245,157: 39.8 against 29.6), and with three pairs a class (M = 5) or fewer the second pass
-// costs what the fewer terms save (2.3M kets: 144 against 159 us).
-constexpr int64_t kFactorMin = 32768;
+// Where the line lies (one stage, direct against factored kernels, us): two launches cost
+// more than one, so small spaces stay direct (M = 7, 19,448 kets: 10.5 / 13.5; 245,157: 38 / 27;
+// M = 9, 35,530: 17.4 / 14.2; M = 11, 16,796: 19.0 / 14.9), and with three pairs a class
+// (M = 5) the second pass costs what the fewer terms save (2.3M kets: 138 / 149).
 constexpr int kFactorMinM = 6;
-
+constexpr int64_t factor_min(int M) { return M >= 9 ? 16384 : 32768; }
 
 static bool build_factored(Space& sp) {
   Tables& t = sp.t;
   const int M = sp.M, nmax = sp.nmax, Q = sp.Q, twoQ = 2 * Q;
   t.fa_on = 0;
-  if (M < kFactorMinM || sp.secOff.back() < kFactorMin || sp.secOff.back() >= (int64_t)kNoIndex) return false;
+  if (M < kFactorMinM || sp.secOff.back() < factor_min(M) || sp.secOff.back() >= (int64_t)kNoIndex) return false;
   const int nc = sp.exact ? 2 * M - 1 : M;
   std::vector<std::vector<std::pair<int, int>>> cls(nc);  // pairs p < q first, then p = q
   for (int d = 0; d < 2; ++d)
@@ -397,10 +396,6 @@ static int build_tables(Space& sp) {
   std::vector<uint32_t>& pq = sp.combos.pq;
   std::vector<double>& G = sp.combos.G;
   std::vector<std::vector<int>>& delta = sp.combos.delta;
-  std::vector<std::vector<int>> dex;    // [combo][16] shifts of the compact exact index
-  // exact momentum: width of mode m's window of suffix momenta, (M-1-m) nmax + 1
-  int exw[16] = {0};
-  for (int m = 1; m < M; ++m) exw[m] = (M - 1 - m) * nmax + 1;
   std::vector<double> gd;
   unsigned char(*pairidx)[16] = sp.combos.pairidx;
   memset(pairidx, 0xff, 256);
@@ -433,7 +428,6 @@ static int build_tables(Space& sp) {
           dn[s] -= 1;
           dn[p] += 1;
           dn[q] += 1;
-          std::vector<int> dx(16, 0);
           for (int m = lo + 1; m <= hi; ++m) {
             int dc = 0, dk = 0;
             for (int e = m; e < M; ++e) {
@@ -441,11 +435,8 @@ static int build_tables(Space& sp) {
               dk += dn[e] * e;
             }
             d[m] = dc * twoQ + modp(dk, Q);
-            // compact exact index: row (rem) by dc, column (skr - m rem) by dk - m dc
-            dx[m] = dc * exw[m] + dk - m * dc;
           }
           delta.push_back(d);
-          dex.push_back(dx);
         }
     }
   annStart.push_back((int)pq.size());
@@ -453,50 +444,16 @@ static int build_tables(Space& sp) {
   t.is_complex = cplx ? 1 : 0;
 
 
-  // shared-memory image: the stage kernels' tables first after the ranking table
-  // (ann .. dsw), so that they stage [E, delta) (mod M) or [ann, sqrt) (exact)
+  // the image that the row kernels stage in shared memory
   size_t off = 0;
-  t.ncp = (std::max(1, t.n_combo) + 3) & ~3;
-  const int nsw = std::max(1, M / 2);  // shift words of a term (modes 1 .. M-1, two per word)
   t.o_cnt = (int)off;
   off = align16(off + sizeof(uint32_t) * (size_t)(M + 1) * (nmax + 1) * Q);
   t.o_E = (int)off;
   off = align16(off + sizeof(int32_t) * (size_t)M * t.rem_w * twoQ);
-  // exact momentum: the compact ranking table, where it and the stage kernels' other
-  // tables and 12 warps' tiles fit a CTA's shared memory and its shifts fit 16 bits
-  t.o_Ex = (int)off;
-  t.ex_smem = 0;
-  if (sp.exact) {
-    size_t exb = 0;
-    int dmax = 0;
-    for (int m = 1; m < M; ++m) {
-      t.ex_w[m] = exw[m];
-      t.ex_base[m] = (int)exb;
-      exb += sizeof(int32_t) * (size_t)t.rem_w * exw[m];
-      dmax = std::max(dmax, 2 * exw[m] + 2 * (M - 1) + 2 * m);
-    }
-    const size_t rows = 64, iw = (size_t)M;
-    size_t wb = iw * rows * 4 + (((size_t)M * rows + 15) & ~(size_t)15) + rows * 4 + rows * 8 + rows +
-                2 * (size_t)(t.n_ann + 2) * 4;
-    wb = (wb + 15) & ~(size_t)15;
-    const size_t rest = 4096 + 32 * (size_t)std::max(1, t.n_combo) * 3 + 16 * (size_t)t.ncp + 1024;
-    if (exb + 12 * wb + rest <= 200 * 1024 && dmax <= 32767) {
-      t.ex_smem = 1;
-      off = align16(off + exb);
-    }
-  }
   t.o_ann = (int)off;
   off = align16(off + sizeof(int32_t) * (size_t)(t.n_ann + 1));
-  t.o_hs = (int)off;
-  off = align16(off + sizeof(int32_t) * (size_t)t.n_ann);
   t.o_pairidx = (int)off;
   off = align16(off + 256);
-  t.o_Gf = (int)off;
-  off = align16(off + sizeof(float) * 4 * (size_t)t.ncp);
-  t.o_dsw = (int)off;
-  off = align16(off + sizeof(uint32_t) * (size_t)std::max(2, nsw) * t.ncp);
-  t.o_dex = (int)off;
-  off = align16(off + (t.ex_smem ? (size_t)32 * std::max(1, t.n_combo) : 0));
   t.o_delta = (int)off;
   off = align16(off + (size_t)(sp.exact ? 32 : 16) * std::max(1, t.n_combo));
   t.o_sqrt = (int)off;
@@ -509,14 +466,12 @@ static int build_tables(Space& sp) {
   off = align16(off + sizeof(double) * (size_t)M);
   t.o_gd = (int)off;
   off = align16(off + sizeof(double) * (size_t)t.n_ann);
-  t.o_sqf = (int)off;
-  off = align16(off + sizeof(float) * 2 * (size_t)(nmax + 3));
   t.blob_bytes = (int)off;
-  // mod M: the stage kernels hold two ranking-table byte offsets per 32-bit word, so
-  // the table must span at most 64 KB (every space within the other limits does but
-  // M = 9 with 97 <= n_max <= 108, whose sectors exceed 2^31 kets anyway)
-  t.sw_ok = (!sp.exact && (int64_t)M * t.rem_w * twoQ * 4 <= 65536) ? 1 : 0;
-  if (!sp.exact && !t.sw_ok) return fail(QB_EUNSUPPORTED, "the ranking table exceeds 64 KB (reduce n_max)");
+  // mod M: the moments kernel holds two ranking-table byte offsets per 32-bit word, so the
+  // table must span at most 64 KB (every space within the other limits does but M = 9 with
+  // 97 <= n_max <= 108, whose sectors exceed 2^31 kets anyway)
+  if (!sp.exact && (int64_t)M * t.rem_w * twoQ * 4 > 65536)
+    return fail(QB_EUNSUPPORTED, "the ranking table exceeds 64 KB (reduce n_max)");
   // exact momentum: the fill counts and the ranking table grow with (M-1) n_max
   // and stay in global memory for every kernel
   t.sm_from = sp.exact ? t.o_ann : 0;
@@ -533,20 +488,6 @@ static int build_tables(Space& sp) {
         if (m >= 1 && rem >= 1 && rem - 1 <= nmax) v = (int32_t)sp.cnt[CI(m - 1, rem - 1, modp(kk - (m - 1), Q))];
         E[((size_t)m * t.rem_w + rr) * twoQ + kk] = v;
       }
-  if (t.ex_smem) {
-    int32_t* Ex = (int32_t*)(b + t.o_Ex);
-    for (int m = 1; m < M; ++m)
-      for (int rr = 0; rr < t.rem_w; ++rr)
-        for (int c = 0; c < t.ex_w[m]; ++c) {
-          const int rem = rr - 2, skr = c + m * rem;
-          int32_t v = 0;
-          if (rem >= 1 && rem - 1 <= nmax) v = (int32_t)sp.cnt[CI(m - 1, rem - 1, modp(skr - (m - 1), Q))];
-          Ex[t.ex_base[m] / 4 + (size_t)rr * t.ex_w[m] + c] = v;
-        }
-    int16_t* dx = (int16_t*)(b + t.o_dex);
-    for (int j = 0; j < t.n_combo; ++j)
-      for (int m = 0; m < 16; ++m) dx[(size_t)j * 16 + m] = (int16_t)dex[j][m];
-  }
   double* sq = (double*)(b + t.o_sqrt);
   for (int k = 0; k < nmax + 3; ++k) sq[k] = std::sqrt((double)k);
   memcpy(b + t.o_pq, pq.data(), sizeof(uint32_t) * pq.size());
@@ -561,43 +502,10 @@ static int build_tables(Space& sp) {
     for (int j = 0; j < t.n_combo; ++j)
       for (int m = 0; m < 16; ++m) dl[(size_t)j * 16 + m] = (uint8_t)(delta[j][m] + kDeltaBias);
   }
-  {  // packed byte shifts: a signed sum, so that the low half's borrow is part of the value
-    int32_t* dw = (int32_t*)(b + t.o_dsw);
-    for (int j = 0; j < t.n_combo; ++j)
-      for (int k = 0; k < std::max(2, nsw); ++k) {
-        const int lo = delta[j][2 * k + 1], hi = (2 * k + 2 < 16) ? delta[j][2 * k + 2] : 0;
-        const int32_t v = (int32_t)(4 * lo + 65536 * 4 * hi);
-        if (k < 2)
-          dw[2 * (size_t)j + k] = v;  // words 0, 1 side by side
-        else
-          dw[(size_t)k * t.ncp + j] = v;  // word k >= 2: column k - 2 after the ncp pairs
-      }
-  }
   memcpy(b + t.o_ann, annStart.data(), sizeof(int32_t) * annStart.size());
-  {  // first combo of each pair whose creation pair comes after it (partners ascend)
-    int32_t* hs = (int32_t*)(b + t.o_hs);
-    for (int a = 0; a < t.n_ann; ++a) {
-      int j = annStart[a];
-      while (j < annStart[a + 1] && (int)pairidx[pq[j] & 0xff][(pq[j] >> 8) & 0xff] < a) ++j;
-      hs[a] = j;
-    }
-  }
   memcpy(b + t.o_pairidx, pairidx, 256);
   memcpy(b + t.o_w, sp.w.data(), sizeof(double) * M);
   memcpy(b + t.o_gd, gd.data(), sizeof(double) * gd.size());
-  // double-float copies: x = hi + lo with hi = fl32(x), lo = fl32(x - hi)
-  auto split = [](double x, float* out) {
-    float h = (float)x;
-    out[0] = h;
-    out[1] = (float)(x - (double)h);
-  };
-  float* sqf = (float*)(b + t.o_sqf);
-  for (int k = 0; k < nmax + 3; ++k) split(std::sqrt((double)k), sqf + 2 * k);
-  float* Gf = (float*)(b + t.o_Gf);
-  for (int j = 0; j < t.n_combo; ++j) {
-    split(G[2 * j], Gf + 2 * j);
-    split(G[2 * j + 1], Gf + 2 * ((size_t)t.ncp + j));
-  }
   return QB_OK;
 }
 
@@ -887,6 +795,7 @@ void qb_space_free(qb_space* space) {
   cudaFree(sp->d_fill);
   cudaFree(sp->d_low);
   cudaFree(sp->d_perm);
+  cudaFree(sp->d_mo);
   cudaFree(sp->d_hpsi);
   for (int k = 0; k < 2; ++k) {
     cudaFree(sp->d_blocks[k]);

@@ -50,31 +50,10 @@ struct Tables {
   int o_G;       // double [n_combo][2]        conj(mult * L^sym_{pq;rs}) (re, im)
   int o_delta;   // uint8  [n_combo][16]       kDeltaBias + flat-index shift of the suffix state at mode m
                  //   (exact: int16 [n_combo][16], the shift itself)
-  int o_Ex;      // exact momentum, when it fits a CTA: the compact ranking table, mode m (1 .. M-1)
-                 //   at byte ex_base[m], int32 [rem_w][ex_w[m]], column skr - m rem (the suffix
-                 //   momentum of mode m lies in [m rem, (M-1) rem]); empty otherwise (o_Ex = o_ann)
-  int ex_smem;   // 1: the stage kernels rank exact-momentum targets in the compact table
-  int ex_w[16];
-  int ex_base[16];
-  int o_dex;     // int16  [n_combo][16]       shifts of the flat compact index per mode (exact, compact)
   int o_ann;     // int32  [n_ann + 1]         first combo of annihilation pair a
-  int o_hs;      // int32  [n_ann]             first combo of pair a whose creation pair (p, q) has a
-                 //   larger pair index: <x|H|x> takes each term once with its reverse
   int o_pairidx; // uint8  [16][16]            pair index of (r <= s)
   int o_w;       // double [M]                 one-body w_p
   int o_gd;      // double [n_ann]             diagonal two-body coefficient mult_rs^2 L^sym_{rs;rs}
-  int o_sqf;     // float2 [nmax+3]            sqrt(k) as a double-float pair (hi, lo)
-  // The stage kernel's per-term tables are column arrays of ncp entries (n_combo
-  // rounded up to a multiple of 4), so that the 32 lanes of a warp, each on its own
-  // term, load 8 or 4 bytes apiece from densely packed rows:
-  int ncp;
-  int o_Gf;      // float2 [2][ncp]            G as double-float pairs: [0][j] (re.hi, re.lo), [1][j] (im.hi, im.lo)
-  int o_dsw;     // uint2 [ncp], then uint32 [nsw - 2][ncp]: byte shifts of the suffix index, two modes
-                 //   per word (nsw = max(1, M / 2) words): word k holds 4 shift(2k+1) + 65536 * 4
-                 //   shift(2k+2) (the ranking table's byte offsets of modes 2k+1 and 2k+2 added in one
-                 //   32-bit add, see the stage kernel); words 0 and 1 side by side, the rest one array
-                 //   per word
-  int sw_ok;     // 1: every byte offset into the ranking table fits 16 bits (required for mod-M momentum)
   const unsigned char* blob;  // device pointer to the image
   // sectors
   int n_sectors;
@@ -158,6 +137,14 @@ struct Tables {
   const uint32_t* fa_basea;    // [lower blocks][fa_rowa] raised target blocks, then the classes' entries (qb_factor.cuh)
   const uint32_t* fa_basec;    // [blocks][fa_Tc] index in the vector of B_k f of the lowered target blocks
   const uint32_t* fa_perm;     // [ceil(fa_low / 32)] order of the rounds (qb_factor.cuh), or NULL
+  // Moments by raised and lowered kets (qb_observe.cu), for spaces that hold every sector up
+  // to nmax (mo_on): rows of 2 mo_w entries per block, the target blocks after a particle is
+  // added to (taken from) each mode, and the places, mo_w / 4 groups of four modes.
+  int mo_on, mo_w;
+  int64_t mo_rows;             // kets of fewer than nmax particles
+  const uint32_t* mo_base;     // [blocks][2 mo_w]
+  const uint2* mo_map;         // [2][mo_w / 4][S]
+  const uint32_t* mo_perm;     // [mo_rows / 32] order of the rounds
   const double* fa_wk;         // [fa_low] their ket weights, or NULL
 };
 // a row of fa_basea: the slots, the classes' entries, the mask of records with a held class
@@ -215,6 +202,7 @@ struct Space {
   uint32_t* d_blocks[2] = {nullptr, nullptr};  // rblk and the block starts of the kets, and of the lower kets
   void* d_hpsi = nullptr;      // FP64 vector of B_k psi (qb_hpsi of a factored space), made by the first call
   std::mutex hpsi_mu;          // held by the call that uses it
+  unsigned char* d_mo = nullptr;  // Tables::mo_*
   uint32_t* d_perm = nullptr;                  // Tables::fa_perm
   uint32_t* d_base[2] = {nullptr, nullptr};    // bases of the blocks, and of the lower blocks
   int64_t scratch_doubles = 0;
@@ -241,22 +229,24 @@ __host__ __device__ inline int nmoments(int M) { return 4 + 2 * M + 4 * M * M; }
 __host__ __device__ inline int nprep(int M) { return M + 2; }
 
 // Scratch layout of a space (doubles), sized at set-up for the largest persistent grid
-// G = SMs * 16:  [0, 2) status word | moment partials [G nmom] | moment sums [nmom] |
-// bilinear / <H> partials [(M + 1) G] | their sums [QB_MAX_MODES + 2] | amplitude table
-// [2 M (nmax + 1)] | initial-state norm [2] | first-pass partials [nprep G] | their sums [nprep]
+// G = SMs * 16:  [0, 2) status word | moment sums [nmom] | <H> sum [2] | first-pass sums [nprep]
+// (these, the first finals_doubles, come back in one copy) | moment partials [G nmom] |
+// bilinear / <H> partials [(M + 1) G] | first-pass partials [nprep G] | amplitude table
+// [2 M (nmax + 1)] | initial-state norm [2]
+// (even, as G is: the amplitude table is read as pairs)
+inline int64_t finals_doubles(int M) { return (2 + nmoments(M) + 2 + nprep(M) + 1) & ~1; }
 inline int64_t scratch_doubles_for(int M, int nmax, int64_t G) {
-  return 2 + G * nmoments(M) + nmoments(M) + (int64_t)(M + 1) * G + QB_MAX_MODES + 2 + 2 * (int64_t)M * (nmax + 1) +
-         2 + G * nprep(M) + nprep(M);
+  return finals_doubles(M) + G * nmoments(M) + (int64_t)(M + 1) * G + G * nprep(M) + 2 * (int64_t)M * (nmax + 1) + 2;
 }
 inline int64_t max_grid_of(const Space& s) { return s.scratch_doubles > 0 ? (int64_t)s.grid_hpsi : 0; }
-inline double* partial_area(const Space& s) { return s.d_scratch + 2; }
-inline double* final_area(const Space& s) { return partial_area(s) + max_grid_of(s) * nmoments(s.M); }
-inline double* dot_area(const Space& s) { return final_area(s) + nmoments(s.M); }
-inline double* dot_final(const Space& s) { return dot_area(s) + (int64_t)(s.M + 1) * max_grid_of(s); }
-inline double* table_area(const Space& s) { return dot_final(s) + QB_MAX_MODES + 2; }
+inline double* final_area(const Space& s) { return s.d_scratch + 2; }
+inline double* dot_final(const Space& s) { return final_area(s) + nmoments(s.M); }
+inline double* prep_final(const Space& s) { return dot_final(s) + 2; }
+inline double* partial_area(const Space& s) { return s.d_scratch + finals_doubles(s.M); }
+inline double* dot_area(const Space& s) { return partial_area(s) + max_grid_of(s) * nmoments(s.M); }
+inline double* prep_area(const Space& s) { return dot_area(s) + (int64_t)(s.M + 1) * max_grid_of(s); }
+inline double* table_area(const Space& s) { return prep_area(s) + max_grid_of(s) * nprep(s.M); }
 inline double* init_final(const Space& s) { return table_area(s) + 2 * (size_t)s.M * (s.nmax + 1); }
-inline double* prep_area(const Space& s) { return init_final(s) + 2; }
-inline double* prep_final(const Space& s) { return prep_area(s) + max_grid_of(s) * nprep(s.M); }
 
 // launchers (qb_kernels.cu); all return a QB_* status
 int launch_hpsi(Space& s, const void* d_v, void* d_out, void* stream);

@@ -531,25 +531,25 @@ __global__ void __launch_bounds__(256) raised_base_kernel(const Tables t, const 
   }
 }
 
-// Order of the lower rounds: within a layer (equal N) of S sectors, which are nearly equal
-// in size, position j of the layer's n rounds is round (j mod S) ceil(n / S) + j / S, the
-// positions beyond the last segment's end moved up.
-__global__ void __launch_bounds__(256) round_order_kernel(const Tables t, const int32_t* lowN, uint32_t* perm) {
-  const int64_t nr = (t.fa_low + 31) / 32;
+// Order of the rounds of kets in sectors (first kets off[nsec + 1], particles secN): within
+// a layer (equal N) of S sectors, which are nearly equal in size, position j of the layer's n
+// rounds is round (j mod S) ceil(n / S) + j / S, the positions beyond the last segment's end
+// moved up.  A layer is the rounds [floor(first / 32), floor(end / 32)) of its kets.
+__global__ void __launch_bounds__(256) round_order_kernel(const int64_t* off, const int32_t* secN, int nsec, int64_t nr,
+                                                           uint32_t* perm) {
   for (int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x; r < nr; r += (int64_t)gridDim.x * 256) {
-    // the layer of round r: the rounds [floor(first / 32), floor(end / 32)) of its kets
-    int lo = 0, hi = t.fa_nlow - 1;
+    int lo = 0, hi = nsec - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (__ldg(t.fa_lowoff + mid) / 32 <= r)
+      if (__ldg(off + mid) / 32 <= r)
         lo = mid;
       else
         hi = mid - 1;
     }
     int a = lo, b = lo;
-    while (a > 0 && lowN[a - 1] == lowN[lo]) --a;
-    while (b + 1 < t.fa_nlow && lowN[b + 1] == lowN[lo]) ++b;
-    const int64_t ra = __ldg(t.fa_lowoff + a) / 32, rb = b + 1 < t.fa_nlow ? __ldg(t.fa_lowoff + b + 1) / 32 : nr;
+    while (a > 0 && secN[a - 1] == secN[lo]) --a;
+    while (b + 1 < nsec && secN[b + 1] == secN[lo]) ++b;
+    const int64_t ra = __ldg(off + a) / 32, rb = b + 1 < nsec ? __ldg(off + b + 1) / 32 : nr;
     const int64_t S = b - a + 1, n = rb - ra, len = (n + S - 1) / S, j = r - ra;
     // full columns: len - 1 of them where the last segment is short
     const int64_t lastlen = n - (S - 1) * len;  // of segment S - 1 (may be <= 0)
@@ -589,6 +589,47 @@ __global__ void __launch_bounds__(kBlock) block_map_kernel(const Tables t, uint1
       else
         map5[(size_t)rec * t.bk_S + f] = place;
     }
+  }
+}
+
+// Tables of the raised moments: suffix shift of one particle more (sign 1) or fewer in mode i
+__device__ __forceinline__ int one_shift(const Tables& t, int i, int m, int sign) {
+  if (i < m) return 0;
+  return sign * 2 * t.Q + (sign > 0 ? i % t.Q : (t.Q - i % t.Q) % t.Q);
+}
+__global__ void __launch_bounds__(kBlock) moment_map_kernel(const Tables t, uint16_t* map) {
+  const int64_t f = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+  Filling F;
+  if (f >= t.bk_S || !filling_of(t, f, F)) return;
+  int32_t sh[kMaxM];
+  for (int q = 0; q < 2 * t.mo_w; ++q) {
+    const int i = q % t.mo_w, sign = q < t.mo_w ? 1 : -1;
+    uint16_t place = 0;
+    if (i < t.M && (sign > 0 || i < t.bk_P || F.occ[i] >= 1)) {
+      for (int m = 0; m < t.M; ++m) sh[m] = one_shift(t, i, m, sign);
+      place = place_of(t, F, sh, 1);
+    }
+    map[((size_t)(q / 4) * t.bk_S + f) * 4 + q % 4] = place;
+  }
+}
+__global__ void __launch_bounds__(256) moment_base_kernel(const Tables t, const uint32_t* start, int64_t nblocks,
+                                                           uint32_t* base) {
+  const int lane = threadIdx.x & 31, w = t.mo_w;  // 2 w <= 32: one entry a lane
+  const int i = lane % w, sign = lane < w ? 1 : -1;
+  const int32_t* E = reinterpret_cast<const int32_t*>(t.blob + t.o_E);
+  for (int64_t b = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5; b < nblocks; b += ((int64_t)gridDim.x * 256) >> 5) {
+    const BlockState s = block_state(t, __ldg(t.occ + start[b]), lane);
+    uint32_t sum = 0;
+    for (int m = 1; m < t.bk_P; ++m)
+      sum += (uint32_t)__ldg(E + __shfl_sync(0xffffffffu, s.my, m) + one_shift(t, i, m, sign));
+    sum += (uint32_t)__ldg(t.bk_EC + __shfl_sync(0xffffffffu, s.my, t.bk_P) + one_shift(t, i, t.bk_P, sign));
+    const int N = s.N + sign, K = (s.K + (sign > 0 ? i : t.Q - i % t.Q)) % t.Q;
+    uint32_t v = kNoIndex;
+    if (lane < 2 * w && i < t.M && N >= 0 && N <= t.nmax) {
+      const int sid = __ldg(t.sec_of + N * t.Q + K);
+      if (sid >= 0) v = (uint32_t)__ldg(t.sec_off + sid + 1) - sum;
+    }
+    if (lane < 2 * w) base[(size_t)b * 2 * w + lane] = v;
   }
 }
 
@@ -750,15 +791,6 @@ __global__ void __launch_bounds__(kBlock) init_table_kernel(const Tables t, cons
     double s = 0.0;
     for (int k = 0; k < kBlock / 32; ++k) s += red[k];
     partial[blockIdx.x] = s;
-  }
-}
-
-// sums partial[0..n)[0..width) over the first index in a fixed order
-__global__ void reduce_partials_kernel(const double* partial, int n, int width, double* out) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < width; c += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < n; ++k) s += partial[(size_t)k * width + c];
-    out[c] = s;
   }
 }
 
@@ -1140,7 +1172,7 @@ int device_setup(Space& s) {
     {
       const int64_t nr = (t.fa_low + 31) / 32;
       QB_CUDA(cudaMalloc(&s.d_perm, sizeof(uint32_t) * (size_t)nr));
-      round_order_kernel<<<base_grid, 256>>>(t, reinterpret_cast<const int32_t*>(at(11)), s.d_perm);
+      round_order_kernel<<<base_grid, 256>>>(t.fa_lowoff, reinterpret_cast<const int32_t*>(at(11)), t.fa_nlow, nr, s.d_perm);
       QB_CUDA(cudaGetLastError());
       t.fa_perm = s.d_perm;
     }
@@ -1151,6 +1183,37 @@ int device_setup(Space& s) {
     QB_CUDA(cudaGetLastError());
     const dim3 grid((unsigned)((t.bk_S + kBlock - 1) / kBlock), (unsigned)std::min(fa_Ta(t) / 4 + t.fa_ng, 8));
     factor_map_kernel<<<grid, kBlock>>>(t, reinterpret_cast<uint16_t*>(at(13)), reinterpret_cast<uint16_t*>(at(14)));
+    QB_CUDA(cudaGetLastError());
+  }
+  // moments by raised kets: odd M with a kernel, every sector from the vacuum to nmax held
+  int layers_end = 0;  // first sector of nmax particles
+  t.mo_on = (s.M == 5 || s.M == 7 || s.M == 9) && s.nmin == 0 && s.nmax >= 1 && s.nmax < 256;
+  if (t.mo_on) {
+    for (int N = 0, i = 0; N <= s.nmax && t.mo_on; ++N) {
+      if (N == s.nmax) layers_end = i;
+      for (int K = 0; K < s.Q; ++K)
+        if (s.cnt[(size_t)N * s.Q + K] > 0) {
+          if (s.secOf[(size_t)N * s.Q + K] < 0) t.mo_on = 0;
+          ++i;
+        }
+    }
+  }
+  if (t.mo_on) {
+    t.mo_w = (s.M + 3) & ~3;
+    t.mo_rows = s.secOff[layers_end];
+    const size_t mapb = ((size_t)2 * t.mo_w * t.bk_S * 2 + 255) & ~(size_t)255;
+    const size_t baseb = ((size_t)nblocks * 2 * t.mo_w * 4 + 255) & ~(size_t)255;
+    const int64_t nr = t.mo_rows / 32;
+    QB_CUDA(cudaMalloc(&s.d_mo, mapb + baseb + 4 * (size_t)std::max<int64_t>(nr, 1)));
+    t.mo_map = reinterpret_cast<const uint2*>(s.d_mo);
+    t.mo_base = reinterpret_cast<const uint32_t*>(s.d_mo + mapb);
+    moment_map_kernel<<<(unsigned)((t.bk_S + kBlock - 1) / kBlock), kBlock>>>(t, reinterpret_cast<uint16_t*>(s.d_mo));
+    moment_base_kernel<<<base_grid, 256>>>(t, start, nblocks, reinterpret_cast<uint32_t*>(s.d_mo + mapb));
+    if (nr > 0) {
+      uint32_t* perm = reinterpret_cast<uint32_t*>(s.d_mo + mapb + baseb);
+      round_order_kernel<<<base_grid, 256>>>(t.sec_off, t.sec_N, t.n_sectors, nr, perm);
+      t.mo_perm = perm;
+    }
     QB_CUDA(cudaGetLastError());
   }
   QB_CUDA(cudaDeviceSynchronize());
@@ -1426,7 +1489,7 @@ int launch_init_table(const Space& s, const double* table_host, int only_N, void
   init_table_kernel<<<grid, kBlock, smem, st>>>(s.t, (const double2*)tab, only_N, (double2*)d_psi, part);
   QB_CUDA(cudaGetLastError());
   double* fin = init_final(s);
-  reduce_partials_kernel<<<1, 32, 0, st>>>(part, grid, 1, fin);
+  sum_rows_kernel<<<1, kSumThreads, 0, st>>>(part, grid, 1, 1.0, false, fin);
   QB_CUDA(cudaGetLastError());
   QB_CUDA(cudaMemcpyAsync(norm2, fin, sizeof(double), cudaMemcpyDeviceToHost, st));
   QB_CUDA(cudaStreamSynchronize(st));
@@ -1540,7 +1603,7 @@ extern "C" int qb_observables_noalloc(qb_space* space, const void* d_psi, qb_obs
   QB_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
   moments_kernel<<<grid, kBlock, smem, st>>>(sp->t, (const double2*)d_psi, part, nmom, status);
   QB_CUDA(cudaGetLastError());
-  reduce_partials_kernel<<<(nmom + 127) / 128, 128, 0, st>>>(part, grid, nmom, fin);
+  sum_rows_kernel<<<nmom, kSumThreads, 0, st>>>(part, grid, nmom, 1.0, false, fin);
   QB_CUDA(cudaGetLastError());
   StageArgs a{};
   a.vin = (const double2*)d_psi;
@@ -1550,7 +1613,7 @@ extern "C" int qb_observables_noalloc(qb_space* space, const void* d_psi, qb_obs
   int gdot = 0;
   rc = sp->t.is_complex ? noalloc_dot<true>(*sp, a, grid, st, &gdot) : noalloc_dot<false>(*sp, a, grid, st, &gdot);
   if (rc) return rc;
-  reduce_partials_kernel<<<1, 32, 0, st>>>(dpart, gdot, 2, dfin);
+  sum_rows_kernel<<<2, kSumThreads, 0, st>>>(dpart, gdot, 2, 1.0, false, dfin);
   QB_CUDA(cudaGetLastError());
   std::vector<double> raw(nmom, 0.0);
   double h2[2];

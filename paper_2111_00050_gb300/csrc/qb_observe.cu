@@ -24,6 +24,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <string>
 
 #include "qb_device.cuh"
@@ -57,15 +58,6 @@ constexpr int kMwSplMax = 3;    // moment entries per lane and pass (<= 96 per p
 #define QB_MW_PIPE 1
 #endif
 __host__ __device__ constexpr int mw_warps(int spl) { return (QB_MW_PIPE && spl == 2) ? QB_MW_WARPS_SPL2 : QB_MW_WARPS; }
-
-// sums partial[0..n)[0..width) over the first index in a fixed order
-__global__ void reduce_rows_kernel(const double* partial, int n, int width, double* out) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < width; c += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < n; ++k) s += partial[(size_t)k * width + c];
-    out[c] = s;
-  }
-}
 
 // FP64 sum over the CTA in a fixed order: lanes by shuffles, then warps in turn;
 // `red` holds one value per warp.  The result is valid in thread 0.
@@ -725,7 +717,222 @@ __global__ void __launch_bounds__(32 * mw_warps(kMwSpl), QB_MW_MIN_BLOCKS) momen
   for (int k = tid; k < nmom; k += kMwBlock) partial[(size_t)blockIdx.x * nmom + k] = row[k];
 }
 
+// ------------------------------------------------------- moments by raised kets
+//
+// A space that holds every sector up to nmax takes the same moments from the kets m of fewer
+// than nmax particles, lanes on consecutive kets:
+//   <a_i>        = sum_m conj(psi(m)) u_i(m),    u_i(m) = (a_i psi)(m)
+//   <a_i^+ a_j>  = sum_m conj(u_i(m)) u_j(m)
+//   <a_i a_j>    = sum_m conj(v_j(m)) u_i(m),    v_j(m) = (a_j^+ psi)(m)
+// so that 14 gathers a ket (M = 7) make the 56 moments, which the entry-per-lane kernel above
+// gathers one by one, ranking each.  In the weighted basis u_i = w(m) sqrt(N + 1) 2^(e_N - e_N+1)
+// f(m + e_i) and v_j = w(m) m_j / sqrt(N) 2^(e_N - e_N-1) f(m - e_j).  The products are
+// double-float, summed over 32 rounds in each lane's registers, then over the warp (each lane
+// ends with one entry) and in FP64.  15.4M kets, M = 7: 4.4 ms in the kernel above, which its
+// scattered gathers and the products' latency limit.
+constexpr int kMoRounds = 32;  // rounds a lane sums in double-float
+template <int MT>
+__host__ __device__ constexpr int mo_threads() {  // registers: four an entry beside the gathered values
+  return MT <= 5 ? 512 : MT <= 7 ? 384 : 256;
+}
+template <int MT, bool AA>
+__host__ __device__ constexpr int mo_entries() {  // A: a_i, then a_i^+ a_j (i < j); AA: a_i a_j (i <= j)
+  return AA ? MT * (MT + 1) / 2 : MT + MT * (MT - 1) / 2;
+}
+
+// acc += conj(p) q for double-float complex p (as factors) and q
+__device__ __forceinline__ void dfc_conj_fma(dfc& acc, dfl pr, dfl pi, float4 q) {
+  dfc_fma(acc, f2_pack(pr.h, pr.h), f2_pack(-pr.h, -pr.h), f2_pack(pr.l, pr.l), f2_pack(q.x, q.y), f2_pack(q.z, q.w));
+  // + pi (q_i, -q_r)
+  dfc_fma(acc, f2_pack(pi.h, -pi.h), f2_pack(-pi.h, pi.h), f2_pack(pi.l, -pi.l), f2_pack(q.y, q.x), f2_pack(q.w, q.z));
+}
+
+// c x for a double-float factor and a double-float complex value
+__device__ __forceinline__ float4 df_scale(dfl c, float4 x) {
+  return df_pack(df_renorm(df_mul(c, df_re(x))), df_renorm(df_mul(c, df_im(x))));
+}
+
+template <int MT, bool AA>
+__global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(const Tables t, const float4* f,
+                                                                              double* partial, int nmom, int* status) {
+  constexpr int NE = mo_entries<MT, AA>(), NC = (NE + 31) / 32, NW = occ_words<MT>(), W4 = (MT + 3) / 4;
+  __shared__ double row[4 + 2 * MT + 4 * MT * MT];
+  __shared__ float2 sc[2][256];  // sqrt(N + 1) 2^(e_N - e_N+1); 2^(e_N - e_N-1) / sqrt(N)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  for (int N = threadIdx.x; N < t.nmax; N += blockDim.x) {
+    const double e0 = __ldg(t.wscale + N).y;  // 2^e_N
+    const dfl up = df_of(sqrt((double)(N + 1)) * e0 * __ldg(t.wscale + N + 1).x);
+    const dfl dn = df_of(N > 0 ? e0 * __ldg(t.wscale + N - 1).x / sqrt((double)N) : 0.0);
+    sc[0][N] = make_float2(up.h, up.l);
+    sc[1][N] = make_float2(dn.h, dn.l);
+  }
+  for (int k = threadIdx.x; k < nmom; k += blockDim.x) row[k] = 0.0;
+  __syncthreads();
+  const int64_t total = t.total, rows = t.mo_rows, nr = (rows + 31) / 32, whole = rows / 32;
+  dfc acc[32 * NC];
+#pragma unroll
+  for (int e = 0; e < 32 * NC; ++e) acc[e] = dfc{0ull, 0ull};
+  double sum_r[NC], sum_i[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) sum_r[c] = sum_i[c] = 0.0;
+  bool bad = false;
+  // each lane of the warp ends with the warp's sum of entry 32 c + lane
+  auto flush = [&]() {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+#pragma unroll
+      for (int s = 16; s >= 1; s >>= 1) {
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int k = 0; k < s; ++k) {
+          if (32 * c + k >= NE) break;  // both halves empty
+          dfc& lo = acc[32 * c + k];
+          dfc& hi = acc[32 * c + k + s];
+          const f2 mh = up ? hi.h : lo.h, ml = up ? hi.l : lo.l, oh = up ? lo.h : hi.h, ol = up ? lo.l : hi.l;
+          dfc m{mh, ml};
+          const f2 rh = __shfl_xor_sync(0xffffffffu, oh, s), rl = __shfl_xor_sync(0xffffffffu, ol, s);
+          dfc_add(m, rh, rl);
+          lo = dfc_renorm(m);
+        }
+      }
+      float hr, hi2, lr, li;
+      f2_unpack(acc[32 * c].h, hr, hi2);
+      f2_unpack(acc[32 * c].l, lr, li);
+      sum_r[c] += (double)hr + (double)lr;
+      sum_i[c] += (double)hi2 + (double)li;
+    }
+#pragma unroll
+    for (int e = 0; e < 32 * NC; ++e) acc[e] = dfc{0ull, 0ull};
+  };
+  int held = 0;
+  for (int64_t rd = nr - 1 - ((int64_t)blockIdx.x * warps + warp); rd >= 0; rd -= (int64_t)gridDim.x * warps) {
+    const int64_t rn = rd < whole && t.mo_perm ? (int64_t)__ldg(t.mo_perm + rd) : rd;
+    const int64_t g = rn * 32 + lane;
+    const bool valid = g < rows;
+    const RoundIn in = load_round(t.occ, t.fill, t.rblk, rn, total, lane);
+    const uint32_t* base = t.mo_base + (size_t)block_of_lane(in, lane, g < total) * (2 * 4 * W4);
+    uint32_t ob[NW];
+    unpack_occ<MT, NW>(t, valid ? in.word : 0ull, ob);
+    int N = 0;
+#pragma unroll
+    for (int k = 0; k < NW; ++k) N += (int)__dp4a(ob[k], 0x01010101u, 0u);
+    const dfl W = valid ? df_of(__ldg(t.wk + g)) : dfl{0.f, 0.f};
+    const float2 cu = sc[0][valid ? N : 0];
+    const dfl wu = df_renorm(df_mul(W, dfl{cu.x, cu.y}));
+    float4 u[MT];
+#pragma unroll
+    for (int k = 0; k < W4; ++k) {
+      const uint4 b = __ldg(reinterpret_cast<const uint4*>(base) + k);
+      const uint2 m = __ldg(t.mo_map + (size_t)k * t.bk_S + in.fill);
+      const uint32_t ix[4] = {b.x + (m.x & 0xffffu), b.y + (m.x >> 16), b.z + (m.y & 0xffffu), b.w + (m.y >> 16)};
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (4 * k + c < MT) {
+          const bool ok = valid && ix[c] < (uint32_t)total;
+          bad |= valid && !ok;
+          u[4 * k + c] = ok ? __ldg(f + ix[c]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < MT; ++i) u[i] = df_scale(wu, u[i]);
+    int e = 0;
+    if constexpr (!AA) {
+      const float4 x = df_scale(W, valid ? __ldg(f + g) : make_float4(0.f, 0.f, 0.f, 0.f));
+#pragma unroll
+      for (int i = 0; i < MT; ++i, ++e) dfc_conj_fma(acc[e], df_re(x), df_im(x), u[i]);
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int j = i + 1; j < MT; ++j, ++e) dfc_conj_fma(acc[e], df_re(u[i]), df_im(u[i]), u[j]);
+    } else {
+      const float2 cd = sc[1][valid ? N : 0];
+      const dfl wd = df_renorm(df_mul(W, dfl{cd.x, cd.y}));
+#pragma unroll
+      for (int k = 0; k < W4; ++k) {
+        const uint4 b = __ldg(reinterpret_cast<const uint4*>(base) + W4 + k);
+        const uint2 m = __ldg(t.mo_map + (size_t)(W4 + k) * t.bk_S + in.fill);
+        const uint32_t ix[4] = {b.x + (m.x & 0xffffu), b.y + (m.x >> 16), b.z + (m.y & 0xffffu), b.w + (m.y >> 16)};
+        float4 v[4];
+        float nj[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (4 * k + c < MT) {
+            nj[c] = occ_float<NW>(ob, 4 * k + c);
+            const bool act = nj[c] != 0.f, ok = act && ix[c] < (uint32_t)total;
+            bad |= act && !ok;
+            v[c] = ok ? __ldg(f + ix[c]) : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (4 * k + c < MT) {
+            const int j = 4 * k + c;
+            const float4 vj = df_scale(df_mul_f(wd, nj[c]), v[c]);
+#pragma unroll
+            for (int i = 0; i <= j; ++i, ++e) dfc_conj_fma(acc[e], df_re(vj), df_im(vj), u[i]);  // entry j (j + 1) / 2 + i
+          }
+      }
+    }
+    if (++held == kMoRounds) {
+      flush();
+      held = 0;
+    }
+  }
+  flush();
+  if (bad) atomicOr(status, 1);
+  // the warps' sums into the CTA's row, one warp at a time (a fixed order)
+  const int oA = 4, oM = 4 + 2 * MT, oAA = 4 + 2 * MT + 2 * MT * MT;
+  for (int w = 0; w < warps; ++w) {
+    if (warp == w) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        int s = 32 * c + lane;
+        if (s >= NE) continue;
+        if (AA) {
+          int j = 0;
+          while ((j + 1) * (j + 2) / 2 <= s) ++j;
+          const int i = s - j * (j + 1) / 2;  // i <= j
+          row[oAA + 2 * (i * MT + j)] += sum_r[c];
+          row[oAA + 2 * (i * MT + j) + 1] += sum_i[c];
+        } else if (s < MT) {
+          row[oA + 2 * s] += sum_r[c];
+          row[oA + 2 * s + 1] += sum_i[c];
+        } else {  // <a_j^dag a_i> = conj <a_i^dag a_j>
+          s -= MT;
+          int i = 0;
+          while (s >= MT - 1 - i) s -= MT - 1 - i++;
+          const int j = i + 1 + s;
+          row[oM + 2 * (i * MT + j)] += sum_r[c];
+          row[oM + 2 * (i * MT + j) + 1] += sum_i[c];
+          row[oM + 2 * (j * MT + i)] += sum_r[c];
+          row[oM + 2 * (j * MT + i) + 1] -= sum_i[c];
+        }
+      }
+    }
+    __syncthreads();
+  }
+  for (int k = threadIdx.x; k < nmom; k += blockDim.x) partial[(size_t)blockIdx.x * nmom + k] = row[k];
+}
+
 // ------------------------------------------------------------------ host side
+
+template <int MT>
+static int launch_raised_moments(const Space& s, const float4* f, cudaStream_t st) {
+  const Tables& t = s.t;
+  const int nmom = nmoments(MT), half = 4 + 2 * MT + 2 * MT * MT;  // columns of a and M; then aa
+  for (int aa = 0; aa < 2; ++aa) {
+    auto k = aa ? raised_moments_kernel<MT, true> : raised_moments_kernel<MT, false>;
+    int warps = 0, grid = 0;
+    int rc = stage_geometry(k, t.mo_rows, 0, mo_threads<MT>() / 32, 0, &warps, &grid);
+    if (rc) return rc;
+    grid = (int)std::min<int64_t>(grid, max_grid_of(s));
+    k<<<grid, 32 * warps, 0, st>>>(t, f, partial_area(s), nmom, reinterpret_cast<int*>(s.d_scratch));
+    QB_CUDA(cudaGetLastError());
+    sum_rows_kernel<<<aa ? nmom - half : half, kSumThreads, 0, st>>>(partial_area(s), grid, nmom, 1.0, false, final_area(s),
+                                                                     aa ? half : 0);
+    QB_CUDA(cudaGetLastError());
+  }
+  return QB_OK;
+}
 
 template <int MT>
 static int launch_prep(const Space& s, const double2* psi, float4* f, double* part, int* grid_out, cudaStream_t st) {
@@ -767,7 +974,7 @@ static int launch_mw(const Space& s, const double2* psi, const float4* f, double
 // 96 and 36); the generic kernel takes any
 template <int MT, int SPL>
 constexpr bool mw_needed() {
-  return MT == 0 || (MT == 5 && SPL == 1) || (MT == 7 && SPL == 2) || (MT == 9 && SPL == 3) ||
+  return MT == 0 || (MT == 5 && SPL <= 2) || (MT == 7 && SPL == 2) || (MT == 9 && SPL == 3) ||
          (MT == 11 && (SPL == 3 || SPL == 2));
 }
 
@@ -789,7 +996,7 @@ static int launch_mw_m(const Space& s, const double2* psi, const float4* f, doub
 // variants take in full passes
 static int tb_pass_entries(int M) {
   switch (M) {
-    case 5: return 32;
+    case 5:
     case 7: return 64;
     case 9: return 96;
     case 11: return 96;
@@ -810,15 +1017,6 @@ static int launch_mw_e(const Space& s, const double2* psi, const float4* f, doub
   }
 }
 
-// acc[c] += weight * sum_k partial[k][c], in a fixed order
-__global__ void accumulate_rows_kernel(const double* partial, int n, int width, double weight, double* acc) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < width; c += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < n; ++k) s += partial[(size_t)k * width + c];
-    acc[c] += weight * s;
-  }
-}
-
 int launch_tb_bilinear(Space& s, const float4* bra, const float4* ket, const int* d_tb, int n_tb, double weight,
                        double* d_acc, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
@@ -830,7 +1028,7 @@ int launch_tb_bilinear(Space& s, const float4* bra, const float4* ket, const int
     int rc = s.t.exact ? launch_mw_e<true>(s, nullptr, bra, partial_area(s), 2 * ne, e0, ne, &gm, st, ket, d_tb)
                        : launch_mw_e<false>(s, nullptr, bra, partial_area(s), 2 * ne, e0, ne, &gm, st, ket, d_tb);
     if (rc) return rc;
-    accumulate_rows_kernel<<<(2 * ne + 127) / 128, 128, 0, st>>>(partial_area(s), gm, 2 * ne, weight, d_acc + 2 * e0);
+    sum_rows_kernel<<<2 * ne, kSumThreads, 0, st>>>(partial_area(s), gm, 2 * ne, weight, true, d_acc + 2 * e0);
     QB_CUDA(cudaGetLastError());
   }
   return QB_OK;
@@ -852,7 +1050,7 @@ int launch_moments(Space& s, const void* d_psi, double* out_host, void* stream) 
     default: rc = launch_prep<0>(s, psi, f, prep_area(s), &gp, st); break;
   }
   if (rc) return rc;
-  reduce_rows_kernel<<<1, 32, 0, st>>>(prep_area(s), gp, npr, prep_final(s));
+  sum_rows_kernel<<<npr, kSumThreads, 0, st>>>(prep_area(s), gp, npr, 1.0, false, prep_final(s));
   QB_CUDA(cudaGetLastError());
   // pass 3: <psi|H|psi> from the weighted copy, w^2 applied per row in FP64
   DfArgs a{};
@@ -868,30 +1066,39 @@ int launch_moments(Space& s, const void* d_psi, double* out_host, void* stream) 
   int g2 = 0;
   rc = stage_launch(s.t, a, 4, 1, s.t.is_complex != 0, st, &g2, false, 0);
   if (rc) return rc;
-  reduce_rows_kernel<<<1, 32, 0, st>>>(a.partial, g2, 1, dot_final(s));
+  sum_rows_kernel<<<1, kSumThreads, 0, st>>>(a.partial, g2, 1, 1.0, false, dot_final(s));
   QB_CUDA(cudaGetLastError());
-  // pass 2: the moments that move the ket, in passes of at most 32 kMwSplMax entries;
-  // each pass's partial rows are summed into its own copy of the moment row
-  const int nent = mw_entries(M), per = 32 * kMwSplMax;
-  const int npass = (nent + per - 1) / per;
-  std::vector<double> mom((size_t)nmom, 0.0), fin((size_t)nmom);
-  for (int p = 0; p < npass; ++p) {
-    const int e0 = p * per, ne = std::min(per, nent - e0);
-    int gm = 0;
-    rc = s.t.exact ? launch_mw_e<true>(s, psi, f, partial_area(s), nmom, e0, ne, &gm, st)
-                   : launch_mw_e<false>(s, psi, f, partial_area(s), nmom, e0, ne, &gm, st);
+  // pass 2: the moments that move the ket, by raised kets or in passes of at most
+  // 32 kMwSplMax entries, each pass's partial rows added to the moment row
+  if (s.t.mo_on) {
+    switch (M) {
+      case 5: rc = launch_raised_moments<5>(s, f, st); break;
+      case 7: rc = launch_raised_moments<7>(s, f, st); break;
+      case 9: rc = launch_raised_moments<9>(s, f, st); break;
+      default: rc = fail(QB_EINTERNAL, "no raised-moments kernel");
+    }
     if (rc) return rc;
-    reduce_rows_kernel<<<(nmom + 127) / 128, 128, 0, st>>>(partial_area(s), gm, nmom, final_area(s));
-    QB_CUDA(cudaGetLastError());
-    QB_CUDA(cudaMemcpyAsync(fin.data(), final_area(s), sizeof(double) * nmom, cudaMemcpyDeviceToHost, st));
-    QB_CUDA(cudaStreamSynchronize(st));
-    for (int k = 0; k < nmom; ++k) mom[k] += fin[k];
+  } else {
+    const int nent = mw_entries(M), per = 32 * kMwSplMax;
+    for (int e0 = 0; e0 < nent; e0 += per) {
+      const int ne = std::min(per, nent - e0);
+      int gm = 0;
+      rc = s.t.exact ? launch_mw_e<true>(s, psi, f, partial_area(s), nmom, e0, ne, &gm, st)
+                     : launch_mw_e<false>(s, psi, f, partial_area(s), nmom, e0, ne, &gm, st);
+      if (rc) return rc;
+      sum_rows_kernel<<<nmom, kSumThreads, 0, st>>>(partial_area(s), gm, nmom, 1.0, e0 > 0, final_area(s));
+      QB_CUDA(cudaGetLastError());
+    }
   }
-  std::vector<double> pre((size_t)npr);
-  double h = 0.0;
-  QB_CUDA(cudaMemcpyAsync(pre.data(), prep_final(s), sizeof(double) * npr, cudaMemcpyDeviceToHost, st));
-  QB_CUDA(cudaMemcpyAsync(&h, dot_final(s), sizeof(double), cudaMemcpyDeviceToHost, st));
+  // the sums and the status word in one copy
+  std::vector<double> fin((size_t)finals_doubles(M));
+  QB_CUDA(cudaMemcpyAsync(fin.data(), s.d_scratch, sizeof(double) * fin.size(), cudaMemcpyDeviceToHost, st));
   QB_CUDA(cudaStreamSynchronize(st));
+  int status = 0;
+  std::memcpy(&status, fin.data(), sizeof(status));
+  if (status) return check_status(s, st);
+  const double *mom = fin.data() + 2, *pre = mom + nmom + 2;
+  double h = mom[nmom];
   for (int k = 0; k < nmom; ++k) out_host[k] = mom[k];
   out_host[0] = pre[0];
   out_host[1] = pre[1];
@@ -904,7 +1111,7 @@ int launch_moments(Space& s, const void* d_psi, double* out_host, void* stream) 
     out_host[oM + 2 * (i * M + i)] = pre[2 + i];
     out_host[oM + 2 * (i * M + i) + 1] = 0.0;
   }
-  return check_status(s, st);
+  return QB_OK;
 }
 
 }  // namespace qb

@@ -111,7 +111,8 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
   a.scale[0] = r.scale;
   a.psi = spsi;
   a.psif = spsif;
-  dfl bil_l{0.f, 0.f}, bil_w[1] = {dfl{0.f, 0.f}};
+  dfl bil_l{0.f, 0.f};
+  dfc bil_w[1] = {dfc{0ull, 0ull}};
   double dot64 = 0.0;
   for (int64_t it = 0; it < r.steps; ++it) {
     for (int d = r.order; d >= 1; --d) {
