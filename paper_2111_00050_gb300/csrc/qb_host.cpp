@@ -539,77 +539,71 @@ static int64_t host_rank(const Space& sp, const int* occ) {
 
 // ---------------------------------------------------------------- eigensolve
 
-// Eigen-decomposition of a Hermitian n x n matrix (n <= QB_MAX_MODES) by cyclic
-// Jacobi rotations on its real 2n x 2n symmetric embedding [[Re, -Im], [Im, Re]].
-// Every eigenvalue appears twice there; eig receives the n distinct-slot values
-// ascending, vec the unit eigenvector of the largest one.
+// Eigen-decomposition of a Hermitian n x n matrix (n <= QB_MAX_MODES) by cyclic complex
+// Jacobi rotations: eig receives the eigenvalues ascending, vec the unit eigenvector of the
+// largest one (its phase is arbitrary).  The rotated-out entries are set to zero, so that a
+// few sweeps end it; on the real 2n x 2n embedding, four times the entries, most of a
+// small space's qb_observables was this (M = 7: 0.4 of 0.56 ms).
 static void hermitian_eig(int n, const double* A /*[n*n] complex*/, double* eig, double* vec /*[n] complex*/) {
-  const int m = 2 * n;
-  std::vector<double> S((size_t)m * m), V((size_t)m * m, 0.0);
+  cd S[QB_MAX_MODES][QB_MAX_MODES], V[QB_MAX_MODES][QB_MAX_MODES];
   for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) {
-      double re = A[2 * (i * n + j)], im = A[2 * (i * n + j) + 1];
-      S[(size_t)i * m + j] = re;
-      S[(size_t)(i + n) * m + (j + n)] = re;
-      S[(size_t)(i + n) * m + j] = im;
-      S[(size_t)i * m + (j + n)] = -im;
+    for (int j = 0; j < n; ++j) {  // the Hermitian part
+      const double re = 0.5 * (A[2 * (i * n + j)] + A[2 * (j * n + i)]);
+      const double im = 0.5 * (A[2 * (i * n + j) + 1] - A[2 * (j * n + i) + 1]);
+      S[i][j] = cd(re, im);
+      V[i][j] = i == j ? 1.0 : 0.0;
     }
-  // symmetrise against rounding in the input
-  for (int i = 0; i < m; ++i)
-    for (int j = i + 1; j < m; ++j) {
-      double v = 0.5 * (S[(size_t)i * m + j] + S[(size_t)j * m + i]);
-      S[(size_t)i * m + j] = S[(size_t)j * m + i] = v;
-    }
-  for (int i = 0; i < m; ++i) V[(size_t)i * m + i] = 1.0;
+  auto mul = [](cd a, cd b) { return cd(a.real() * b.real() - a.imag() * b.imag(), a.real() * b.imag() + a.imag() * b.real()); };
   for (int sweep = 0; sweep < 100; ++sweep) {
     double off = 0.0, tot = 0.0;
-    for (int i = 0; i < m; ++i)
-      for (int j = 0; j < m; ++j) {
-        double v = S[(size_t)i * m + j] * S[(size_t)i * m + j];
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j) {
+        const double v = std::norm(S[i][j]);
         tot += v;
         if (i != j) off += v;
       }
     if (off <= 1e-32 * tot || off == 0.0) break;
-    for (int p = 0; p < m - 1; ++p)
-      for (int q = p + 1; q < m; ++q) {
-        double apq = S[(size_t)p * m + q];
-        if (apq == 0.0) continue;
-        double app = S[(size_t)p * m + p], aqq = S[(size_t)q * m + q];
-        double theta = (aqq - app) / (2.0 * apq);
-        double tt = (theta >= 0 ? 1.0 : -1.0) / (std::fabs(theta) + std::sqrt(theta * theta + 1.0));
-        double c = 1.0 / std::sqrt(tt * tt + 1.0), s = tt * c;
-        for (int k = 0; k < m; ++k) {  // columns p, q
-          double skp = S[(size_t)k * m + p], skq = S[(size_t)k * m + q];
-          S[(size_t)k * m + p] = c * skp - s * skq;
-          S[(size_t)k * m + q] = s * skp + c * skq;
+    for (int p = 0; p < n - 1; ++p)
+      for (int q = p + 1; q < n; ++q) {
+        const double m = std::abs(S[p][q]);
+        if (m == 0.0) continue;
+        const cd ph = S[p][q] / m;  // e^{i phi}
+        const double app = S[p][p].real(), aqq = S[q][q].real();
+        const double theta = (aqq - app) / (2.0 * m);
+        const double tt = (theta >= 0 ? 1.0 : -1.0) / (std::fabs(theta) + std::sqrt(theta * theta + 1.0));
+        const double c = 1.0 / std::sqrt(tt * tt + 1.0), s = tt * c;
+        const cd sp = s * ph, sm = std::conj(sp);
+        // columns: u_p = c e_p - s e^{-i phi} e_q, u_q = s e^{i phi} e_p + c e_q
+        for (int k = 0; k < n; ++k) {
+          const cd x = S[k][p], y = S[k][q];
+          S[k][p] = c * x - mul(sm, y);
+          S[k][q] = mul(sp, x) + c * y;
+          const cd vx = V[k][p], vy = V[k][q];
+          V[k][p] = c * vx - mul(sm, vy);
+          V[k][q] = mul(sp, vx) + c * vy;
         }
-        for (int k = 0; k < m; ++k) {  // rows p, q
-          double spk = S[(size_t)p * m + k], sqk = S[(size_t)q * m + k];
-          S[(size_t)p * m + k] = c * spk - s * sqk;
-          S[(size_t)q * m + k] = s * spk + c * sqk;
+        for (int k = 0; k < n; ++k) {  // rows: the adjoint
+          const cd x = S[p][k], y = S[q][k];
+          S[p][k] = c * x - mul(sp, y);
+          S[q][k] = mul(sm, x) + c * y;
         }
-        for (int k = 0; k < m; ++k) {
-          double vkp = V[(size_t)k * m + p], vkq = V[(size_t)k * m + q];
-          V[(size_t)k * m + p] = c * vkp - s * vkq;
-          V[(size_t)k * m + q] = s * vkp + c * vkq;
-        }
+        S[p][q] = S[q][p] = 0.0;
+        S[p][p] = S[p][p].real();
+        S[q][q] = S[q][q].real();
       }
   }
-  std::vector<int> order(m);
-  for (int i = 0; i < m; ++i) order[i] = i;
-  std::sort(order.begin(), order.end(), [&](int a, int b) { return S[(size_t)a * m + a] < S[(size_t)b * m + b]; });
-  for (int k = 0; k < n; ++k)
-    eig[k] = 0.5 * (S[(size_t)order[2 * k] * m + order[2 * k]] + S[(size_t)order[2 * k + 1] * m + order[2 * k + 1]]);
-  int top = order[m - 1];
+  int order[QB_MAX_MODES];
+  for (int i = 0; i < n; ++i) order[i] = i;
+  std::sort(order, order + n, [&](int a, int b) { return S[a][a].real() < S[b][b].real(); });
+  for (int k = 0; k < n; ++k) eig[k] = S[order[k]][order[k]].real();
+  const int top = order[n - 1];
   double nrm = 0.0;
-  for (int i = 0; i < n; ++i) {
-    double x = V[(size_t)i * m + top], y = V[(size_t)(i + n) * m + top];
-    vec[2 * i] = x;
-    vec[2 * i + 1] = y;
-    nrm += x * x + y * y;
-  }
+  for (int i = 0; i < n; ++i) nrm += std::norm(V[i][top]);
   nrm = std::sqrt(nrm);
-  for (int i = 0; i < 2 * n; ++i) vec[i] /= nrm;
+  for (int i = 0; i < n; ++i) {
+    vec[2 * i] = V[i][top].real() / nrm;
+    vec[2 * i + 1] = V[i][top].imag() / nrm;
+  }
 }
 
 // Derived observables of Sec. II C-E from the raw moments.
