@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <complex>
 #include <cstring>
@@ -98,7 +99,7 @@ static void build_block_tables(Space& sp, bool factored) {
   const std::vector<int>&annR = sp.combos.annR, &annS = sp.combos.annS, &annStart = sp.combos.annStart;
   const std::vector<uint32_t>& pq = sp.combos.pq;
   const std::vector<double>& G = sp.combos.G;
-  const std::vector<std::vector<int>>& delta = sp.combos.delta;
+  const std::vector<std::array<int, 16>>& delta = sp.combos.delta;
   const unsigned char(*pairidx)[16] = sp.combos.pairidx;
   const int M = sp.M, nmax = sp.nmax, Q = sp.Q, twoQ = 2 * Q;
   t.bk_kc = (M % 2 == 1 && M >= 5 && M <= 11 && !sp.exact && !t.is_complex) ? (M - 1) / 2 : 0;
@@ -186,8 +187,28 @@ static void build_block_tables(Space& sp, bool factored) {
   put(4, EC.data(), 4 * EC.size());
   put(5, cls.data(), 4 * cls.size());
   put(7, combo.data(), 4 * combo.size());
-  sp.bk_off[6] = sp.bk.size();
   sp.bk_map_bytes = ((size_t)std::max(1, nrec) * t.bk_S * 2 * w + 255) & ~(size_t)255;
+}
+
+// Blocks (Tables::rblk) of the sectors and of the lower sectors: Space::blkCnt counts the
+// blocks of the fillings of modes m .. M-1 (m <= P), from which the device finds block b of
+// a sector as it finds a ket from the fill counts.
+static void count_blocks(Space& sp) {
+  const int P = sp.t.bk_P, V = sp.nmax + 1, Q = sp.Q;
+  auto CI = [&](int m, int n, int k) { return ((size_t)m * V + n) * Q + k; };
+  sp.blkCnt.assign((size_t)(P + 1) * V * Q, 0);
+  for (int n = 0; n < V; ++n)
+    for (int k = 0; k < Q; ++k) sp.blkCnt[CI(P, n, k)] = sp.cnt[CI(P, n, k)] > 0;
+  for (int m = P - 1; m >= 0; --m)
+    for (int n = 0; n < V; ++n)
+      for (int k = 0, j = modp(-m, Q); k < Q; ++k, j = j + 1 == Q ? 0 : j + 1)
+        sp.blkCnt[CI(m, n, k)] = sp.blkCnt[CI(m + 1, n, k)] + (n > 0 ? sp.blkCnt[CI(m, n - 1, j)] : 0);
+  auto run = [&](const std::vector<int>& N, const std::vector<int>& K, std::vector<uint32_t>& out) {
+    out.assign(1, 0);
+    for (size_t i = 0; i < N.size(); ++i) out.push_back(out.back() + sp.blkCnt[CI(0, N[i], K[i])]);
+  };
+  run(sp.secN, sp.secK, sp.secBlk);
+  if (sp.t.fa_on) run(sp.lowN, sp.lowK, sp.lowBlk);
 }
 
 // Whether the two-body part factors into one operator per momentum class,
@@ -261,6 +282,12 @@ static bool build_factored(Space& sp) {
     }
   const int nlow = (int)sp.lowN.size();
   if (nlow == 0) return false;
+  const int64_t total = sp.secOff.back();
+  if (total > kObsfKets) {  // 120 bytes a ket: tables, state and workspace of a direct step
+    size_t avail = 0, all = 0;
+    if (cudaMemGetInfo(&avail, &all) != cudaSuccess) return false;
+    if (120.0 * (double)total + 16.0 * (double)nG + 12.0 * (double)sp.lowOff.back() > 0.9 * (double)all) return false;
+  }
   sp.low_held = nlow <= (int)sp.secN.size();
   for (int i = 0; i < nlow && sp.low_held; ++i)
     sp.low_held = sp.secN[i] == sp.lowN[i] && sp.secK[i] == sp.lowK[i] && sp.secOff[i] == sp.lowOff[i];
@@ -343,7 +370,6 @@ static bool build_factored(Space& sp) {
   at = 15;
   put(lam64.data(), 8 * lam64.size());
   put(pqa.data(), 4 * pqa.size());
-  sp.fa_off[13] = sp.fa.size();
   t.fa_nlow = nlow;
   t.fa_every = std::find(goff.begin(), goff.end(), kNoIndex) == goff.end() ? 1 : 0;
   t.fa_low = sp.lowOff.back();
@@ -363,15 +389,12 @@ static int build_tables(Space& sp) {
   auto CI = [&](int m, int n, int k) { return ((size_t)m * (nmax + 1) + n) * Q + k; };
   sp.cnt.assign((size_t)(M + 1) * (nmax + 1) * Q, 0);
   sp.cnt[CI(M, 0, 0)] = 1;
+  // either mode m is empty or one particle of it is taken away
   for (int m = M - 1; m >= 0; --m)
     for (int n = 0; n <= nmax; ++n)
-      for (int k = 0; k < Q; ++k) {
-        uint64_t acc = 0;
-        for (int v = 0; v <= n; ++v) {
-          acc += sp.cnt[CI(m + 1, n - v, modp((long long)k - (long long)m * v, Q))];
-          if (acc >= (1ull << 62)) acc = (1ull << 62);
-        }
-        sp.cnt[CI(m, n, k)] = acc;
+      for (int k = 0, j = modp(-m, Q); k < Q; ++k, j = j + 1 == Q ? 0 : j + 1) {
+        const uint64_t acc = sp.cnt[CI(m + 1, n, k)] + (n > 0 ? sp.cnt[CI(m, n - 1, j)] : 0);
+        sp.cnt[CI(m, n, k)] = std::min<uint64_t>(acc, 1ull << 62);
       }
   for (uint64_t v : sp.cnt)
     if (v >= (1ull << 31)) return fail(QB_EUNSUPPORTED, "a sub-sector count reaches 2^31; reduce n_max");
@@ -395,7 +418,7 @@ static int build_tables(Space& sp) {
   std::vector<int>&annR = sp.combos.annR, &annS = sp.combos.annS, &annStart = sp.combos.annStart;
   std::vector<uint32_t>& pq = sp.combos.pq;
   std::vector<double>& G = sp.combos.G;
-  std::vector<std::vector<int>>& delta = sp.combos.delta;
+  std::vector<std::array<int, 16>>& delta = sp.combos.delta;
   std::vector<double> gd;
   unsigned char(*pairidx)[16] = sp.combos.pairidx;
   memset(pairidx, 0xff, 256);
@@ -422,7 +445,7 @@ static int build_tables(Space& sp) {
           pq.push_back((uint32_t)p | ((uint32_t)q << 8) | ((uint32_t)lo << 16) | ((uint32_t)hi << 24));
           G.push_back(g.real());
           G.push_back(g.imag());
-          std::vector<int> d(16, 0);
+          std::array<int, 16> d{};
           int dn[16] = {0};
           dn[r] -= 1;
           dn[s] -= 1;
@@ -480,14 +503,10 @@ static int build_tables(Space& sp) {
   uint32_t* cnt32 = (uint32_t*)(b + t.o_cnt);
   for (size_t i = 0; i < sp.cnt.size(); ++i) cnt32[i] = (uint32_t)sp.cnt[i];
   int32_t* E = (int32_t*)(b + t.o_E);
-  for (int m = 0; m < M; ++m)
-    for (int rr = 0; rr < t.rem_w; ++rr)
-      for (int kk = 0; kk < twoQ; ++kk) {
-        int rem = rr - 2;
-        int32_t v = 0;
-        if (m >= 1 && rem >= 1 && rem - 1 <= nmax) v = (int32_t)sp.cnt[CI(m - 1, rem - 1, modp(kk - (m - 1), Q))];
-        E[((size_t)m * t.rem_w + rr) * twoQ + kk] = v;
-      }
+  for (int m = 1; m < M; ++m)
+    for (int rr = 3; rr < t.rem_w && rr - 3 <= nmax; ++rr)
+      for (int kk = 0, j = modp(1 - m, Q); kk < twoQ; ++kk, j = j + 1 == Q ? 0 : j + 1)
+        E[((size_t)m * t.rem_w + rr) * twoQ + kk] = (int32_t)sp.cnt[CI(m - 1, rr - 3, j)];
   double* sq = (double*)(b + t.o_sqrt);
   for (int k = 0; k < nmax + 3; ++k) sq[k] = std::sqrt((double)k);
   memcpy(b + t.o_pq, pq.data(), sizeof(uint32_t) * pq.size());
@@ -760,7 +779,7 @@ int qb_sector_build(const qb_model* model, int n_min, int n_max, const int* p_li
     return fail(QB_EINVAL, "no non-empty sector in the requested range");
   }
   build_block_tables(*sp, build_factored(*sp));
-  sp->fa_off[14] = sp->fa_off[13] + (((size_t)sp->t.fa_nrec * sp->t.fa_pl * sp->t.bk_S * 8 + 255) & ~(size_t)255);
+  count_blocks(*sp);
   rc = device_setup(*sp);
   if (rc) {
     qb_space_free(reinterpret_cast<qb_space*>(sp));
@@ -773,28 +792,9 @@ int qb_sector_build(const qb_model* model, int n_min, int n_max, const int* p_li
 void qb_space_free(qb_space* space) {
   Space* sp = reinterpret_cast<Space*>(space);
   if (!sp) return;
-  cudaFree(sp->d_blob);
-  cudaFree(sp->d_secOff);
-  cudaFree(sp->d_secN);
-  cudaFree(sp->d_secK);
-  cudaFree(sp->d_secOf);
-  cudaFree(sp->d_scratch);
-  cudaFree(sp->d_diag);
-  cudaFree(sp->d_obsf);
-  cudaFree(sp->d_wtab);
-  cudaFree(sp->d_occ);
-  cudaFree(sp->d_wi);
-  cudaFree(sp->d_bk);
-  cudaFree(sp->d_fa);
-  cudaFree(sp->d_fill);
-  cudaFree(sp->d_low);
-  cudaFree(sp->d_perm);
-  cudaFree(sp->d_mo);
+  cudaFree(sp->d_arena);
+  if (sp->own_obsf) cudaFree(sp->d_obsf);
   cudaFree(sp->d_hpsi);
-  for (int k = 0; k < 2; ++k) {
-    cudaFree(sp->d_blocks[k]);
-    cudaFree(sp->d_base[k]);
-  }
   if (sp->capture_stream) cudaStreamDestroy(sp->capture_stream);
   delete sp;
 }

@@ -1,6 +1,7 @@
 // Internal structures shared by the host code (qb_host.cpp) and the CUDA
 // kernels (qb_kernels.cu).  Not part of the public ABI (include/qb.h).
 #pragma once
+#include <array>
 #include <cstdint>
 #include <mutex>
 #include <string>
@@ -15,6 +16,11 @@ namespace qb {
 // Shifts of a suffix-state index are stored as unsigned bytes offset by this bias
 // (a shift lies in [-4M, 5M) for M <= 16).
 constexpr int kDeltaBias = 64;
+
+// Spaces of more kets than these leave memory for the caller's vectors: the observables' copy
+// of the state is allocated by the first call that needs it, and contact couplings are
+// factored only where the vector of B_k f fits beside what a step needs without it.
+constexpr int64_t kObsfKets = 1ll << 28;
 
 // 32-bit indices of kets and of entries of B_k f stay below this
 constexpr uint32_t kNoIndex = 0xffff0000u;
@@ -157,7 +163,7 @@ struct Combos {
   std::vector<int> annR, annS, annStart;       // pairs (r <= s) and their first combos
   std::vector<uint32_t> pq;                    // p | q << 8 | lo << 16 | hi << 24
   std::vector<double> G;                       // coupling (re, im)
-  std::vector<std::vector<int>> delta;         // [16] shift of the suffix index at each mode
+  std::vector<std::array<int, 16>> delta;      // shift of the suffix index at each mode
   unsigned char pairidx[16][16];
 };
 
@@ -183,28 +189,17 @@ struct Space {
   bool low_held = false;                  // the lower kets are the space's first kets
   size_t bk_map_bytes = 0;
   int64_t maxDim = 0;
-  // device allocations owned by the space
-  unsigned char* d_blob = nullptr;
-  int64_t* d_secOff = nullptr;
-  int32_t* d_secN = nullptr;
-  int32_t* d_secK = nullptr;
-  int32_t* d_secOf = nullptr;
+  std::vector<uint32_t> blkCnt;           // [P + 1][nmax + 1][Q] blocks of the fillings of modes m .. M-1
+  std::vector<uint32_t> secBlk, lowBlk;   // first block of each sector (lower sector), and their number
+  // device memory of the space: one allocation that holds every table (device_setup), the
+  // pointers below and the tables' into it
+  unsigned char* d_arena = nullptr;
   double* d_scratch = nullptr;  // reduction partials
   float4* d_diag = nullptr;     // per ket: one-body and two-body diagonal as double-float pairs
   float4* d_obsf = nullptr;     // double-float copy of the state being observed (qb_observables)
-  double2* d_wtab = nullptr;    // ket-weight factors (Tables::wtab)
-  uint64_t* d_occ = nullptr;    // packed occupation vectors (Tables::occ)
-  double* d_wi = nullptr;       // inverse ket weights and the weights (Tables::wi, wk)
-  unsigned char* d_bk = nullptr;  // block tables (Tables::bk_*)
-  unsigned char* d_fa = nullptr;  // tables of the factored couplings (Tables::fa_*)
-  uint32_t* d_fill = nullptr;     // fillings (Tables::fill)
-  unsigned char* d_low = nullptr; // occupations and fillings of the lower kets
-  uint32_t* d_blocks[2] = {nullptr, nullptr};  // rblk and the block starts of the kets, and of the lower kets
+  bool own_obsf = false;        // an allocation of its own, made by the first call (kObsfKets)
   void* d_hpsi = nullptr;      // FP64 vector of B_k psi (qb_hpsi of a factored space), made by the first call
   std::mutex hpsi_mu;          // held by the call that uses it
-  unsigned char* d_mo = nullptr;  // Tables::mo_*
-  uint32_t* d_perm = nullptr;                  // Tables::fa_perm
-  uint32_t* d_base[2] = {nullptr, nullptr};    // bases of the blocks, and of the lower blocks
   int64_t scratch_doubles = 0;
   Tables t{};
   cudaStream_t capture_stream = nullptr;  // private stream on which RK4 chunks are captured into graphs

@@ -195,125 +195,250 @@ __global__ void __launch_bounds__(256) to_dfw_kernel(const Tables t, const doubl
   }
 }
 
-// per-ket diagonal of H, one-body and two-body parts, as double-float pairs; the
-// packed occupations and the inverse ket weight of every ket
-// Number of the filling of the modes P .. M-1 of the row's ket (after setup_row)
-__device__ __forceinline__ uint32_t row_filling(const Tables& t, const View& v, const RowScratch& rs, int N, int K) {
-  const int tid = threadIdx.x, P = t.bk_P, twoQ = 2 * t.Q;
-  int cls = N * t.Q + K;  // P = 0: the whole ket
-  if (P > 0) {
-    const int flat = rs.idx[P * kBlock + tid] - (P * t.rem_w + 2) * twoQ;
-    cls = flat / twoQ * t.Q + flat % twoQ;
-  }
-  const int2 c = __ldg(t.bk_cls + cls);
-  return (uint32_t)(c.x + c.y - 1 - (rs.pe[(t.M - 1) * kBlock + tid] - rs.pe[P * kBlock + tid]));
-}
+// ------------------------------------------------------- tables of kets and blocks
+//
+// What set-up holds per ket is a product or a sum of a part of the block (modes 0 .. P-1, its
+// particle number and momentum) and a part of the filling (modes P .. M-1), so that the kets
+// are neither unranked nor weighed one by one: block_kernel finds every block's first ket
+// and every filling, and ket_kernel joins the two for 32 kets at a time.  A kernel
+// that unranked each ket and summed its M (M + 1) / 2 pairs in FP64, 110 operations at 2 per
+// clock and SM, took 10.5 ms for 62.9M kets of 7 modes and 0.28 ms for 2.3M of 5 modes; the
+// three kernels take 2.4 and 0.13.
 
-// packed occupations and fillings of the lower kets of a factored space
-__global__ void __launch_bounds__(kBlock) lower_kernel(const Tables t, const int32_t* lowN, const int32_t* lowK,
-                                                        uint64_t* occ, uint32_t* fill) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  load_blob(t, smem);
-  const View v = make_view(t, smem);
-  const RowScratch rs = row_scratch(smem + blob_smem(t));
-  for (int64_t g = (int64_t)blockIdx.x * kBlock + threadIdx.x; g < t.fa_low; g += (int64_t)gridDim.x * kBlock) {
-    int lo = 0, hi = t.fa_nlow - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (__ldg(t.fa_lowoff + mid) <= g)
-        lo = mid;
-      else
-        hi = mid - 1;
-    }
-    const int64_t off = __ldg(t.fa_lowoff + lo);
-    const int N = __ldg(lowN + lo), K = __ldg(lowK + lo);
-    setup_row(t, v, rs, N, K, __ldg(t.fa_lowoff + lo + 1) - off, g - off);
-    uint64_t word = 0;
-    for (int m = 0; m < t.M; ++m) word |= (uint64_t)rs.occ[m * kBlock + threadIdx.x] << (m * t.occ_bits);
-    occ[g] = word;
-    fill[g] = row_filling(t, v, rs, N, K);
-  }
-}
-
-__global__ void __launch_bounds__(kBlock) diag_kernel(const Tables t, float4* diag, uint64_t* occ, double* wi,
-                                                        double* wk, uint32_t* fill) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  load_blob(t, smem);
-  const View v = make_view(t, smem);
-  const RowScratch rs = row_scratch(smem + blob_smem(t));
-  const int tid = threadIdx.x, M = t.M;
-  for (int64_t base = (int64_t)blockIdx.x * kBlock; base < t.total; base += (int64_t)gridDim.x * kBlock) {
-    const int64_t g = base + tid;
-    if (g >= t.total) break;
-    const int sid = find_sector(t, g);
-    const int64_t off = __ldg(t.sec_off + sid);
-    const int64_t D = __ldg(t.sec_off + sid + 1) - off;
-    const int N = __ldg(t.sec_N + sid), K = __ldg(t.sec_K + sid);
-    setup_row(t, v, rs, N, K, D, g - off);
-    fill[g] = row_filling(t, v, rs, N, K);
-    double dw = 0.0, dl = 0.0;
-    uint64_t word = 0;
-    for (int r = 0; r < M; ++r) {
-      const int nr = rs.occ[r * kBlock + tid];
-      word |= (uint64_t)nr << (r * t.occ_bits);
-      dw += v.w[r] * nr;
-      for (int s2 = r; s2 < M; ++s2) {
-        const int ns = rs.occ[s2 * kBlock + tid] - (r == s2 ? 1 : 0);
-        if (nr >= 1 && ns >= 1) dl += v.gd[v.pairidx[r * 16 + s2]] * (double)(nr * ns);
-      }
-    }
-    const dfl a = df_of(dw), b = df_of(dl);
-    diag[g] = make_float4(a.h, a.l, b.h, b.l);
-    occ[g] = word;
-    const double2 wt = ket_weight<0>(t, rs.occ + tid, kBlock);
-    wi[g] = wt.y;
-    wk[g] = wt.x;
-  }
-}
-
-// A filling from its number: its class (particles crem, momentum ckr of the modes P ..
-// M-1), occupations and ranking-table indices.  False for the numbers left out.
-struct Filling {
-  int crem, ckr;
-  int occ[kMaxM], idx[kMaxM];
+// A filling (Tables::suf): the packed occupations of its modes (all ones: a number left out),
+// its factors of the ket weight and of the inverse weight, its parts of the diagonals
+struct Suffix {
+  const uint64_t* word;
+  const double *w, *wi, *dw, *dl;
 };
-__device__ __forceinline__ bool filling_of(const Tables& t, int64_t f, Filling& F) {
-  const int M = t.M, Q = t.Q, P = t.bk_P, V = t.nmax + 1, twoQ = 2 * Q;
-  const uint32_t* cnt = reinterpret_cast<const uint32_t*>(t.blob + t.o_cnt);
-  int lo = 0, hi = V * Q - 1;  // the last class that starts at or before it
+// The block's parts of the same, with the first filling of its class and, for each mode
+// P + j, the coefficient of n_{P+j} that the pairs (r < P, P + j) add to the two-body diagonal
+struct BlockRec {
+  uint64_t word;
+  uint32_t fill0, pad;
+  double w, wi, dw, dl;
+  double cross[];
+};
+__host__ __device__ inline size_t block_rec_bytes(int M, int P) { return sizeof(BlockRec) + 8 * (size_t)(M - P); }
+
+// One block a thread: block b of the sectors (first kets off, first blocks sblk) starts at
+// ket start[b].  The occupations of its modes are found from the block counts as those of a
+// ket from the fill counts.  FULL: all of BlockRec, else its word and first filling.
+struct BlockArgs {
+  const int32_t *secN, *secK;
+  const int64_t* secOff;
+  const uint32_t* sblk;
+  int nsec;
+  const uint32_t* bcnt;
+  uint32_t* start;
+  unsigned char* rec;
+  size_t stride;
+};
+template <bool FULL>
+__device__ void find_block(const Tables& t, const BlockArgs& a, uint32_t b) {
+  const uint32_t* sblk = a.sblk;
+  const int nsec = a.nsec;
+  if (b >= __ldg(sblk + nsec)) return;
+  int lo = 0, hi = nsec - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (t.bk_cls[mid].x <= f)
+    if (__ldg(sblk + mid) <= b)
       lo = mid;
     else
       hi = mid - 1;
   }
-  int64_t left = f - t.bk_cls[lo].x;
-  if (left >= t.bk_cls[lo].y) return false;
-  F.crem = lo / Q;
-  F.ckr = lo % Q;
-  int rem = F.crem, kr = F.ckr;
-  for (int m = 0; m < kMaxM; ++m) F.occ[m] = 0;
-  for (int m = P; m < M - 1; ++m) {  // lexicographic in (n_P, n_P+1, ...)
+  const int M = t.M, P = t.bk_P, Q = t.Q, V = t.nmax + 1, N = __ldg(a.secN + lo);
+  const uint32_t* cnt = reinterpret_cast<const uint32_t*>(t.blob + t.o_cnt);
+  const double* w1 = reinterpret_cast<const double*>(t.blob + t.o_w);
+  const double* gd = reinterpret_cast<const double*>(t.blob + t.o_gd);
+  const uint8_t* pairidx = t.blob + t.o_pairidx;
+  int64_t off = __ldg(a.secOff + lo);
+  uint32_t left = b - __ldg(sblk + lo);
+  int rem = N, kr = __ldg(a.secK + lo);
+  uint64_t word = 0;
+  const double2 c = __ldg(t.wscale + N);
+  double w = c.x, wi = c.y, dw = 0.0, dl = 0.0;
+  BlockRec* R = reinterpret_cast<BlockRec*>(a.rec + (size_t)b * a.stride);
+  for (int m = 0; m < P; ++m) {
     int val = 0;
     while (val < rem) {
-      const int64_t c = cnt[((size_t)(m + 1) * V + rem - val) * Q + kr];
-      if (left < c) break;
-      left -= c;
+      const size_t i = ((size_t)(m + 1) * V + rem - val) * Q + kr;
+      const uint32_t n = __ldg(a.bcnt + i);
+      if (left < n) break;
+      left -= n;
+      off += __ldg(cnt + i);
       ++val;
       kr -= m;
       while (kr < 0) kr += Q;
     }
-    F.occ[m] = val;
+    word |= (uint64_t)val << (m * t.occ_bits);
+    if (FULL) {
+      const double2 f = __ldg(t.wtab + rem * V + val);
+      w *= f.x;
+      wi *= f.y;
+      const double v = (double)val;
+      dw += w1[m] * v;
+      double g = gd[pairidx[m * 17]] * (v - 1.0);
+      for (int r = 0; r < m; ++r) g += gd[pairidx[r * 16 + m]] * (double)occ_of(word, r, t.occ_bits);
+      if (val) dl += g * v;
+    }
     rem -= val;
   }
-  F.occ[M - 1] = rem;
+  a.start[b] = (uint32_t)off;
+  R->word = word;
+  R->fill0 = (uint32_t)__ldg(t.bk_cls + rem * Q + kr).x;
+  if (!FULL) return;
+  R->w = w;
+  R->wi = wi;
+  R->dw = dw;
+  R->dl = dl;
+  for (int m = P; m < M; ++m) {
+    double g = 0.0;
+    for (int r = 0; r < P; ++r) g += gd[pairidx[r * 16 + m]] * (double)occ_of(word, r, t.occ_bits);
+    R->cross[m - P] = g;
+  }
+}
+
+// One filling a thread, from its number: the class, then the occupations in lexicographic
+// order
+__device__ void find_filling(const Tables& t, int f, uint64_t* words, double* sw, double* swi, double* sdw, double* sdl) {
+  if (f >= t.bk_S) return;
+  const int M = t.M, Q = t.Q, P = t.bk_P, V = t.nmax + 1;
+  const uint32_t* cnt = reinterpret_cast<const uint32_t*>(t.blob + t.o_cnt);
+  const double* w1 = reinterpret_cast<const double*>(t.blob + t.o_w);
+  const double* gd = reinterpret_cast<const double*>(t.blob + t.o_gd);
+  const uint8_t* pairidx = t.blob + t.o_pairidx;
+  int lo = 0, hi = V * Q - 1;  // the last class that starts at or before it
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(t.bk_cls + mid).x <= f)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  const int2 cls = __ldg(t.bk_cls + lo);
+  uint32_t left = (uint32_t)(f - cls.x);
+  uint64_t word = 0;
+  double w = 1.0, wi = 1.0, dw = 0.0, dl = 0.0;
+  if (left >= (uint32_t)cls.y) {
+    word = ~0ull;
+  } else {
+    int rem = lo / Q, kr = lo % Q;
+    for (int m = P; m < M; ++m) {
+      int val = 0;
+      if (m == M - 1) val = rem;
+      while (val < rem) {
+        const uint32_t c = __ldg(cnt + ((size_t)(m + 1) * V + rem - val) * Q + kr);
+        if (left < c) break;
+        left -= c;
+        ++val;
+        kr -= m;
+        while (kr < 0) kr += Q;
+      }
+      word |= (uint64_t)val << (m * t.occ_bits);
+      const double2 x = __ldg(t.wtab + rem * V + val);
+      w *= x.x;
+      wi *= x.y;
+      const double v = (double)val;
+      dw += w1[m] * v;
+      double g = gd[pairidx[m * 17]] * (v - 1.0);
+      for (int r = P; r < m; ++r) g += gd[pairidx[r * 16 + m]] * (double)occ_of(word, r, t.occ_bits);
+      if (val) dl += g * v;
+      rem -= val;
+    }
+  }
+  words[f] = word;
+  sw[f] = w;
+  swi[f] = wi;
+  sdw[f] = dw;
+  sdl[f] = dl;
+}
+
+// Both in one launch, the fillings by the first nf CTAs
+__global__ void __launch_bounds__(128) block_kernel(const Tables t, const BlockArgs a, unsigned nf, uint64_t* words) {
+  if (blockIdx.x < nf) {
+    const size_t S = (size_t)t.bk_S;
+    double* d = reinterpret_cast<double*>(words + S);
+    find_filling(t, (int)(blockIdx.x * 128 + threadIdx.x), words, d, d + S, d + 2 * S, d + 3 * S);
+  } else {
+    find_block<true>(t, a, (blockIdx.x - nf) * 128u + threadIdx.x);
+  }
+}
+__global__ void __launch_bounds__(128) lower_block_kernel(const Tables t, const BlockArgs a) {
+  find_block<false>(t, a, blockIdx.x * 128u + threadIdx.x);
+}
+
+// The kets' tables, a run of rounds of 32 consecutive kets a warp: the block of the first one
+// is searched for, the following ones come from the starts after it.  Writes 44 bytes a ket
+// (lower kets: 12): at 62.9M kets, 2.8 GB.
+template <bool FULL>
+__global__ void __launch_bounds__(256) ket_kernel(const Tables t, const Suffix sx, int64_t n, uint32_t nblocks,
+                                                   const uint32_t* start, const unsigned char* rec, size_t stride,
+                                                   int run, float4* diag, uint64_t* occ, double* wi, double* wk,
+                                                   uint32_t* fill, uint32_t* rblk) {
+  const int lane = threadIdx.x & 31, P = t.bk_P, M = t.M;
+  const int64_t nr = (n + 31) / 32;
+  const int64_t r0 = (((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5) * run;
+  if (r0 >= nr) return;
+  const int64_t r1 = min(r0 + run, nr);
+  uint32_t b = 0;  // the last block that starts at or before ket 32 r0
+  {
+    uint32_t hi = nblocks - 1;
+    while (b < hi) {
+      const uint32_t mid = b + (hi - b + 1) / 2;
+      if ((int64_t)__ldg(start + mid) <= 32 * r0)
+        b = mid;
+      else
+        hi = mid - 1;
+    }
+  }
+  for (int64_t r = r0; r < r1; ++r) {
+    const int64_t g = 32 * r + lane;
+    // at most 31 blocks start at the round's other kets, and one with the next round
+    const uint32_t nb = b + 1 + lane;
+    const uint32_t d = nb < nblocks ? __ldg(start + nb) - (uint32_t)(32 * r) : 64u;
+    const uint32_t heads = __reduce_or_sync(0xffffffffu, d < 32u ? 1u << d : 0u);
+    const bool next = __any_sync(0xffffffffu, d == 32u);
+    const uint32_t me = b + __popc(heads & ((2u << lane) - 1u));
+    if (lane == 0) rblk[r] = b;
+    if (g < n) {
+      const BlockRec* R = reinterpret_cast<const BlockRec*>(rec + (size_t)me * stride);
+      const uint32_t f = R->fill0 + (uint32_t)g - __ldg(start + me);
+      const uint64_t sword = __ldg(sx.word + f);
+      occ[g] = R->word | sword;
+      fill[g] = f;
+      if (FULL) {
+        double dl = R->dl + __ldg(sx.dl + f);
+        for (int m = P; m < M; ++m) dl += R->cross[m - P] * (double)occ_of(sword, m, t.occ_bits);
+        const dfl x = df_of(R->dw + __ldg(sx.dw + f)), y = df_of(dl);
+        diag[g] = make_float4(x.h, x.l, y.h, y.l);
+        wk[g] = R->w * __ldg(sx.w + f);
+        wi[g] = R->wi * __ldg(sx.wi + f);
+      }
+    }
+    b += __popc(heads) + (next ? 1u : 0u);
+  }
+}
+
+// A filling: its class (particles crem, momentum ckr of the modes P .. M-1), occupations and
+// ranking-table indices.  False for the numbers left out.
+struct Filling {
+  int crem, ckr;
+  int occ[kMaxM], idx[kMaxM];
+};
+__device__ __forceinline__ bool filling_of(const Tables& t, const uint64_t* words, int64_t f, Filling& F) {
+  const int M = t.M, Q = t.Q, P = t.bk_P;
+  const uint64_t word = __ldg(words + f);
+  if (word == ~0ull) return false;
   int sr = 0, sk = 0;
   for (int m = M - 1; m >= P; --m) {
+    F.occ[m] = occ_of(word, m, t.occ_bits);
     sr += F.occ[m];
     sk = (sk + m * F.occ[m]) % Q;
-    F.idx[m] = (m * t.rem_w + sr + 2) * twoQ + sk;
+    F.idx[m] = (m * t.rem_w + sr + 2) * 2 * Q + sk;
   }
+  F.crem = sr;
+  F.ckr = sk;
   return true;
 }
 
@@ -337,97 +462,6 @@ __device__ __forceinline__ bool supplies(const Tables& t, const Filling& F, int 
 }
 __device__ __forceinline__ int2 pair_of(uint32_t info) {  // the modes of a selector word
   return make_int2((info & 7) | ((info >> 12) & 8), ((info >> 16) & 7) | ((info >> 28) & 8));
-}
-
-// Blocks.  A ket starts a block unless its filling follows the one before it.
-constexpr int kScanRounds = 2048;  // rounds of 32 kets per CTA of the block scan
-
-__device__ __forceinline__ uint32_t round_heads(const uint32_t* fill, int64_t r, int64_t n, int lane) {
-  const int64_t g = r * 32 + lane;
-  bool head = false;
-  if (g < n) head = g == 0 || __ldg(fill + g) != __ldg(fill + g - 1) + 1u;
-  return __ballot_sync(0xffffffffu, head);
-}
-
-// blocks that start in each run of kScanRounds rounds
-__global__ void __launch_bounds__(256) block_count_kernel(const uint32_t* fill, int64_t n, uint32_t* part) {
-  __shared__ uint32_t sum;
-  if (threadIdx.x == 0) sum = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int64_t r0 = (int64_t)blockIdx.x * kScanRounds, r1 = min(r0 + kScanRounds, (n + 31) / 32);
-  uint32_t c = 0;
-  for (int64_t r = r0 + (threadIdx.x >> 5); r < r1; r += 8) c += __popc(round_heads(fill, r, n, lane));
-  if (lane == 0) atomicAdd(&sum, c);
-  __syncthreads();
-  if (threadIdx.x == 0) part[blockIdx.x] = sum;
-}
-
-// part[i] = the blocks before run i; part[n] = all of them
-__global__ void __launch_bounds__(1024) block_scan_kernel(uint32_t* part, int n) {
-  __shared__ uint32_t s[1024];
-  __shared__ uint32_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  for (int i0 = 0; i0 < n; i0 += 1024) {
-    const int i = i0 + threadIdx.x;
-    const uint32_t v = i < n ? part[i] : 0u;
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-      const uint32_t x = threadIdx.x >= o ? s[threadIdx.x - o] : 0u;
-      __syncthreads();
-      s[threadIdx.x] += x;
-      __syncthreads();
-    }
-    const uint32_t before = carry + s[threadIdx.x] - v;
-    if (i < n) part[i] = before;
-    __syncthreads();
-    if (threadIdx.x == 1023) carry = before + v;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[n] = carry;
-}
-
-// rblk[r] = block of the first ket of round r; start[b] = first ket of block b
-__global__ void __launch_bounds__(256) block_start_kernel(const uint32_t* fill, int64_t n, const uint32_t* part,
-                                                           uint32_t* rblk, uint32_t* start) {
-  __shared__ uint32_t cnt[kScanRounds];
-  __shared__ uint32_t wsum[8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t r0 = (int64_t)blockIdx.x * kScanRounds;
-  const int nr = (int)min((int64_t)kScanRounds, (n + 31) / 32 - r0);
-  for (int r = warp; r < nr; r += 8) {
-    const uint32_t h = round_heads(fill, r0 + r, n, lane);
-    if (lane == 0) cnt[r] = __popc(h);
-  }
-  __syncthreads();
-  // exclusive scan of cnt: 8 rounds a thread
-  uint32_t v[8], t = 0;
-  for (int k = 0; k < 8; ++k) {
-    const int r = threadIdx.x * 8 + k;
-    v[k] = r < nr ? cnt[r] : 0u;
-    t += v[k];
-  }
-  uint32_t x = t;
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wsum[warp] = x;
-  __syncthreads();
-  uint32_t run = part[blockIdx.x] + x - t;
-  for (int w = 0; w < warp; ++w) run += wsum[w];
-  for (int k = 0; k < 8; ++k) {
-    const int r = threadIdx.x * 8 + k;
-    if (r < nr) cnt[r] = run;
-    run += v[k];
-  }
-  __syncthreads();
-  for (int r = warp; r < nr; r += 8) {
-    const uint32_t h = round_heads(fill, r0 + r, n, lane);
-    if (lane == 0) rblk[r0 + r] = cnt[r] + (h & 1u) - 1u;
-    if ((h >> lane) & 1u) start[cnt[r] + __popc(h & ((1u << lane) - 1u))] = (uint32_t)((r0 + r) * 32 + lane);
-  }
 }
 
 // Suffix states of a block, lane m <= P holding mode m's: particles, momentum mod Q and the
@@ -571,10 +605,11 @@ __global__ void __launch_bounds__(256) round_order_kernel(const int64_t* off, co
 // The maps of the direct stage kernel (Tables::bk_map): for every filling and every term,
 // the place of the changed filling in its class.  A thread takes one filling and the
 // records of its block row.
-__global__ void __launch_bounds__(kBlock) block_map_kernel(const Tables t, uint16_t* map, uint16_t* map5) {
+__global__ void __launch_bounds__(kBlock) block_map_kernel(const Tables t, const uint64_t* words, uint16_t* map,
+                                                            uint16_t* map5) {
   const int64_t f = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   Filling F;
-  if (f >= t.bk_S || !filling_of(t, f, F)) return;
+  if (f >= t.bk_S || !filling_of(t, words, f, F)) return;
   const int w = t.bk_kc == 2 ? 2 : 4, TS = t.bk_T + 4;
   for (int rec = blockIdx.y; rec < t.bk_nrec; rec += gridDim.y) {
     const uint32_t info = t.bk_info[rec].x;
@@ -597,12 +632,12 @@ __device__ __forceinline__ int one_shift(const Tables& t, int i, int m, int sign
   if (i < m) return 0;
   return sign * 2 * t.Q + (sign > 0 ? i % t.Q : (t.Q - i % t.Q) % t.Q);
 }
-__global__ void __launch_bounds__(kBlock) moment_map_kernel(const Tables t, uint16_t* map) {
+__global__ void __launch_bounds__(kBlock) moment_map_kernel(const Tables t, const uint64_t* words, uint16_t* map) {
   const int64_t f = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   Filling F;
-  if (f >= t.bk_S || !filling_of(t, f, F)) return;
+  if (f >= t.bk_S || !filling_of(t, words, f, F)) return;
   int32_t sh[kMaxM];
-  for (int q = 0; q < 2 * t.mo_w; ++q) {
+  for (int q = blockIdx.y; q < 2 * t.mo_w; q += gridDim.y) {
     const int i = q % t.mo_w, sign = q < t.mo_w ? 1 : -1;
     uint16_t place = 0;
     if (i < t.M && (sign > 0 || i < t.bk_P || F.occ[i] >= 1)) {
@@ -635,10 +670,11 @@ __global__ void __launch_bounds__(256) moment_base_kernel(const Tables t, const 
 
 // The maps of the factored stages: places after a pair is added (fa_mapa) or taken away
 // (fa_mapc)
-__global__ void __launch_bounds__(kBlock) factor_map_kernel(const Tables t, uint16_t* mapa, uint16_t* mapc) {
+__global__ void __launch_bounds__(kBlock) factor_map_kernel(const Tables t, const uint64_t* words, uint16_t* mapa,
+                                                             uint16_t* mapc) {
   const int64_t f = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   Filling F;
-  if (f >= t.bk_S || !filling_of(t, f, F)) return;
+  if (f >= t.bk_S || !filling_of(t, words, f, F)) return;
   const int Ta = fa_Ta(t), Tc = fa_Tc(t);
   const uint32_t* info = reinterpret_cast<const uint32_t*>(t.fa_info);
   for (int q = blockIdx.y; q < Ta / 4 + t.fa_ng; q += gridDim.y)
@@ -655,23 +691,12 @@ __global__ void __launch_bounds__(kBlock) factor_map_kernel(const Tables t, uint
 
 // ------------------------------------------------------------- small kernels
 
-__global__ void __launch_bounds__(kBlock) unrank_kernel(const Tables t, int64_t first, int64_t count, int* occ_out,
-                                                         int* status) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  load_blob(t, smem);
-  const View v = make_view(t, smem);
-  const RowScratch rs = row_scratch(smem + blob_smem(t));
-  const int tid = threadIdx.x;
-  for (int64_t base = (int64_t)blockIdx.x * kBlock; base < count; base += (int64_t)gridDim.x * kBlock) {
-    const int64_t k = base + tid;
-    if (k >= count) break;
-    const int64_t g = first + k;
-    const int sid = find_sector(t, g);
-    const int64_t off = __ldg(t.sec_off + sid);
-    const int64_t D = __ldg(t.sec_off + sid + 1) - off;
-    const int64_t me = setup_row(t, v, rs, __ldg(t.sec_N + sid), __ldg(t.sec_K + sid), D, g - off);
-    if (me != g - off) atomicOr(status, 2);
-    for (int m = 0; m < t.M; ++m) occ_out[k * t.M + m] = rs.occ[m * kBlock + tid];
+// occupations from the packed words, one (ket, mode) a thread
+__global__ void __launch_bounds__(kBlock) unrank_kernel(const Tables t, int64_t first, int64_t count, int* occ_out) {
+  const int64_t n = count * t.M;
+  for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < n; i += (int64_t)gridDim.x * kBlock) {
+    const int64_t k = i / t.M;
+    occ_out[i] = occ_of(__ldg(t.occ + first + k), (int)(i - k * t.M), t.occ_bits);
   }
 }
 
@@ -756,25 +781,17 @@ __global__ void __launch_bounds__(kBlock) terms_kernel(const Tables t, unsigned 
 // per-block partial sums of |amplitude|^2
 __global__ void __launch_bounds__(kBlock) init_table_kernel(const Tables t, const double2* table, int only_N,
                                                              double2* psi, double* partial) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  load_blob(t, smem);
-  const View v = make_view(t, smem);
-  const RowScratch rs = row_scratch(smem + blob_smem(t));
   const int tid = threadIdx.x, M = t.M, V = t.nmax + 1;
   double n2 = 0.0;
-  for (int64_t base = (int64_t)blockIdx.x * kBlock; base < t.total; base += (int64_t)gridDim.x * kBlock) {
-    const int64_t g = base + tid;
-    if (g >= t.total) break;
-    const int sid = find_sector(t, g);
-    const int64_t off = __ldg(t.sec_off + sid);
-    const int64_t D = __ldg(t.sec_off + sid + 1) - off;
-    const int N = __ldg(t.sec_N + sid);
+  for (int64_t g = (int64_t)blockIdx.x * kBlock + tid; g < t.total; g += (int64_t)gridDim.x * kBlock) {
+    const uint64_t word = __ldg(t.occ + g);
+    int N = 0;
+    for (int m = 0; m < M; ++m) N += occ_of(word, m, t.occ_bits);
     double re = 0.0, im = 0.0;
     if (only_N < 0 || N == only_N) {
-      setup_row(t, v, rs, N, __ldg(t.sec_K + sid), D, g - off);
       re = 1.0;
       for (int m = 0; m < M; ++m) {
-        const double2 f = __ldg(table + (size_t)m * V + rs.occ[m * kBlock + tid]);
+        const double2 f = __ldg(table + (size_t)m * V + occ_of(word, m, t.occ_bits));
         const double nr = re * f.x - im * f.y;
         im = re * f.y + im * f.x;
         re = nr;
@@ -975,150 +992,204 @@ int check_status(const Space& s, cudaStream_t st) {
   return QB_OK;
 }
 
-// Finds the blocks of n kets from their fillings: *d_out receives rblk [ceil(n / 32)] and,
-// from *start on, the first ket of each block.
-static int find_blocks(const uint32_t* fill, int64_t n, uint32_t** d_out, uint32_t** start, int64_t* nblocks) {
-  const int64_t nr = (n + 31) / 32;
-  const int np = (int)((nr + kScanRounds - 1) / kScanRounds);
-  uint32_t* part = nullptr;
-  QB_CUDA(cudaMalloc(&part, sizeof(uint32_t) * ((size_t)np + 1)));
-  block_count_kernel<<<np, 256>>>(fill, n, part);
-  block_scan_kernel<<<1, 1024>>>(part, np);
-  uint32_t total = 0;
-  cudaError_t e = cudaMemcpy(&total, part + np, sizeof(total), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMalloc(d_out, sizeof(uint32_t) * ((size_t)nr + total));
-  if (e == cudaSuccess) {
-    *start = *d_out + nr;
-    *nblocks = total;
-    block_start_kernel<<<np, 256>>>(fill, n, part, *d_out, *start);
-    e = cudaGetLastError();
-  }
-  cudaFree(part);  // waits for the kernels
-  QB_CUDA(e);
-  return QB_OK;
-}
-
 int device_setup(Space& s) {
   QB_CUDA(cudaGetDevice(&s.device));
-  const size_t nsec = s.secN.size();
-  QB_CUDA(cudaMalloc(&s.d_blob, s.blob.size()));
-  QB_CUDA(cudaMemcpy(s.d_blob, s.blob.data(), s.blob.size(), cudaMemcpyHostToDevice));
-  QB_CUDA(cudaMalloc(&s.d_secOff, sizeof(int64_t) * (nsec + 1)));
-  QB_CUDA(cudaMemcpy(s.d_secOff, s.secOff.data(), sizeof(int64_t) * (nsec + 1), cudaMemcpyHostToDevice));
-  QB_CUDA(cudaMalloc(&s.d_secN, sizeof(int32_t) * nsec));
-  QB_CUDA(cudaMemcpy(s.d_secN, s.secN.data(), sizeof(int32_t) * nsec, cudaMemcpyHostToDevice));
-  QB_CUDA(cudaMalloc(&s.d_secK, sizeof(int32_t) * nsec));
-  QB_CUDA(cudaMemcpy(s.d_secK, s.secK.data(), sizeof(int32_t) * nsec, cudaMemcpyHostToDevice));
-  QB_CUDA(cudaMalloc(&s.d_secOf, sizeof(int32_t) * s.secOf.size()));
-  QB_CUDA(cudaMemcpy(s.d_secOf, s.secOf.data(), sizeof(int32_t) * s.secOf.size(), cudaMemcpyHostToDevice));
   Tables& t = s.t;
-  t.blob = s.d_blob;
-  t.n_sectors = (int)nsec;
-  t.sec_off = s.d_secOff;
-  t.sec_N = s.d_secN;
-  t.sec_K = s.d_secK;
-  t.sec_of = s.d_secOf;
+  const int M = s.M, V = s.nmax + 1, nsec = (int)s.secN.size();
+  t.n_sectors = nsec;
   t.total = s.secOff.back();
-  if (row_smem(t) + (size_t)(kBlock / 32) * nmoments(s.M) * 8 > 227 * 1024)
+  if (row_smem(t) + (size_t)(kBlock / 32) * nmoments(M) * 8 > 227 * 1024)
     return fail(QB_EUNSUPPORTED, "tables too large for shared memory (reduce n_max or M)");
+  if (t.total >= (int64_t)kNoIndex) return fail(QB_EUNSUPPORTED, "the space exceeds 2^32 - 2^16 kets");
+  // sqrt(C(rem, k)): the binomial exactly in 128 bits while it fits (rem <= 125:
+  // C(125, 62) < 2^122), then one rounding to double, one correctly rounded sqrt
+  // and one division; beyond, by the recurrence C(rem, k) = C(rem, k-1) (rem-k+1) / k
+  // in long double (at least 64 significant bits: the accumulated relative error
+  // of at most 2 rem roundings stays far below a double's half-ulp)
+  std::vector<double2> wt((size_t)V * V, make_double2(0.0, 0.0));
+  for (int rem = 0; rem < V; ++rem) {
+    unsigned __int128 c = 1;
+    long double cl = 1.0L;
+    for (int k = 0; k <= rem; ++k) {
+      if (k > 0) {
+        if (rem <= 125)
+          c = c * (unsigned __int128)(rem - k + 1) / (unsigned __int128)k;
+        else
+          cl = cl * (long double)(rem - k + 1) / (long double)k;
+      }
+      const double r = rem <= 125 ? std::sqrt((double)c) : (double)std::sqrt(cl);
+      wt[(size_t)rem * V + k] = make_double2(r, 1.0 / r);
+    }
+  }
+  // after the table: the per-N centring powers of two (Tables::wscale)
+  for (int N = 0; N < V; ++N) {
+    const int e = (int)std::floor(0.5 * log2_max_ket_weight(M, N) + 0.5);
+    wt.push_back(make_double2(std::ldexp(1.0, -e), std::ldexp(1.0, e)));
+  }
+  t.occ_bits = 1;
+  while ((1 << t.occ_bits) <= s.nmax) ++t.occ_bits;  // M * occ_bits <= 64 (checked by qb_sector_build)
+
+  // One allocation holds everything, as one copy brings what the host made: each allocation
+  // and its release cost 20 to 50 us, twenty of them half of a small space's set-up.
+  size_t bytes = 0;
+  auto take = [&](size_t n) {
+    const size_t at = bytes;
+    bytes = (bytes + n + 255) & ~(size_t)255;
+    return at;
+  };
+  struct Part {
+    size_t at;
+    const void* p;
+    size_t n;
+  };
+  std::vector<Part> parts;
+  auto give = [&](const void* p, size_t n) {
+    parts.push_back({take(n), p, n});
+    return parts.back().at;
+  };
+  const size_t o_blob = give(s.blob.data(), s.blob.size());
+  const size_t o_secOff = give(s.secOff.data(), sizeof(int64_t) * (nsec + 1));
+  const size_t o_secN = give(s.secN.data(), sizeof(int32_t) * nsec);
+  const size_t o_secK = give(s.secK.data(), sizeof(int32_t) * nsec);
+  const size_t o_secOf = give(s.secOf.data(), sizeof(int32_t) * s.secOf.size());
+  const size_t o_wtab = give(wt.data(), sizeof(double2) * wt.size());
+  const size_t o_bk = give(s.bk.data(), s.bk.size());
+  const size_t o_fa = t.fa_on ? give(s.fa.data(), s.fa.size()) : 0;
+  const size_t o_bcnt = give(s.blkCnt.data(), sizeof(uint32_t) * s.blkCnt.size());
+  const size_t o_sblk = give(s.secBlk.data(), sizeof(uint32_t) * (nsec + 1));
+  const size_t o_lblk = t.fa_on ? give(s.lowBlk.data(), sizeof(uint32_t) * s.lowBlk.size()) : 0;
+  const size_t image = bytes;
   // scratch: status + partials for the largest persistent grid of any reduction
   int sms = 0;
   QB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s.device));
   const int64_t max_grid = (int64_t)sms * 16;
   s.grid_hpsi = (int)max_grid;
-  s.scratch_doubles = scratch_doubles_for(s.M, s.nmax, max_grid);
-  QB_CUDA(cudaMalloc(&s.d_scratch, sizeof(double) * s.scratch_doubles));
-  QB_CUDA(cudaMemset(s.d_scratch, 0, sizeof(double) * s.scratch_doubles));
-  QB_CUDA(cudaMalloc(&s.d_diag, sizeof(float4) * (size_t)t.total));
-  QB_CUDA(cudaMalloc(&s.d_obsf, sizeof(float4) * (size_t)t.total));
-  QB_CUDA(cudaMalloc(&s.d_occ, sizeof(uint64_t) * (size_t)t.total));
-  QB_CUDA(cudaMalloc(&s.d_wi, 2 * sizeof(double) * (size_t)t.total));
-  t.wi = s.d_wi;
-  t.wk = s.d_wi + t.total;
-  t.occ_bits = 1;
-  while ((1 << t.occ_bits) <= s.nmax) ++t.occ_bits;  // M * occ_bits <= 64 (checked by qb_sector_build)
-  t.occ = s.d_occ;
-  {
-    // sqrt(C(rem, k)): the binomial exactly in 128 bits while it fits (rem <= 125:
-    // C(125, 62) < 2^122), then one rounding to double, one correctly rounded sqrt
-    // and one division; beyond, by the recurrence C(rem, k) = C(rem, k-1) (rem-k+1) / k
-    // in long double (at least 64 significant bits: the accumulated relative error
-    // of at most 2 rem roundings stays far below a double's half-ulp)
-    const int V = s.nmax + 1;
-    std::vector<double2> wt((size_t)V * V, make_double2(0.0, 0.0));
-    for (int rem = 0; rem < V; ++rem) {
-      unsigned __int128 c = 1;
-      long double cl = 1.0L;
-      for (int k = 0; k <= rem; ++k) {
-        if (k > 0) {
-          if (rem <= 125)
-            c = c * (unsigned __int128)(rem - k + 1) / (unsigned __int128)k;
-          else
-            cl = cl * (long double)(rem - k + 1) / (long double)k;
-        }
-        const double r = rem <= 125 ? std::sqrt((double)c) : (double)std::sqrt(cl);
-        wt[(size_t)rem * V + k] = make_double2(r, 1.0 / r);
-      }
-    }
-    // after the table: the per-N centring powers of two (Tables::wscale)
-    for (int N = 0; N < V; ++N) {
-      const int e = (int)std::floor(0.5 * log2_max_ket_weight(s.M, N) + 0.5);
-      wt.push_back(make_double2(std::ldexp(1.0, -e), std::ldexp(1.0, e)));
-    }
-    QB_CUDA(cudaMalloc(&s.d_wtab, sizeof(double2) * wt.size()));
-    QB_CUDA(cudaMemcpy(s.d_wtab, wt.data(), sizeof(double2) * wt.size(), cudaMemcpyHostToDevice));
-    t.wtab = s.d_wtab;
-    t.wscale = s.d_wtab + (size_t)V * V;
-  }
-  {
-    const size_t five = t.bk_kc == 5 ? (size_t)t.bk_nrec * t.bk_S * 2 : 0;
-    QB_CUDA(cudaMalloc(&s.d_bk, s.bk_off[6] + (t.fa_on ? 0 : s.bk_map_bytes + five)));
-    QB_CUDA(cudaMemcpy(s.d_bk, s.bk.data(), s.bk.size(), cudaMemcpyHostToDevice));
-    t.bk_info = reinterpret_cast<const uint2*>(s.d_bk + s.bk_off[0]);
-    t.bk_G = reinterpret_cast<const float2*>(s.d_bk + s.bk_off[1]);
-    t.bk_Gi = reinterpret_cast<const float2*>(s.d_bk + s.bk_off[2]);
-    t.bk_psh = reinterpret_cast<const int32_t*>(s.d_bk + s.bk_off[3]);
-    t.bk_EC = reinterpret_cast<const int32_t*>(s.d_bk + s.bk_off[4]);
-    t.bk_cls = reinterpret_cast<const int2*>(s.d_bk + s.bk_off[5]);
-    t.bk_combo = reinterpret_cast<const uint32_t*>(s.d_bk + s.bk_off[7]);
-    t.bk_map = s.d_bk + s.bk_off[6];
-    t.bk_map5 = reinterpret_cast<const uint16_t*>(s.d_bk + s.bk_off[6] + s.bk_map_bytes);
-    QB_CUDA(cudaMalloc(&s.d_fill, sizeof(uint32_t) * (size_t)t.total));
-    t.fill = s.d_fill;
-  }
-  {
-    const size_t smem = row_smem(t);
-    int grid = 0;
-    int rc = persistent_grid(diag_kernel, smem, t.total, &grid);
-    if (rc) return rc;
-    diag_kernel<<<grid, kBlock, smem>>>(t, s.d_diag, s.d_occ, s.d_wi, s.d_wi + t.total, s.d_fill);
-    QB_CUDA(cudaGetLastError());
-  }
-  uint32_t* start = nullptr;
-  int64_t nblocks = 0;
-  {
-    int rc = find_blocks(s.d_fill, t.total, &s.d_blocks[0], &start, &nblocks);
-    if (rc) return rc;
-    t.rblk = s.d_blocks[0];
-    const size_t T = t.fa_on ? (size_t)fa_Tc(t) : (size_t)t.bk_T;
-    QB_CUDA(cudaMalloc(&s.d_base[0], sizeof(uint32_t) * (size_t)nblocks * T));
-  }
-  const int base_grid = sms * 8;
-  base_kernel<<<base_grid, 256>>>(t, start, nblocks, s.d_base[0], reinterpret_cast<int*>(s.d_scratch));
-  QB_CUDA(cudaGetLastError());
+  s.scratch_doubles = scratch_doubles_for(M, s.nmax, max_grid);
+  const size_t o_scratch = take(sizeof(double) * s.scratch_doubles);
+  const size_t n = (size_t)t.total, nr = (n + 31) / 32;
+  // (the observables' copy of the state with it, but of the largest spaces: kObsfKets)
+  const bool obsf = t.total <= kObsfKets;
+  const size_t o_diag = take(16 * n), o_obsf = take(obsf ? 16 * n : 0), o_occ = take(8 * n), o_wi = take(16 * n);
+  const size_t o_fill = take(4 * n), o_rblk = take(4 * nr);
+  const size_t S = (size_t)t.bk_S, o_suf = take(40 * S);
+  const uint32_t nblocks = s.secBlk.back();
+  const size_t stride = block_rec_bytes(M, t.bk_P);
+  const size_t o_start = take(4 * (size_t)nblocks);
+  // the blocks' records are read before the rows of bases are written over them
+  const size_t o_base = take((size_t)nblocks * std::max(stride, sizeof(uint32_t) * (t.fa_on ? fa_Tc(t) : t.bk_T)));
+  size_t o_map = 0, o_map5 = 0;
   if (!t.fa_on) {
-    t.bk_base = s.d_base[0];
+    o_map = take(s.bk_map_bytes);
+    o_map5 = take(t.bk_kc == 5 ? (size_t)t.bk_nrec * S * 2 : 0);
+  }
+  // lower kets: the space's first ones, or their own
+  const size_t low = t.fa_on ? (size_t)t.fa_low : 0, lnr = (low + 31) / 32;
+  const uint32_t lblocks = !t.fa_on ? 0 : s.low_held ? s.secBlk[t.fa_nlow] : s.lowBlk.back();
+  size_t o_mapa = 0, o_mapc = 0, o_perm = 0, o_basea = 0, o_locc = 0, o_lfill = 0, o_lrblk = 0, o_lstart = 0;
+  if (t.fa_on) {
+    o_mapa = take((size_t)t.fa_nrec * t.fa_pl * S * 8);
+    o_mapc = take((size_t)t.fa_ng * S * 8);
+    o_perm = take(4 * lnr);
+    o_basea = take((size_t)lblocks * std::max(sizeof(BlockRec), sizeof(uint32_t) * fa_rowa(t)));
+    if (!s.low_held) {
+      o_locc = take(8 * low);
+      o_lfill = take(4 * low);
+      o_lrblk = take(4 * lnr);
+      o_lstart = take(4 * (size_t)lblocks);
+    }
+  }
+  // moments by raised kets: odd M with a kernel, every sector from the vacuum to nmax held
+  int layers_end = 0;  // first sector of nmax particles
+  t.mo_on = (M == 5 || M == 7 || M == 9) && s.nmin == 0 && s.nmax >= 1 && s.nmax < 256;
+  for (int N = 0, i = 0; N <= s.nmax && t.mo_on; ++N) {
+    if (N == s.nmax) layers_end = i;
+    for (int K = 0; K < s.Q; ++K)
+      if (s.cnt[(size_t)N * s.Q + K] > 0) {
+        if (s.secOf[(size_t)N * s.Q + K] < 0) t.mo_on = 0;
+        ++i;
+      }
+  }
+  size_t o_mmap = 0, o_mbase = 0, o_mperm = 0;
+  int64_t mnr = 0;
+  if (t.mo_on) {
+    t.mo_w = (M + 3) & ~3;
+    t.mo_rows = s.secOff[layers_end];
+    mnr = t.mo_rows / 32;
+    o_mmap = take((size_t)2 * t.mo_w * S * 2);
+    o_mbase = take((size_t)nblocks * 2 * t.mo_w * 4);
+    o_mperm = take(4 * (size_t)mnr);
+  }
+
+  QB_CUDA(cudaMalloc(&s.d_arena, bytes));
+  unsigned char* A = s.d_arena;
+  {
+    std::vector<unsigned char> img(image, 0);
+    for (const Part& p : parts)
+      if (p.n) memcpy(img.data() + p.at, p.p, p.n);
+    QB_CUDA(cudaMemcpy(A, img.data(), image, cudaMemcpyHostToDevice));
+  }
+  s.d_scratch = reinterpret_cast<double*>(A + o_scratch);
+  QB_CUDA(cudaMemsetAsync(s.d_scratch, 0, sizeof(double) * s.scratch_doubles));
+  auto u32 = [&](size_t o) { return reinterpret_cast<uint32_t*>(A + o); };
+  auto i32 = [&](size_t o) { return reinterpret_cast<const int32_t*>(A + o); };
+  s.d_diag = reinterpret_cast<float4*>(A + o_diag);
+  s.d_obsf = obsf ? reinterpret_cast<float4*>(A + o_obsf) : nullptr;
+  uint64_t* occ = reinterpret_cast<uint64_t*>(A + o_occ);
+  double* wi = reinterpret_cast<double*>(A + o_wi);
+  t.blob = A + o_blob;
+  t.sec_off = reinterpret_cast<const int64_t*>(A + o_secOff);
+  t.sec_N = i32(o_secN);
+  t.sec_K = i32(o_secK);
+  t.sec_of = i32(o_secOf);
+  t.wi = wi;
+  t.wk = wi + n;
+  t.occ = occ;
+  t.wtab = reinterpret_cast<const double2*>(A + o_wtab);
+  t.wscale = t.wtab + (size_t)V * V;
+  auto bk = [&](int k) { return A + o_bk + s.bk_off[k]; };
+  t.bk_info = reinterpret_cast<const uint2*>(bk(0));
+  t.bk_G = reinterpret_cast<const float2*>(bk(1));
+  t.bk_Gi = reinterpret_cast<const float2*>(bk(2));
+  t.bk_psh = reinterpret_cast<const int32_t*>(bk(3));
+  t.bk_EC = reinterpret_cast<const int32_t*>(bk(4));
+  t.bk_cls = reinterpret_cast<const int2*>(bk(5));
+  t.bk_combo = reinterpret_cast<const uint32_t*>(bk(7));
+  t.fill = u32(o_fill);
+  t.rblk = u32(o_rblk);
+
+  Suffix sx{};
+  {
+    uint64_t* words = reinterpret_cast<uint64_t*>(A + o_suf);
+    double* d = reinterpret_cast<double*>(words + S);
+    sx = Suffix{words, d, d + S, d + 2 * S, d + 3 * S};
+  }
+  // a run of rounds a warp: 8, fewer where the kets don't fill the SMs' 64 warps
+  auto run_of = [&](size_t rounds) { return (int)std::max<size_t>(1, std::min<size_t>(8, rounds / ((size_t)sms * 64))); };
+  auto grid_of = [&](size_t rounds) { return (unsigned)(((rounds + run_of(rounds) - 1) / run_of(rounds) + 7) / 8); };
+  uint32_t* start = u32(o_start);
+  const unsigned nf = (unsigned)((S + 127) / 128);
+  block_kernel<<<nf + (nblocks + 127) / 128, 128>>>(
+      t, BlockArgs{t.sec_N, t.sec_K, t.sec_off, u32(o_sblk), nsec, u32(o_bcnt), start, A + o_base, stride}, nf,
+      reinterpret_cast<uint64_t*>(A + o_suf));
+  ket_kernel<true><<<grid_of(nr), 256>>>(t, sx, t.total, nblocks, start, A + o_base, stride, run_of(nr), s.d_diag, occ, wi,
+                                         wi + n, u32(o_fill), u32(o_rblk));
+  QB_CUDA(cudaGetLastError());
+  const int base_grid = sms * 8;
+  base_kernel<<<base_grid, 256>>>(t, start, nblocks, u32(o_base), reinterpret_cast<int*>(s.d_scratch));
+  QB_CUDA(cudaGetLastError());
+  const unsigned fill_grid = (unsigned)((S + kBlock - 1) / kBlock);
+  if (!t.fa_on) {
+    t.bk_base = u32(o_base);
+    t.bk_map = A + o_map;
+    t.bk_map5 = reinterpret_cast<const uint16_t*>(A + o_map5);
     if (t.bk_nrec > 0) {
-      const dim3 grid((unsigned)((t.bk_S + kBlock - 1) / kBlock), (unsigned)std::min(t.bk_nrec, 8));
-      block_map_kernel<<<grid, kBlock>>>(t, reinterpret_cast<uint16_t*>(s.d_bk + s.bk_off[6]),
-                                         const_cast<uint16_t*>(t.bk_map5));
+      const dim3 grid(fill_grid, (unsigned)std::min(t.bk_nrec, 8));
+      block_map_kernel<<<grid, kBlock>>>(t, sx.word, reinterpret_cast<uint16_t*>(A + o_map),
+                                         reinterpret_cast<uint16_t*>(A + o_map5));
       QB_CUDA(cudaGetLastError());
     }
   } else {
-    const size_t total_bytes = s.fa_off[14] + (size_t)t.fa_ng * t.bk_S * 8;
-    QB_CUDA(cudaMalloc(&s.d_fa, total_bytes));
-    QB_CUDA(cudaMemcpy(s.d_fa, s.fa.data(), s.fa.size(), cudaMemcpyHostToDevice));
-    auto at = [&](int k) { return s.d_fa + s.fa_off[k]; };
+    auto at = [&](int k) { return A + o_fa + s.fa_off[k]; };
     t.fa_rec = reinterpret_cast<const uint2*>(at(0));
     t.fa_lam = reinterpret_cast<const float2*>(at(1));
     t.fa_ka = reinterpret_cast<const int32_t*>(at(2));
@@ -1130,89 +1201,49 @@ int device_setup(Space& s) {
     t.fa_lowof = reinterpret_cast<const int32_t*>(at(8));
     t.fa_lowoff = reinterpret_cast<const int64_t*>(at(9));
     t.fa_goff = reinterpret_cast<const uint32_t*>(at(10));
-    t.fa_basec = s.d_base[0];
     t.fa_lam64 = reinterpret_cast<const double*>(at(15));
     t.fa_pqa = reinterpret_cast<const uint32_t*>(at(16));
-    t.fa_mapa = reinterpret_cast<const uint2*>(at(13));
-    t.fa_mapc = reinterpret_cast<const uint2*>(at(14));
+    t.fa_mapa = reinterpret_cast<const uint2*>(A + o_mapa);
+    t.fa_mapc = reinterpret_cast<const uint2*>(A + o_mapc);
+    t.fa_basec = u32(o_base);
+    t.fa_basea = u32(o_basea);
+    t.fa_perm = u32(o_perm);
+    const int32_t *lowN = reinterpret_cast<const int32_t*>(at(11)), *lowK = reinterpret_cast<const int32_t*>(at(12));
     uint32_t* lstart = start;
-    int64_t lblocks = nblocks;
     if (s.low_held) {
-      t.fa_occ = s.d_occ;
-      t.fa_fill = s.d_fill;
+      t.fa_occ = t.occ;
+      t.fa_fill = t.fill;
       t.fa_wk = t.wk;
       t.fa_rblk = t.rblk;
-      // the lower kets' blocks are the first ones: up to the block of the ket after them
-      if (t.fa_low < t.total) {
-        const int64_t r = t.fa_low / 32;
-        uint32_t first = 0, f[32];
-        const int n = (int)(t.fa_low - 32 * r) + 1;
-        QB_CUDA(cudaMemcpy(&first, t.rblk + r, sizeof(first), cudaMemcpyDeviceToHost));
-        QB_CUDA(cudaMemcpy(f, s.d_fill + 32 * r, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
-        lblocks = first;
-        for (int k = 1; k < n; ++k) lblocks += f[k] != f[k - 1] + 1u;
-      }
     } else {
-      QB_CUDA(cudaMalloc(&s.d_low, (size_t)t.fa_low * 12));
-      uint64_t* occ = reinterpret_cast<uint64_t*>(s.d_low);
-      uint32_t* fill = reinterpret_cast<uint32_t*>(occ + t.fa_low);
-      t.fa_occ = occ;
-      t.fa_fill = fill;
+      lstart = u32(o_lstart);
+      t.fa_occ = reinterpret_cast<const uint64_t*>(A + o_locc);
+      t.fa_fill = u32(o_lfill);
       t.fa_wk = nullptr;
-      int grid = 0;
-      int rc = persistent_grid(lower_kernel, row_smem(t), t.fa_low, &grid);
-      if (rc) return rc;
-      lower_kernel<<<grid, kBlock, row_smem(t)>>>(t, reinterpret_cast<const int32_t*>(at(11)),
-                                                  reinterpret_cast<const int32_t*>(at(12)), occ, fill);
+      t.fa_rblk = u32(o_lrblk);
+      lower_block_kernel<<<(lblocks + 127) / 128, 128>>>(
+          t, BlockArgs{lowN, lowK, t.fa_lowoff, u32(o_lblk), t.fa_nlow, u32(o_bcnt), lstart, A + o_basea, sizeof(BlockRec)});
+      ket_kernel<false><<<grid_of(lnr), 256>>>(t, sx, t.fa_low, lblocks, lstart, A + o_basea, sizeof(BlockRec), run_of(lnr),
+                                               nullptr, reinterpret_cast<uint64_t*>(A + o_locc), nullptr, nullptr,
+                                               u32(o_lfill), u32(o_lrblk));
       QB_CUDA(cudaGetLastError());
-      rc = find_blocks(fill, t.fa_low, &s.d_blocks[1], &lstart, &lblocks);
-      if (rc) return rc;
-      t.fa_rblk = s.d_blocks[1];
     }
-    {
-      const int64_t nr = (t.fa_low + 31) / 32;
-      QB_CUDA(cudaMalloc(&s.d_perm, sizeof(uint32_t) * (size_t)nr));
-      round_order_kernel<<<base_grid, 256>>>(t.fa_lowoff, reinterpret_cast<const int32_t*>(at(11)), t.fa_nlow, nr, s.d_perm);
-      QB_CUDA(cudaGetLastError());
-      t.fa_perm = s.d_perm;
-    }
-    QB_CUDA(cudaMalloc(&s.d_base[1], sizeof(uint32_t) * (size_t)lblocks * fa_rowa(t)));
-    t.fa_basea = s.d_base[1];
-    lowered_base_kernel<<<base_grid, 256>>>(t, start, nblocks, s.d_base[0]);
-    raised_base_kernel<<<base_grid, 256>>>(t, lstart, lblocks, s.d_base[1]);
-    QB_CUDA(cudaGetLastError());
-    const dim3 grid((unsigned)((t.bk_S + kBlock - 1) / kBlock), (unsigned)std::min(fa_Ta(t) / 4 + t.fa_ng, 8));
-    factor_map_kernel<<<grid, kBlock>>>(t, reinterpret_cast<uint16_t*>(at(13)), reinterpret_cast<uint16_t*>(at(14)));
+    round_order_kernel<<<base_grid, 256>>>(t.fa_lowoff, lowN, t.fa_nlow, (int64_t)lnr, u32(o_perm));
+    lowered_base_kernel<<<base_grid, 256>>>(t, start, nblocks, u32(o_base));
+    raised_base_kernel<<<base_grid, 256>>>(t, lstart, lblocks, u32(o_basea));
+    const dim3 grid(fill_grid, (unsigned)std::min(fa_Ta(t) / 4 + t.fa_ng, 8));
+    factor_map_kernel<<<grid, kBlock>>>(t, sx.word, reinterpret_cast<uint16_t*>(A + o_mapa),
+                                        reinterpret_cast<uint16_t*>(A + o_mapc));
     QB_CUDA(cudaGetLastError());
   }
-  // moments by raised kets: odd M with a kernel, every sector from the vacuum to nmax held
-  int layers_end = 0;  // first sector of nmax particles
-  t.mo_on = (s.M == 5 || s.M == 7 || s.M == 9) && s.nmin == 0 && s.nmax >= 1 && s.nmax < 256;
   if (t.mo_on) {
-    for (int N = 0, i = 0; N <= s.nmax && t.mo_on; ++N) {
-      if (N == s.nmax) layers_end = i;
-      for (int K = 0; K < s.Q; ++K)
-        if (s.cnt[(size_t)N * s.Q + K] > 0) {
-          if (s.secOf[(size_t)N * s.Q + K] < 0) t.mo_on = 0;
-          ++i;
-        }
-    }
-  }
-  if (t.mo_on) {
-    t.mo_w = (s.M + 3) & ~3;
-    t.mo_rows = s.secOff[layers_end];
-    const size_t mapb = ((size_t)2 * t.mo_w * t.bk_S * 2 + 255) & ~(size_t)255;
-    const size_t baseb = ((size_t)nblocks * 2 * t.mo_w * 4 + 255) & ~(size_t)255;
-    const int64_t nr = t.mo_rows / 32;
-    QB_CUDA(cudaMalloc(&s.d_mo, mapb + baseb + 4 * (size_t)std::max<int64_t>(nr, 1)));
-    t.mo_map = reinterpret_cast<const uint2*>(s.d_mo);
-    t.mo_base = reinterpret_cast<const uint32_t*>(s.d_mo + mapb);
-    moment_map_kernel<<<(unsigned)((t.bk_S + kBlock - 1) / kBlock), kBlock>>>(t, reinterpret_cast<uint16_t*>(s.d_mo));
-    moment_base_kernel<<<base_grid, 256>>>(t, start, nblocks, reinterpret_cast<uint32_t*>(s.d_mo + mapb));
-    if (nr > 0) {
-      uint32_t* perm = reinterpret_cast<uint32_t*>(s.d_mo + mapb + baseb);
-      round_order_kernel<<<base_grid, 256>>>(t.sec_off, t.sec_N, t.n_sectors, nr, perm);
-      t.mo_perm = perm;
+    t.mo_map = reinterpret_cast<const uint2*>(A + o_mmap);
+    t.mo_base = u32(o_mbase);
+    moment_map_kernel<<<dim3(fill_grid, 8), kBlock>>>(t, sx.word, reinterpret_cast<uint16_t*>(A + o_mmap));
+    moment_base_kernel<<<base_grid, 256>>>(t, start, nblocks, u32(o_mbase));
+    if (mnr > 0) {
+      round_order_kernel<<<base_grid, 256>>>(t.sec_off, t.sec_N, t.n_sectors, mnr, u32(o_mperm));
+      t.mo_perm = u32(o_mperm);
     }
     QB_CUDA(cudaGetLastError());
   }
@@ -1436,11 +1467,10 @@ int launch_to_df(const void* psi, void* psif, int64_t n, void* stream) {
 
 int launch_unrank(const Space& s, int64_t first, int64_t count, int* d_occ, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
-  const size_t smem = row_smem(s.t);
   int grid = 0;
-  int rc = persistent_grid(unrank_kernel, smem, count, &grid);
+  int rc = persistent_grid(unrank_kernel, 0, count * s.M, &grid);
   if (rc) return rc;
-  unrank_kernel<<<grid, kBlock, smem, st>>>(s.t, first, count, d_occ, reinterpret_cast<int*>(s.d_scratch));
+  unrank_kernel<<<grid, kBlock, 0, st>>>(s.t, first, count, d_occ);
   QB_CUDA(cudaGetLastError());
   return check_status(s, st);
 }
@@ -1478,15 +1508,14 @@ int launch_terms(const Space& s, int64_t* terms, int64_t* tuples, void* stream) 
 int launch_init_table(const Space& s, const double* table_host, int only_N, void* d_psi, double* norm2,
                       void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
-  const size_t smem = row_smem(s.t);
   int grid = 0;
-  int rc = persistent_grid(init_table_kernel, smem, s.t.total, &grid);
+  int rc = persistent_grid(init_table_kernel, 0, s.t.total, &grid);
   if (rc) return rc;
   double* part = partial_area(s);
   double* tab = table_area(s);
   const size_t tab_bytes = sizeof(double) * 2 * (size_t)s.M * (s.nmax + 1);
   QB_CUDA(cudaMemcpyAsync(tab, table_host, tab_bytes, cudaMemcpyHostToDevice, st));
-  init_table_kernel<<<grid, kBlock, smem, st>>>(s.t, (const double2*)tab, only_N, (double2*)d_psi, part);
+  init_table_kernel<<<grid, kBlock, 0, st>>>(s.t, (const double2*)tab, only_N, (double2*)d_psi, part);
   QB_CUDA(cudaGetLastError());
   double* fin = init_final(s);
   sum_rows_kernel<<<1, kSumThreads, 0, st>>>(part, grid, 1, 1.0, false, fin);

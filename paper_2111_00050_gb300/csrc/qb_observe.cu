@@ -1038,6 +1038,10 @@ int launch_moments(Space& s, const void* d_psi, double* out_host, void* stream) 
   cudaStream_t st = (cudaStream_t)stream;
   const int M = s.M, nmom = nmoments(M), npr = nprep(M);
   const double2* psi = (const double2*)d_psi;
+  if (!s.d_obsf) {
+    QB_CUDA(cudaMalloc(&s.d_obsf, sizeof(float4) * (size_t)s.t.total));
+    s.own_obsf = true;
+  }
   float4* f = s.d_obsf;
   // pass 1: weighted copy, norm, <N>, <n_i>
   int gp = 0;
