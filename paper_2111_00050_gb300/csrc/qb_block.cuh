@@ -58,6 +58,29 @@ __device__ __forceinline__ float occ_float23(const uint32_t (&ob)[NW], uint32_t 
   if constexpr (NW == 4) w = __byte_perm(m8 ? ob[2] : ob[0], m8 ? ob[3] : ob[1], m);
   return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7650u));
 }
+// Values that a stage reads once (the kets' words and fillings, the diagonal, the vectors of the
+// epilogue) are not kept in L1, whose lines the gathers, the maps and the bases reuse.  One step
+// of the M = 9, N = 27 long-range space (23.5M kets) 20.8 -> 20.3 ms, 20 steps with gradient of
+// the M = 5, 2.3M-ket space 48.0 -> 47.1; maps read that way cost as much again (55.7).
+__device__ __forceinline__ float4 ld_once(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ uint64_t ld_once(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.u64 %0, [%1];" : "=l"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_once(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
 template <int NW>
 __device__ __forceinline__ float occ_float(const uint32_t (&ob)[NW], int m) {
   return occ_float23<NW>(ob, (uint32_t)(m & 7), m >= 8) - 8388608.0f;
@@ -150,7 +173,8 @@ __device__ __forceinline__ void add_record(dfc& acc, const float4 (&x)[Rec<KC>::
 // Everything of a ket's row that the epilogue needs, and the epilogue: forms the
 // stage's output (or the bilinears, or the <x|H|x> summand) from the off-diagonal sum.
 // WHOLE: acc is the whole two-body part (factored couplings), else its off-diagonal part.
-template <int MT, int B, int KIND, bool WHOLE, int NW>
+// RESIDENT: the state's vectors lie in shared memory.
+template <int MT, int B, int KIND, bool WHOLE, int NW, bool RESIDENT = false>
 __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a, int mode, int64_t gr, int64_t ri,
                                                const dfc (&acc)[B], const uint32_t (&ob)[NW], dfl& bil_l, dfc* bil_w,
                                                double& dot64) {
@@ -158,7 +182,7 @@ __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a,
   constexpr int kMB = (MT > 0) ? MT : 16;
   const int M = (MT > 0) ? MT : t.M;
   const int64_t total = t.total;
-  const float4 dg4 = a.diag[gr];
+  const float4 dg4 = ld_once(a.diag + gr);
   const dfl zf{a.zf.x, a.zf.y};
   // the ket weight where true values are formed
   double2 wk = make_double2(1.0, 1.0);
@@ -187,7 +211,7 @@ __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a,
     if (BIL && b == 0) {
       // H_L x (two-body part at scale 1) and the pair vector of this row, as true
       // values: each factor times w (w^2 alone may leave the fp32 range)
-      const float4 pp = a.pair[ri];
+      const float4 pp = ld_once(a.pair + ri);
       const dfl wd = df_of(wk.x);
       const dfl dl{dg4.z, dg4.w};
       const dfl lr = df_mul(wd, WHOLE ? acc_r : df_add(df_mul(dl, df_re(xo)), acc_r));
@@ -211,7 +235,8 @@ __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a,
     if (mode == 0 || mode == 2) {
       dfl orr = df_mul(zf, hi), oi = df_neg(df_mul(zf, hr));  // z H x with z = -i zre
       if (mode == 0) {
-        const float4 p0 = a.psif[(size_t)b * total + ri];
+        const float4* pf = a.psif + (size_t)b * total + ri;
+        const float4 p0 = RESIDENT ? *pf : ld_once(pf);
         orr = df_add(df_re(p0), orr);
         oi = df_add(df_im(p0), oi);
       }
@@ -220,7 +245,7 @@ __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a,
       double sr = a.zre * df_to(hi), si = -a.zre * df_to(hr);
       if (mode == 3) {
         for (int k = 0; k < a.nbasef; ++k) {
-          const float4 e = a.basef[k][(size_t)b * total + ri];
+          const float4 e = ld_once(a.basef[k] + (size_t)b * total + ri);
           sr += df_to(df_re(e));
           si += df_to(df_im(e));
         }
@@ -245,8 +270,8 @@ __device__ __forceinline__ RoundIn load_round(const uint64_t* occ, const uint32_
                                               int64_t n, int lane) {
   RoundIn in;
   const int64_t g = min(r * 32 + lane, n - 1);
-  in.word = __ldg(occ + g);
-  in.fill = __ldg(fill + g);
+  in.word = ld_once(occ + g);
+  in.fill = ld_once(fill + g);
   in.first = __ldg(rblk + r);
   return in;
 }
@@ -384,22 +409,34 @@ __global__ void __launch_bounds__((U > 1 ? 256 : blk_max_threads<B, KIND>()), 1)
         }
       };
       if constexpr (FIX && U == 1 && B == 1 && !CPLX && MT <= kUnrollM) {
-        // unrolled: the pairs are constants, a pair's factor is one product of two registers
+        // unrolled: the pairs are constants, a pair's factor is one product of two registers; the
+        // maps and bases two records ahead (one ahead: one stage of 245,157 kets at M = 7 37.7 us,
+        // now 36.2; reading the next targets into L1 or L2 by prefetch as well: 41.1)
         constexpr OrderedPairs<MT> pr{};
         constexpr int NR = MT * (MT + 1) / 2;
         float nf[MT];
 #pragma unroll
         for (int m = 0; m < MT; ++m) nf[m] = occ_float<NW>(ob, m);
         load(0, mcur, bcur);
+        uint32_t rkn[NT];
+        auto targets = [&](uint32_t (&k)[NT]) {
+          k[0] = bcur[0].a.x + (mcur[0].a.x & 0xffffu);
+          k[1] = bcur[0].a.y + (mcur[0].a.x >> 16);
+          if constexpr (NT > 2) k[2] = bcur[0].a.z + (mcur[0].a.y & 0xffffu);
+          if constexpr (NT > 3) k[3] = bcur[0].a.w + (mcur[0].a.y >> 16);
+          if constexpr (NT > 4) k[4] = bcur[0].b + mcur[0].b;
+        };
+        targets(rkn);
+        load(1, mcur, bcur);
 #pragma unroll
         for (int rec = 0; rec < NR; ++rec) {
           uint32_t rk[NT];
-          rk[0] = bcur[0].a.x + (mcur[0].a.x & 0xffffu);
-          rk[1] = bcur[0].a.y + (mcur[0].a.x >> 16);
-          if constexpr (NT > 2) rk[2] = bcur[0].a.z + (mcur[0].a.y & 0xffffu);
-          if constexpr (NT > 3) rk[3] = bcur[0].a.w + (mcur[0].a.y >> 16);
-          if constexpr (NT > 4) rk[4] = bcur[0].b + mcur[0].b;
-          if (rec + 1 < NR) load(rec + 1, mcur, bcur);
+#pragma unroll
+          for (int c = 0; c < NT; ++c) rk[c] = rkn[c];
+          if (rec + 1 < NR) {
+            targets(rkn);
+            if (rec + 2 < NR) load(rec + 2, mcur, bcur);
+          }
           const float Af = pr.r[rec] != pr.s[rec] ? nf[pr.r[rec]] * nf[pr.s[rec]] : nf[pr.r[rec]] * (nf[pr.r[rec]] - 1.f);
           uint32_t top = rk[0];
 #pragma unroll

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
             if (KC > 0 || (info.x & 0x80u)) acc[0] = dfc_renorm(acc[0]);
           }
         }
-        if (valid) stage_epilogue<MT, 1, KIND_STAGE, false, NW>(t, a, d == 1 ? 1 : 0, off + i, i, acc, ob, bil_l, bil_w, dot64);
+        if (valid) stage_epilogue<MT, 1, KIND_STAGE, false, NW, true>(t, a, d == 1 ? 1 : 0, off + i, i, acc, ob, bil_l, bil_w, dot64);
       }
       __syncthreads();
     }
