@@ -203,7 +203,7 @@ struct AdjointLayout {
   double* acc;      // [M + 1]
   double* fin;      // [2 (M + 1)]
   int n_tb;         // two-body operators of the coupling gradient
-  int* tb;          // [n_tb] a1 | a2 << 8 | c1 << 16 | c2 << 24
+  int* tb;          // [n_tb] a1 | a2 << 8 | c1 << 16 | c2 << 24, or the operators' columns (tb_columns)
   double* tbacc;    // [2 n_tb] weighted sums of <forward stage vector, O costate>
   int64_t bytes;
 };
@@ -381,7 +381,9 @@ static int adjoint_impl(qb_space* space, const double* z, double scale, double d
   QB_CUDA(cudaMemsetAsync(L.acc, 0, 8 * (kMaxM + 1), st));
   const std::vector<int> ops = two_body_ops(M, sp->t.Q);
   if (grad_L) {
-    QB_CUDA(cudaMemcpy(L.tb, ops.data(), 4 * ops.size(), cudaMemcpyHostToDevice));
+    // the operators, or (by blocks) their columns
+    const std::vector<int> tb = sp->t.fa_on ? ops : tb_columns(*sp, ops);
+    QB_CUDA(cudaMemcpy(L.tb, tb.data(), 4 * tb.size(), cudaMemcpyHostToDevice));
     QB_CUDA(cudaMemsetAsync(L.tbacc, 0, 16 * ops.size(), st));
   }
 
@@ -408,7 +410,8 @@ static int adjoint_impl(qb_space* space, const double* z, double scale, double d
       QB_CUDA(cudaGetLastError());
       // coupling gradient: <forward stage vector, O costate> for every two-body O
       if (grad_L) {
-        r = launch_tb_bilinear(*sp, a.pair, a.vin, L.tb, L.n_tb, weight, L.tbacc, stream);
+        r = sp->t.fa_on ? launch_tb_bilinear(*sp, a.pair, a.vin, L.tb, L.n_tb, weight, L.tbacc, stream)
+                        : launch_tb_blocks(*sp, a.pair, a.vin, L.tb, L.n_tb, weight, L.tbacc, st);
         if (r) return r;
       }
     }

@@ -262,6 +262,11 @@ int launch_moments(Space& s, const void* d_psi, double* out_host, void* stream);
 // bra and ket are weighted double-float vectors of the space (as the stage kernels hold them)
 int launch_tb_bilinear(Space& s, const float4* bra, const float4* ket, const int* d_tb, int n_tb, double weight,
                        double* d_acc, void* stream);
+// The same by blocks of kets, for spaces with the direct stage tables (fa_on = 0): tb_columns
+// gives each operator's column of the partial sums, which the launch takes as d_tb
+std::vector<int> tb_columns(const Space& s, const std::vector<int>& ops);
+int launch_tb_blocks(const Space& s, const float4* bra, const float4* ket, const int* cols, int n_ops, double weight,
+                     double* acc, cudaStream_t st);
 int64_t workspace_bytes(const Space& s, int batch);
 // psi (FP64 complex) -> double-float copy (float4 per ket)
 int launch_to_df(const void* psi, void* psif, int64_t n, void* stream);
