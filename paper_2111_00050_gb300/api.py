@@ -170,7 +170,8 @@ class Space:
         check(lib().qb_evolve(self._h, _dptr(psi), float(dt), int(steps), _dptr(work), _stream()))
 
     def set_resident_max(self, kets: int) -> None:
-        """qb_space_set_resident_max: sectors up to `kets` kets run shared-memory resident (0: never)."""
+        """qb_space_set_resident_max: sectors up to `kets` kets run shared-memory resident (0: every
+        stage is a launch, no small space runs all its steps in one)."""
         check(lib().qb_space_set_resident_max(self._h, int(kets)))
 
     def set_order(self, order: int) -> None:

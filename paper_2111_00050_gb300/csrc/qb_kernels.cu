@@ -1342,6 +1342,23 @@ static int rk4_issue(Space& s, DfArgs& a, double dt, int64_t steps, float4* w1, 
   return QB_OK;
 }
 
+// Cooperative launches of every space on a device run one after the other, whatever their
+// streams: each waits for the event of the one before.
+int coop_order(const void* kernel, int grid, int threads, void** args, size_t smem, cudaStream_t st) {
+  constexpr int kDevices = 64;
+  static std::mutex mu;
+  static cudaEvent_t last[kDevices] = {};
+  int dev = 0;
+  QB_CUDA(cudaGetDevice(&dev));
+  if (dev >= kDevices) return fail(QB_EUNSUPPORTED, "device number");
+  std::lock_guard<std::mutex> lock(mu);
+  if (!last[dev]) QB_CUDA(cudaEventCreateWithFlags(&last[dev], cudaEventDisableTiming));
+  QB_CUDA(cudaStreamWaitEvent(st, last[dev], 0));
+  QB_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), args, smem, st));
+  QB_CUDA(cudaEventRecord(last[dev], st));
+  return QB_OK;
+}
+
 template <int B>
 static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int64_t steps, float4* w1, float4* w2,
                     float4* psif, cudaStream_t st, bool plain = false) {
@@ -1368,18 +1385,28 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
     QB_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, s.device));
     QB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s.device));
     const int cap = (int)std::min<int64_t>((s.maxDim + 3) & ~int64_t(3), 65536);
-    if (s.maxDim <= std::min(s.resident_max_kets, resident_most(s.t)) && s.t.total <= 64LL * sms && resident_smem(s.t, cap) + 1024 <= (size_t)optin) {
-      ResArgs r{};
-      r.psi = psi;
-      r.psif = psif;
-      r.diag = s.d_diag;
-      r.scale = a.scale[0];
-      r.dt = dt;
-      r.steps = steps;
-      r.order = s.order;
-      r.cap = cap;
-      r.status = a.status;
+    ResArgs r{};
+    r.psi = psi;
+    r.psif = psif;
+    r.diag = s.d_diag;
+    r.scale = a.scale[0];
+    r.dt = dt;
+    r.steps = steps;
+    r.order = s.order;
+    r.cap = cap;
+    r.w1 = w1;
+    r.w2 = w2;
+    r.barrier = reinterpret_cast<uint32_t*>(s.d_scratch + 1);
+    r.status = a.status;
+    if (s.maxDim <= std::min(s.resident_max_kets, resident_most(s.t)) && s.t.total <= 64LL * sms && resident_smem(s.t, cap) + 1024 <= (size_t)optin)
       return resident_launch(s.t, r, (int)std::min<int64_t>(1024, (s.maxDim + 31) & ~int64_t(31)), st);
+    // One cooperative launch where the kets find a thread each.
+    if (s.resident_max_kets > 0 && grid_reg_fits(s.t, sms)) {
+      switch (s.M) {
+        case 5: return grid_launch_m5(s.t, r, st);
+        case 7: return grid_launch_m7(s.t, r, st);
+        default: break;
+      }
     }
   }
   if (steps < 2 * kGraphSteps) return rk4_issue<B>(s, a, dt, steps, w1, w2, psif, st, false);

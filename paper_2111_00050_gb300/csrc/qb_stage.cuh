@@ -13,6 +13,8 @@
 
 namespace qb {
 
+int coop_order(const void* kernel, int grid, int threads, void** args, size_t smem, cudaStream_t st);
+
 struct ResArgs {
   double2* psi;        // global psi [total]
   float4* psif;        // global double-float copy of psi in the weighted basis [total] (read, written back)
@@ -22,6 +24,8 @@ struct ResArgs {
   int64_t steps;
   int order;           // Taylor order of a step (stages per step)
   int cap;             // kets per sector the shared buffers hold (a multiple of 4)
+  float4 *w1, *w2;     // stage vectors [total] and counter of the cooperative launch
+  uint32_t* barrier;
   int* status;
 };
 
@@ -170,6 +174,27 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
   }
 }
 
+// Barrier of a cooperative grid: the CTAs arrive at a counter and wait until `target` have.
+// The wait is bounded (a minute or so, longer than another stream's kernel should hold the
+// SMs that the grid's last CTAs wait for): on its end the status is set and every CTA leaves.
+constexpr uint32_t kSpinLimit = 1u << 27;
+__device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target, int* status) {
+  __syncthreads();
+  int late = 0;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(counter, 1u);
+    uint32_t seen, n = 0;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
+    } while (seen < target && ++n < kSpinLimit);
+    late = seen < target;
+    if (late) atomicOr(status, 8);
+    __threadfence();
+  }
+  return __syncthreads_or(late) == 0;
+}
+
 // Sectors of at most reg_kets(M) kets with a fixed partner count: one ket a thread, its
 // targets, pair factors, psi and weights in registers for the whole call, so that a stage
 // reads shared memory for the gathered values (and the couplings, by broadcast) only.  The
@@ -178,18 +203,28 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
 // (general kernel 3.1; 4.6 when every stage ranked its targets).
 constexpr int reg_kets(int M) { return M == 5 ? 512 : 256; }  // 126 registers a thread, 202 (M = 7), 255 (M = 9)
 
-template <int MT>
+//
+// GRID: the same over the whole space, one CTA an SM in a cooperative launch, for spaces whose
+// sectors are too large for a CTA but whose kets all find a thread.  The stage vectors lie in
+// global memory (L2), with a grid barrier in the place of the CTA's.  Launched stage by stage
+// such a space pays for the launch, its tables and its chain of dependent reads every time (us a
+// stage, stage launches / grid): M = 5, 3,060 kets 5.5 / 3.5, 33,649 kets 6.8 / 4.1, 53,130 kets
+// 8.2 / 5.1; M = 7, 19,448 kets 10.1 / 4.5, 27,132 kets 10.2 / 6.1.  M = 9 does not fit its
+// registers (12,870 kets 12.2 / 12.1) and stays with the stage launches.
+template <int MT, bool GRID>
 __global__ void __launch_bounds__(reg_kets(MT), 1) resident_reg_kernel(const Tables t, const ResArgs r) {
   constexpr int KC = (MT - 1) / 2, NT = Rec<KC>::n, RW = Rec<KC>::w, NW = occ_words<MT>();
   constexpr int NR = MT * (MT + 1) / 2;
   static_assert(KC >= 2 && KC <= 4, "two or four 16-bit targets a record");
   const int T = t.bk_T;
   float2* sG = reinterpret_cast<float2*>(blk_smem);
-  float4* buf = reinterpret_cast<float4*>(blk_smem + blk_smem_bytes(t, false));  // [2][cap]
-  const int i = threadIdx.x;
-  for (int k = i; k < T; k += blockDim.x) sG[k] = __ldg(t.bk_G + k);
-  const int64_t off = __ldg(t.sec_off + blockIdx.x);
-  const int D = (int)(__ldg(t.sec_off + blockIdx.x + 1) - off);
+  // two vectors of the stages: [2][cap] in shared memory, or the workspace's
+  float4* const buf0 = GRID ? r.w1 : reinterpret_cast<float4*>(blk_smem + blk_smem_bytes(t, false));
+  float4* const buf1 = GRID ? r.w2 : buf0 + r.cap;
+  const int i = GRID ? (int)(blockIdx.x * blockDim.x + threadIdx.x) : (int)threadIdx.x;
+  for (int k = threadIdx.x; k < T; k += blockDim.x) sG[k] = __ldg(t.bk_G + k);
+  const int64_t off = GRID ? 0 : __ldg(t.sec_off + blockIdx.x);
+  const int D = (int)(GRID ? t.total : __ldg(t.sec_off + blockIdx.x + 1) - off);
   const bool valid = i < D;
   const int64_t g = off + (valid ? i : 0);
   uint32_t ix[NR][RW / 2];
@@ -198,7 +233,7 @@ __global__ void __launch_bounds__(reg_kets(MT), 1) resident_reg_kernel(const Tab
   float4 pf = r.psif[g];
   const float4 dg4 = __ldg(r.diag + g);
   const double wk = __ldg(t.wk + g), wi = __ldg(t.wi + g);
-  bool bad = D > r.cap;
+  bool bad = !GRID && D > r.cap;
   {
     uint32_t ob[NW];
     unpack_occ<MT, NW>(t, valid ? __ldg(t.occ + g) : 0ull, ob);
@@ -231,16 +266,22 @@ __global__ void __launch_bounds__(reg_kets(MT), 1) resident_reg_kernel(const Tab
     }
   }
   if (bad) atomicOr(r.status, 1);
-  if (D > r.cap) return;  // not reached: the host sizes the buffers for the largest sector
+  if (!GRID && D > r.cap) return;  // not reached: the host sizes the buffers for the largest sector
   const dfl sc{r.scale.x, r.scale.y};
   const dfl dg = df_add(dfl{dg4.x, dg4.y}, df_mul(sc, dfl{dg4.z, dg4.w}));
   float4 own = pf;
   int cur = 0;
-  if (valid) buf[i] = pf;
-  __syncthreads();
+  uint32_t round = 0;
+  auto sync = [&]() -> bool {  // false: the grid's barrier gave up
+    if (GRID) return grid_barrier(r.barrier, ++round * gridDim.x, r.status);
+    __syncthreads();
+    return true;
+  };
+  if (valid) buf0[i] = pf;
+  if (!sync()) return;
   for (int64_t it = 0; it < r.steps; ++it) {
     for (int d = r.order; d >= 1; --d) {
-      const float4* vin = buf + cur * r.cap;
+      const float4* vin = cur ? buf1 : buf0;
       dfc acc{0ull, 0ull};
 #pragma unroll
       for (int rec = 0; rec < NR; ++rec) {
@@ -269,8 +310,8 @@ __global__ void __launch_bounds__(reg_kets(MT), 1) resident_reg_kernel(const Tab
         own = pf = df_pack(df_of(psi.x * wi), df_of(psi.y * wi));
       }
       cur ^= 1;
-      if (valid) buf[cur * r.cap + i] = own;
-      __syncthreads();
+      if (valid) (cur ? buf1 : buf0)[i] = own;
+      if (!sync()) return;
     }
   }
   if (valid) {
@@ -281,7 +322,7 @@ __global__ void __launch_bounds__(reg_kets(MT), 1) resident_reg_kernel(const Tab
 
 template <int MT>
 int resident_reg_launch(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {
-  auto k = resident_reg_kernel<MT>;
+  auto k = resident_reg_kernel<MT, false>;
   const size_t smem = blk_smem_bytes(t, false) + (size_t)r.cap * 32;
   int per = 0, sms = 0;
   const int rc = occupancy_cached(k, smem, &per, &sms, threads);
@@ -289,6 +330,36 @@ int resident_reg_launch(const Tables& t, const ResArgs& r, int threads, cudaStre
   k<<<t.n_sectors, threads, smem, st>>>(t, r);
   QB_CUDA(cudaGetLastError());
   return QB_OK;
+}
+
+// The cooperative launch.  Two of them on different streams are kept in order by an event
+// (coop_order): each needs every SM, and CTAs of both must not wait for one another's places.
+template <int MT>
+int grid_reg_launch(const Tables& t, const ResArgs& r0, cudaStream_t st) {
+  auto k = resident_reg_kernel<MT, true>;
+  const size_t smem = blk_smem_bytes(t, false);
+  int per = 0, sms = 0;
+  const int rc = occupancy_cached(k, smem, &per, &sms, reg_kets(MT));
+  if (rc) return rc;
+  ResArgs r = r0;
+  Tables tt = t;
+  const int threads = ((int)((t.total + sms - 1) / sms) + 31) & ~31;
+  const int grid = (int)((t.total + threads - 1) / threads);
+  // the barrier's counter: 31 bits of arrivals a launch
+  const int64_t most = (int64_t)0x7fffffff / ((int64_t)grid * r.order) - 1;
+  void* args[] = {&tt, &r};
+  for (int64_t left = r0.steps; left > 0; left -= r.steps) {
+    r.steps = std::min(left, most);
+    QB_CUDA(cudaMemsetAsync(r.barrier, 0, sizeof(uint32_t), st));
+    const int e = coop_order(reinterpret_cast<const void*>(k), grid, threads, args, smem, st);
+    if (e) return e;
+  }
+  return QB_OK;
+}
+// Whether every ket finds a thread and a 16-bit target
+inline bool grid_reg_fits(const Tables& t, int sms) {
+  return !t.fa_on && (t.M == 5 || t.M == 7) && t.bk_kc > 0 &&
+         t.total <= std::min<int64_t>(65536, (int64_t)sms * reg_kets(t.M));
 }
 
 template <int MT, bool FIX, bool CPLX>
@@ -318,6 +389,8 @@ int resident_launch_m7(const Tables&, const ResArgs&, int, cudaStream_t);
 int resident_launch_m9(const Tables&, const ResArgs&, int, cudaStream_t);
 int resident_launch_m11(const Tables&, const ResArgs&, int, cudaStream_t);
 int resident_launch_any(const Tables&, const ResArgs&, int, cudaStream_t);
+int grid_launch_m5(const Tables&, const ResArgs&, cudaStream_t);
+int grid_launch_m7(const Tables&, const ResArgs&, cudaStream_t);
 
 // Every sector resident, `threads` threads each.
 inline int resident_launch(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {

@@ -9,4 +9,5 @@ int resident_launch_m7(const Tables& t, const ResArgs& r, int threads, cudaStrea
   if (threads <= reg_kets(7)) return resident_reg_launch<7>(t, r, threads, st);
   return resident_launch_k<7, true, false>(t, r, threads, st);
 }
+int grid_launch_m7(const Tables& t, const ResArgs& r, cudaStream_t st) { return grid_reg_launch<7>(t, r, st); }
 }  // namespace qb
