@@ -45,6 +45,22 @@ STAGE_NCU_ISSUE_ACTIVE = 0.670
 STAGE_NCU_L1_WAVEFRONTS = 0.920
 
 
+def _factored(W, qs):
+    """Whether the stages of this space run in two passes (contact couplings: one real number per
+    momentum class, spaces of enough kets)."""
+    if W.M < 6 or qs.total < (16384 if W.M >= 9 else 32768):
+        return False
+    L = np.asarray(W.L)
+    L = 0.25 * (L + L.transpose(1, 0, 2, 3) + L.transpose(0, 1, 3, 2) + L.transpose(1, 0, 3, 2))
+    pairs = [(p, q) for p in range(W.M) for q in range(p, W.M)]
+    for k in range(W.M):
+        cls = [a for a in pairs if sum(a) % W.M == k]
+        vals = {complex(L[a + b]) for a in cls for b in cls}
+        if len(vals) > 1 or any(v.imag for v in vals):
+            return False
+    return True
+
+
 def _peaks():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -565,8 +581,9 @@ def main():
     value = job_throughput(world, 4 * terms, ms_step)
     steps_per_s = 1e3 / ms_step
 
-    # ---- dominant kernel: one fused RK4 stage == one H psi over all sectors; a step is
-    # four launches of it, timed above with CUDA events on the launching stream
+    # ---- dominant kernels: one fused RK4 stage == one H psi over all sectors; a step is
+    # four of them, timed above with CUDA events on the launching stream
+    factored = _factored(W, qs)
     stage_time = ms_step * 1e-3 / 4
     flops = 4.0 * terms  # >= 2 FP64 FMA per term (real coefficient x complex amplitude)
     achieved = flops / stage_time / 1e12
@@ -592,7 +609,8 @@ def main():
         "frac": achieved / dfma_tflops, "peak_kind": "measured DFMA rate of this GPU (qb_measure_fp64_fma)",
         "peak_unit_count": FP64_PEAK_TFLOPS, "frac_of_unit_count": achieved / FP64_PEAK_TFLOPS,
         "traffic": STAGE_DRAM_BYTES_PER_KET * qs.total if args.config == "batched_coherent" else None,
-        "kernel": f"stage_df_kernel<{W.M},1,0,0,1,{qs.tile_shape}> (one RK4 stage = one H psi over all sectors, weighted basis)",
+        "kernel": (f"ann_kernel + cre_kernel<{W.M},0>" if factored else f"blk_stage_kernel<{W.M}>") +
+                  " (one RK4 stage = one H psi over all sectors, weighted basis)",
         "stage_ms": stage_time * 1e3,
         "peak_note": "FP64-equivalent flops (2 FMA/term) vs the FP64 FMA rate measured on this GPU; the "
                      "kernel itself runs double-float on the FP32/ALU pipes (FP64 pipe idle), so frac > 1 "
@@ -602,8 +620,8 @@ def main():
         "fp64_hpsi_ms": fp64_ms,
         "ncu_issue_active": STAGE_NCU_ISSUE_ACTIVE if args.config == "batched_coherent" else None,
         "ncu_l1_data_pipe": STAGE_NCU_L1_WAVEFRONTS if args.config == "batched_coherent" else None,
-        "ncu_note": "issue-slot and L1/shared data-pipe wavefront utilisation of the stage kernel from the "
-                    "ncu capture at n_tot=12 (profiles/stage_df_kernel_batched_coherent_ntot12.md)",
+        "ncu_note": "issue-slot and L1 utilisation of the creation pass, the longer of a stage's two kernels, from "
+                    "the ncu capture at n_tot=12 (profiles/factored_stage_batched_coherent_ntot12.md)",
     }
 
     # ---- plain path: one launch per sector per stage, same workload and arithmetic
@@ -693,10 +711,9 @@ def main():
             "observables_ms": obs_ms, "observables_kets_per_s": qs.total / (obs_ms * 1e-3),
             "evolve_observe_2_steps_3_obs_ms": evobs_ms, "breaktime_us": bt_us, "breaktime_flag": bt[1],
             "meanfield_ms": mf_ms, "meanfield_steps": W.steps}
-    # kernel launches of the timed call: four stage launches per step, the weighted copy,
-    # and the resident kernel when some sector is small enough
-    resident = resident_max > 0 and int(qs.dims[0]) <= resident_max  # leading sectors run resident
-    launches = 4 * args.steps + 1 + (1 if resident else 0)
+    # kernel launches of the timed call: four stages per step, of two kernels each where the
+    # couplings factor, and the weighted copy
+    launches = 4 * args.steps * (2 if factored else 1) + 1
 
     line = {
         "metric": "H_psi_terms_per_s", "value": value, "unit": "terms/s", "n_gpus": world, "steps": args.steps,

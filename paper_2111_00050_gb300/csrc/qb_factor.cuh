@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
   auto round_of = [&](int64_t r) { return perm ? (int64_t)__ldg(perm + max(r, r0)) : max(r, r0); };
   int64_t rn = round_of(rd), rn2 = round_of(rd - step);
   RoundIn next = load_round(t.fa_occ, t.fa_fill, t.fa_rblk, rn, t.fa_low, lane);
+  chain_wait();
   for (; rd >= r0; rd -= step) {
       const int64_t g = rn * 32 + lane;
       const bool valid = g >= a.low0 && g < a.low1;
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
         bad |= act && !ok;
 #pragma unroll
         for (int c = 0; c < NS; ++c)
-          if (ok && (NT > 0 || c < n)) x[c] = __ldg(a.vin + ix[c]);
+          if (ok && (NT > 0 || c < n)) x[c] = a.vin[ix[c]];
         if constexpr (NT > 0) {
           acc = dfc{f2_pack(x[0].x, x[0].y), f2_pack(x[0].z, x[0].w)};
         } else {
@@ -205,6 +206,7 @@ __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
   const int64_t r0 = a.row0 / 32, step = (int64_t)gridDim.x * warps;
   int64_t rd = (a.row1 - 1) / 32 - ((int64_t)blockIdx.x * warps + warp);
   RoundIn next = load_round(t.occ, t.fill, t.rblk, max(rd, r0), t.total, lane);
+  chain_wait();
   for (; rd >= r0; rd -= step) {
       const int64_t g = rd * 32 + lane;
       const bool valid = g >= a.row0 && g < a.row1;
@@ -245,7 +247,7 @@ __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
             A[c] = i < NO ? nf[pr.r[i]] * nf[pr.s[i]] : nf[pr.r[i]] * (nf[pr.r[i]] - 1.f);  // exact
             const bool act = A[c] != 0.f, ok = act && ix[c] < nG;
             bad |= act && !ok;
-            if (ok) x[c] = __ldg(a.g + ix[c]);
+            if (ok) x[c] = a.g[ix[c]];
           }
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
                    (occ_float23<NW>(ob, sel[c] >> 16, (sel[c] & 0x80000000u) != 0u) - del[c]);  // exact
             const bool act = A[c] != 0.f, ok = act && ix[c] < nG;
             bad |= act && !ok;
-            if (ok) x[c] = __ldg(a.g + ix[c]);
+            if (ok) x[c] = a.g[ix[c]];
           }
 #pragma unroll
           for (int c = 0; c < 4; ++c)
@@ -309,8 +311,7 @@ int ann_launch(const Tables& t, const DfArgs& a, int shape, cudaStream_t st, int
   int grid = 0, warps = 0;
   const int rc = stage_geometry(k, a.low1 - a.low0, shape, 32, smem, &warps, &grid);
   if (rc) return rc;
-  k<<<grid, 32 * warps, smem, st>>>(t, a);
-  QB_CUDA(cudaGetLastError());
+  QB_CUDA(chain_launch(k, grid, 32 * warps, smem, st, t, a));
   if (grid_out) *grid_out = grid;
   return QB_OK;
 }
@@ -322,8 +323,7 @@ int cre_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream
   int grid = 0, warps = 0;
   const int rc = stage_geometry(k, a.row1 - a.row0, shape, blk_max_threads<1, KIND>() / 32, smem, &warps, &grid);
   if (rc) return rc;
-  k<<<grid, 32 * warps, smem, st>>>(t, a, mode);
-  QB_CUDA(cudaGetLastError());
+  QB_CUDA(chain_launch(k, grid, 32 * warps, smem, st, t, a, mode));
   if (grid_out) *grid_out = grid;
   return QB_OK;
 }
