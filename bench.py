@@ -35,14 +35,14 @@ import workloads as wl  # noqa: E402
 # FP64 peak from unit counts and clock: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz; the
 # roofline uses the DFMA rate measured on the GPU by the run itself (qb_measure_fp64_fma)
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# DRAM bytes per ket of one stage launch (the first stage of a step), from an ncu capture
-# of the current stage kernel (batched coherent at n_tot=12: 617.2 MB read + 226.8 MB
-# written over 15,380,937 kets); scaled by kets
-STAGE_DRAM_BYTES_PER_KET = (617.219072e6 + 226.820352e6) / 15380937
-# the same capture's issue-slot and L1 data-pipe utilisation (the kernel's real limits:
-# the FP64 pipe is idle)
-STAGE_NCU_ISSUE_ACTIVE = 0.670
-STAGE_NCU_L1_WAVEFRONTS = 0.920
+# DRAM bytes per ket of one stage (both passes of the first stage of a step), from an ncu
+# capture of the current kernels (batched coherent at n_tot=12: 339.7 MB read + 1094.2 MB written
+# by the annihilation pass, 1881.2 + 233.9 by the creation pass, 15,380,937 kets); scaled by kets
+STAGE_DRAM_BYTES_PER_KET = (339.699e6 + 1094.183e6 + 1881.227e6 + 233.866e6) / 15380937
+# the same capture's issue-slot and L1 data-pipe utilisation of the creation pass, the longer one
+# (the kernels' real limits: the FP64 pipe is idle)
+STAGE_NCU_ISSUE_ACTIVE = 0.614
+STAGE_NCU_L1_WAVEFRONTS = 0.454
 
 
 def _factored(W, qs):

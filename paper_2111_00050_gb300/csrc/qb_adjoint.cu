@@ -99,13 +99,13 @@ __global__ void __launch_bounds__(kBlock) seed_kernel(const Tables t, const Seed
         // (a_j psi)_n = sqrt(n_j + 1) psi[n + e_j]
         const double2 pu = psi_at(t, v, rs, a.psi, N, K, 1, e, up, a.status);
         const double2 tu = cmul(a.ca[j], pu);
-        const double su = sqrt((double)(nj + 1));
+        const double su = v.sq[nj + 1];
         r.x += su * tu.x;
         r.y += su * tu.y;
         if (nj >= 1) {  // (a_j^dag psi)_n = sqrt(n_j) psi[n - e_j]
           const double2 pd = psi_at(t, v, rs, a.psi, N, K, 1, e, dnn, a.status);
           const double2 td = cmul(a.cad[j], pd);
-          const double sd = sqrt((double)nj);
+          const double sd = v.sq[nj];
           r.x += sd * td.x;
           r.y += sd * td.y;
         }
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kBlock) seed_kernel(const Tables t, const Seed
           const double2 p = psi_at(t, v, rs, a.psi, N, K, 2, e, dn, a.status);
           const double2 cij = cmul(cconj(a.xi[i]), a.xi[j]);
           const double2 tt = cmul(cij, p);
-          const double s = sqrt((double)ni * (double)(occ[j * kBlock] + 1));
+          const double s = v.sq[ni] * v.sq[occ[j * kBlock] + 1];
           r.x += s * tt.x;
           r.y += s * tt.y;
         }
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kBlock) mixed_kernel(const Tables t, const dou
       int e[1] = {k}, dn[1] = {-1};
       const double2 p = psi_at(t, v, rs, ket, N, K, 1, e, dn, status);
       const double2 tt = cmul(b, p);
-      const double sq = sqrt((double)nk);
+      const double sq = v.sq[nk];
       acc[2 * (k + 1)] += sq * tt.x;
       acc[2 * (k + 1) + 1] += sq * tt.y;
     }

@@ -757,14 +757,12 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
                                                                               double* partial, int nmom, int* status) {
   constexpr int NE = mo_entries<MT, AA>(), NC = (NE + 31) / 32, NW = occ_words<MT>(), W4 = (MT + 3) / 4;
   __shared__ double row[4 + 2 * MT + 4 * MT * MT];
-  __shared__ float2 sc[2][256];  // sqrt(N + 1) 2^(e_N - e_N+1); 2^(e_N - e_N-1) / sqrt(N)
+  __shared__ double sc[2][256];  // sqrt(N + 1) 2^(e_N - e_N+1); 2^(e_N - e_N-1) / sqrt(N)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   for (int N = threadIdx.x; N < t.nmax; N += blockDim.x) {
     const double e0 = __ldg(t.wscale + N).y;  // 2^e_N
-    const dfl up = df_of(sqrt((double)(N + 1)) * e0 * __ldg(t.wscale + N + 1).x);
-    const dfl dn = df_of(N > 0 ? e0 * __ldg(t.wscale + N - 1).x / sqrt((double)N) : 0.0);
-    sc[0][N] = make_float2(up.h, up.l);
-    sc[1][N] = make_float2(dn.h, dn.l);
+    sc[0][N] = sqrt((double)(N + 1)) * e0 * __ldg(t.wscale + N + 1).x;
+    sc[1][N] = N > 0 ? e0 * __ldg(t.wscale + N - 1).x / sqrt((double)N) : 0.0;
   }
   for (int k = threadIdx.x; k < nmom; k += blockDim.x) row[k] = 0.0;
   __syncthreads();
@@ -816,9 +814,9 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
     int N = 0;
 #pragma unroll
     for (int k = 0; k < NW; ++k) N += (int)__dp4a(ob[k], 0x01010101u, 0u);
-    const dfl W = valid ? df_of(__ldg(t.wk + g)) : dfl{0.f, 0.f};
-    const float2 cu = sc[0][valid ? N : 0];
-    const dfl wu = df_renorm(df_mul(W, dfl{cu.x, cu.y}));
+    // (a factor of N rounded to 48 bits by itself would err alike in all kets of N)
+    const double wk = valid ? __ldg(t.wk + g) : 0.0;
+    const dfl wu = df_of(wk * sc[0][valid ? N : 0]);
     float4 u[MT];
 #pragma unroll
     for (int k = 0; k < W4; ++k) {
@@ -837,7 +835,7 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
     for (int i = 0; i < MT; ++i) u[i] = df_scale(wu, u[i]);
     int e = 0;
     if constexpr (!AA) {
-      const float4 x = df_scale(W, valid ? __ldg(f + g) : make_float4(0.f, 0.f, 0.f, 0.f));
+      const float4 x = df_scale(df_of(wk), valid ? __ldg(f + g) : make_float4(0.f, 0.f, 0.f, 0.f));
 #pragma unroll
       for (int i = 0; i < MT; ++i, ++e) dfc_conj_fma(acc[e], df_re(x), df_im(x), u[i]);
 #pragma unroll
@@ -845,8 +843,7 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
 #pragma unroll
         for (int j = i + 1; j < MT; ++j, ++e) dfc_conj_fma(acc[e], df_re(u[i]), df_im(u[i]), u[j]);
     } else {
-      const float2 cd = sc[1][valid ? N : 0];
-      const dfl wd = df_renorm(df_mul(W, dfl{cd.x, cd.y}));
+      const dfl wd = df_of(wk * sc[1][valid ? N : 0]);
 #pragma unroll
       for (int k = 0; k < W4; ++k) {
         const uint4 b = __ldg(reinterpret_cast<const uint4*>(base) + W4 + k);
