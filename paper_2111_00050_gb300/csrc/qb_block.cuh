@@ -41,10 +41,10 @@ enum { KIND_STAGE = 0, KIND_BIL = 1, KIND_DOT = 2 };
 
 extern __shared__ __align__(16) unsigned char blk_smem[];
 
-// words of occupation bytes, four modes a word
+// words of occupation bytes, four modes a word (two at least: occ_float23)
 template <int MT>
 __host__ __device__ constexpr int occ_words() {
-  return MT > 0 ? (MT + 3) / 4 : 4;
+  return MT > 0 ? (MT > 4 ? (MT + 3) / 4 : 2) : 4;
 }
 
 // 2^23 + n_m as a float, exactly: the byte becomes the last one of 2^23.  The mode is in

@@ -60,6 +60,10 @@ CASES = {
     "direct_m11": (11, 6, 6, None, "long", False, 8008),
     "direct_m4": (4, 0, 20, None, "hermitian", False, 10626),
     "direct_m6": (6, 0, 9, None, "hermitian", False, 5005),
+    "direct_m7_complex": (7, 0, 8, None, "hermitian", False, 6435),
+    "direct_m8": (8, 0, 7, None, "hermitian", False, 6435),
+    "direct_m5_exact": (5, 0, 14, None, "long", True, 11628),
+    "factored_m8_exact": (8, 0, 10, None, "contact", True, 43758),
     "factored_m6": (6, 0, 14, None, "contact", False, 38760),
     "factored_m8": (8, 0, 10, None, "contact", False, 43758),
 }
