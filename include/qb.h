@@ -109,13 +109,14 @@ const char* qb_last_error(void);
  * current device, with the tables the space owns: per ket the diagonal of H
  * (16 B), the occupation vector packed into 64 bits (8 B), the ket weight and its
  * inverse (8 B each) and the number of its last modes' filling (4 B), plus a
- * double-float copy of an observed state (16 B per ket); and the ranking tables of
- * the stages (a few bytes per ket).
+ * double-float copy of an observed state (16 B per ket; above 2^28 kets it is allocated
+ * by the first qb_observables); and the ranking tables of the stages (a few bytes per ket).
  * Limits: 1 <= M <= QB_MAX_MODES; M * bits(n_max) <= 64; n_max <= 250;
  * the largest ket weight sqrt(n_max! / prod_m n_m!) over occupations of n_max
  * particles at most 2^160 (the RK4 stages hold psi / w(n) as fp32 pairs, with the
  * weights of each N centred on 1 by a power of two; e.g. n_max <= 206 for M = 3,
- * n_max <= 143 for M = 5); every sector dimension < 2^31; with exact momentum
+ * n_max <= 143 for M = 5); every sector dimension < 2^31, their sum < 2^32 - 2^16; with
+ * exact momentum
  * (M-1) n_max + 1 <= 6553 (the term shifts are 16-bit), and batched sweeps
  * (batch > 1) are not built.
  * Errors: QB_EINVAL for a bad model or range, QB_EUNSUPPORTED beyond the limits,
@@ -168,7 +169,9 @@ int qb_init_field_number(qb_space* space, const double* z, int n_tot, void* d_ps
  * vectors (at most M per ket, for one member). */
 int64_t qb_workspace_bytes(const qb_space* space, int batch);
 
-/* out = H psi for one state vector (d_out and d_psi distinct, device). */
+/* out = H psi for one state vector (d_out and d_psi distinct, device).  For a coupling that
+ * is one real number per momentum class the space allocates the annihilated vectors' memory
+ * (16 bytes an entry) at the first call; without it the rows are formed one by one. */
 int qb_hpsi(qb_space* space, const void* d_psi, void* d_out, void* stream);
 
 /* `steps` RK4 steps of size dt of d psi/dt = -i H psi, in place on d_psi.

@@ -18,7 +18,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libqb.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["qb_host.cpp", "qb_kernels.cu", "qb_adjoint.cu", "qb_stage_m5.cu", "qb_stage_m7.cu", "qb_stage_m9.cu", "qb_stage_m11.cu",
-           "qb_stage_any.cu", "qb_factor_m5.cu", "qb_factor_m7.cu", "qb_factor_m9.cu", "qb_factor_m11.cu",
+           "qb_stage_any.cu", "qb_factor_m7.cu", "qb_factor_m9.cu", "qb_factor_m11.cu",
            "qb_factor_any.cu", "qb_diag.cu", "qb_observe.cu", "qb_hpsi.cu", "qb_couple.cu"]
 HEADERS = ["qb_internal.h", "qb_device.cuh", "qb_block.cuh", "qb_factor.cuh", "qb_stage.cuh", os.path.join("..", "..", "include", "qb.h"),
            os.path.join("..", "..", "include", "qb_diag.h")]

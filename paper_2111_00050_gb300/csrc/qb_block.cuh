@@ -641,7 +641,6 @@ int stage_launch_m7(const Tables&, const DfArgs&, int, int, bool, int, cudaStrea
 int stage_launch_m9(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
 int stage_launch_m11(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
 int stage_launch_any(const Tables&, const DfArgs&, int, int, bool, bool, int, cudaStream_t, int*);
-int fac_launch_m5(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
 int fac_launch_m7(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
 int fac_launch_m9(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
 int fac_launch_m11(const Tables&, const DfArgs&, int, int, bool, int, cudaStream_t, int*);
@@ -655,7 +654,6 @@ inline int stage_launch(const Tables& t, const DfArgs& a, int mode, int B, bool 
                         int* grid_out = nullptr, bool bil = false, int shape = 0) {
   if (t.fa_on) {
     switch (t.M) {
-      case 5: return fac_launch_m5(t, a, mode, B, bil, shape, st, grid_out);
       case 7: return fac_launch_m7(t, a, mode, B, bil, shape, st, grid_out);
       case 9: return fac_launch_m9(t, a, mode, B, bil, shape, st, grid_out);
       case 11: return fac_launch_m11(t, a, mode, B, bil, shape, st, grid_out);

@@ -6,8 +6,8 @@
 // t the ket n with r, s taken away and p, q added: the target that the direct stage kernel
 // ranks for the same term.  f_n w_n^2 is formed by two products (w_n^2 alone may leave the fp32
 // range).  A task is one to four records (pairs (r, s) with their partners), up to eight
-// sums, over a share of the kets; sums over 32 kets of a lane are double-float, the lanes',
-// warps' and CTAs' are FP64 in a fixed order.
+// sums, over a share of the kets; the sums of a warp over up to 32 rounds are double-float, those
+// of the warps' flushes, the warps and the CTAs FP64, in a fixed order.
 //
 // Bound by the issue of the 24 packed operations of a complex product and of what they take
 // (57% of the issue slots, 16 warps an SM).  The 45 operators of 435,897 kets at M = 5: 74 us;

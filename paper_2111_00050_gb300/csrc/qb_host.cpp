@@ -294,7 +294,7 @@ static bool build_factored(Space& sp) {
 
   // annihilation records
   const bool fix = M % 2 == 1 && !sp.exact;
-  t.fa_nt = fix && M >= 5 && M <= 11 ? (M + 1) / 2 : 0;
+  t.fa_nt = fix && M <= 11 ? (M + 1) / 2 : 0;
   t.fa_pl = t.fa_nt > 4 ? 2 : 1;
   const int per = t.fa_nt > 0 ? t.fa_nt : 4;
   std::vector<uint32_t> rec;

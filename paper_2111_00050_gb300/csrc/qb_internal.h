@@ -180,9 +180,9 @@ struct Space {
   std::vector<int> secOf;                 // [(nmax+1) * Q]
   std::vector<unsigned char> blob;        // host copy of the shared-memory image
   Combos combos;
-  std::vector<unsigned char> bk;          // block tables but the maps (image of d_bk's first bytes)
-  size_t bk_off[8] = {0};                 // byte offsets of info, G, Gi, psh, EC, cls, the maps and combo in d_bk
-  std::vector<unsigned char> fa;          // tables of the factored couplings but the maps (image of d_fa's first bytes)
+  std::vector<unsigned char> bk;          // block tables but the maps and bases
+  size_t bk_off[8] = {0};                 // byte offsets of info, G, Gi, psh, EC, cls, (6 unused) and combo in bk
+  std::vector<unsigned char> fa;          // tables of the factored couplings but the maps and bases
   size_t fa_off[17] = {0};
   std::vector<int> lowN, lowK;            // lower sectors
   std::vector<int64_t> lowOff;
@@ -268,8 +268,6 @@ std::vector<int> tb_columns(const Space& s, const std::vector<int>& ops);
 int launch_tb_blocks(const Space& s, const float4* bra, const float4* ket, const int* cols, int n_ops, double weight,
                      double* acc, cudaStream_t st);
 int64_t workspace_bytes(const Space& s, int batch);
-// psi (FP64 complex) -> double-float copy (float4 per ket)
-int launch_to_df(const void* psi, void* psif, int64_t n, void* stream);
 // psi [B][total] -> double-float copy in the weighted basis f = psi / w(n) (the stages' basis)
 int launch_to_dfw(const Space& s, const void* psi, void* psif, int B, void* stream);
 // observables of Sec. II C-E from the raw moments (host)

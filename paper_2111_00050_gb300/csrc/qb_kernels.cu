@@ -174,14 +174,6 @@ __global__ void __launch_bounds__(kBlock) hpsi_kernel(const Tables t, const Stag
 }
 
 
-// psi (FP64) -> double-float copy
-__global__ void to_df_kernel(const double2* psi, float4* out, int64_t n) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    const double2 x = psi[k];
-    out[k] = df_pack(df_of(x.x), df_of(x.y));
-  }
-}
-
 // psi (FP64, [B][total]) -> double-float copy in the weighted basis, f = psi / w(n),
 // with the inverse weights of the per-ket table (coalesced, no unranking)
 template <int MT>
@@ -1482,12 +1474,6 @@ int launch_to_dfw(const Space& s, const void* psi, void* psif, int B, void* stre
     default: break;
   }
   k<<<grid, 256, 0, (cudaStream_t)stream>>>(s.t, (const double2*)psi, (float4*)psif, B);
-  QB_CUDA(cudaGetLastError());
-  return QB_OK;
-}
-
-int launch_to_df(const void* psi, void* psif, int64_t n, void* stream) {
-  to_df_kernel<<<1216, 256, 0, (cudaStream_t)stream>>>((const double2*)psi, (float4*)psif, n);
   QB_CUDA(cudaGetLastError());
   return QB_OK;
 }
