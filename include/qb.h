@@ -193,8 +193,9 @@ int qb_evolve_batch(qb_space* space, void* d_psi, int batch, const double* scale
  * every step of the call in one launch, in registers and shared memory.  A space of 5 or
  * 7 modes without factored couplings whose kets all find a thread (152 SMs: 65,536 and
  * 38,912 kets) runs in one cooperative launch, one thread a ket, with a grid barrier
- * between stages; such launches of one device run one after the other, whatever their
- * streams.  Other spaces run stage by stage, the launches captured into CUDA graphs in
+ * between stages.  Such launches of one device take turns, whatever their spaces, streams
+ * and threads: a call whose turn does not come in about the time that its own launch would
+ * take runs stage by stage instead.  Other spaces run stage by stage, the launches captured into CUDA graphs in
  * chunks of 32 steps.  0 disables both; the default is 1024.  Results do not depend on the
  * setting: every ket goes through the same arithmetic. */
 int qb_space_set_resident_max(qb_space* space, int resident_max_kets);

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <mutex>
 #include <string>
@@ -1334,26 +1335,24 @@ static int rk4_issue(Space& s, DfArgs& a, double dt, int64_t steps, float4* w1, 
   return QB_OK;
 }
 
-// Cooperative launches of every space on a device run one after the other, whatever their
-// streams: each waits for the event of the one before.
-int coop_order(const void* kernel, int grid, int threads, void** args, size_t smem, cudaStream_t st) {
+// Cooperative launches take turns: one call at a time on a device holds the turn, from before it
+// clears its barrier's counter until its stream is drained.  (Two at once could each hold the
+// SMs that the other's last CTAs need, and calls on one space share its counter.)  The turn is
+// a host lock and leaves nothing on the streams: a wait for another stream's event can close a
+// circle of waits with the caller's own, and an event that a caller's stream capture has taken
+// up refuses every later wait.  A call waits for it about as long as its own launch would run
+// (5 us a stage), between a millisecond and a second, and then goes stage by stage.
+static std::unique_lock<std::timed_mutex> coop_turn(const Space& s, int64_t steps) {
   constexpr int kDevices = 64;
-  static std::mutex mu;
-  static cudaEvent_t last[kDevices] = {};
-  int dev = 0;
-  QB_CUDA(cudaGetDevice(&dev));
-  if (dev >= kDevices) return fail(QB_EUNSUPPORTED, "device number");
-  std::lock_guard<std::mutex> lock(mu);
-  if (!last[dev]) QB_CUDA(cudaEventCreateWithFlags(&last[dev], cudaEventDisableTiming));
-  QB_CUDA(cudaStreamWaitEvent(st, last[dev], 0));
-  QB_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), args, smem, st));
-  QB_CUDA(cudaEventRecord(last[dev], st));
-  return QB_OK;
+  static std::timed_mutex turn[kDevices];
+  if (s.device < 0 || s.device >= kDevices) return {};
+  const int64_t us = std::min<int64_t>(std::max<int64_t>(5 * s.order * std::min<int64_t>(steps, 1000000), 1000), 1000000);
+  return std::unique_lock<std::timed_mutex>(turn[s.device], std::chrono::microseconds(us));
 }
 
 template <int B>
 static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int64_t steps, float4* w1, float4* w2,
-                    float4* psif, cudaStream_t st, bool plain = false) {
+                    float4* psif, cudaStream_t st, bool plain, std::unique_lock<std::timed_mutex>& turn) {
   {
     // the stages run in the weighted basis f = psi / w
     int rc = launch_to_dfw(s, psi, psif, B, st);
@@ -1394,11 +1393,8 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
       return resident_launch(s.t, r, (int)std::min<int64_t>(1024, (s.maxDim + 31) & ~int64_t(31)), st);
     // One cooperative launch where the kets find a thread each.
     if (s.resident_max_kets > 0 && grid_reg_fits(s.t, sms)) {
-      switch (s.M) {
-        case 5: return grid_launch_m5(s.t, r, st);
-        case 7: return grid_launch_m7(s.t, r, st);
-        default: break;
-      }
+      turn = coop_turn(s, steps);
+      if (turn.owns_lock()) return s.M == 5 ? grid_launch_m5(s.t, r, st) : grid_launch_m7(s.t, r, st);
     }
   }
   if (steps < 2 * kGraphSteps) return rk4_issue<B>(s, a, dt, steps, w1, w2, psif, st, false);
@@ -1447,15 +1443,19 @@ int launch_rk4(Space& s, void* d_psi, int batch, const double* scale, double dt,
   float4* w1 = (float4*)d_work;
   float4* w2 = w1 + n;
   float4* psif = w2 + n;
+  std::unique_lock<std::timed_mutex> turn;  // of a cooperative launch, held until the stream is drained
   int rc;
   switch (batch) {
-    case 1: rc = rk4_loop<1>(s, psi, scale, dt, steps, w1, w2, psif, st, plain); break;
-    case 2: rc = rk4_loop<2>(s, psi, scale, dt, steps, w1, w2, psif, st, plain); break;
-    case 4: rc = rk4_loop<4>(s, psi, scale, dt, steps, w1, w2, psif, st, plain); break;
-    case 8: rc = rk4_loop<8>(s, psi, scale, dt, steps, w1, w2, psif, st, plain); break;
+    case 1: rc = rk4_loop<1>(s, psi, scale, dt, steps, w1, w2, psif, st, plain, turn); break;
+    case 2: rc = rk4_loop<2>(s, psi, scale, dt, steps, w1, w2, psif, st, plain, turn); break;
+    case 4: rc = rk4_loop<4>(s, psi, scale, dt, steps, w1, w2, psif, st, plain, turn); break;
+    case 8: rc = rk4_loop<8>(s, psi, scale, dt, steps, w1, w2, psif, st, plain, turn); break;
     default: return fail(QB_EINVAL, "batch must be 1, 2, 4 or 8");
   }
-  if (rc) return rc;
+  if (rc) {
+    if (turn.owns_lock()) cudaStreamSynchronize(st);
+    return rc;
+  }
   return check_status(s, st);
 }
 

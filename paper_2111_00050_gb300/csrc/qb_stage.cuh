@@ -13,8 +13,6 @@
 
 namespace qb {
 
-int coop_order(const void* kernel, int grid, int threads, void** args, size_t smem, cudaStream_t st);
-
 struct ResArgs {
   double2* psi;        // global psi [total]
   float4* psif;        // global double-float copy of psi in the weighted basis [total] (read, written back)
@@ -332,8 +330,8 @@ int resident_reg_launch(const Tables& t, const ResArgs& r, int threads, cudaStre
   return QB_OK;
 }
 
-// The cooperative launch.  Two of them on different streams are kept in order by an event
-// (coop_order): each needs every SM, and CTAs of both must not wait for one another's places.
+// The cooperative launch, by the call that holds the device's turn (coop_turn): it needs every
+// SM, and the barrier's counter is the space's.
 template <int MT>
 int grid_reg_launch(const Tables& t, const ResArgs& r0, cudaStream_t st) {
   auto k = resident_reg_kernel<MT, true>;
@@ -351,8 +349,7 @@ int grid_reg_launch(const Tables& t, const ResArgs& r0, cudaStream_t st) {
   for (int64_t left = r0.steps; left > 0; left -= r.steps) {
     r.steps = std::min(left, most);
     QB_CUDA(cudaMemsetAsync(r.barrier, 0, sizeof(uint32_t), st));
-    const int e = coop_order(reinterpret_cast<const void*>(k), grid, threads, args, smem, st);
-    if (e) return e;
+    QB_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k), dim3(grid), dim3(threads), args, smem, st));
   }
   return QB_OK;
 }

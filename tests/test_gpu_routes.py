@@ -1,0 +1,88 @@
+"""Calls that meet on one space or one device, and the routes' limits and refusals.
+
+Where two runs take the same arithmetic they are compared bit for bit; against the oracle the
+tolerances are those of test_gpu_blocks.py.
+"""
+import ctypes
+import threading
+
+import numpy as np
+import pytest
+
+import oracle as orc
+import workloads as wl
+from helpers import random_state, rel_err, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def _space(M, hi, lo=0, kind="contact", **kw):
+    import paper_2111_00050_gb300 as qb
+
+    L = wl.long_range_coupling(M, 0.02) if kind == "long" else wl.contact_coupling(M, -0.02)
+    return qb.Space(M, wl.dispersion_quadratic(M) * 0.3, L, lo, hi, **kw)
+
+
+@pytest.mark.parametrize("threads", [2, 4])
+def test_threads_evolve_states_of_one_space(threads):
+    """A thread, a stream, a state and a workspace each on one space of the cooperative launch
+    (33,649 kets): the states of one call after the other, bit for bit."""
+    import torch
+
+    qs = _space(5, 18)
+    assert qs.total == 33649
+    want = [to_dev(random_state(qs.total, k)) for k in range(threads)]
+    got = [x.clone() for x in want]
+    for x in want:
+        for steps in (1, 20, 70, 3):
+            qs.evolve(x, 1e-3, steps)
+    work = [qs.workspace() for _ in range(threads)]
+    streams = [torch.cuda.Stream() for _ in range(threads)]
+    torch.cuda.synchronize()
+    errors = []
+
+    def run(k):
+        try:
+            with torch.cuda.stream(streams[k]):
+                for steps in (1, 20, 70, 3):
+                    qs.evolve(got[k], 1e-3, steps, work[k])
+        except Exception as e:  # noqa: BLE001 (reported by the main thread)
+            errors.append(e)
+
+    pool = [threading.Thread(target=run, args=(k,)) for k in range(threads)]
+    for t in pool:
+        t.start()
+    for t in pool:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
+    assert all(bool((g == e).all()) for g, e in zip(got, want))
+
+
+def test_a_call_under_capture_leaves_nothing_behind():
+    """A call on a stream that its caller captures ends in an error (its status is read by the
+    host); the next call, on any stream, is as if it had not been."""
+    import torch
+
+    import paper_2111_00050_gb300 as qb
+
+    rt = ctypes.CDLL("libcudart.so.13")
+    qs = _space(5, 18)
+    x = to_dev(random_state(qs.total, 1))
+    want = x.clone()
+    qs.set_resident_max(0)  # stage by stage
+    qs.evolve(want, 1e-3, 5)
+    qs.set_resident_max(1024)
+    work = qs.workspace()
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    handle, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    assert rt.cudaStreamBeginCapture(handle, 1) == 0  # thread-local mode
+    with torch.cuda.stream(stream), pytest.raises(qb.QbError):
+        qs.evolve(x, 1e-3, 5, work)
+    rt.cudaStreamEndCapture(handle, ctypes.byref(graph))
+    if graph.value:
+        rt.cudaGraphDestroy(graph)
+    rt.cudaGetLastError()
+    qs.evolve(x, 1e-3, 5, work)
+    assert bool((x == want).all())
