@@ -41,7 +41,7 @@ extern "C" {
 #define QB_EINVAL 1       /* bad argument: size, alignment, range, non-Hermitian or non-conserving L */
 #define QB_ENOMEM 2       /* a device or host allocation failed */
 #define QB_ECUDA 3        /* a CUDA runtime call or kernel launch failed */
-#define QB_ETIMEOUT 4     /* a bounded device-side wait ran out */
+#define QB_ETIMEOUT 4     /* a bounded device-side wait ran out (qb_evolve: d_psi is then undefined) */
 #define QB_EINTERNAL 5    /* a device-side consistency check failed (rank out of range, ...) */
 #define QB_EUNSUPPORTED 6 /* outside the compiled limits (M > QB_MAX_MODES, packed occupation > 64 bits) */
 
@@ -195,9 +195,11 @@ int qb_evolve_batch(qb_space* space, void* d_psi, int batch, const double* scale
  * 38,912 kets) runs in one cooperative launch, one thread a ket, with a grid barrier
  * between stages.  Such launches of one device take turns, whatever their spaces, streams
  * and threads: a call whose turn does not come in about the time that its own launch would
- * take runs stage by stage instead.  Other spaces run stage by stage, the launches captured into CUDA graphs in
- * chunks of 32 steps.  0 disables both; the default is 1024.  Results do not depend on the
- * setting: every ket goes through the same arithmetic. */
+ * take runs stage by stage instead.  The barrier's waits are bounded (about a minute): a call
+ * whose wait runs out, as behind another stream's kernel that does not give up its SMs, returns
+ * QB_ETIMEOUT and leaves d_psi undefined.  Other spaces run stage by stage, the launches
+ * captured into CUDA graphs in chunks of 32 steps.  0 disables both; the default is 1024.
+ * Results do not depend on the setting: every ket goes through the same arithmetic. */
 int qb_space_set_resident_max(qb_space* space, int resident_max_kets);
 
 /* Execution tuning of the RK4 stages of qb_evolve, qb_evolve_plain and

@@ -1,5 +1,5 @@
 /*
- * qb_diag -- diagnostics and measurement helpers of the qb library.  Neither
+ * qb_diag -- diagnostics and measurement helpers of the qb library.  No
  * call computes anything of the paper's method (arXiv:2111.00050 has no
  * counterpart); they serve error-path tests and the roofline denominators of
  * the benchmark.  Conventions as in qb.h (status codes, void* streams).
@@ -26,6 +26,13 @@ extern "C" {
  * be NULL) without clearing it.  A nonzero set_bits lets a test exercise the error
  * path of the next call without any device fault.  Synchronises the stream. */
 int qb_space_status(qb_space* space, int set_bits, int* status, void* stream);
+
+/* Polls of a thread block at a barrier of qb_evolve's cooperative launch (qb.h,
+ * qb_space_set_resident_max) before it gives up and the call returns QB_ETIMEOUT;
+ * 2^27 (about a minute) after qb_sector_build.  With 0 every wait runs out at the
+ * first barrier, before any state is written, which lets a test exercise that path.
+ * Later calls on the space take it. */
+int qb_space_set_wait_polls(qb_space* space, uint32_t polls);
 
 /* FP64 fused multiply-add rate of the current GPU, for the roofline denominator
  * of FP64-equivalent work: a grid of 8 CTAs per SM of 256 threads, each running 8

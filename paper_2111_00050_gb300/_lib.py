@@ -96,6 +96,7 @@ SIGNATURES = {
                                     ctypes.c_int, _c_double_p]),
     # include/qb_diag.h
     "qb_space_status": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, _c_int_p, ctypes.c_void_p]),
+    "qb_space_set_wait_polls": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_uint32]),
     "qb_measure_fp64_fma": (ctypes.c_int, [ctypes.c_int, _c_double_p, ctypes.c_void_p]),
 }
 

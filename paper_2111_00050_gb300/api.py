@@ -131,6 +131,11 @@ class Space:
         check(lib().qb_space_status(self._h, int(set_bits), ctypes.byref(st), _stream()))
         return int(st.value)
 
+    def set_wait_polls(self, polls: int) -> None:
+        """qb_space_set_wait_polls: polls at a barrier of the cooperative launch before evolve
+        ends in QB_ETIMEOUT (0: at once)."""
+        check(lib().qb_space_set_wait_polls(self._h, int(polls)))
+
     def terms(self):
         t, u = ctypes.c_int64(), ctypes.c_int64()
         check(lib().qb_space_terms(self._h, ctypes.byref(t), ctypes.byref(u), _stream()))

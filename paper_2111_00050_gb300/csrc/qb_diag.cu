@@ -1,5 +1,5 @@
 // Diagnostics and measurement helpers (include/qb_diag.h): the device status
-// word of a space, and the FP64 FMA rate of the GPU for the roofline denominator.
+// word of a space, the limit of its bounded waits, and the FP64 FMA rate of the GPU for the roofline denominator.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -47,6 +47,13 @@ extern "C" int qb_space_status(qb_space* space, int set_bits, int* status, void*
     QB_CUDA(cudaStreamSynchronize(st));
   }
   if (status) *status = h;
+  return QB_OK;
+}
+
+extern "C" int qb_space_set_wait_polls(qb_space* space, uint32_t polls) {
+  Space* sp = reinterpret_cast<Space*>(space);
+  if (!sp) return fail(QB_EINVAL, "space is NULL");
+  sp->wait_polls = polls;
   return QB_OK;
 }
 

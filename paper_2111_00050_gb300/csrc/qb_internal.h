@@ -22,6 +22,9 @@ constexpr int kDeltaBias = 64;
 // factored only where the vector of B_k f fits beside what a step needs without it.
 constexpr int64_t kObsfKets = 1ll << 28;
 
+// Polls of a grid barrier before its CTA gives up: a minute or so
+constexpr uint32_t kWaitPolls = 1u << 27;
+
 // 32-bit indices of kets and of entries of B_k f stay below this
 constexpr uint32_t kNoIndex = 0xffff0000u;
 
@@ -205,6 +208,7 @@ struct Space {
   cudaStream_t capture_stream = nullptr;  // private stream on which RK4 chunks are captured into graphs
   int resident_max_kets = 1024;           // spaces whose sectors are all up to this size run shared-memory resident
   int order = 4;                          // Taylor order of a time step (4: RK4)
+  uint32_t wait_polls = kWaitPolls;       // of a cooperative launch's CTA at a barrier
   int tile_shape = 0;                     // tile shape of the single-state stage kernel (qb_stage.cuh)
   int device = 0;
   int grid_hpsi = 0;  // persistent grid sizes per kernel family
@@ -224,7 +228,8 @@ __host__ __device__ inline int nmoments(int M) { return 4 + 2 * M + 4 * M * M; }
 __host__ __device__ inline int nprep(int M) { return M + 2; }
 
 // Scratch layout of a space (doubles), sized at set-up for the largest persistent grid
-// G = SMs * 16:  [0, 2) status word | moment sums [nmom] | <H> sum [2] | first-pass sums [nprep]
+// G = SMs * 16:  status word (first half of [0, 1)), counter and status of the cooperative
+// launch ([1, 2)) | moment sums [nmom] | <H> sum [2] | first-pass sums [nprep]
 // (these, the first finals_doubles, come back in one copy) | moment partials [G nmom] |
 // bilinear / <H> partials [(M + 1) G] | first-pass partials [nprep G] | amplitude table
 // [2 M (nmax + 1)] | initial-state norm [2]

@@ -1387,13 +1387,15 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
     r.cap = cap;
     r.w1 = w1;
     r.w2 = w2;
-    r.barrier = reinterpret_cast<uint32_t*>(s.d_scratch + 1);
     r.status = a.status;
     if (s.maxDim <= std::min(s.resident_max_kets, resident_most(s.t)) && s.t.total <= 64LL * sms && resident_smem(s.t, cap) + 1024 <= (size_t)optin)
       return resident_launch(s.t, r, (int)std::min<int64_t>(1024, (s.maxDim + 31) & ~int64_t(31)), st);
     // One cooperative launch where the kets find a thread each.
     if (s.resident_max_kets > 0 && grid_reg_fits(s.t, sms)) {
       turn = coop_turn(s, steps);
+      r.barrier = reinterpret_cast<uint32_t*>(s.d_scratch + 1);
+      r.status = reinterpret_cast<int*>(r.barrier) + 1;
+      r.polls = s.wait_polls;
       if (turn.owns_lock()) return s.M == 5 ? grid_launch_m5(s.t, r, st) : grid_launch_m7(s.t, r, st);
     }
   }
@@ -1454,6 +1456,15 @@ int launch_rk4(Space& s, void* d_psi, int batch, const double* scale, double dt,
   }
   if (rc) {
     if (turn.owns_lock()) cudaStreamSynchronize(st);
+    return rc;
+  }
+  if (turn.owns_lock()) {  // with the launch's own status, which no other call on the space reads or clears
+    int h[4];
+    QB_CUDA(cudaMemcpyAsync(h, s.d_scratch, sizeof(h), cudaMemcpyDeviceToHost, st));
+    QB_CUDA(cudaStreamSynchronize(st));
+    rc = h[0] ? check_status(s, st) : QB_OK;
+    if (h[3] & kLate) return fail(QB_ETIMEOUT, "a wait between the stages of a cooperative launch ran out");
+    if (h[3]) return fail(QB_EINTERNAL, "device-side consistency check failed (status " + std::to_string(h[3]) + ")");
     return rc;
   }
   return check_status(s, st);

@@ -24,6 +24,8 @@ struct ResArgs {
   int cap;             // kets per sector the shared buffers hold (a multiple of 4)
   float4 *w1, *w2;     // stage vectors [total] and counter of the cooperative launch
   uint32_t* barrier;
+  uint32_t polls;      // of a CTA at a barrier before it gives up
+  bool later;          // not the call's first launch
   int* status;
 };
 
@@ -173,21 +175,21 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
 }
 
 // Barrier of a cooperative grid: the CTAs arrive at a counter and wait until `target` have.
-// The wait is bounded (a minute or so, longer than another stream's kernel should hold the
-// SMs that the grid's last CTAs wait for): on its end the status is set and every CTA leaves.
-constexpr uint32_t kSpinLimit = 1u << 27;
-__device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target, int* status) {
+// The wait is bounded (kWaitPolls, a minute or so, longer than another stream's kernel should
+// hold the SMs that the grid's last CTAs wait for): on its end kLate is set in the launch's
+// status and the CTA leaves, as every other one does at the next barrier.
+constexpr int kLate = 8;
+__device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target, uint32_t polls, int* status) {
   __syncthreads();
   int late = 0;
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(counter, 1u);
-    uint32_t seen, n = 0;
-    do {
+    uint32_t seen = 0;
+    for (uint32_t n = 0; n < polls && seen < target; ++n)
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
-    } while (seen < target && ++n < kSpinLimit);
     late = seen < target;
-    if (late) atomicOr(status, 8);
+    if (late) atomicOr(status, kLate);
     __threadfence();
   }
   return __syncthreads_or(late) == 0;
@@ -215,6 +217,8 @@ __global__ void __launch_bounds__(reg_kets(MT), 1) resident_reg_kernel(const Tab
   constexpr int NR = MT * (MT + 1) / 2;
   static_assert(KC >= 2 && KC <= 4, "two or four 16-bit targets a record");
   const int T = t.bk_T;
+  // a launch after one of the same call that gave up does nothing
+  if (GRID && r.later && __syncthreads_or(threadIdx.x == 0 && (*reinterpret_cast<volatile int*>(r.status) & kLate) != 0)) return;
   float2* sG = reinterpret_cast<float2*>(blk_smem);
   // two vectors of the stages: [2][cap] in shared memory, or the workspace's
   float4* const buf0 = GRID ? r.w1 : reinterpret_cast<float4*>(blk_smem + blk_smem_bytes(t, false));
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(reg_kets(MT), 1) resident_reg_kernel(const Tab
   int cur = 0;
   uint32_t round = 0;
   auto sync = [&]() -> bool {  // false: the grid's barrier gave up
-    if (GRID) return grid_barrier(r.barrier, ++round * gridDim.x, r.status);
+    if (GRID) return grid_barrier(r.barrier, ++round * gridDim.x, r.polls, r.status);
     __syncthreads();
     return true;
   };
@@ -331,7 +335,7 @@ int resident_reg_launch(const Tables& t, const ResArgs& r, int threads, cudaStre
 }
 
 // The cooperative launch, by the call that holds the device's turn (coop_turn): it needs every
-// SM, and the barrier's counter is the space's.
+// SM, and the barrier's counter and the status beside it are the space's.
 template <int MT>
 int grid_reg_launch(const Tables& t, const ResArgs& r0, cudaStream_t st) {
   auto k = resident_reg_kernel<MT, true>;
@@ -348,7 +352,8 @@ int grid_reg_launch(const Tables& t, const ResArgs& r0, cudaStream_t st) {
   void* args[] = {&tt, &r};
   for (int64_t left = r0.steps; left > 0; left -= r.steps) {
     r.steps = std::min(left, most);
-    QB_CUDA(cudaMemsetAsync(r.barrier, 0, sizeof(uint32_t), st));
+    r.later = left < r0.steps;
+    QB_CUDA(cudaMemsetAsync(r.barrier, 0, (r.later ? 1 : 2) * sizeof(uint32_t), st));  // the status once
     QB_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k), dim3(grid), dim3(threads), args, smem, st));
   }
   return QB_OK;

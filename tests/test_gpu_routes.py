@@ -86,3 +86,27 @@ def test_a_call_under_capture_leaves_nothing_behind():
     rt.cudaGetLastError()
     qs.evolve(x, 1e-3, 5, work)
     assert bool((x == want).all())
+
+
+@pytest.mark.parametrize("M,hi", [(5, 18), (7, 10)])
+def test_a_wait_that_runs_out_is_reported(M, hi):
+    """With no polls every thread block gives up at the first barrier and leaves: QB_ETIMEOUT, for
+    this call alone; the calls after it, with the limit back, are as if it had not been."""
+    import paper_2111_00050_gb300 as qb
+
+    qs = _space(M, hi)
+    x = to_dev(random_state(qs.total, 2))
+    want = x.clone()
+    qs.evolve(want, 1e-3, 5)
+    y = x.clone()
+    qs.set_wait_polls(0)
+    for steps in (1, 40):
+        with pytest.raises(qb.QbError) as e:
+            qs.evolve(y, 1e-3, steps)
+        assert e.value.code == qb._lib.QB_ETIMEOUT
+    assert qs.status() == 0
+    qs.observables(x)
+    qs.set_wait_polls(1 << 27)
+    y.copy_(x)
+    qs.evolve(y, 1e-3, 5)
+    assert bool((y == want).all())
