@@ -102,6 +102,7 @@ class Space:
         self.order = 4
         self.tile_shape = 0
         self.tuning = None
+        self._work_bytes = {}  # qb_workspace_bytes by batch
 
     def __del__(self):
         h = getattr(self, "_h", None)
@@ -167,11 +168,23 @@ class Space:
         n = int(lib().qb_workspace_bytes(self._h, int(batch)))
         return torch.empty(n // 16, dtype=torch.complex128, device="cuda")
 
+    def _work(self, work: Optional[torch.Tensor], batch: int, steps: int) -> torch.Tensor:
+        """The caller's workspace, if it holds what `batch` states of this space take (the size
+        depends on the couplings too, not only on the kets), or one of its own."""
+        if work is None:
+            return self.workspace(batch)
+        need = self._work_bytes.get(batch)
+        if need is None:
+            need = self._work_bytes[batch] = int(lib().qb_workspace_bytes(self._h, batch))
+        if steps > 0 and work.numel() * work.element_size() < need:
+            raise ValueError("workspace too small for this space (Space.workspace)")
+        return work
+
     def hpsi(self, psi: torch.Tensor, out: torch.Tensor) -> None:
         check(lib().qb_hpsi(self._h, _dptr(psi), _dptr(out), _stream()))
 
     def evolve(self, psi: torch.Tensor, dt: float, steps: int, work: Optional[torch.Tensor] = None) -> None:
-        work = self.workspace(1) if work is None else work
+        work = self._work(work, 1, steps)
         check(lib().qb_evolve(self._h, _dptr(psi), float(dt), int(steps), _dptr(work), _stream()))
 
     def set_resident_max(self, kets: int) -> None:
@@ -228,13 +241,13 @@ class Space:
         return best
 
     def evolve_plain(self, psi: torch.Tensor, dt: float, steps: int, work: Optional[torch.Tensor] = None) -> None:
-        work = self.workspace(1) if work is None else work
+        work = self._work(work, 1, steps)
         check(lib().qb_evolve_plain(self._h, _dptr(psi), float(dt), int(steps), _dptr(work), _stream()))
 
     def evolve_batch(self, psi: torch.Tensor, scale, dt: float, steps: int,
                      work: Optional[torch.Tensor] = None) -> None:
         sc = _f64(scale)
-        work = self.workspace(sc.size) if work is None else work
+        work = self._work(work, int(sc.size), steps)
         check(lib().qb_evolve_batch(self._h, _dptr(psi), int(sc.size),
                                     sc.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), float(dt), int(steps),
                                     _dptr(work), _stream()))
@@ -281,7 +294,7 @@ class Space:
 
     def evolve_observe(self, psi: torch.Tensor, dt: float, steps: int, obs_every: int,
                        work: Optional[torch.Tensor] = None) -> list:
-        work = self.workspace(1) if work is None else work
+        work = self._work(work, 1, steps)
         n = steps // obs_every + 1
         arr = (QbObs * n)()
         check(lib().qb_evolve_observe(self._h, _dptr(psi), float(dt), int(steps), int(obs_every), arr, _dptr(work),

@@ -110,3 +110,37 @@ def test_a_wait_that_runs_out_is_reported(M, hi):
     y.copy_(x)
     qs.evolve(y, 1e-3, 5)
     assert bool((y == want).all())
+
+
+@pytest.mark.parametrize("kind", ["long", "contact"])
+def test_a_workspace_that_is_too_small_is_refused(kind):
+    """Two spaces over the same kets can differ in what they take (a contact coupling adds the
+    annihilated vectors): a workspace of the smaller one is refused, not written past its end."""
+    import torch
+
+    qs = _space(7, 12, kind=kind)
+    base = torch.empty(3 * qs.total, dtype=torch.complex128, device="cuda")
+    x = to_dev(random_state(qs.total, 1))
+    want = x.clone()
+    qs.evolve(want, 1e-3, 2)
+    calls = {
+        "evolve": lambda y, work: qs.evolve(y, 1e-3, 2, work),
+        "evolve_plain": lambda y, work: qs.evolve_plain(y, 1e-3, 2, work),
+        "evolve_observe": lambda y, work: qs.evolve_observe(y, 1e-3, 2, 1, work),
+        "evolve_batch": lambda y, work: qs.evolve_batch(y, [1.0], 1e-3, 2, work),
+    }
+    work = qs.workspace()
+    assert (work.numel() > base.numel()) == (kind == "contact")
+    for name, call in calls.items():
+        for w in (base, work[1:]):
+            y = x.clone()
+            if w is base and kind == "long":
+                call(y, w)
+                assert bool((y == want).all()), name
+            else:
+                with pytest.raises(ValueError):
+                    call(y, w)
+                assert bool((y == x).all()), name
+    qs.evolve(x, 1e-3, 0, work[1:])  # no steps take no workspace
+    with pytest.raises(ValueError):
+        qs.evolve_batch(torch.stack([x, x]), [1.0, 2.0], 1e-3, 2, work)
