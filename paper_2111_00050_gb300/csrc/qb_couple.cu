@@ -5,9 +5,10 @@
 //   <bra, a_p^dag a_q^dag a_r a_s ket> = sum_n conj(b_t) k f_n w_n^2,  k = n_r (n_s - [r = s]),
 // t the ket n with r, s taken away and p, q added: the target that the direct stage kernel
 // ranks for the same term.  f_n w_n^2 is formed by two products (w_n^2 alone may leave the fp32
-// range).  A task is one to four records (pairs (r, s) with their partners), up to eight
-// sums, over a share of the kets; the sums of a warp over up to 32 rounds are double-float, those
-// of the warps' flushes, the warps and the CTAs FP64, in a fixed order.
+// range), the weight with a third part (dft_mul).  A task is one to four records (pairs (r, s) with their partners), up to eight
+// sums, over a share of the kets; the sums of a lane over up to 32 kets are double-float, those of
+// the lanes of three floats (tfc_add, more bits than FP64), those of the warps' flushes, the
+// warps and the CTAs FP64, in a fixed order.
 //
 // Bound by the issue of the 24 packed operations of a complex product and of what they take
 // (57% of the issue slots, 16 warps an SM).  The 45 operators of 435,897 kets at M = 5: 74 us;
@@ -70,6 +71,9 @@ __global__ void __launch_bounds__(32 * kTbWarps, 2) tb_kernel(const Tables t, co
   // more add the four lanes of a column (all eight columns by FP64 shuffles took longer than
   // the products where a warp has few rounds)
   auto flush = [&]() {
+    f2 rest[kTbCols];  // third parts (tfc_add)
+#pragma unroll
+    for (int j = 0; j < kTbCols; ++j) rest[j] = 0ull;
 #pragma unroll
     for (int w = kTbCols / 2; w >= 1; w >>= 1) {
       const bool up = (lane & (4 * w)) != 0;
@@ -77,22 +81,21 @@ __global__ void __launch_bounds__(32 * kTbWarps, 2) tb_kernel(const Tables t, co
       for (int j = 0; j < kTbCols / 2; ++j) {
         if (j >= w) break;
         const dfc mine = up ? acc[j + w] : acc[j], other = up ? acc[j] : acc[j + w];
+        const f2 rmine = up ? rest[j + w] : rest[j], rother = up ? rest[j] : rest[j + w];
         acc[j] = mine;
-        dfc_add(acc[j], __shfl_xor_sync(0xffffffffu, other.h, 4 * w), __shfl_xor_sync(0xffffffffu, other.l, 4 * w));
-        acc[j] = dfc_renorm(acc[j]);
+        rest[j] = rmine;
+        tfc_add(acc[j], rest[j], __shfl_xor_sync(0xffffffffu, other.h, 4 * w), __shfl_xor_sync(0xffffffffu, other.l, 4 * w),
+                w < kTbCols / 2 ? __shfl_xor_sync(0xffffffffu, rother, 4 * w) : 0ull);
       }
     }
 #pragma unroll
-    for (int o = 2; o >= 1; o >>= 1) {
-      dfc_add(acc[0], __shfl_xor_sync(0xffffffffu, acc[0].h, o), __shfl_xor_sync(0xffffffffu, acc[0].l, o));
-      acc[0] = dfc_renorm(acc[0]);
-    }
+    for (int o = 2; o >= 1; o >>= 1)
+      tfc_add(acc[0], rest[0], __shfl_xor_sync(0xffffffffu, acc[0].h, o), __shfl_xor_sync(0xffffffffu, acc[0].l, o),
+              __shfl_xor_sync(0xffffffffu, rest[0], o));
     if ((lane & 3) == 0) {  // column lane / 4
-      float rh, ih, rl, il;
-      f2_unpack(acc[0].h, rh, ih);
-      f2_unpack(acc[0].l, rl, il);
-      sum[warp][lane / 2] += (double)rh + (double)rl;
-      sum[warp][lane / 2 + 1] += (double)ih + (double)il;
+      const double2 v = tfc_to(acc[0], rest[0]);
+      sum[warp][lane / 2] += v.x;
+      sum[warp][lane / 2 + 1] += v.y;
     }
 #pragma unroll
     for (int j = 0; j < kTbCols; ++j) acc[j] = dfc{0ull, 0ull};
@@ -107,7 +110,7 @@ __global__ void __launch_bounds__(32 * kTbWarps, 2) tb_kernel(const Tables t, co
   for (; rd < nr; rd += step) {
     const RoundIn in = next;
     const float4 kv = knext;
-    const dfl wd = df_of(wnext);
+    const dft wd = dft_of(wnext);
     const int64_t g = rd * 32 + lane;
     const bool valid = g < total;
     {
@@ -116,7 +119,7 @@ __global__ void __launch_bounds__(32 * kTbWarps, 2) tb_kernel(const Tables t, co
       knext = __ldg(ket + gn);
       wnext = __ldg(t.wk + gn);
     }
-    const dfl yr = df_mul(df_mul(df_re(kv), wd), wd), yi = df_mul(df_mul(df_im(kv), wd), wd);
+    const dfl yr = dft_mul(wd, dft_mul(wd, df_re(kv))), yi = dft_mul(wd, dft_mul(wd, df_im(kv)));
     const f2 yh = f2_pack(yr.h, yi.h), yl = f2_pack(yr.l, yi.l);
     uint32_t ob[NW];
     unpack_occ<MT, NW>(t, valid ? in.word : 0ull, ob);  // an invalid lane: no pair acts

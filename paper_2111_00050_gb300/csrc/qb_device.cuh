@@ -247,6 +247,9 @@ __device__ __forceinline__ int64_t rank_changed(const Tables& t, const View& v, 
 struct dfl {
   float h, l;
 };
+struct dft {  // and what the low part rounds off, below 2^-48 of the value
+  float h, l, r;
+};
 
 // The split by integers: FP64 conversions and sums run at the FP64 rate (2 a clock and SM),
 // which bounds what forms a weighted copy.  The 24 leading bits rounded to nearest are the
@@ -255,7 +258,7 @@ struct dfl {
 // One stage of the 42-ket sector 1.12 -> 1.06 us, 100 steps of 245,157 kets at M = 7 14.8 ->
 // 14.6 ms; the inverse by integers (two parts put together) costs the bilinear stages more
 // than it saves.
-__device__ __forceinline__ dfl df_of(double x) {
+__device__ __forceinline__ dft dft_of(double x) {
   const uint32_t hw = (uint32_t)__double2hiint(x), lw = (uint32_t)__double2loint(x), ex = (hw >> 20) & 0x7ffu;
   if (ex - 920u < 230u) {
     const int up = (int)((lw >> 28) & 1u);  // the first bit left off
@@ -263,11 +266,19 @@ __device__ __forceinline__ dfl df_of(double x) {
     const int rest = (int)(lw & 0x1fffffffu) - (up << 29);
     const uint32_t sign = hw & 0x80000000u;
     const float scale = __uint_as_float(sign | ((ex - 919u) << 23));  // 2^(e - 23)
-    return {__uint_as_float(sign | top), __fmul_rn(__fmul_rn((float)rest, 0x1p-29f), scale)};
+    const float low = (float)rest;
+    return {__uint_as_float(sign | top), __fmul_rn(__fmul_rn(low, 0x1p-29f), scale),
+            __fmul_rn(__fmul_rn((float)(rest - (int)low), 0x1p-29f), scale)};
   }
-  if (((hw << 1) | lw) == 0u) return {__uint_as_float(hw), 0.f};  // most kets of a number state
+  if (((hw << 1) | lw) == 0u) return {__uint_as_float(hw), 0.f, 0.f};  // most kets of a number state
   const float h = __double2float_rn(x);
-  return {h, __double2float_rn(x - (double)h)};
+  const double d = x - (double)h;
+  const float l = __double2float_rn(d);
+  return {h, l, __double2float_rn(d - (double)l)};
+}
+__device__ __forceinline__ dfl df_of(double x) {
+  const dft a = dft_of(x);
+  return {a.h, a.l};
 }
 __device__ __forceinline__ double df_to(dfl a) { return (double)a.h + (double)a.l; }
 __device__ __forceinline__ dfl df_neg(dfl a) { return {-a.h, -a.l}; }
@@ -287,6 +298,17 @@ __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
   e = fmaf(a.h, b.l, e);
   e = fmaf(a.l, b.h, e);
   return {p, e};
+}
+
+// a * b, unnormalised, for a factor that many b share: the rounding of its low part would err
+// alike in all of them.  (The third part comes first: added to a sum that is rounded already, it
+// would be lost in the same way each time.)
+__device__ __forceinline__ dfl dft_mul(dft a, dfl b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = __fmul_rn(a.r, b.h);
+  e = fmaf(a.l, b.h, e);
+  e = fmaf(a.h, b.l, e);
+  return {p, __fadd_rn(e, fmaf(a.h, b.h, -p))};
 }
 
 // acc += c * x; acc.h carries the TwoSum, acc.l gathers every rounding error
@@ -401,6 +423,32 @@ __device__ __forceinline__ void dfc_fma_int(dfc& acc, f2 a2, f2 na2, f2 xh, f2 x
 __device__ __forceinline__ dfc dfc_renorm(dfc a) {
   const f2 h = f2_add(a.h, a.l);
   return {h, f2_sub(a.l, f2_sub(h, a.h))};
+}
+
+// a + b and its rounding error (TwoSum)
+__device__ __forceinline__ f2 f2_two_sum(f2 a, f2 b, f2& err) {
+  const f2 s = f2_add(a, b), bb = f2_sub(s, a);
+  err = f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb));
+  return s;
+}
+
+// acc + rest += x + xr, sums of three floats each: what the sums of the high and the low parts
+// round off goes into the third part, some 70 bits in all.  Adds up the lanes' double-float sums
+// where those of FP64 (2 a clock and SM) would cost more than the products.
+__device__ __forceinline__ void tfc_add(dfc& acc, f2& rest, f2 xh, f2 xl, f2 xr) {
+  f2 eh, el, em;
+  acc.h = f2_two_sum(acc.h, xh, eh);
+  acc.l = f2_two_sum(acc.l, xl, el);
+  acc.l = f2_two_sum(acc.l, eh, em);
+  rest = f2_add(f2_add(rest, xr), f2_add(el, em));
+}
+// the two values in FP64
+__device__ __forceinline__ double2 tfc_to(dfc a, f2 rest) {
+  float h0, h1, l0, l1, r0, r1;
+  f2_unpack(a.h, h0, h1);
+  f2_unpack(a.l, l0, l1);
+  f2_unpack(rest, r0, r1);
+  return make_double2((double)h0 + ((double)l0 + (double)r0), (double)h1 + ((double)l1 + (double)r1));
 }
 
 // Arguments of one stage launch.  With z = -i zre and x the gathered vector

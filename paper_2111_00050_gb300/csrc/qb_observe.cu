@@ -18,7 +18,8 @@
 // Every sum over kets is FP64: per-thread FP64 accumulators in kernels 1 and 3, and
 // where a term is a double-float product (n_i |psi|^2 in kernel 1, the gathered
 // moments in kernel 2) the products of 32 kets are summed in double-float and each
-// such partial is added to an FP64 accumulator.  CTA rows and the sum over CTAs are
+// such partial is added to an FP64 accumulator, or by raised kets (below) to a sum of
+// three floats over a warp and that to FP64.  CTA rows and the sum over CTAs are
 // FP64 in a fixed order (deterministic).
 #include <cuda_runtime.h>
 
@@ -726,11 +727,18 @@ __global__ void __launch_bounds__(32 * mw_warps(kMwSpl), QB_MW_MIN_BLOCKS) momen
 //   <a_i a_j>    = sum_m conj(v_j(m)) u_i(m),    v_j(m) = (a_j^+ psi)(m)
 // so that 14 gathers a ket (M = 7) make the 56 moments, which the entry-per-lane kernel above
 // gathers one by one, ranking each.  In the weighted basis u_i = w(m) sqrt(N + 1) 2^(e_N - e_N+1)
-// f(m + e_i) and v_j = w(m) m_j / sqrt(N) 2^(e_N - e_N-1) f(m - e_j).  The products are
-// double-float, summed over 32 rounds in each lane's registers, then over the warp (each lane
-// ends with one entry) and in FP64.  15.4M kets, M = 7: 4.4 ms in the kernel above, which its
-// scattered gathers and the products' latency limit.
+// f(m + e_i) and v_j = w(m) m_j / sqrt(N) 2^(e_N - e_N-1) f(m - e_j).  15.4M kets, M = 7: 4.4 ms in
+// the kernel above, which its scattered gathers and the products' latency limit.
+//
+// The products are double-float, summed over the 32 kets of 32 rounds in each lane's registers,
+// as the kernel above sums 32 kets; then over the lanes as sums of three floats (tfc_add, more
+// bits than FP64; each lane ends with one entry) and in FP64.  The weights enter with a third
+// part (dft_mul): they take few values, whose rounding to 48 bits erred alike in many kets.
+// Positive states of 11,440 kets, M = 7, relative to 64 bits: 7.7e-16 with double-float sums of
+// the lanes and weights of 48 bits, 2.0e-16 so, 4.1e-16 in the kernel above; qb_observables of
+// 15.4M kets 2.92 / 3.01 ms.
 constexpr int kMoRounds = 32;  // rounds a lane sums in double-float
+constexpr int kMoRenorm = 16;  // and after which its sums are renormalised
 template <int MT>
 __host__ __device__ constexpr int mo_threads() {  // registers: four an entry beside the gathered values
   return MT <= 5 ? 512 : MT <= 7 ? 384 : 256;
@@ -748,8 +756,8 @@ __device__ __forceinline__ void dfc_conj_fma(dfc& acc, dfl pr, dfl pi, float4 q)
 }
 
 // c x for a double-float factor and a double-float complex value
-__device__ __forceinline__ float4 df_scale(dfl c, float4 x) {
-  return df_pack(df_renorm(df_mul(c, df_re(x))), df_renorm(df_mul(c, df_im(x))));
+__device__ __forceinline__ float4 df_scale(dft c, float4 x) {
+  return df_pack(df_renorm(dft_mul(c, df_re(x))), df_renorm(dft_mul(c, df_im(x))));
 }
 
 template <int MT, bool AA>
@@ -778,26 +786,29 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
   auto flush = [&]() {
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
+      f2 rest[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) rest[k] = 0ull;
 #pragma unroll
       for (int s = 16; s >= 1; s >>= 1) {
         const bool up = (lane & s) != 0;
 #pragma unroll
         for (int k = 0; k < s; ++k) {
           if (32 * c + k >= NE) break;  // both halves empty
-          dfc& lo = acc[32 * c + k];
-          dfc& hi = acc[32 * c + k + s];
+          const dfc lo = acc[32 * c + k], hi = acc[32 * c + k + s];
           const f2 mh = up ? hi.h : lo.h, ml = up ? hi.l : lo.l, oh = up ? lo.h : hi.h, ol = up ? lo.l : hi.l;
+          const f2 rl = rest[k], rh = rest[k + s], orest = up ? rl : rh;
           dfc m{mh, ml};
-          const f2 rh = __shfl_xor_sync(0xffffffffu, oh, s), rl = __shfl_xor_sync(0xffffffffu, ol, s);
-          dfc_add(m, rh, rl);
-          lo = dfc_renorm(m);
+          f2 r = up ? rh : rl;
+          tfc_add(m, r, __shfl_xor_sync(0xffffffffu, oh, s), __shfl_xor_sync(0xffffffffu, ol, s),
+                  s < 16 ? __shfl_xor_sync(0xffffffffu, orest, s) : 0ull);
+          acc[32 * c + k] = m;
+          rest[k] = r;
         }
       }
-      float hr, hi2, lr, li;
-      f2_unpack(acc[32 * c].h, hr, hi2);
-      f2_unpack(acc[32 * c].l, lr, li);
-      sum_r[c] += (double)hr + (double)lr;
-      sum_i[c] += (double)hi2 + (double)li;
+      const double2 v = tfc_to(acc[32 * c], rest[0]);
+      sum_r[c] += v.x;
+      sum_i[c] += v.y;
     }
 #pragma unroll
     for (int e = 0; e < 32 * NC; ++e) acc[e] = dfc{0ull, 0ull};
@@ -814,9 +825,9 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
     int N = 0;
 #pragma unroll
     for (int k = 0; k < NW; ++k) N += (int)__dp4a(ob[k], 0x01010101u, 0u);
-    // (a factor of N rounded to 48 bits by itself would err alike in all kets of N)
+    // (the few values that the weights take, rounded to 48 bits, would err alike in many kets)
     const double wk = valid ? __ldg(t.wk + g) : 0.0;
-    const dfl wu = df_of(wk * sc[0][valid ? N : 0]);
+    const dft wu = dft_of(wk * sc[0][valid ? N : 0]);
     float4 u[MT];
 #pragma unroll
     for (int k = 0; k < W4; ++k) {
@@ -835,7 +846,7 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
     for (int i = 0; i < MT; ++i) u[i] = df_scale(wu, u[i]);
     int e = 0;
     if constexpr (!AA) {
-      const float4 x = df_scale(df_of(wk), valid ? __ldg(f + g) : make_float4(0.f, 0.f, 0.f, 0.f));
+      const float4 x = df_scale(dft_of(wk), valid ? __ldg(f + g) : make_float4(0.f, 0.f, 0.f, 0.f));
 #pragma unroll
       for (int i = 0; i < MT; ++i, ++e) dfc_conj_fma(acc[e], df_re(x), df_im(x), u[i]);
 #pragma unroll
@@ -843,7 +854,7 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
 #pragma unroll
         for (int j = i + 1; j < MT; ++j, ++e) dfc_conj_fma(acc[e], df_re(u[i]), df_im(u[i]), u[j]);
     } else {
-      const dfl wd = df_of(wk * sc[1][valid ? N : 0]);
+      const dft wd = dft_of(wk * sc[1][valid ? N : 0]);
 #pragma unroll
       for (int k = 0; k < W4; ++k) {
         const uint4 b = __ldg(reinterpret_cast<const uint4*>(base) + W4 + k);
@@ -863,13 +874,18 @@ __global__ void __launch_bounds__(mo_threads<MT>(), 1) raised_moments_kernel(con
         for (int c = 0; c < 4; ++c)
           if (4 * k + c < MT) {
             const int j = 4 * k + c;
-            const float4 vj = df_scale(df_mul_f(wd, nj[c]), v[c]);
+            const dfl wn = df_mul_f(dfl{wd.h, wd.l}, nj[c]);
+            const float4 vj = df_scale(dft{wn.h, wn.l, wd.r * nj[c]}, v[c]);
 #pragma unroll
             for (int i = 0; i <= j; ++i, ++e) dfc_conj_fma(acc[e], df_re(vj), df_im(vj), u[i]);  // entry j (j + 1) / 2 + i
           }
       }
     }
-    if (++held == kMoRounds) {
+    if (++held % kMoRenorm == 0) {
+#pragma unroll
+      for (int e = 0; e < NE; ++e) acc[e] = dfc_renorm(acc[e]);
+    }
+    if (held == kMoRounds) {
       flush();
       held = 0;
     }
