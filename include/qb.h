@@ -234,10 +234,13 @@ int qb_evolve_plain(qb_space* space, void* d_psi, double dt, int64_t steps, void
  * from the FP64 state; the moments that move a ket (<a_i>, <a_i^dag a_j>,
  * <a_i a_j>) as double-float products (about 48 significant bits) of the state and
  * its weighted double-float copy, summed in double-float over 32 kets at a time and
- * added in FP64 or in sums of three floats (some 70 bits); <H> from the weighted double-float H psi, each row's contribution
- * formed and summed in FP64, with every off-diagonal term of H taken once together
- * with its Hermitian reverse (half the terms of an H psi).  The space's weighted-copy buffer (16 B per ket) is
- * overwritten.  Relative errors are of order 1e-14. */
+ * added in FP64 or in sums of three floats (some 70 bits); <H> from the weighted
+ * copy, each row's conj(f) (H f) formed in double-float with every off-diagonal term of H
+ * taken once together with its Hermitian reverse (half the terms of an H psi), or, where a
+ * contact coupling is factored (qb_workspace_bytes), each lower ket's sum over the momentum
+ * classes of lam_k |B_k f|^2; either multiplied by the squared ket weight and summed in FP64.
+ * The space's weighted-copy buffer (16 B per ket) is overwritten.  Relative to the sum of
+ * the terms' magnitudes the moments and <H> are off by some 1e-15. */
 int qb_observables(qb_space* space, const void* d_psi, qb_obs* out, void* stream);
 
 /* Evolution with observation: series[0] is the initial state, series[k] the

@@ -14,7 +14,8 @@
 //     (a_i^dag a_j), n_i n_j or n_i (n_i - 1) (a_i a_j): the square roots of the
 //     ladder operators cancel against the ratio of ket weights.
 //  3. the double-float stage kernel in its <x|H|x> mode on f, each row's
-//     Re(conj(f_n) (W^-1 H W f)_n) multiplied by w_n^2 in FP64.
+//     Re(conj(f_n) (W^-1 H W f)_n) multiplied by w_n^2 in FP64; of a factored coupling
+//     its annihilation pass, each lower ket's sum_k lam_k |B_k f|^2 times the same.
 // Every sum over kets is FP64: per-thread FP64 accumulators in kernels 1 and 3, and
 // where a term is a double-float product (n_i |psi|^2 in kernel 1, the gathered
 // moments in kernel 2) the products of 32 kets are summed in double-float and each
