@@ -110,7 +110,8 @@ const char* qb_last_error(void);
  * (16 B), the occupation vector packed into 64 bits (8 B), the ket weight and its
  * inverse (8 B each) and the number of its last modes' filling (4 B), plus a
  * double-float copy of an observed state (16 B per ket; above 2^28 kets it is allocated
- * by the first qb_observables); and the ranking tables of the stages (a few bytes per ket).
+ * by the first qb_observables); and the ranking tables of the stages (a few bytes per ket up
+ * to 9 modes, at most some 250 with 16, at most 16 of 2^29 kets and more).
  * Limits: 1 <= M <= QB_MAX_MODES; M * bits(n_max) <= 64; n_max <= 250;
  * the largest ket weight sqrt(n_max! / prod_m n_m!) over occupations of n_max
  * particles at most 2^160 (the RK4 stages hold psi / w(n) as fp32 pairs, with the

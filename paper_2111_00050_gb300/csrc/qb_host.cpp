@@ -92,7 +92,29 @@ static int prepare_model(const qb_model* model, std::vector<double>& w, std::vec
 // read beside the gathers and should stay in L2.  One step of the M = 9, N = 27 long-range
 // space (23.5M kets) takes 22.8 ms with 6 MB, 21.5 with 24 and 21.8 with 80; of the M = 7,
 // n_tot = 16 contact space 24.3, 23.9 and 23.9.
+//
+// With many modes that leaves blocks of a few kets, each with a row of bases for hundreds of
+// terms (M = 16, n_max = 14, long-range: 2.4 KB a ket, 345 GB).  Where the rows would take more
+// than kBaseBytes a ket, or than kBaseRoom in all and 16 bytes a ket, the suffix grows on while
+// maps and rows together shrink (that space, 145M kets: 9 GB).  It costs no time: one step of
+// M = 16, 5.3M kets, 1,486 B a ket 25.2 ms, 274 B 25.3; M = 13, 1.1M kets, 702 B 4.15, 279 B 4.06;
+// M = 12, 2.7M kets, 368 B 7.12, 212 B 7.06.
 constexpr int64_t kMapBytes = 24ll << 20;
+constexpr int64_t kBaseBytes = 256, kBaseRoom = 8ll << 30;
+
+// Blocks of the fillings of modes m .. M-1 (m <= P): [P + 1][nmax + 1][Q]
+static std::vector<uint32_t> block_counts(const Space& sp, int P) {
+  const int V = sp.nmax + 1, Q = sp.Q;
+  auto CI = [&](int m, int n, int k) { return ((size_t)m * V + n) * Q + k; };
+  std::vector<uint32_t> c((size_t)(P + 1) * V * Q, 0);
+  for (int n = 0; n < V; ++n)
+    for (int k = 0; k < Q; ++k) c[CI(P, n, k)] = sp.cnt[CI(P, n, k)] > 0;
+  for (int m = P - 1; m >= 0; --m)
+    for (int n = 0; n < V; ++n)
+      for (int k = 0, j = modp(-m, Q); k < Q; ++k, j = j + 1 == Q ? 0 : j + 1)
+        c[CI(m, n, k)] = c[CI(m + 1, n, k)] + (n > 0 ? c[CI(m, n - 1, j)] : 0);
+  return c;
+}
 
 static void build_block_tables(Space& sp, bool factored) {
   Tables& t = sp.t;
@@ -121,19 +143,41 @@ static void build_block_tables(Space& sp, bool factored) {
   // map bytes per filling (factored: the pairs added, four a group, and taken away)
   const int64_t per_fill = factored ? 8 * ((M * (M + 1) / 2 + 3) / 4 + (sp.exact ? 2 * M : M) * ((M + 8) / 8))
                                     : (int64_t)std::max(1, nrec) * (t.bk_kc == 5 ? 10 : 2 * w);
-  int P = M - 1;
-  for (int q = M - 1; q >= 0; --q) {
-    int64_t S = 0, big = 0;
+  // fillings of the modes q .. M-1 with their gaps; -1: a class exceeds 16-bit places
+  auto fillings = [&](int q) {
+    int64_t S = 0;
     for (int n = 0; n <= nmax; ++n)
       for (int k = 0; k < Q; ++k) {
         const int64_t c = (int64_t)sp.cnt[CI(q, n, k)];
+        if (c > 65535) return (int64_t)-1;
         S += c + 1;
-        big = std::max(big, c);
       }
-    if (q < M - 1 && (big > 65535 || S * per_fill > kMapBytes)) break;
-    P = q;
-    t.bk_S = (int)S;
+    return S;
+  };
+  auto row_bytes = [&](int q) {  // bytes of the rows of bases
+    const std::vector<uint32_t> c = block_counts(sp, q);
+    int64_t rows = 0, low = 0;
+    for (size_t i = 0; i < sp.secN.size(); ++i) rows += c[CI(0, sp.secN[i], sp.secK[i])];
+    if (!factored) return 4ll * t.bk_T * rows;
+    for (size_t i = 0; i < sp.lowN.size(); ++i) low += c[CI(0, sp.lowN[i], sp.lowK[i])];
+    return 4ll * (fa_Tc(t) * rows + fa_rowa(t) * low);
+  };
+  int P = M - 1;
+  int64_t S = fillings(P);
+  while (P > 0) {
+    const int64_t s = fillings(P - 1);
+    if (s < 0 || s * per_fill > kMapBytes) break;
+    --P;
+    S = s;
   }
+  const int64_t total = sp.secOff.back(), room = std::min(kBaseBytes * total, std::max(kBaseRoom, 16 * total));
+  for (int64_t rows = row_bytes(P); P > 0 && rows > room; --P) {
+    const int64_t s = fillings(P - 1), next = row_bytes(P - 1);
+    if (s < 0 || s > 0x7fffffff || s * per_fill + next >= S * per_fill + rows) break;
+    S = s;
+    rows = next;
+  }
+  t.bk_S = (int)S;
   t.bk_P = P;
 
   std::vector<uint32_t> info(2 * (size_t)std::max(1, nrec));
@@ -190,19 +234,12 @@ static void build_block_tables(Space& sp, bool factored) {
   sp.bk_map_bytes = ((size_t)std::max(1, nrec) * t.bk_S * 2 * w + 255) & ~(size_t)255;
 }
 
-// Blocks (Tables::rblk) of the sectors and of the lower sectors: Space::blkCnt counts the
-// blocks of the fillings of modes m .. M-1 (m <= P), from which the device finds block b of
-// a sector as it finds a ket from the fill counts.
+// Blocks (Tables::rblk) of the sectors and of the lower sectors, from whose counts the device
+// finds block b of a sector as it finds a ket from the fill counts.
 static void count_blocks(Space& sp) {
-  const int P = sp.t.bk_P, V = sp.nmax + 1, Q = sp.Q;
+  const int V = sp.nmax + 1, Q = sp.Q;
   auto CI = [&](int m, int n, int k) { return ((size_t)m * V + n) * Q + k; };
-  sp.blkCnt.assign((size_t)(P + 1) * V * Q, 0);
-  for (int n = 0; n < V; ++n)
-    for (int k = 0; k < Q; ++k) sp.blkCnt[CI(P, n, k)] = sp.cnt[CI(P, n, k)] > 0;
-  for (int m = P - 1; m >= 0; --m)
-    for (int n = 0; n < V; ++n)
-      for (int k = 0, j = modp(-m, Q); k < Q; ++k, j = j + 1 == Q ? 0 : j + 1)
-        sp.blkCnt[CI(m, n, k)] = sp.blkCnt[CI(m + 1, n, k)] + (n > 0 ? sp.blkCnt[CI(m, n - 1, j)] : 0);
+  sp.blkCnt = block_counts(sp, sp.t.bk_P);
   auto run = [&](const std::vector<int>& N, const std::vector<int>& K, std::vector<uint32_t>& out) {
     out.assign(1, 0);
     for (size_t i = 0; i < N.size(); ++i) out.push_back(out.back() + sp.blkCnt[CI(0, N[i], K[i])]);

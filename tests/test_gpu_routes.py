@@ -24,6 +24,18 @@ def _space(M, hi, lo=0, kind="contact", **kw):
     return qb.Space(M, wl.dispersion_quadratic(M) * 0.3, L, lo, hi, **kw)
 
 
+def _rk4(qs, x, dt, steps):
+    """The Horner steps by FP64 H psi (qb_hpsi, compared with the oracle by itself)."""
+    out = qs.empty_state()
+    for _ in range(steps):
+        v = x
+        for d in (4, 3, 2, 1):
+            qs.hpsi(v, out)
+            v = x - (1j * dt / d) * out
+        x = v
+    return x
+
+
 @pytest.mark.parametrize("threads", [2, 4])
 def test_threads_evolve_states_of_one_space(threads):
     """A thread, a stream, a state and a workspace each on one space of the cooperative launch
@@ -214,3 +226,34 @@ def test_energy_of_factored_couplings_takes_the_weights_in_fp64(M, hi, kets):
         x, h = x.astype(np.longdouble), h.astype(np.longdouble)
         err.append(float((qs.observables(psi)["H"] * (x * x).sum() - (x * h).sum()) / np.abs(x * h).sum()))
     assert np.sqrt(np.mean(np.square(err))) <= 7e-16
+
+
+@pytest.mark.parametrize("M,hi,kets", [(16, 6, 74613), (14, 7, 116280)])
+def test_many_modes_against_the_oracle(M, hi, kets):
+    """Hundreds of terms a ket, and blocks of more modes than the maps' line asks for: H psi and
+    two steps."""
+    qs = _space(M, hi, kind="long")
+    assert qs.total == kets
+    os_ = orc.Space(M, qs.sectors)
+    w, L = wl.dispersion_quadratic(M) * 0.3, wl.long_range_coupling(M, 0.02)
+    x = random_state(qs.total, M)
+    y = qs.empty_state()
+    qs.hpsi(to_dev(x), y)
+    ref = orc.apply_h(os_, w, L, x)
+    assert rel_err(to_host(y), ref) <= 1e-13
+    psi = to_dev(x)
+    dt = 0.2 / max(1.0, np.linalg.norm(ref))
+    qs.evolve(psi, dt, 2)
+    assert rel_err(to_host(psi), to_host(_rk4(qs, to_dev(x), dt, 2))) <= 1e-11
+
+
+def test_tables_of_many_modes_stay_small():
+    """14 modes, 4.5M kets: with blocks of three kets, each with a row of 840 bases, the space took
+    5 GB.  60 bytes a ket, rows of at most 256 and half a gigabyte of maps and sums are 1.9."""
+    import torch
+
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    qs = _space(14, 11, kind="long")
+    assert qs.total == 4457400
+    assert free - torch.cuda.mem_get_info()[0] <= (60 + 256) * qs.total + (1 << 29)
