@@ -13,6 +13,7 @@ import pytest
 import oracle as orc
 import workloads as wl
 from helpers import random_state, rel_err, to_dev, to_host
+from test_gpu_blocks import CASES, _coupling
 
 pytestmark = pytest.mark.gpu
 
@@ -257,3 +258,96 @@ def test_tables_of_many_modes_stay_small():
     qs = _space(14, 11, kind="long")
     assert qs.total == 4457400
     assert free - torch.cuda.mem_get_info()[0] <= (60 + 256) * qs.total + (1 << 29)
+
+
+@pytest.mark.parametrize("name", CASES)
+def test_norm_particles_and_energy_of_every_route(name):
+    """Norm, <N> and <H> (direct rows, or factored couplings' lower kets) against the oracle: FP64
+    sums of products of 48 bits, 1e-12 of what they sum."""
+    import paper_2111_00050_gb300 as qb
+
+    M, lo, hi, momenta, kind, exact, _ = CASES[name]
+    w, L = wl.dispersion_quadratic(M) * 0.3, _coupling(kind, M, exact)
+    qs = qb.Space(M, w, L, lo, hi, momenta, exact=exact)
+    os_ = orc.Space(M, qs.sectors, exact=exact)
+    x = random_state(qs.total, 11) * 1.5
+    got, hx = qs.observables(to_dev(x)), orc.apply_h(os_, w, L, x)
+    norm, N = np.sum(np.abs(x) ** 2), os_.basis.sum(1)
+    assert abs(got["norm"] - norm) <= 1e-12 * norm
+    assert abs(got["N"] - np.sum(np.abs(x) ** 2 * N) / norm) <= 1e-12 * max(1, hi)
+    assert abs(got["H"] - np.vdot(x, hx).real / norm) <= 1e-12 * np.sum(np.abs(x * hx)) / norm
+
+
+# M, n_max, coupling, kets: more rounds of 32 kets than 16 warps an SM take at once, so that every
+# shape but the first two is a launch of its own, in the direct kernel of two and three partners
+# (unrolled) and of four, the generic one, and both passes of factored couplings
+SHAPES = [(5, 24, "contact", 118755), (7, 14, "long", 116280), (9, 10, "long", 92378), (4, 40, "contact", 135751),
+          (7, 14, "contact", 116280), (8, 12, "contact", 125970)]
+
+
+@pytest.mark.parametrize("M,hi,kind,kets", SHAPES)
+def test_tile_shapes_of_stage_launches_are_bit_identical(M, hi, kind, kets):
+    """70 steps (a graph of 32 replayed once, and single launches) under every shape, and one launch
+    a sector."""
+    import paper_2111_00050_gb300 as qb
+
+    qs = _space(M, hi, kind=kind)
+    assert qs.total == kets
+    x = to_dev(random_state(qs.total, 4))
+    want = x.clone()
+    qs.evolve(want, 1e-4, 70)
+    for shape in range(1, qb._lib.QB_TILE_SHAPES):
+        qs.set_tile_shape(shape)
+        y = x.clone()
+        qs.evolve(y, 1e-4, 70)
+        assert bool((y == want).all()), shape
+    qs.set_tile_shape(0)
+    qs.evolve_plain(x, 1e-4, 70)
+    assert bool((x == want).all())
+
+
+@pytest.mark.parametrize("B", [2, 4, 8])
+@pytest.mark.parametrize("M,lo,hi", [(7, 0, 12), (11, 7, 7)])
+def test_sweeps_of_factored_couplings(M, lo, hi, B):
+    """The members of a sweep take their passes in turn through one vector: each against the oracle
+    under its own coupling (the bound of three steps in test_gpu_blocks.py), and 70 steps against
+    a space of that coupling alone (a coupling scaled in the kernel or in the tables: 1e-11)."""
+    import torch
+
+    import paper_2111_00050_gb300 as qb
+
+    w, L = wl.dispersion_quadratic(M) * 0.3, wl.contact_coupling(M, -0.02)
+    qs = qb.Space(M, w, L, lo, hi)
+    os_ = orc.Space(M, qs.sectors)
+    scale = [0.25 * (b + 1) * (-1) ** b for b in range(B)]
+    x = [random_state(qs.total, 20 + b) for b in range(B)]
+    dt = 0.2 / max(1.0, np.linalg.norm(orc.apply_h(os_, w, 2 * L, x[0])))
+    psi = torch.stack([to_dev(v) for v in x])
+    qs.evolve_batch(psi, scale, dt, 3)
+    for b in (0, B - 1):
+        assert rel_err(to_host(psi[b]), orc.rk4(os_, w, scale[b] * L, x[b], dt, 3)) <= 1e-11, b
+    psi = torch.stack([to_dev(v) for v in x])
+    qs.evolve_batch(psi, scale, dt, 70)
+    for b in range(B):
+        alone = to_dev(x[b])
+        qb.Space(M, w, scale[b] * L, lo, hi).evolve(alone, dt, 70)
+        assert rel_err(to_host(psi[b]), to_host(alone)) <= 1e-11, b
+
+
+@pytest.mark.parametrize("M,lo,hi,exact", [(7, 0, 12, False), (7, 14, 14, False), (9, 0, 8, False), (11, 7, 7, False),
+                                           (7, 0, 12, True)])
+def test_factored_steps_by_graph(M, lo, hi, exact):
+    """70 steps of factored couplings (a replayed graph) and the same by one launch a sector, bit for
+    bit, and by FP64 H psi: 280 stages, each off by some 2^-44 of its increment, 1e-11."""
+    import paper_2111_00050_gb300 as qb
+
+    w, L = wl.dispersion_quadratic(M) * 0.3, wl.contact_coupling(M, -0.02, exact=exact)
+    qs = qb.Space(M, w, L, lo, hi, exact=exact)
+    x, out = to_dev(random_state(qs.total, 6)), qs.empty_state()
+    qs.hpsi(x, out)
+    dt = 0.2 / max(1.0, float(out.norm()))
+    a, b = x.clone(), x.clone()
+    qs.evolve(a, dt, 70)
+    qs.evolve_plain(b, dt, 70)
+    assert bool((a == b).all())
+    assert rel_err(to_host(a), to_host(_rk4(qs, x, dt, 70))) <= 1e-11
