@@ -558,6 +558,165 @@ __global__ void __launch_bounds__((U > 1 ? 256 : blk_max_threads<B, KIND>()), 1)
   if constexpr (BIL) bil_reduce<kMB>(a, M, bil_l, bil_w);
 }
 
+// The records that a ket takes part in, one after the other: the pairs (r, s) of its occupied
+// modes in order, each with its records.
+struct RecordWalk {
+  uint32_t occ, two, rm, sm;  // modes with a particle, with two; modes r and s still to come
+  int r, rec;
+  __device__ __forceinline__ RecordWalk(const Tables& t, uint64_t word) : occ(0u), two(0u), sm(0u), r(0), rec(-1) {
+    for (int m = 0; m < t.M; ++m) {
+      const int n = occ_of(word, m, t.occ_bits);
+      occ |= (n > 0 ? 1u : 0u) << m;
+      two |= (n > 1 ? 1u : 0u) << m;
+    }
+    rm = occ;
+  }
+  // the next record in rec; false when there is none (first: first record of each pair)
+  __device__ __forceinline__ bool next(const uint2* sinfo, const uint16_t* first) {
+    if (rec >= 0 && (sinfo[rec].x & 0x80u) == 0u) {
+      ++rec;
+      return true;
+    }
+    while ((rm | sm) != 0u) {
+      if (sm == 0u) {
+        r = __ffs(rm) - 1;
+        rm &= rm - 1;
+        sm = occ & (~0u << r);
+        if (((two >> r) & 1u) == 0u) sm &= ~(1u << r);
+        continue;
+      }
+      const int s = __ffs(sm) - 1;
+      sm &= sm - 1;
+      const uint32_t f = first[r * 16 + s];
+      if (f != 0xffffu) {
+        rec = (int)f;
+        return true;
+      }
+    }
+    return false;
+  }
+};
+// first[r * 16 + s]: the first record of the pair, or 0xffff (a CTA's threads together, between
+// two barriers)
+constexpr size_t kFirstBytes = 512;
+__device__ __forceinline__ void first_records(const uint2* sinfo, int nrec, uint16_t* first) {
+  for (int i = threadIdx.x; i < 256; i += blockDim.x) first[i] = 0xffffu;
+  __syncthreads();
+  for (int i = threadIdx.x; i < nrec; i += blockDim.x) {
+    const uint32_t x = sinfo[i].x;
+    if (i == 0 || (sinfo[i - 1].x & 0x80u) != 0u)
+      first[((x & 7) | ((x >> 12) & 8)) * 16 + (((x >> 16) & 7) | ((x >> 28) & 8))] = (uint16_t)i;
+  }
+  __syncthreads();
+}
+
+// The same stage with each lane on the records of its own ket instead of all lanes on every
+// record in step: scattered reads of maps, bases and couplings, but no work for pairs that a ket
+// lacks, which with many modes and few particles are nearly all.  A pair that a ket lacks adds
+// zero in the kernel above, so that the states agree bit for bit.  The lanes stay together in the
+// products where a sweep's members share a record whose partners vary (IN_STEP): with four
+// members, M = 10, 184,756 kets, a stage 292 us apart, 280 in step; with two 172 and 189.
+template <int KC, int B, bool CPLX, int KIND>
+__global__ void __launch_bounds__((blk_max_threads<B, KIND>()), 1)
+    sparse_stage_kernel(const Tables t, const DfArgs a, const int mode) {
+  constexpr int NT = Rec<KC>::n, RW = Rec<KC>::w, NW = occ_words<0>();
+  constexpr bool BIL = (KIND == KIND_BIL), IN_STEP = KC == 0 && B >= 4;
+  const int T = t.bk_T, nrec = t.bk_nrec;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  float2* sG = reinterpret_cast<float2*>(blk_smem);
+  float2* sGi = sG + T;
+  uint2* sinfo = reinterpret_cast<uint2*>(sG + (CPLX ? 2 : 1) * T);
+  uint16_t* first = reinterpret_cast<uint16_t*>(blk_smem + blk_smem_bytes(t, CPLX));
+  for (int i = threadIdx.x; i < T; i += blockDim.x) {
+    sG[i] = __ldg(t.bk_G + i);
+    if (CPLX) sGi[i] = __ldg(t.bk_Gi + i);
+  }
+  for (int i = threadIdx.x; i < nrec; i += blockDim.x) sinfo[i] = __ldg(t.bk_info + i);
+  __syncthreads();
+  first_records(sinfo, nrec, first);
+
+  const int64_t total = t.total;
+  dfl bil_l{0.f, 0.f};
+  dfc bil_w[BIL ? 8 : 1];
+#pragma unroll
+  for (int q = 0; q < (BIL ? 8 : 1); ++q) bil_w[q] = dfc{0ull, 0ull};
+  double dot64 = 0.0;
+  const int64_t r0 = a.row0 / 32, step = (int64_t)gridDim.x * warps;
+  int64_t rd = (a.row1 - 1) / 32 - ((int64_t)blockIdx.x * warps + warp);
+  RoundIn in_next = load_round(t.occ, t.fill, t.rblk, max(rd, r0), total, lane);
+  chain_wait();
+  for (; rd >= r0; rd -= step) {
+    const int64_t g = rd * 32 + lane;
+    const bool valid = g >= a.row0 && g < a.row1;
+    const RoundIn in = in_next;
+    in_next = load_round(t.occ, t.fill, t.rblk, max(rd - step, r0), total, lane);
+    const uint32_t* base = t.bk_base + (size_t)block_of_lane(in, lane, g < total) * T;
+    uint32_t ob[NW];
+    unpack_occ<0, NW>(t, valid ? in.word : 0ull, ob);
+    const unsigned char* mp = t.bk_map + (size_t)in.fill * (2 * RW);
+    const uint16_t* mp5 = t.bk_map5 + in.fill;
+    dfc acc[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) acc[b] = dfc{0ull, 0ull};
+    bool bad = false;
+    RecordWalk walk(t, valid ? in.word : 0ull);
+    MapRec<KC> m{};
+    BaseRec<KC> bs{};
+    bool act = walk.next(sinfo, first);
+    auto load = [&]() {
+      if (act) {
+        m = load_map<KC>(mp + (size_t)walk.rec * t.bk_S * (2 * RW), mp5 + (size_t)walk.rec * t.bk_S);
+        bs = load_base<KC>(base, walk.rec, nrec);
+      }
+    };
+    load();
+    while (__any_sync(0xffffffffu, act)) {
+      const bool on = act;
+      const int rec = walk.rec;
+      uint32_t rk[NT];
+      rk[0] = bs.a.x + (m.a.x & 0xffffu);
+      rk[1] = bs.a.y + (m.a.x >> 16);
+      if constexpr (NT > 2) rk[2] = bs.a.z + (m.a.y & 0xffffu);
+      if constexpr (NT > 3) rk[3] = bs.a.w + (m.a.y >> 16);
+      if constexpr (NT > 4) rk[4] = bs.b + m.b;
+      if (on) act = walk.next(sinfo, first);
+      load();
+      if (!IN_STEP && !on) continue;
+      const int ri = on ? rec : 0;
+      const uint2 info = sinfo[ri];
+      const float Af = (occ_float23<NW>(ob, info.x, (info.x & 0x8000u) != 0u) - 8388608.0f) *
+                       (occ_float23<NW>(ob, info.x >> 16, (info.x & 0x80000000u) != 0u) - __uint_as_float(info.y));
+      const int n = !on ? 0 : KC == 0 ? (int)((info.x >> 4) & 7) : NT;
+      uint32_t top = rk[0];
+#pragma unroll
+      for (int c = 1; c < NT; ++c)
+        if (KC > 0 || c < n) top = max(top, rk[c]);
+      const bool ok = on && top < (uint32_t)total;
+      bad |= on && !ok;
+      if (!IN_STEP && !ok) continue;
+      const int terms = IN_STEP ? __reduce_max_sync(0xffffffffu, n) : n;  // beyond n: zeros
+      const bool done = on && (KC > 0 || (info.x & 0x80u) != 0u);
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        float4 x[NT];
+#pragma unroll
+        for (int c = 0; c < NT; ++c)
+          x[c] = (!IN_STEP || ok) && (KC > 0 || c < n) ? a.vin[(size_t)b * total + rk[c]] : make_float4(0.f, 0.f, 0.f, 0.f);
+        add_record<KC, CPLX, false>(acc[b], x, sG, sGi, ri, nrec, terms, 0, IN_STEP && !on ? 0.f : Af);
+        if (IN_STEP) {
+          const dfc sum = dfc_renorm(acc[b]);
+          if (done) acc[b] = sum;
+        } else if (done) {
+          acc[b] = dfc_renorm(acc[b]);
+        }
+      }
+    }
+    if (bad) atomicOr(a.status, 1);
+    if (valid) stage_epilogue<0, B, KIND, false, NW>(t, a, mode, g, g, acc, ob, bil_l, bil_w, dot64);
+  }
+  if constexpr (BIL) bil_reduce<16>(a, t.M, bil_l, bil_w);
+}
+
 // Tile shapes: warps per CTA (a warp takes 32 kets at a time)
 constexpr int kTileShapes = 5;
 __host__ __device__ constexpr int tile_warps(int ts) { return ts == 1 ? 16 : ts == 2 ? 24 : ts == 3 ? 12 : ts == 4 ? 8 : 32; }
@@ -600,8 +759,40 @@ int blk_launch_u(const Tables& t, const DfArgs& a, int mode, int shape, cudaStre
   return QB_OK;
 }
 
+template <int KC, int B, bool CPLX, int KIND>
+int sparse_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream_t st, int* grid_out) {
+  auto k = sparse_stage_kernel<KC, B, CPLX, KIND>;
+  const size_t smem = blk_smem_bytes(t, CPLX) + kFirstBytes;
+  int warps = 0, grid = 0;
+  const int rc = stage_geometry(k, a.row1 - a.row0, shape, blk_max_threads<B, KIND>() / 32, smem, &warps, &grid);
+  if (rc) return rc;
+  QB_CUDA(chain_launch(k, grid, 32 * warps, smem, st, t, a, mode));
+  if (grid_out) *grid_out = grid;
+  return QB_OK;
+}
+// Share of a space's records that a ket takes part in on average (Tables::bk_share), up to which
+// each lane walks its own ket's.  One stage, all records in step / own records (us): one state, M =
+// 12, 18,564 kets (share 0.10) 53 / 21; M = 10, 19,448 kets (0.15) 32 / 29; M = 8, 6,435 (0.2) 15 /
+// 19; M = 9, 5,005 (0.14) 11 / 13; M = 11, 167,960 (0.19) 125 / 71, 16,796 of one momentum (0.24)
+// 18 / 45.  Two members, M = 9, 92,378 (0.26) 66 / 53, M = 7, 19,448 (0.33) 18 / 24; four, M = 10, 184,756
+// (0.24) 355 / 280, M = 7, 245,157 (0.47) 127 / 128; eight, M = 5, 1.2M kets (0.79) 521 / 459.  Partners
+// that vary, eight members: M = 6, 5,005 kets (0.34) 56 / 66.  With bilinears (a gradient of
+// three steps), M = 12, 18,564 kets 3.1 / 2.0 ms, M = 11, 31,824 (0.14) 1.8 / 2.2.
+template <int KC, int B, int KIND>
+constexpr float sparse_share() {
+  if (KIND == KIND_BIL) return KC == 0 ? 0.16f : KC >= 4 ? 0.1f : 0.f;
+  if (B == 1) return KC == 0 ? 0.16f : KC == 4 ? 0.12f : KC == 5 ? 0.2f : 0.f;
+  if (B == 2) return KC == 0 ? 0.25f : KC >= 4 ? 0.37f : 0.18f;
+  if (KC == 0) return 0.3f;
+  return B == 4 ? 0.45f : 2.f;  // eight: always
+}
+
 template <int MT, bool FIX, int B, bool CPLX, int KIND>
 int blk_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream_t st, int* grid_out) {
+  constexpr int KC = FIX ? (MT - 1) / 2 : 0;
+  if constexpr (KIND != KIND_DOT && sparse_share<KC, B, KIND>() > 0.f)
+    if (t.bk_share < sparse_share<KC, B, KIND>())
+      return sparse_launch<KC, B, CPLX, KIND>(t, a, mode, shape, st, grid_out);
   if constexpr (FIX && B == 1 && KIND == KIND_STAGE) {
     int dev = 0, sms = 0;
     QB_CUDA(cudaGetDevice(&dev));
@@ -629,7 +820,21 @@ int blk_launch_kind(const Tables& t, const DfArgs& a, int mode, int B, bool bil,
     case 1: return blk_launch<MT, FIX, 1, false, KIND_STAGE>(t, a, mode, shape, st, grid);
     case 2: return blk_launch<MT, FIX, 2, false, KIND_STAGE>(t, a, mode, shape, st, grid);
     case 4: return blk_launch<MT, FIX, 4, false, KIND_STAGE>(t, a, mode, shape, st, grid);
-    case 8: return blk_launch<MT, FIX, 8, false, KIND_STAGE>(t, a, mode, shape, st, grid);
+    case 8:
+      if constexpr (!FIX)
+        if (t.bk_share < sparse_share<0, 8, KIND_STAGE>()) {  // as two groups of four (eight at once
+          DfArgs h = a;                                       // M = 10, 184,756 kets: 626 us, so 559)
+          const int rc = blk_launch<MT, FIX, 4, false, KIND_STAGE>(t, h, mode, shape, st, grid);
+          if (rc) return rc;
+          const size_t n = 4 * (size_t)t.total;
+          h.vin += n;
+          h.out += n;
+          if (h.psi) h.psi += n;
+          if (h.psif) h.psif += n;
+          for (int b = 0; b < 4; ++b) h.scale[b] = a.scale[b + 4];
+          return blk_launch<MT, FIX, 4, false, KIND_STAGE>(t, h, mode, shape, st, grid);
+        }
+      return blk_launch<MT, FIX, 8, false, KIND_STAGE>(t, a, mode, shape, st, grid);
     default: return fail(QB_EINVAL, "batch must be 1, 2, 4 or 8");
   }
 }

@@ -179,6 +179,21 @@ static void build_block_tables(Space& sp, bool factored) {
   }
   t.bk_S = (int)S;
   t.bk_P = P;
+  // A ket takes part in the records of a pair (r, s) if it is a ket of two particles fewer with
+  // them added.
+  {
+    std::vector<int> of(annR.size(), 0);
+    int most = 0;
+    for (const Record& R : recs) most = std::max(most, ++of[R.pair]);
+    double taken = 0.0;
+    for (size_t i = 0; i < sp.secN.size(); ++i)
+      for (size_t a = 0; a < annR.size() && sp.secN[i] >= 2; ++a)
+        taken += (double)of[a] * (double)sp.cnt[CI(0, sp.secN[i] - 2, modp((long long)sp.secK[i] - annR[a] - annS[a], Q))];
+    t.bk_share = nrec > 0 ? (float)(taken / ((double)nrec * (double)sp.secOff.back())) : 1.f;
+    // (p modes occupied, of which nmax / 2 twice at most)
+    const int64_t p = std::min(M, nmax);
+    t.bk_most = (int)std::min<int64_t>(nrec, most * (p * (p - 1) / 2 + std::min(M, nmax / 2)));
+  }
 
   std::vector<uint32_t> info(2 * (size_t)std::max(1, nrec));
   std::vector<float> Gr(2 * (size_t)t.bk_T, 0.f), Gi(2 * (size_t)t.bk_T, 0.f);

@@ -98,6 +98,8 @@ struct Tables {
                             //   left out after each class
   const uint32_t* fill;     // [total] number of the filling of every ket
   int bk_nrec;              // records
+  float bk_share;           // share of the records that a ket takes part in, on average
+  int bk_most;              // records that a ket takes part in, at most
   int bk_T;                 // term slots (a multiple of 4): record i holds [w i, w i + w), w = 2 for
                             //   bk_kc = 2, else 4; a fifth partner sits at 4 n_rec + i
   const uint32_t* rblk;     // [ceil(total / 32)] block of every 32nd ket

@@ -29,19 +29,29 @@ struct ResArgs {
   int* status;
 };
 
-// bytes of one ket's target indices: w 16-bit entries a record, and the fifth partner's
+// Whether the resident kernel keeps each ket's own records alone (SPARSE): where a ket takes part
+// in few of them (Tables::bk_share).  One stage, every record / own records (us): M = 16, 969 kets
+// (share 0.02) 63 / 2.9; M = 9, 220 kets (0.05; the register kernel) 7.7 / 1.8; M = 8, 495 (0.09) 12.5
+// / 3.2; M = 6, 210 (0.13) 7.0 / 3.1, 1,287 (0.36) 9.4 / 9.0; M = 4, 495 (0.42) 3.5 / 3.8.
+inline bool resident_sparse(const Tables& t) { return t.bk_share < 0.3f && t.bk_kc != 2 && t.bk_kc != 3; }
+
+// bytes of one ket's target indices: w 16-bit entries a record, and the fifth partner's; of its
+// own records alone, their numbers and how many there are
 inline size_t resident_index_bytes(const Tables& t) {
-  return (size_t)t.bk_nrec * (t.bk_kc == 2 ? 4 : t.bk_kc == 5 ? 10 : 8);
+  const size_t rec = t.bk_kc == 2 ? 4 : t.bk_kc == 5 ? 10 : 8;
+  return resident_sparse(t) ? t.bk_most * (rec + 2) + 2 : t.bk_nrec * rec;
 }
 
 // Shared memory of the resident kernel holding `cap` kets per sector.
 inline size_t resident_smem(const Tables& t, int cap) {
-  return blk_smem_bytes(t, t.is_complex != 0) + (size_t)cap * (64 + resident_index_bytes(t));
+  return blk_smem_bytes(t, t.is_complex != 0) + (size_t)cap * (64 + resident_index_bytes(t)) +
+         (resident_sparse(t) ? kFirstBytes : 0);
 }
 
-template <int MT, bool FIX, bool CPLX>
+// SPARSE: a ket's targets are kept for the records that it takes part in, with their numbers, and
+// the lanes walk each its own; else for every record, which the lanes walk in step.
+template <int MT, int KC, bool CPLX, bool SPARSE>
 __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const ResArgs r) {
-  constexpr int KC = FIX ? (MT - 1) / 2 : 0;
   constexpr int NT = Rec<KC>::n, RW = Rec<KC>::w, NW = occ_words<MT>();
   const int T = t.bk_T, nrec = t.bk_nrec, cap = r.cap;
   float2* sG = reinterpret_cast<float2*>(blk_smem);
@@ -51,8 +61,12 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
   float4* spsif = reinterpret_cast<float4*>(spsi + cap);
   float4* sw1 = spsif + cap;
   float4* sw2 = sw1 + cap;
-  uint16_t* sidx = reinterpret_cast<uint16_t*>(sw2 + cap);      // [nrec][cap][RW]
-  uint16_t* sidx5 = sidx + (size_t)nrec * cap * RW;             // [nrec][cap]
+  const int rows = SPARSE ? t.bk_most : nrec;
+  uint16_t* sidx = reinterpret_cast<uint16_t*>(sw2 + cap);      // [rows][cap][RW]
+  uint16_t* sidx5 = sidx + (size_t)rows * cap * RW;             // [rows][cap]
+  uint16_t* srec = sidx5 + (NT > 4 ? (size_t)rows * cap : 0);   // [rows][cap] numbers of the records
+  uint16_t* scnt = srec + (size_t)rows * cap;                   // [cap]
+  uint16_t* first = scnt + cap;                                 // [256]
   const int tid = threadIdx.x, nthr = blockDim.x;
   for (int i = tid; i < T; i += nthr) {
     sG[i] = __ldg(t.bk_G + i);
@@ -60,6 +74,7 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
   }
   for (int i = tid; i < nrec; i += nthr) sinfo[i] = __ldg(t.bk_info + i);
   __syncthreads();
+  if (SPARSE) first_records(sinfo, nrec, first);
   const int64_t off = __ldg(t.sec_off + blockIdx.x);
   const int D = (int)(__ldg(t.sec_off + blockIdx.x + 1) - off);
   if (D > cap) {  // not reached: the host sizes the buffers for the largest sector
@@ -73,8 +88,9 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
     const int64_t g = off + i;
     spsi[i] = r.psi[g];
     spsif[i] = r.psif[g];  // the weighted double-float copy
+    const uint64_t word = __ldg(t.occ + g);
     uint32_t ob[NW];
-    unpack_occ<MT, NW>(t, __ldg(t.occ + g), ob);
+    unpack_occ<MT, NW>(t, word, ob);
     uint32_t blk = __ldg(t.rblk + g / 32), f = __ldg(t.fill + g / 32 * 32);
     for (int64_t k = g / 32 * 32 + 1; k <= g; ++k) {  // blocks begun since the round's first ket
       const uint32_t fk = __ldg(t.fill + k);
@@ -82,7 +98,16 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
       f = fk;
     }
     const uint32_t* base = t.bk_base + (size_t)blk * T;
-    for (int rec = 0; rec < nrec; ++rec) {
+    RecordWalk walk(t, SPARSE ? word : 0ull);
+    int row = 0;
+    for (;; ++row) {
+      if (SPARSE ? !walk.next(sinfo, first) : row == nrec) break;
+      if (SPARSE && row == rows) {  // not reached: bk_most bounds them
+        bad = true;
+        break;
+      }
+      const int rec = SPARSE ? walk.rec : row;
+      if (SPARSE) srec[(size_t)row * cap + i] = (uint16_t)rec;
       const uint2 info = sinfo[rec];
       const float Af = (occ_float23<NW>(ob, info.x, (info.x & 0x8000u) != 0u) - 8388608.0f) *
                        (occ_float23<NW>(ob, info.x >> 16, (info.x & 0x80000000u) != 0u) - __uint_as_float(info.y));
@@ -101,11 +126,12 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
           }
         }
         if (c < 4)
-          sidx[((size_t)rec * cap + i) * RW + c] = (uint16_t)k;
+          sidx[((size_t)row * cap + i) * RW + c] = (uint16_t)k;
         else
-          sidx5[(size_t)rec * cap + i] = (uint16_t)k;
+          sidx5[(size_t)row * cap + i] = (uint16_t)k;
       }
     }
+    if (SPARSE) scnt[i] = (uint16_t)row;
   }
   if (bad) atomicOr(r.status, 1);
   __syncthreads();
@@ -138,18 +164,20 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
         for (int c = 0; c < NT; ++c) x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         const uint16_t* ip = sidx + (size_t)ii * RW;
         const uint16_t* ip5 = sidx5 + ii;
-        for (int rec = 0; rec < nrec; ++rec) {
+        const int cnt = !SPARSE ? nrec : valid ? (int)scnt[ii] : 0;
+        for (int row = 0; SPARSE ? __any_sync(0xffffffffu, row < cnt) : row < nrec; ++row) {
+          const int rec = !SPARSE ? row : row < cnt ? (int)srec[(size_t)row * cap + ii] : 0;
           const uint2 info = sinfo[rec];
           const float Af = (occ_float23<NW>(ob, info.x, (info.x & 0x8000u) != 0u) - 8388608.0f) *
                            (occ_float23<NW>(ob, info.x >> 16, (info.x & 0x80000000u) != 0u) - __uint_as_float(info.y));
-          const bool act = Af != 0.f;
-          if (__any_sync(0xffffffffu, act)) {
+          const bool act = SPARSE ? row < cnt : Af != 0.f;
+          if (SPARSE ? act : (bool)__any_sync(0xffffffffu, act)) {
             const int n = KC == 0 ? (int)((info.x >> 4) & 7) : NT;
             uint2 k2 = make_uint2(0u, 0u);
             if constexpr (RW == 2)
-              k2.x = *reinterpret_cast<const uint32_t*>(ip + (size_t)rec * cap * RW);
+              k2.x = *reinterpret_cast<const uint32_t*>(ip + (size_t)row * cap * RW);
             else
-              k2 = *reinterpret_cast<const uint2*>(ip + (size_t)rec * cap * RW);
+              k2 = *reinterpret_cast<const uint2*>(ip + (size_t)row * cap * RW);
             if (act) {  // a lane that lacks the pair keeps its last values
               x[0] = vin[k2.x & 0xffffu];
               if (KC > 0 || n > 1) x[1] = vin[k2.x >> 16];
@@ -157,7 +185,7 @@ __global__ void __launch_bounds__(1024, 1) resident_kernel(const Tables t, const
                 if (KC > 0 || n > 2) x[2] = vin[k2.y & 0xffffu];
               if constexpr (NT > 3)
                 if (KC > 0 || n > 3) x[3] = vin[k2.y >> 16];
-              if constexpr (NT > 4) x[4] = vin[ip5[(size_t)rec * cap]];
+              if constexpr (NT > 4) x[4] = vin[ip5[(size_t)row * cap]];
             }
             add_record<KC, CPLX, false>(acc[0], x, sG, sGi, rec, nrec, n, 0, Af);
             if (KC > 0 || (info.x & 0x80u)) acc[0] = dfc_renorm(acc[0]);
@@ -364,9 +392,9 @@ inline bool grid_reg_fits(const Tables& t, int sms) {
          t.total <= std::min<int64_t>(65536, (int64_t)sms * reg_kets(t.M));
 }
 
-template <int MT, bool FIX, bool CPLX>
+template <int MT, int KC, bool CPLX, bool SPARSE>
 int resident_launch_k(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {
-  auto k = resident_kernel<MT, FIX, CPLX>;
+  auto k = resident_kernel<MT, KC, CPLX, SPARSE>;
   const size_t smem = resident_smem(t, r.cap);
   int per = 0, sms = 0;
   const int rc = occupancy_cached(k, smem, &per, &sms, threads);  // raises the function's shared-memory limit

@@ -28,7 +28,10 @@ int stage_launch_any(const Tables& t, const DfArgs& a, int mode, int B, bool cpl
   return stage_of<true>(t, a, mode, shape, st, grid);
 }
 int resident_launch_any(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {
-  return t.is_complex ? resident_launch_k<0, false, true>(t, r, threads, st)
-                      : resident_launch_k<0, false, false>(t, r, threads, st);
+  if (resident_sparse(t))
+    return t.is_complex ? resident_launch_k<0, 0, true, true>(t, r, threads, st)
+                        : resident_launch_k<0, 0, false, true>(t, r, threads, st);
+  return t.is_complex ? resident_launch_k<0, 0, true, false>(t, r, threads, st)
+                      : resident_launch_k<0, 0, false, false>(t, r, threads, st);
 }
 }  // namespace qb

@@ -6,8 +6,7 @@ int stage_launch_m5(const Tables& t, const DfArgs& a, int mode, int B, bool bil,
   return blk_launch_kind<5, true>(t, a, mode, B, bil, shape, st, grid);
 }
 int resident_launch_m5(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {
-  if (threads <= reg_kets(5)) return resident_reg_launch<5>(t, r, threads, st);
-  return resident_launch_k<5, true, false>(t, r, threads, st);
+  return resident_reg_launch<5>(t, r, threads, st);
 }
 int grid_launch_m5(const Tables& t, const ResArgs& r, cudaStream_t st) { return grid_reg_launch<5>(t, r, st); }
 }  // namespace qb

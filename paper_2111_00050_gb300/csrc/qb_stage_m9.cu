@@ -6,7 +6,7 @@ int stage_launch_m9(const Tables& t, const DfArgs& a, int mode, int B, bool bil,
   return blk_launch_kind<9, true>(t, a, mode, B, bil, shape, st, grid);
 }
 int resident_launch_m9(const Tables& t, const ResArgs& r, int threads, cudaStream_t st) {
-  if (threads <= reg_kets(9)) return resident_reg_launch<9>(t, r, threads, st);
-  return resident_launch_k<9, true, false>(t, r, threads, st);
+  return resident_sparse(t) ? resident_launch_k<0, 4, false, true>(t, r, threads, st)
+                            : resident_reg_launch<9>(t, r, threads, st);
 }
 }  // namespace qb

@@ -351,3 +351,57 @@ def test_factored_steps_by_graph(M, lo, hi, exact):
     qs.evolve_plain(b, dt, 70)
     assert bool((a == b).all())
     assert rel_err(to_host(a), to_host(_rk4(qs, x, dt, 70))) <= 1e-11
+
+
+# M, n_max, coupling, exact: few particles in many modes, where each lane walks its own ket's
+# records, resident (the first row) and stage by stage, and next to the lines between the two
+FEW = [(16, 3, "long", False), (12, 3, "hermitian", False), (11, 3, "contact", False), (9, 3, "long", False),
+       (8, 4, "contact", True), (6, 4, "long", False),
+       (14, 5, "long", False), (12, 5, "hermitian", False), (11, 5, "long", False), (10, 5, "long", True), (9, 5, "long", False)]
+
+
+@pytest.mark.parametrize("M,hi,kind,exact", FEW)
+def test_few_particles_in_many_modes(M, hi, kind, exact):
+    """H psi and three steps against the oracle (the bounds of test_gpu_blocks.py); 33 and 70 steps in
+    one launch, stage by stage and sector by sector, bit for bit."""
+    import paper_2111_00050_gb300 as qb
+
+    w, L = wl.dispersion_quadratic(M) * 0.3, _coupling(kind, M, exact)
+    qs = qb.Space(M, w, L, 0, hi, exact=exact)
+    os_ = orc.Space(M, qs.sectors, exact=exact)
+    x = random_state(qs.total, M)
+    y = qs.empty_state()
+    qs.hpsi(to_dev(x), y)
+    ref = orc.apply_h(os_, w, L, x)
+    assert rel_err(to_host(y), ref) <= 1e-13
+    dt = 0.2 / max(1.0, np.linalg.norm(ref))
+    psi = to_dev(x)
+    qs.evolve(psi, dt, 3)
+    assert rel_err(to_host(psi), orc.rk4(os_, w, L, x, dt, 3)) <= 1e-11
+    for steps in (33, 70):
+        runs = [to_dev(x) for _ in range(3)]
+        qs.evolve(runs[0], dt, steps)
+        qs.set_resident_max(0)
+        qs.evolve(runs[1], dt, steps)
+        qs.evolve_plain(runs[2], dt, steps)
+        qs.set_resident_max(1024)
+        assert bool((runs[0] == runs[1]).all()) and bool((runs[0] == runs[2]).all())
+
+
+@pytest.mark.parametrize("B", [2, 4, 8])
+@pytest.mark.parametrize("M,hi,kind", [(4, 9, "long"), (5, 10, "contact"), (6, 9, "long"), (7, 6, "long"), (7, 10, "long"),
+                                       (8, 7, "contact"), (9, 6, "long"), (10, 6, "long"), (11, 5, "long"), (12, 4, "long"),
+                                       (13, 4, "contact")])
+def test_members_of_a_sweep_equal_single_runs(M, hi, kind, B):
+    """The number of members decides whether all lanes take every record or each its own ket's: the
+    states of the members one by one, bit for bit."""
+    import torch
+
+    qs = _space(M, hi, kind=kind)
+    x = [to_dev(random_state(qs.total, b)) for b in range(B)]
+    scale = [0.3 * (b + 1) * (-1) ** b for b in range(B)]
+    psi = torch.stack(x)
+    qs.evolve_batch(psi, scale, 1e-3, 5)
+    for b in range(B):
+        qs.evolve_batch(x[b], [scale[b]], 1e-3, 5)
+        assert bool((psi[b] == x[b]).all()), b
