@@ -17,6 +17,12 @@
 
 namespace qb {
 
+// Share of the records (Tables::bk_share) up to which each lane walks its own ket's.  All records in
+// step / own (us): M = 16, 969 kets (0.02) 216 / 57; M = 14, 116,280 (0.1) 711 / 255; M = 11, 167,960
+// (0.19) 588 / 306; M = 8, 43,758 (0.29) 118 / 107; M = 6, 5,005 (0.34) 44 / 48; M = 7, 50,388 (0.39)
+// 93 / 83, M = 6, 38,760 (0.48) 52 / 56.
+constexpr float kHpsiShare = 0.3f;
+
 struct HpsiArgs {
   const double2* psi;
   double2* out;
@@ -47,7 +53,9 @@ __device__ __forceinline__ double row_diag(const Tables& t, const uint32_t (&ob)
   return d + dl;
 }
 
-template <int KC, bool CPLX>
+// SPARSE: each lane walks the records of its own ket (qb_block.cuh, sparse_stage_kernel), with the
+// same sums.
+template <int KC, bool CPLX, bool SPARSE>
 __global__ void __launch_bounds__(512, 2) hpsi_direct_kernel(const Tables t, const HpsiArgs a) {
   constexpr int NT = Rec<KC>::n, RW = Rec<KC>::w;
   const int T = t.bk_T, nrec = t.bk_nrec, M = t.M;
@@ -68,6 +76,8 @@ __global__ void __launch_bounds__(512, 2) hpsi_direct_kernel(const Tables t, con
   }
   for (int i = threadIdx.x; i < nrec; i += blockDim.x) sinfo[i] = __ldg(t.bk_info + i);
   __syncthreads();
+  uint16_t* first = reinterpret_cast<uint16_t*>(spq + T);
+  if (SPARSE) first_records(sinfo, nrec, first);
   const int64_t total = t.total, step = (int64_t)gridDim.x * warps;
   int64_t rd = (total - 1) / 32 - ((int64_t)blockIdx.x * warps + warp);
   for (; rd >= 0; rd -= step) {
@@ -83,26 +93,32 @@ __global__ void __launch_bounds__(512, 2) hpsi_direct_kernel(const Tables t, con
     bool bad = false;
     MapRec<KC> mcur;
     BaseRec<KC> bcur;
-    if (nrec > 0) {
-      mcur = load_map<KC>(mp, mp5);
-      bcur = load_base<KC>(base, 0, nrec);
-    }
-    for (int rec = 0; rec < nrec; ++rec) {
-      const int nx = min(rec + 1, nrec - 1);
-      const MapRec<KC> mnext = load_map<KC>(mp + (size_t)nx * t.bk_S * (2 * RW), mp5 + (size_t)nx * t.bk_S);
-      const BaseRec<KC> bnext = load_base<KC>(base, nx, nrec);
+    RecordWalk walk(t, SPARSE && valid ? in.word : 0ull);
+    auto load = [&](int rec) {
+      mcur = load_map<KC>(mp + (size_t)rec * t.bk_S * (2 * RW), mp5 + (size_t)rec * t.bk_S);
+      bcur = load_base<KC>(base, rec, nrec);
+    };
+    bool on = SPARSE ? walk.next(sinfo, first) : nrec > 0;
+    if (on) load(SPARSE ? walk.rec : 0);
+    // (a lane without a further record of its own waits at the loop's end)
+    for (int at = 0; SPARSE ? on : at < nrec; ++at) {
+      const int rec = SPARSE ? walk.rec : at;
+      const MapRec<KC> mnow = mcur;
+      const BaseRec<KC> bnow = bcur;
+      if (SPARSE) on = walk.next(sinfo, first);
+      if (!SPARSE || on) load(SPARSE ? walk.rec : min(at + 1, nrec - 1));
       const uint2 info = sinfo[rec];
       const int r = (int)((info.x & 7) | ((info.x >> 12) & 8)), s = (int)(((info.x >> 16) & 7) | ((info.x >> 28) & 8));
       const int nr = occ_int<4>(ob, r), ns = occ_int<4>(ob, s) - (r == s ? 1 : 0);
       const bool act = nr >= 1 && ns >= 1;
-      if (__any_sync(0xffffffffu, act)) {
+      if (SPARSE ? act : (bool)__any_sync(0xffffffffu, act)) {
         const int n = KC == 0 ? (int)((info.x >> 4) & 7) : NT;
         uint32_t rk[NT];
-        rk[0] = bcur.a.x + (mcur.a.x & 0xffffu);
-        rk[1] = bcur.a.y + (mcur.a.x >> 16);
-        if constexpr (NT > 2) rk[2] = bcur.a.z + (mcur.a.y & 0xffffu);
-        if constexpr (NT > 3) rk[3] = bcur.a.w + (mcur.a.y >> 16);
-        if constexpr (NT > 4) rk[4] = bcur.b + mcur.b;
+        rk[0] = bnow.a.x + (mnow.a.x & 0xffffu);
+        rk[1] = bnow.a.y + (mnow.a.x >> 16);
+        if constexpr (NT > 2) rk[2] = bnow.a.z + (mnow.a.y & 0xffffu);
+        if constexpr (NT > 3) rk[3] = bnow.a.w + (mnow.a.y >> 16);
+        if constexpr (NT > 4) rk[4] = bnow.b + mnow.b;
         uint32_t top = rk[0];
 #pragma unroll
         for (int c = 1; c < NT; ++c)
@@ -139,9 +155,8 @@ __global__ void __launch_bounds__(512, 2) hpsi_direct_kernel(const Tables t, con
           }
         }
       }
-      mcur = mnext;
-      bcur = bnext;
     }
+    __syncwarp();
     if (bad) atomicOr(a.status, 1);
     if (valid) {
       const double dg = row_diag<true>(t, ob, sw, sgd);
@@ -307,7 +322,8 @@ static int hpsi_run(K k, const Tables& t, const HpsiArgs& a, int64_t rows, int m
 template <int KC, bool CPLX>
 static int hpsi_direct(const Tables& t, const HpsiArgs& a, cudaStream_t st) {
   const size_t smem = (((size_t)(t.nmax + 3 + t.M + t.n_ann) * 8 + 15) & ~(size_t)15) + (size_t)t.bk_T * 20 + (size_t)t.bk_nrec * 8;
-  return hpsi_run(hpsi_direct_kernel<KC, CPLX>, t, a, t.total, 16, smem, st);
+  if (t.bk_share < kHpsiShare) return hpsi_run(hpsi_direct_kernel<KC, CPLX, true>, t, a, t.total, 16, smem + kFirstBytes, st);
+  return hpsi_run(hpsi_direct_kernel<KC, CPLX, false>, t, a, t.total, 16, smem, st);
 }
 
 int launch_hpsi(Space& s, const void* d_v, void* d_out, void* stream) {
