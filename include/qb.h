@@ -167,7 +167,8 @@ int qb_init_field_number(qb_space* space, const double* z, int n_tot, void* d_ps
 /* Bytes of device workspace qb_evolve / qb_evolve_batch need for `batch`
  * state vectors: 48 per ket and member, plus, for a coupling that is one real number
  * per momentum class (a contact interaction), 16 for every entry of the annihilated
- * vectors (at most M per ket, for one member). */
+ * vectors: one per momentum class and ket of two particles fewer, at most M per ket (exact
+ * momentum: 2 M - 1); for every member where that is 256 MB in all, else for one. */
 int64_t qb_workspace_bytes(const qb_space* space, int batch);
 
 /* out = H psi for one state vector (d_out and d_psi distinct, device).  For a coupling that
@@ -183,7 +184,8 @@ int qb_evolve(qb_space* space, void* d_psi, double dt, int64_t steps, void* d_wo
 
 /* Batched sweep: `batch` state vectors d_psi[batch][total], member b evolving
  * under H_b = H_w + scale[b] * H_L (one-body part unchanged, two-body part
- * scaled).  All sectors of all members advance in one launch per RK4 stage.
+ * scaled).  All sectors of all members advance in one launch per RK4 stage; with a contact
+ * coupling (see qb_workspace_bytes) in two, or, of large spaces, two for each member.
  * scale: host [batch].  d_work: qb_workspace_bytes(space, batch) bytes. */
 int qb_evolve_batch(qb_space* space, void* d_psi, int batch, const double* scale, double dt, int64_t steps,
                     void* d_work, void* stream);

@@ -69,12 +69,12 @@ __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.launch_dependents;");
 }
 template <typename... P, typename... A>
-inline cudaError_t chain_launch(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t st, A... args) {
+inline cudaError_t chain_launch(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t c{};
-  c.gridDim = dim3((unsigned)grid);
+  c.gridDim = grid;
   c.blockDim = dim3((unsigned)block);
   c.dynamicSmemBytes = smem;
   c.stream = st;
@@ -198,11 +198,12 @@ __device__ __forceinline__ void add_record(dfc& acc, const float4 (&x)[Rec<KC>::
 // Everything of a ket's row that the epilogue needs, and the epilogue: forms the
 // stage's output (or the bilinears, or the <x|H|x> summand) from the off-diagonal sum.
 // WHOLE: acc is the whole two-body part (factored couplings), else its off-diagonal part.
-// RESIDENT: the state's vectors lie in shared memory.
+// RESIDENT: the state's vectors lie in shared memory.  gr: the ket; ri: its entry of the vectors;
+// member: of the sweep, the first of B.
 template <int MT, int B, int KIND, bool WHOLE, int NW, bool RESIDENT = false>
 __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a, int mode, int64_t gr, int64_t ri,
                                                const dfc (&acc)[B], const uint32_t (&ob)[NW], dfl& bil_l, dfc* bil_w,
-                                               double& dot64) {
+                                               double& dot64, int member = 0) {
   constexpr bool BIL = (KIND == KIND_BIL), DOT = (KIND == KIND_DOT);
   constexpr int kMB = (MT > 0) ? MT : 16;
   const int M = (MT > 0) ? MT : t.M;
@@ -221,7 +222,7 @@ __device__ __forceinline__ void stage_epilogue(const Tables& t, const DfArgs& a,
       acc_r = dfl{2.f * acc_r.h, 2.f * acc_r.l};
       acc_i = dfl{2.f * acc_i.h, 2.f * acc_i.l};
     }
-    const dfl sc{a.scale[b].x, a.scale[b].y};
+    const dfl sc{a.scale[b + member].x, a.scale[b + member].y};
     const dfl dg = WHOLE ? dfl{dg4.x, dg4.y} : df_add(dfl{dg4.x, dg4.y}, df_mul(sc, dfl{dg4.z, dg4.w}));
     const float4 xo = a.vin[(size_t)b * total + ri];
     const dfl hr = df_add(df_mul(dg, df_re(xo)), df_mul(sc, acc_r));

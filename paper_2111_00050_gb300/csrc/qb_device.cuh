@@ -473,7 +473,8 @@ struct DfArgs {
   const float4* diag;  // per ket (w.hi, w.lo, L.hi, L.lo)
   float2 scale[8];     // two-body scale per member, double-float
   int64_t row0, row1;  // kets [row0, row1) of the launch (every sector: 0, total)
-  float4* g;           // factored couplings: B_k of the gathered vector(s), [B][fa_nG]
+  float4* g;           // factored couplings: B_k of the gathered vector(s), [g_members][fa_nG]
+  int g_members;       // members of a sweep with a vector each; else they take one in turn
   int64_t low0, low1;  // and the lower kets [low0, low1) that the launch fills (every one: 0, fa_low)
   double zre;          // z = -i zre
   float2 zf;           // zre as double-float

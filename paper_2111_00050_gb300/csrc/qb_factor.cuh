@@ -29,7 +29,8 @@ inline size_t ann_smem_bytes(const Tables& t) { return ((size_t)t.fa_nrec * 8 + 
 // rest squared in FP64: the weight rounded to 48 bits erred alike in the many kets that share it
 // (positive states of 245,157 kets, M = 7, against 64 bits 1.1e-15, now 4e-16, the direct form 7e-16).
 // EVERY: every record of every lower ket is taken (all momenta held).
-template <int NT, bool DOT, bool EVERY>
+// SIDE: member blockIdx.y of a sweep, with a vector of its own (here and below).
+template <int NT, bool DOT, bool EVERY, bool SIDE>
 __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfArgs a) {
   constexpr int PL = NT > 4 ? 2 : 1;       // groups of four pairs a record
   constexpr int NS = NT > 0 ? NT : 4;      // pairs of a record
@@ -41,6 +42,8 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
   for (int i = threadIdx.x; i < nc; i += blockDim.x) slam[i] = __ldg(t.fa_lam + i);
   __syncthreads();
   const int64_t total = t.total;
+  const float4* vin = a.vin + (SIDE ? (size_t)blockIdx.y * total : 0);
+  float4* g_out = a.g + (SIDE ? (size_t)blockIdx.y * t.fa_nG : 0);
   double dot64 = 0.0;
 
   // Rounds of a layer are taken in an order that walks its sectors side by side (fa_perm):
@@ -123,7 +126,7 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
         bad |= act && !ok;
 #pragma unroll
         for (int c = 0; c < NS; ++c)
-          if (ok && (NT > 0 || c < n)) x[c] = a.vin[ix[c]];
+          if (ok && (NT > 0 || c < n)) x[c] = vin[ix[c]];
         if constexpr (NT > 0) {
           acc = dfc{f2_pack(x[0].x, x[0].y), f2_pack(x[0].z, x[0].w)};
         } else {
@@ -151,7 +154,7 @@ __global__ void __launch_bounds__(1024, 1) ann_kernel(const Tables t, const DfAr
           } else {
             gr = df_renorm(df_mul(dfl{lm.x, lm.y}, gr));
             gi = df_renorm(df_mul(dfl{lm.x, lm.y}, gi));
-            if (ok) a.g[__ldg(gb + k) + (uint32_t)g] = df_pack(gr, gi);
+            if (ok) g_out[__ldg(gb + k) + (uint32_t)g] = df_pack(gr, gi);
           }
           acc = dfc{0ull, 0ull};
         }
@@ -189,7 +192,7 @@ struct PairList {
 
 inline size_t cre_smem_bytes(const Tables& t) { return (size_t)fa_Tc(t) * 12; }
 
-template <int MT, int KIND>
+template <int MT, int KIND, bool SIDE>
 __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
     cre_kernel(const Tables t, const DfArgs a, const int mode) {
   constexpr int NW = occ_words<MT>();
@@ -204,6 +207,7 @@ __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
   for (int i = threadIdx.x; i < 2 * ng; i += blockDim.x) scoef[i] = __ldg(t.fa_coef + i);
   __syncthreads();
   const uint32_t nG = (uint32_t)t.fa_nG;
+  const float4* g_in = a.g + (SIDE ? (size_t)blockIdx.y * nG : 0);
   dfl bil_l{0.f, 0.f};
   dfc bil_w[BIL ? (kMB + 1) / 2 : 1];
 #pragma unroll
@@ -254,7 +258,7 @@ __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
             A[c] = i < NO ? nf[pr.r[i]] * nf[pr.s[i]] : nf[pr.r[i]] * (nf[pr.r[i]] - 1.f);  // exact
             const bool act = A[c] != 0.f, ok = act && ix[c] < nG;
             bad |= act && !ok;
-            if (ok) x[c] = a.g[ix[c]];
+            if (ok) x[c] = g_in[ix[c]];
           }
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
@@ -293,7 +297,7 @@ __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
                    (occ_float23<NW>(ob, sel[c] >> 16, (sel[c] & 0x80000000u) != 0u) - del[c]);  // exact
             const bool act = A[c] != 0.f, ok = act && ix[c] < nG;
             bad |= act && !ok;
-            if (ok) x[c] = a.g[ix[c]];
+            if (ok) x[c] = g_in[ix[c]];
           }
 #pragma unroll
           for (int c = 0; c < 4; ++c)
@@ -306,58 +310,66 @@ __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
         }
       }
       if (bad) atomicOr(a.status, 1);
-      if (valid) stage_epilogue<MT, 1, KIND, true, NW>(t, a, mode, g, g, acc, ob, bil_l, bil_w, dot64);
+      if (valid)
+        stage_epilogue<MT, 1, KIND, true, NW>(t, a, mode, g, SIDE ? g + (int64_t)blockIdx.y * t.total : g, acc, ob, bil_l,
+                                              bil_w, dot64, SIDE ? (int)blockIdx.y : 0);
   }
   if constexpr (BIL) bil_reduce<kMB>(a, M, bil_l, bil_w);
 }
 
-template <int NT, bool DOT>
-int ann_launch(const Tables& t, const DfArgs& a, int shape, cudaStream_t st, int* grid_out) {
-  auto k = t.fa_every ? ann_kernel<NT, DOT, true> : ann_kernel<NT, DOT, false>;
+template <int NT, bool DOT, bool SIDE>
+int ann_launch(const Tables& t, const DfArgs& a, int members, int shape, cudaStream_t st, int* grid_out) {
+  auto k = t.fa_every ? ann_kernel<NT, DOT, true, SIDE> : ann_kernel<NT, DOT, false, SIDE>;
   const size_t smem = ann_smem_bytes(t);
   int grid = 0, warps = 0;
   const int rc = stage_geometry(k, a.low1 - a.low0, shape, 32, smem, &warps, &grid);
   if (rc) return rc;
-  QB_CUDA(chain_launch(k, grid, 32 * warps, smem, st, t, a));
+  QB_CUDA(chain_launch(k, dim3((unsigned)grid, (unsigned)members), 32 * warps, smem, st, t, a));
   if (grid_out) *grid_out = grid;
   return QB_OK;
 }
 
-template <int MT, int KIND>
-int cre_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream_t st, int* grid_out) {
-  auto k = cre_kernel<MT, KIND>;
+template <int MT, int KIND, bool SIDE>
+int cre_launch(const Tables& t, const DfArgs& a, int mode, int members, int shape, cudaStream_t st, int* grid_out) {
+  auto k = cre_kernel<MT, KIND, SIDE>;
   const size_t smem = cre_smem_bytes(t);
   int grid = 0, warps = 0;
   const int rc = stage_geometry(k, a.row1 - a.row0, shape, blk_max_threads<1, KIND>() / 32, smem, &warps, &grid);
   if (rc) return rc;
-  QB_CUDA(chain_launch(k, grid, 32 * warps, smem, st, t, a, mode));
+  QB_CUDA(chain_launch(k, dim3((unsigned)grid, (unsigned)members), 32 * warps, smem, st, t, a, mode));
   if (grid_out) *grid_out = grid;
   return QB_OK;
 }
 
 // One stage of a factored space: NT pairs a class (0: any), MT modes (0: any).  The members
-// of a sweep take their two passes one after the other, through one vector g.
+// of a sweep take a pass in one launch with a vector g each (side_by_side), or their two passes
+// one after the other through one.
 template <int MT, int NT>
 int fac_launch(const Tables& t, const DfArgs& a0, int mode, int B, bool bil, int shape, cudaStream_t st, int* grid) {
   if (mode < 0 || mode > 4) return fail(QB_EINTERNAL, "bad stage mode");
   if (mode == 4) {
     if (B != 1) return fail(QB_EUNSUPPORTED, "the <x|H|x> reduction runs one state at a time");
-    return ann_launch<NT, true>(t, a0, shape, st, grid);
+    return ann_launch<NT, true, false>(t, a0, 1, shape, st, grid);
   }
   if (bil && B != 1) return fail(QB_EUNSUPPORTED, "bilinear stages run one state at a time");
   if (B != 1 && t.exact) return fail(QB_EUNSUPPORTED, "exact momentum: batched sweeps are not built");
   if (B != 1 && B != 2 && B != 4 && B != 8) return fail(QB_EINVAL, "batch must be 1, 2, 4 or 8");
-  for (int b = 0; b < B; ++b) {
+  const int members = B > 1 && a0.g_members >= B ? B : 1;
+  for (int b = 0; b < B; b += members) {
     DfArgs a = a0;
     a.vin += (size_t)b * t.total;
     if (a.psif) a.psif += (size_t)b * t.total;
     if (a.psi) a.psi += (size_t)b * t.total;
     a.out += (size_t)b * t.total;
-    a.scale[0] = a0.scale[b];
+    if (b > 0) a.scale[0] = a0.scale[b];
     int rc = QB_OK;
-    if (a.low1 > a.low0) rc = ann_launch<NT, false>(t, a, shape, st, nullptr);
+    if (a.low1 > a.low0)
+      rc = members > 1 ? ann_launch<NT, false, true>(t, a, members, shape, st, nullptr)
+                       : ann_launch<NT, false, false>(t, a, 1, shape, st, nullptr);
     if (rc) return rc;
-    rc = bil ? cre_launch<MT, KIND_BIL>(t, a, mode, shape, st, grid) : cre_launch<MT, KIND_STAGE>(t, a, mode, shape, st, grid);
+    rc = bil           ? cre_launch<MT, KIND_BIL, false>(t, a, mode, 1, shape, st, grid)
+         : members > 1 ? cre_launch<MT, KIND_STAGE, true>(t, a, mode, members, shape, st, grid)
+                       : cre_launch<MT, KIND_STAGE, false>(t, a, mode, 1, shape, st, grid);
     if (rc) return rc;
   }
   return QB_OK;

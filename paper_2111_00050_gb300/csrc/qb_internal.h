@@ -275,6 +275,7 @@ std::vector<int> tb_columns(const Space& s, const std::vector<int>& ops);
 int launch_tb_blocks(const Space& s, const float4* bra, const float4* ket, const int* cols, int n_ops, double weight,
                      double* acc, cudaStream_t st);
 int64_t workspace_bytes(const Space& s, int batch);
+int side_by_side(const Space& s, int batch);  // members of a sweep with a vector of B_k f each
 // psi [B][total] -> double-float copy in the weighted basis f = psi / w(n) (the stages' basis)
 int launch_to_dfw(const Space& s, const void* psi, void* psif, int B, void* stream);
 // observables of Sec. II C-E from the raw moments (host)

@@ -1244,10 +1244,20 @@ int device_setup(Space& s) {
   return QB_OK;
 }
 
+// Members of a sweep whose vectors of B_k f lie side by side, so that each of the two passes is
+// one launch for all of them: all, where that takes 256 MB at most.  A pass over so few kets is
+// one or two waves of the SMs, and eight in turn pay for that and for the launch eight times (one
+// stage of eight members, us: M = 16, 20,349 kets 312, side by side 86; M = 7, 50,388 104 / 36; M = 11,
+// 167,960 361 / 186, M = 7, 245,157 202 / 175; M = 9, 817,190, beyond the line, 691 / 686).
+constexpr int64_t kSideEntries = 16ll << 20;
+int side_by_side(const Space& s, int batch) {
+  return batch * s.t.fa_nG <= kSideEntries ? batch : 1;
+}
+
 // workspace: two double-float stage vectors and the double-float copy of psi,
-// each [batch][total] x 16 bytes, and for factored couplings the vector of B_k f
+// each [batch][total] x 16 bytes, and for factored couplings the vectors of B_k f
 int64_t workspace_bytes(const Space& s, int batch) {
-  return 16 * (3 * (int64_t)batch * s.secOff.back() + (s.t.fa_on ? s.t.fa_nG : 0));
+  return 16 * (3 * (int64_t)batch * s.secOff.back() + (s.t.fa_on ? side_by_side(s, batch) * s.t.fa_nG : 0));
 }
 
 template <int MODE, int B, bool CPLX>
@@ -1367,6 +1377,7 @@ static int rk4_loop(Space& s, double2* psi, const double* scale, double dt, int6
   a.psi = psi;
   a.psif = psif;
   a.g = psif + (size_t)B * s.t.total;
+  a.g_members = side_by_side(s, B);
   a.status = reinterpret_cast<int*>(s.d_scratch);
   a.nbasef = 0;
   if (plain) return rk4_issue<B>(s, a, dt, steps, w1, w2, psif, st, true);
