@@ -190,7 +190,7 @@ struct PairList {
   }
 };
 
-inline size_t cre_smem_bytes(const Tables& t) { return (size_t)fa_Tc(t) * 12; }
+inline size_t cre_smem_bytes(const Tables& t, int MT) { return MT > 0 ? 0 : (size_t)fa_Tc(t) * 12; }
 
 template <int MT, int KIND, bool SIDE>
 __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
@@ -203,9 +203,11 @@ __global__ void __launch_bounds__((blk_max_threads<1, KIND>()), 1)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   uint4* sinfo = reinterpret_cast<uint4*>(blk_smem);
   float4* scoef = reinterpret_cast<float4*>(sinfo + ng);
-  for (int i = threadIdx.x; i < ng; i += blockDim.x) sinfo[i] = __ldg(t.fa_info + i);
-  for (int i = threadIdx.x; i < 2 * ng; i += blockDim.x) scoef[i] = __ldg(t.fa_coef + i);
-  __syncthreads();
+  if constexpr (MT == 0) {  // else the pairs are constants
+    for (int i = threadIdx.x; i < ng; i += blockDim.x) sinfo[i] = __ldg(t.fa_info + i);
+    for (int i = threadIdx.x; i < 2 * ng; i += blockDim.x) scoef[i] = __ldg(t.fa_coef + i);
+    __syncthreads();
+  }
   const uint32_t nG = (uint32_t)t.fa_nG;
   const float4* g_in = a.g + (SIDE ? (size_t)blockIdx.y * nG : 0);
   dfl bil_l{0.f, 0.f};
@@ -332,7 +334,7 @@ int ann_launch(const Tables& t, const DfArgs& a, int members, int shape, cudaStr
 template <int MT, int KIND, bool SIDE>
 int cre_launch(const Tables& t, const DfArgs& a, int mode, int members, int shape, cudaStream_t st, int* grid_out) {
   auto k = cre_kernel<MT, KIND, SIDE>;
-  const size_t smem = cre_smem_bytes(t);
+  const size_t smem = cre_smem_bytes(t, MT);
   int grid = 0, warps = 0;
   const int rc = stage_geometry(k, a.row1 - a.row0, shape, blk_max_threads<1, KIND>() / 32, smem, &warps, &grid);
   if (rc) return rc;

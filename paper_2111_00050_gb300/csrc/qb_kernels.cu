@@ -26,14 +26,12 @@ namespace qb {
 
 // ------------------------------------------------------------ H psi kernels
 
-enum { MODE_HPSI = 0, MODE_STAGE = 1, MODE_DOT = 2 };
+enum { MODE_HPSI = 0, MODE_DOT = 1 };
 
 struct StageArgs {
   const double2* vin;  // gathered vector(s) [B][total]
-  const double2* psi;  // psi(s) [B][total] (stage mode)
   double2* out;        // output(s) [B][total]
   double scale[8];     // two-body scale per member
-  double zre;          // stage factor  -i dt / d  = (0, -dt/d): out = psi + (dt/d) * (Im Hv, -Re Hv)
   double* partial;     // MODE_DOT: [gridDim.x][2]
   int* status;         // device status word (bounds violations)
 };
@@ -139,10 +137,6 @@ __global__ void __launch_bounds__(kBlock) hpsi_kernel(const Tables t, const Stag
       const double hi = dg * x.y + sc * acc_im[b];
       if (MODE == MODE_HPSI) {
         a.out[(size_t)b * total + g] = make_double2(hr, hi);
-      } else if (MODE == MODE_STAGE) {
-        const double2 p0 = a.psi[(size_t)b * total + g];
-        // psi + (-i dt/d) * Hv,  zre = dt/d
-        a.out[(size_t)b * total + g] = make_double2(p0.x + a.zre * hi, p0.y - a.zre * hr);
       } else {
         // <x | Hx> contribution: conj(x) * Hx
         dot_re += x.x * hr + x.y * hi;
