@@ -45,22 +45,6 @@ STAGE_NCU_ISSUE_ACTIVE = 0.614
 STAGE_NCU_L1_WAVEFRONTS = 0.454
 
 
-def _factored(W, qs):
-    """Whether the stages of this space run in two passes (contact couplings: one real number per
-    momentum class, spaces of enough kets)."""
-    if W.M < 6 or qs.total < (16384 if W.M >= 9 else 32768):
-        return False
-    L = np.asarray(W.L)
-    L = 0.25 * (L + L.transpose(1, 0, 2, 3) + L.transpose(0, 1, 3, 2) + L.transpose(1, 0, 3, 2))
-    pairs = [(p, q) for p in range(W.M) for q in range(p, W.M)]
-    for k in range(W.M):
-        cls = [a for a in pairs if sum(a) % W.M == k]
-        vals = {complex(L[a + b]) for a in cls for b in cls}
-        if len(vals) > 1 or any(v.imag for v in vals):
-            return False
-    return True
-
-
 def _peaks():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -583,7 +567,7 @@ def main():
 
     # ---- dominant kernels: one fused RK4 stage == one H psi over all sectors; a step is
     # four of them, timed above with CUDA events on the launching stream
-    factored = _factored(W, qs)
+    factored = int(qb.lib().qb_workspace_bytes(qs._h, 1)) > 48 * qs.total  # annihilated vectors: two passes a stage
     stage_time = ms_step * 1e-3 / 4
     flops = 4.0 * terms  # >= 2 FP64 FMA per term (real coefficient x complex amplitude)
     achieved = flops / stage_time / 1e12
@@ -609,7 +593,7 @@ def main():
         "frac": achieved / dfma_tflops, "peak_kind": "measured DFMA rate of this GPU (qb_measure_fp64_fma)",
         "peak_unit_count": FP64_PEAK_TFLOPS, "frac_of_unit_count": achieved / FP64_PEAK_TFLOPS,
         "traffic": STAGE_DRAM_BYTES_PER_KET * qs.total if args.config == "batched_coherent" else None,
-        "kernel": (f"ann_kernel + cre_kernel<{W.M},0>" if factored else f"blk_stage_kernel<{W.M}>") +
+        "kernel": (f"ann_kernel + cre_kernel<{W.M}>" if factored else f"blk_stage_kernel<{W.M}>") +
                   " (one RK4 stage = one H psi over all sectors, weighted basis)",
         "stage_ms": stage_time * 1e3,
         "peak_note": "FP64-equivalent flops (2 FMA/term) vs the FP64 FMA rate measured on this GPU; the "
