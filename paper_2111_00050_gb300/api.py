@@ -221,7 +221,7 @@ class Space:
         sector runs through the stage kernel), then the resident threshold among
         `candidates`.  Keeps the fastest of each and returns the threshold; the chosen
         shape is in self.tile_shape and both, with every timing, in self.tuning."""
-        work = self.workspace(1) if work is None else work
+        work = self._work(work, 1, steps)
         trial = psi.clone()
         shapes = range(_lib.QB_TILE_SHAPES) if shapes is None else shapes
         self.set_resident_max(0)

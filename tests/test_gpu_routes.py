@@ -157,6 +157,8 @@ def test_a_workspace_that_is_too_small_is_refused(kind):
                 assert bool((y == x).all()), name
     qs.evolve(x, 1e-3, 0, work[1:])  # no steps take no workspace
     with pytest.raises(ValueError):
+        qs.autotune(1e-3, x, steps=1, work=work[1:])
+    with pytest.raises(ValueError):
         qs.evolve_batch(torch.stack([x, x]), [1.0, 2.0], 1e-3, 2, work)
 
 
