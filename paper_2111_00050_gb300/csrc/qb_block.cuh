@@ -791,17 +791,21 @@ constexpr float sparse_share() {
 template <int MT, bool FIX, int B, bool CPLX, int KIND>
 int blk_launch(const Tables& t, const DfArgs& a, int mode, int shape, cudaStream_t st, int* grid_out) {
   constexpr int KC = FIX ? (MT - 1) / 2 : 0;
-  if constexpr (KIND != KIND_DOT && sparse_share<KC, B, KIND>() > 0.f)
-    if (t.bk_share < sparse_share<KC, B, KIND>())
-      return sparse_launch<KC, B, CPLX, KIND>(t, a, mode, shape, st, grid_out);
-  if constexpr (FIX && B == 1 && KIND == KIND_STAGE) {
-    int dev = 0, sms = 0;
-    QB_CUDA(cudaGetDevice(&dev));
-    QB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if ((a.row1 - a.row0) / 32 <= (int64_t)sms * kFewWarps)
-      return blk_launch_u<MT, FIX, B, CPLX, KIND, 4>(t, a, mode, shape, st, grid_out);
+  constexpr float line = KIND == KIND_DOT ? 0.f : sparse_share<KC, B, KIND>();
+  if constexpr (line > 1.f) {
+    return sparse_launch<KC, B, CPLX, KIND>(t, a, mode, shape, st, grid_out);
+  } else {
+    if constexpr (line > 0.f)
+      if (t.bk_share < line) return sparse_launch<KC, B, CPLX, KIND>(t, a, mode, shape, st, grid_out);
+    if constexpr (FIX && B == 1 && KIND == KIND_STAGE) {
+      int dev = 0, sms = 0;
+      QB_CUDA(cudaGetDevice(&dev));
+      QB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+      if ((a.row1 - a.row0) / 32 <= (int64_t)sms * kFewWarps)
+        return blk_launch_u<MT, FIX, B, CPLX, KIND, 4>(t, a, mode, shape, st, grid_out);
+    }
+    return blk_launch_u<MT, FIX, B, CPLX, KIND, 1>(t, a, mode, shape, st, grid_out);
   }
-  return blk_launch_u<MT, FIX, B, CPLX, KIND, 1>(t, a, mode, shape, st, grid_out);
 }
 
 // the kinds and batch sizes of one kernel family (real or complex couplings)
