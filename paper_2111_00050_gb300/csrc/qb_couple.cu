@@ -5,15 +5,16 @@
 //   <bra, a_p^dag a_q^dag a_r a_s ket> = sum_n conj(b_t) k f_n w_n^2,  k = n_r (n_s - [r = s]),
 // t the ket n with r, s taken away and p, q added: the target that the direct stage kernel
 // ranks for the same term.  f_n w_n^2 is formed by two products (w_n^2 alone may leave the fp32
-// range), the weight with a third part (dft_mul).  A task is one to four records (pairs (r, s) with their partners), up to eight
-// sums, over a share of the kets; the sums of a lane over up to 32 kets are double-float, those of
-// the lanes of three floats (tfc_add, more bits than FP64), those of the warps' flushes, the
-// warps and the CTAs FP64, in a fixed order.
+// range), the weight with a third part (dft_mul).  A task is one to four records (pairs (r, s)
+// with their partners), up to eight sums, over a share of the kets; the sums of a lane over up to
+// 32 kets are double-float, those of the lanes of three floats (tfc_add, more bits than FP64), those
+// of the warps' flushes, the warps and the CTAs FP64, in a fixed order.
 //
 // Bound by the issue of the 24 packed operations of a complex product and of what they take
-// (57% of the issue slots, 16 warps an SM).  The 45 operators of 435,897 kets at M = 5: 74 us;
-// the moments kernel, one entry a lane and every target ranked anew from the ranking table,
-// took 145 us, a form that gathered record by record 94.
+// (58% of the issue slots, 16 warps an SM).  The 45 operators of 435,897 kets at M = 5: 77 us
+// (lanes added in double-float and weights of 48 bits: 74); the moments kernel, one entry a lane and
+// every target ranked anew from the ranking table, took 145 us, a form that gathered record by
+// record 94.
 #include <cuda_runtime.h>
 
 #include <algorithm>
