@@ -154,8 +154,7 @@ static void build_block_tables(Space& sp, bool factored) {
       }
     return S;
   };
-  auto row_bytes = [&](int q) {  // bytes of the rows of bases
-    const std::vector<uint32_t> c = block_counts(sp, q);
+  auto row_bytes = [&](const std::vector<uint32_t>& c) {  // of bases, from the counts of blocks
     int64_t rows = 0, low = 0;
     for (size_t i = 0; i < sp.secN.size(); ++i) rows += c[CI(0, sp.secN[i], sp.secK[i])];
     if (!factored) return 4ll * t.bk_T * rows;
@@ -171,24 +170,30 @@ static void build_block_tables(Space& sp, bool factored) {
     S = s;
   }
   const int64_t total = sp.secOff.back(), room = std::min(kBaseBytes * total, std::max(kBaseRoom, 16 * total));
-  for (int64_t rows = row_bytes(P); P > 0 && rows > room; --P) {
-    const int64_t s = fillings(P - 1), next = row_bytes(P - 1);
+  sp.blkCnt = block_counts(sp, P);
+  for (int64_t rows = row_bytes(sp.blkCnt); P > 0 && rows > room; --P) {
+    std::vector<uint32_t> counts = block_counts(sp, P - 1);
+    const int64_t s = fillings(P - 1), next = row_bytes(counts);
     if (s < 0 || s > 0x7fffffff || s * per_fill + next >= S * per_fill + rows) break;
+    sp.blkCnt.swap(counts);
     S = s;
     rows = next;
   }
   t.bk_S = (int)S;
   t.bk_P = P;
   // A ket takes part in the records of a pair (r, s) if it is a ket of two particles fewer with
-  // them added.
+  // them added: summed by the pairs' momentum classes.
   {
-    std::vector<int> of(annR.size(), 0);
+    std::vector<int> of(annR.size(), 0), in_class(std::min(Q, 2 * M - 1), 0);
     int most = 0;
-    for (const Record& R : recs) most = std::max(most, ++of[R.pair]);
+    for (const Record& R : recs) {
+      most = std::max(most, ++of[R.pair]);
+      ++in_class[(annR[R.pair] + annS[R.pair]) % Q];
+    }
     double taken = 0.0;
     for (size_t i = 0; i < sp.secN.size(); ++i)
-      for (size_t a = 0; a < annR.size() && sp.secN[i] >= 2; ++a)
-        taken += (double)of[a] * (double)sp.cnt[CI(0, sp.secN[i] - 2, modp((long long)sp.secK[i] - annR[a] - annS[a], Q))];
+      for (int k = 0; k < (int)in_class.size() && sp.secN[i] >= 2; ++k)
+        taken += (double)in_class[k] * (double)sp.cnt[CI(0, sp.secN[i] - 2, sp.secK[i] - k + (sp.secK[i] < k ? Q : 0))];
     t.bk_share = nrec > 0 ? (float)(taken / ((double)nrec * (double)sp.secOff.back())) : 1.f;
     // (p modes occupied, of which nmax / 2 twice at most)
     const int64_t p = std::min(M, nmax);
@@ -254,7 +259,6 @@ static void build_block_tables(Space& sp, bool factored) {
 static void count_blocks(Space& sp) {
   const int V = sp.nmax + 1, Q = sp.Q;
   auto CI = [&](int m, int n, int k) { return ((size_t)m * V + n) * Q + k; };
-  sp.blkCnt = block_counts(sp, sp.t.bk_P);
   auto run = [&](const std::vector<int>& N, const std::vector<int>& K, std::vector<uint32_t>& out) {
     out.assign(1, 0);
     for (size_t i = 0; i < N.size(); ++i) out.push_back(out.back() + sp.blkCnt[CI(0, N[i], K[i])]);
